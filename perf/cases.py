@@ -152,6 +152,11 @@ def solenoidal(seed):
     return g.curl_modes(k, a, ph, 0.1 / np.linalg.norm(v, axis=1).max())
 
 
+def padded(params):
+    """The parameters as one flat array: every one starts at a multiple of four (gnn_layout)."""
+    return torch.cat([torch.nn.functional.pad(w.reshape(-1), (0, -w.numel() % 4)) for w in params])
+
+
 def weights(case, seed):
     """The network's parameters, in the order of gnn_layout: We, be, (Ws, Wm, b) per layer, Wd, bd."""
     C = (case["pt"] + 1) * len(multi_indices(case["p"]))
@@ -213,7 +218,7 @@ def prepare(case, seed):
         state["ups"] = torch.empty_like(state["vbar"])
     elif kind.startswith("gnn"):
         s.gnn_init(hidden=HIDDEN, layers=LAYERS, bf16=case["bf16"], seed=0)
-        s.gnn_params(np.concatenate([w.reshape(-1).numpy() for w in weights(case, seed)]))
+        s.gnn_params(padded(weights(case, seed)).numpy())
         state["z"] = s.pressure_empty()
     return state
 
@@ -538,7 +543,7 @@ def exact_network(S, case, seed, data):
     for r, t in zip(data["R"].chunk(case["pairs"]), data["T"].chunk(case["pairs"])):
         loss = loss + (net(r) - t.reshape(S.ne, -1)).square().sum() / t.square().sum() / case["pairs"]
     grads = torch.autograd.grad(loss, params)
-    return {"loss": float(loss), "grad": torch.cat([d.reshape(-1) for d in grads]).cpu().numpy()}
+    return {"loss": float(loss), "grad": padded(grads).cpu().numpy()}
 
 
 def exact(case, seed):
