@@ -72,8 +72,9 @@ __global__ void __launch_bounds__(256) k_dense(int ne, int K, int O, const float
     }
 }
 
-// m_i = Sum_{f} h_{nbr(i,f)}  (symmetric adjacency: also the adjoint of itself)
-__global__ void k_gather(int ne, int H, const int* __restrict__ nbr4, const float* __restrict__ h, float* __restrict__ m) {
+// m_i = Sum_{f} h_{nbr(i,f)} (+ add_i)  (symmetric adjacency: also the adjoint of itself)
+__global__ void k_gather(int ne, int H, const int* __restrict__ nbr4, const float* __restrict__ h, float* __restrict__ m,
+                         const float* __restrict__ add = nullptr) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)ne * H; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = e / H;
     const int c = (int)(e % H);
@@ -82,7 +83,7 @@ __global__ void k_gather(int ne, int H, const int* __restrict__ nbr4, const floa
       const int n = nbr4[4 * i + f];
       if (n >= 0) s += h[(size_t)n * H + c];
     }
-    m[e] = s;
+    m[e] = add ? s + add[e] : s;
   }
 }
 
@@ -93,17 +94,22 @@ __global__ void k_relu_back(int64_t n, const float* __restrict__ pre, const floa
 }
 
 // Weight gradient partials: part[chunk][o][k] = Sum_{i in chunk} D[i][o] X[i][k]; bias partial
-// (k == K slot) = Sum_i D[i][o].  Fixed chunking -> deterministic after k_wgrad_reduce.
-constexpr int kChunk = 1024;
-__global__ void __launch_bounds__(256) k_wgrad(int ne, int O, int K, const float* __restrict__ D, const float* __restrict__ X,
-                                               float* __restrict__ part) {
+// (k == K slot) = Sum_i D[i][o].  Fixed chunking -> deterministic after k_wgrad_reduce.  A chunk is the K
+// range of one CTA: the smallest multiple of 64 tets, at least 128, that leaves one CTA per SM (chunks of
+// 1,024 kept 6 of 152 SMs busy at 6,000 tets).
+static int wgrad_chunk(int64_t ne) {
+  const int64_t c = (ne + 152 * 64 - 1) / (152 * 64) * 64;
+  return (int)(c < 128 ? 128 : c);
+}
+__global__ void __launch_bounds__(256) k_wgrad(int ne, int chunk_len, int O, int K, const float* __restrict__ D,
+                                               const float* __restrict__ X, float* __restrict__ part) {
   __shared__ float Ds[kK][kT + 1];
   __shared__ float Xs[kK][kT + 1];
   const int chunk = blockIdx.x, o0 = blockIdx.y * kT, k0 = blockIdx.z * kT;
   const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
   float acc[4][4] = {};
   float bacc[4] = {0, 0, 0, 0};
-  const int ibeg = chunk * kChunk, iend = min(ne, ibeg + kChunk);
+  const int ibeg = chunk * chunk_len, iend = min(ne, ibeg + chunk_len);
   for (int i0 = ibeg; i0 < iend; i0 += kK) {
     for (int idx = threadIdx.x; idx < kK * kT; idx += blockDim.x) {
       const int r = idx / kT, c = idx % kT;
@@ -133,16 +139,27 @@ __global__ void __launch_bounds__(256) k_wgrad(int ne, int O, int K, const float
     if (blockIdx.z == 0 && tx == 0) part[chunk * stride + (size_t)o * (K + 1) + K] = bacc[p];
   }
 }
-// out_W[o][k] (+)= Sum_chunks part; out_b[o] (+)= Sum_chunks part[..][K]
-__global__ void k_wgrad_reduce(int nchunk, int O, int K, const float* __restrict__ part, float scale, float* __restrict__ gW,
-                               float* __restrict__ gb) {
-  const size_t stride = (size_t)O * (K + 1);
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)stride; e += (int64_t)gridDim.x * blockDim.x) {
-    float s = 0.0f;
-    for (int c = 0; c < nchunk; ++c) s += part[c * stride + e];
-    const int o = (int)(e / (K + 1)), k = (int)(e % (K + 1));
-    if (k < K) gW[(size_t)o * K + k] += scale * s;
-    else if (gb) gb[o] += scale * s;
+// out_W[o][k] (+)= Sum_chunks part; out_b[o] (+)= Sum_chunks part[..][K].  A block takes 32 entries; its 8
+// warps sum every eighth chunk each (a thread that walked all chunks alone was bound by load latency).
+__global__ void __launch_bounds__(256) k_wgrad_reduce(int nchunk, int O, int K, const float* __restrict__ part, float scale,
+                                                      float* __restrict__ gW, float* __restrict__ gb) {
+  __shared__ float red[8][32];
+  const int stride = O * (K + 1);
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, e = blockIdx.x * 32 + lane;
+  float s = 0.0f;
+  if (e < stride) {
+#pragma unroll 4
+    for (int c = w; c < nchunk; c += 8) s += part[(size_t)c * stride + e];
+  }
+  red[w][lane] = s;
+  __syncthreads();
+  if (w == 0 && e < stride) {
+    float t = 0.0f;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) t += red[q][lane];
+    const int o = e / (K + 1), k = e - o * (K + 1);
+    if (k < K) gW[(size_t)o * K + k] += scale * t;
+    else if (gb) gb[o] += scale * t;
   }
 }
 
@@ -193,10 +210,26 @@ __global__ void k_gnn_sumsq(int64_t n, const double* __restrict__ r, double* par
     part[blockIdx.x] = t;
   }
 }
-__global__ void k_gnn_scale(int nparts, const double* part, int64_t n, double* s_out) {
-  if (threadIdx.x == 0 && blockIdx.x == 0) {
+// the sum of the block's 256 values, in a fixed order (every thread gets it; one thread adds the eight
+// warp sums: binary64 additions by all threads would occupy the binary64 pipe)
+__device__ __forceinline__ double gnn_block_sum(double v) {
+  __shared__ double red[9];
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  __syncthreads();
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
     double t = 0.0;
-    for (int k = 0; k < nparts; ++k) t += part[k];
+    for (int k = 0; k < 8; ++k) t += red[k];
+    red[8] = t;
+  }
+  __syncthreads();
+  return red[8];
+}
+// one block of 256 threads (one thread walking the 256 partials took 13 us)
+__global__ void __launch_bounds__(256) k_gnn_scale(int nparts, const double* part, int64_t n, double* s_out) {
+  const double t = gnn_block_sum(threadIdx.x < nparts ? part[threadIdx.x] : 0.0);
+  if (threadIdx.x == 0) {
     const double s = sqrt(t / (double)n);
     s_out[0] = s > 0.0 ? s : 1.0;
   }
@@ -262,21 +295,15 @@ __global__ void k_gnn_lossdiff(int64_t n, const float* __restrict__ out, const d
     part[2 * blockIdx.x + 1] = tb;
   }
 }
-__global__ void k_scale_f(int64_t n, const double* __restrict__ part2, int nparts, float* __restrict__ v, double* loss) {
-  // v *= 2 / Sum t^2 ; loss += Sum diff^2 / Sum t^2  (one thread finishes the reduction first)
-  __shared__ double fac;
-  if (threadIdx.x == 0) {
-    double a = 0.0, b = 0.0;
-    for (int k = 0; k < nparts; ++k) { a += part2[2 * k]; b += part2[2 * k + 1]; }
-    fac = b > 0.0 ? 2.0 / b : 0.0;
-    if (blockIdx.x == 0) loss[0] += b > 0.0 ? a / b : 0.0;
-  }
-  __syncthreads();
-  const float f = (float)fac;
+// v *= 2 / Sum t^2; loss += Sum diff^2 / Sum t^2.  Every block (256 threads) reduces the 256 partial pairs
+// itself, all threads at once (one thread per block walking them took 45 us).
+__global__ void __launch_bounds__(256) k_scale_f(int64_t n, const double* __restrict__ part2, int nparts,
+                                                 float* __restrict__ v, double* loss) {
+  const bool in = threadIdx.x < nparts;
+  const double a = gnn_block_sum(in ? part2[2 * threadIdx.x] : 0.0), b = gnn_block_sum(in ? part2[2 * threadIdx.x + 1] : 0.0);
+  if (blockIdx.x == 0 && threadIdx.x == 0) loss[0] += b > 0.0 ? a / b : 0.0;
+  const float f = (float)(b > 0.0 ? 2.0 / b : 0.0);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) v[e] *= f;
-}
-__global__ void k_fadd(int64_t n, const float* __restrict__ a, float* __restrict__ b) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) b[e] += a[e];
 }
 __global__ void k_to_bf16(int64_t n, const float* __restrict__ a, __nv_bfloat16* __restrict__ b) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
@@ -315,50 +342,72 @@ namespace stdg {
 static cudaStream_t S(stdg_solver* s) { return s->stream; }
 static const int kGB = 1216;
 
-template <typename TW>
-static void dense(stdg_solver* s, int K, int O, const float* A, const void* W, int wt, const float* b, int acc, int relu,
-                  float* pre, float* Y) {
-  const int ne = (int)s->ne;
+static const void* wptr(const GnnState& n, int64_t off) {   // working-copy weights at `off`
+  return n.bf16 ? static_cast<const void*>(static_cast<const __nv_bfloat16*>(n.wc) + off)
+                : static_cast<const void*>(static_cast<const float*>(n.wc) + off);
+}
+static TcGemmArgs dense_args(stdg_solver* s, int K, int O, const float* A, const void* W, int wt, float* Y) {
+  TcGemmArgs a{};
+  a.M = (int)s->ne; a.N = O; a.K = K;
+  a.A = A; a.lda = K; a.a_kmajor = 1;
+  a.B = W; a.b_bf16 = 1; a.ldb = wt ? O : K; a.b_kmajor = wt ? 0 : 1;
+  a.D = Y; a.ldd = O; a.err = s->derr;
+  return a;
+}
+// Y = A W^T (wt == 0: W [O][K]) or A W (wt == 1: W [K][O]), + b, ReLU.  bfloat16 weights: the product on the
+// tensor cores (activations rounded to bfloat16, binary32 sums).
+static void dense(stdg_solver* s, int K, int O, const float* A, int64_t woff, int wt, const float* b, int relu, float* pre,
+                  float* Y) {
+  GnnState& n = *s->gnn;
   ++s->nlaunch;
-  if constexpr (sizeof(TW) == 2) {
-    // bfloat16 weights: the product on the tensor cores (activations rounded to bfloat16, binary32 sums)
-    TcGemmArgs a{};
-    a.M = ne; a.N = O; a.K = K; a.ksplit = 0;
-    a.A = A; a.sAm = K; a.sAk = 1;
-    a.B = W; a.b_bf16 = 1;
-    if (wt) { a.sBn = 1; a.sBk = O; } else { a.sBn = K; a.sBk = 1; }
-    a.D = Y; a.ldd = O; a.dsplit = 0;
-    a.bias = b; a.accumulate = acc; a.relu = relu; a.pre = pre; a.err = s->derr;
+  if (n.bf16) {
+    TcGemmArgs a = dense_args(s, K, O, A, wptr(n, woff), wt, Y);
+    a.bias = b; a.relu = relu; a.pre = pre;
     launch_tc_gemm(a, S(s));
     return;
   }
+  const int ne = (int)s->ne;
   dim3 grid((ne + kT - 1) / kT, (O + kT - 1) / kT);
-  k_dense<TW><<<grid, 256, 0, S(s)>>>(ne, K, O, A, static_cast<const TW*>(W), wt, b, acc, relu, pre, Y);
+  k_dense<float><<<grid, 256, 0, S(s)>>>(ne, K, O, A, static_cast<const float*>(wptr(n, woff)), wt, b, 0, relu, pre, Y);
 }
-static void dense_any(stdg_solver* s, int K, int O, const float* A, int64_t woff, int wt, const float* b, int acc,
-                      int relu, float* pre, float* Y) {
+// a message-passing layer Y = relu(h Ws^T + m Wm^T + b): with bfloat16 weights one launch whose
+// accumulator takes both products (the sum stays in tensor memory instead of a trip through Y)
+static void dense_pair(stdg_solver* s, const float* h, const float* m, int64_t wsoff, int64_t wmoff, const float* b,
+                       float* pre, float* Y) {
   GnnState& n = *s->gnn;
-  if (n.bf16) dense<__nv_bfloat16>(s, K, O, A, static_cast<__nv_bfloat16*>(n.wc) + woff, wt, b, acc, relu, pre, Y);
-  else dense<float>(s, K, O, A, static_cast<float*>(n.wc) + woff, wt, b, acc, relu, pre, Y);
+  const int H = n.H, ne = (int)s->ne;
+  if (n.bf16) {
+    TcGemmArgs a = dense_args(s, H, H, h, wptr(n, wsoff), 0, Y);
+    a.A2 = m; a.lda2 = H; a.B2 = wptr(n, wmoff); a.ldb2 = H; a.K2 = H;
+    a.bias = b; a.relu = 1; a.pre = pre;
+    ++s->nlaunch;
+    launch_tc_gemm(a, S(s));
+    return;
+  }
+  dim3 grid((ne + kT - 1) / kT, (H + kT - 1) / kT);
+  s->nlaunch += 2;
+  k_dense<float><<<grid, 256, 0, S(s)>>>(ne, H, H, h, static_cast<const float*>(wptr(n, wsoff)), 0, b, 0, 0, nullptr, Y);
+  k_dense<float><<<grid, 256, 0, S(s)>>>(ne, H, H, m, static_cast<const float*>(wptr(n, wmoff)), 0, nullptr, 1, 1, pre, Y);
 }
 static void wgrad(stdg_solver* s, int O, int K, const float* D, const float* Xin, int64_t goff, int64_t gboff) {
   GnnState& n = *s->gnn;
-  const int ne = (int)s->ne;
-  const int nchunk = (ne + kChunk - 1) / kChunk;
+  const int ne = (int)s->ne, chunk = wgrad_chunk(ne);
+  const int nchunk = (ne + chunk - 1) / chunk;
   if (n.bf16 && K + 1 <= 256) {
     // on the tensor cores: part[chunk][o][k] = Sum_{i in chunk} D[i][o] X[i][k], k = K the bias column
     TcGemmArgs a{};
-    a.M = O; a.N = K + 1; a.K = ne; a.ksplit = kChunk;
-    a.A = D; a.sAm = 1; a.sAk = O;
-    a.B = Xin; a.sBn = 1; a.sBk = K; a.b_bf16 = 0; a.b_ones_last = 1;
+    a.M = O; a.N = K + 1; a.K = ne; a.ksplit = chunk;
+    a.A = D; a.lda = O; a.a_kmajor = 0;
+    a.B = Xin; a.ldb = K; a.b_kmajor = 0; a.b_ones_last = 1;
     a.D = n.wpart; a.ldd = K + 1; a.dsplit = (int64_t)O * (K + 1);
     a.err = s->derr;
     launch_tc_gemm(a, S(s));
   } else {
     dim3 grid(nchunk, (O + kT - 1) / kT, (K + kT - 1) / kT);
-    k_wgrad<<<grid, 256, 0, S(s)>>>(ne, O, K, D, Xin, n.wpart);
+    k_wgrad<<<grid, 256, 0, S(s)>>>(ne, chunk, O, K, D, Xin, n.wpart);
   }
-  k_wgrad_reduce<<<kGB, 256, 0, S(s)>>>(nchunk, O, K, n.wpart, 1.0f, n.g + goff, gboff >= 0 ? n.g + gboff : nullptr);
+  k_wgrad_reduce<<<(O * (K + 1) + 31) / 32, 256, 0, S(s)>>>(nchunk, O, K, n.wpart, 1.0f, n.g + goff,
+                                                            gboff >= 0 ? n.g + gboff : nullptr);
   s->nlaunch += 2;
 }
 
@@ -367,19 +416,18 @@ static void gnn_forward(stdg_solver* s, const double* r) {
   GnnState& n = *s->gnn;
   const int64_t nv = s->ne * (int64_t)n.C;
   k_gnn_sumsq<<<256, 256, 0, S(s)>>>(nv, r, n.part);
-  k_gnn_scale<<<1, 32, 0, S(s)>>>(256, n.part, nv, n.sdev);
+  k_gnn_scale<<<1, 256, 0, S(s)>>>(256, n.part, nv, n.sdev);
   k_gnn_features<<<kGB, 256, 0, S(s)>>>((int)s->ne, n.C, n.G, r, n.geom, n.sdev, n.X);
   s->nlaunch += 3;
-  dense_any(s, n.F, n.H, n.X, n.off[0], 0, n.w + n.off[1], 0, 1, n.pre0, n.h[0]);
+  dense(s, n.F, n.H, n.X, n.off[0], 0, n.w + n.off[1], 1, n.pre0, n.h[0]);
   for (int l = 0; l < n.L; ++l) {
     k_gather<<<kGB, 256, 0, S(s)>>>((int)s->ne, n.H, s->gnbr, n.h[l], n.mb[l]);
     ++s->nlaunch;
     const int64_t base = 2 + 3 * (int64_t)l;
-    dense_any(s, n.H, n.H, n.h[l], n.off[base], 0, n.w + n.off[base + 2], 0, 0, nullptr, n.h[l + 1]);
-    dense_any(s, n.H, n.H, n.mb[l], n.off[base + 1], 0, nullptr, 1, 1, n.pre[l], n.h[l + 1]);
+    dense_pair(s, n.h[l], n.mb[l], n.off[base], n.off[base + 1], n.w + n.off[base + 2], n.pre[l], n.h[l + 1]);
   }
   const int64_t dbase = 2 + 3 * (int64_t)n.L;
-  dense_any(s, n.H, n.C, n.h[n.L], n.off[dbase], 0, n.w + n.off[dbase + 1], 0, 0, nullptr, n.out);
+  dense(s, n.H, n.C, n.h[n.L], n.off[dbase], 0, n.w + n.off[dbase + 1], 0, nullptr, n.out);
 }
 
 // loss of one pair and accumulation of its gradients into n.g (loss added into n.loss[0])
@@ -387,22 +435,21 @@ static void gnn_backward(stdg_solver* s, const double* t) {
   GnnState& n = *s->gnn;
   const int64_t nv = s->ne * (int64_t)n.C, nh = s->ne * (int64_t)n.H;
   k_gnn_lossdiff<<<256, 256, 0, S(s)>>>(nv, n.out, n.sdev, t, n.dout, n.part);
-  k_scale_f<<<kGB, 256, 0, S(s)>>>(nv, n.part, 256, n.dout, n.loss);
+  k_scale_f<<<304, 256, 0, S(s)>>>(nv, n.part, 256, n.dout, n.loss);
   s->nlaunch += 2;
   const int64_t dbase = 2 + 3 * (int64_t)n.L;
   wgrad(s, n.C, n.H, n.dout, n.h[n.L], n.off[dbase], n.off[dbase + 1]);
-  dense_any(s, n.C, n.H, n.dout, n.off[dbase], 1, nullptr, 0, 0, nullptr, n.dh);
+  dense(s, n.C, n.H, n.dout, n.off[dbase], 1, nullptr, 0, nullptr, n.dh);
   for (int l = n.L - 1; l >= 0; --l) {
     const int64_t base = 2 + 3 * (int64_t)l;
     k_relu_back<<<kGB, 256, 0, S(s)>>>(nh, n.pre[l], n.dh, n.dpre);
     ++s->nlaunch;
     wgrad(s, n.H, n.H, n.dpre, n.h[l], n.off[base], n.off[base + 2]);
     wgrad(s, n.H, n.H, n.dpre, n.mb[l], n.off[base + 1], -1);
-    dense_any(s, n.H, n.H, n.dpre, n.off[base], 1, nullptr, 0, 0, nullptr, n.t1);
-    dense_any(s, n.H, n.H, n.dpre, n.off[base + 1], 1, nullptr, 0, 0, nullptr, n.t2);
-    k_gather<<<kGB, 256, 0, S(s)>>>((int)s->ne, n.H, s->gnbr, n.t2, n.dh);
-    k_fadd<<<kGB, 256, 0, S(s)>>>(nh, n.t1, n.dh);
-    s->nlaunch += 2;
+    dense(s, n.H, n.H, n.dpre, n.off[base], 1, nullptr, 0, nullptr, n.t1);
+    dense(s, n.H, n.H, n.dpre, n.off[base + 1], 1, nullptr, 0, nullptr, n.t2);
+    k_gather<<<kGB, 256, 0, S(s)>>>((int)s->ne, n.H, s->gnbr, n.t2, n.dh, n.t1);
+    ++s->nlaunch;
   }
   k_relu_back<<<kGB, 256, 0, S(s)>>>(nh, n.pre0, n.dh, n.dpre);
   ++s->nlaunch;
@@ -520,7 +567,8 @@ extern "C" stdg_status stdg_gnn_init(stdg_solver* s, int hidden, int layers, int
   for (auto& p : n->h) if ((e = dev_alloc(s, (void**)&p, ne * H * sizeof(float))) != STDG_OK) return e;
   for (auto& p : n->mb) if ((e = dev_alloc(s, (void**)&p, ne * H * sizeof(float))) != STDG_OK) return e;
   for (auto& p : n->pre) if ((e = dev_alloc(s, (void**)&p, ne * H * sizeof(float))) != STDG_OK) return e;
-  const int nchunk = (int)((ne + kChunk - 1) / kChunk);
+  const size_t chunk = (size_t)wgrad_chunk((int64_t)ne);
+  const int nchunk = (int)((ne + chunk - 1) / chunk);
   const int64_t wmax = std::max<int64_t>({(int64_t)H * (F + 1), (int64_t)C * (H + 1), (int64_t)H * (H + 1)});
   if ((e = dev_alloc(s, (void**)&n->wpart, (size_t)nchunk * wmax * sizeof(float))) != STDG_OK) return e;
   if ((e = dev_alloc(s, (void**)&n->sdev, 8 * sizeof(double))) != STDG_OK) return e;

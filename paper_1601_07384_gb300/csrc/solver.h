@@ -197,16 +197,19 @@ int mg_launches(const stdg_solver* s);       // kernel launches per application
 int mg_partial_blocks();
 int mg_levels(const stdg_solver* s, int* sizes, int cap);
 void mg_free(stdg_solver* s);
-// Dense layer products on the tensor cores (tcgemm.cu): D (+)= A B^T with bfloat16 operands
+// Dense layer products on the tensor cores (tcgemm.cu): D = A B^T (+ A2 B2^T) with bfloat16 operands
 struct TcGemmArgs {
-  int M, N, K, ksplit;                       // CTA (x, z) covers rows [128 x, ...) and k in [z ksplit, ...)
-  const float* A; int64_t sAm, sAk;          // A(m, k) = A[m sAm + k sAk]
-  const void* B; int64_t sBn, sBk;           // B(n, k) = B[n sBn + k sBk]
-  int b_bf16;                                // B elements are bfloat16 (else binary32)
+  int M, N, K, ksplit;                       // CTA (x, y) covers rows [128 x, ...) and k in [y ksplit, ...)
+  const float* A; int64_t lda; int a_kmajor; // A(m, k) = A[m lda + k] (a_kmajor) or A[k lda + m]
+  const void* B; int64_t ldb; int b_kmajor;  // B(n, k) = B[n ldb + k] (b_kmajor) or B[k ldb + n]
+  int b_bf16;                                // B and B2 elements are bfloat16 (else binary32)
   int b_ones_last;                           // B(N - 1, k) = 1 (a bias column of a weight gradient)
+  const float* A2; int64_t lda2;             // second pair of operands, laid out as the first (or null)
+  const void* B2; int64_t ldb2;
+  int K2;
   float* D; int64_t ldd, dsplit;             // D(m, n) of K range z at D[z dsplit + m ldd + n]
   const float* bias;                         // + bias[n]
-  int accumulate, relu;                      // D = (D +) A B^T (+ bias), then max(., 0)
+  int relu;                                  // then max(., 0)
   float* pre;                                // pre-activation (before ReLU), if not null
   int* err;                                  // set to 1 when a bounded wait gives up
 };
