@@ -77,17 +77,16 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
     if (s->opt.precision < 0 || s->opt.precision > 3) { delete s; set_error("unknown precision %d", opts->precision); return STDG_EINVAL; }
   }
   {
-    // "tma": block-staged TMA operator kernels; "warp": one warp per staged tet; default: CTAs of
-    // several warps per staged tet
+    // "tma" / "warp": the block-staged TMA operator kernels / one warp per staged tet, with binary32
+    // pairs for the binary64-accurate pressure operator; default: the warp kernels for the binary32
+    // operators, fixed point for the binary64-accurate ones
     const char* k = std::getenv("STDG_OP_KERNEL");
     s->op_warp = (k && std::strcmp(k, "tma") == 0) ? 0 : 1;
-    s->op_cta = (k && std::strcmp(k, "warp") == 0) ? 0 : 1;
+    s->op_pairs = (k && (std::strcmp(k, "tma") == 0 || std::strcmp(k, "warp") == 0)) ? 1 : 0;
     const char* mi = std::getenv("STDG_MIXED_INNER");   // binary32 iterations per outer mixed step
     if (mi && std::atoi(mi) > 0 && std::atoi(mi) <= 1000) s->mix_inner = s->mix_inner_mg = std::atoi(mi);
     const char* mm = std::getenv("STDG_MIXED_M");       // directions kept by the outer flexible CG
     if (mm && std::atoi(mm) > 0 && std::atoi(mm) <= 16) s->mix_m = std::atoi(mm);
-    const char* dw = std::getenv("STDG_DF_MIN_WARPS");  // pair kernel used when this many warps fit per SM
-    if (dw && std::atoi(dw) > 0 && std::atoi(dw) <= 64) s->df_min_warps = std::atoi(dw);
     const char* vi = std::getenv("STDG_VISC_INNER64");
     s->visc_inner64 = vi && std::atoi(vi) == 1;
     const char* ck = std::getenv("STDG_CONV_KERNEL");  // "generic": no compile-time-degree convection kernel
@@ -176,6 +175,10 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   TRY(dev_alloc(s, (void**)&s->Aoff, (size_t)m->nf * NN * sizeof(double)));
   TRY(dev_alloc(s, (void**)&s->Bdiag, (size_t)m->ne * NN * sizeof(double)));
   TRY(dev_alloc(s, (void**)&s->Bvisc, (size_t)m->ne * NN * sizeof(double)));
+  TRY(dev_alloc(s, (void**)&s->eB, (size_t)m->ne * sizeof(uint16_t)));
+  TRY(dev_alloc(s, (void**)&s->eA, (size_t)m->nf * sizeof(uint16_t)));
+  TRY(dev_alloc(s, (void**)&s->eQ, (size_t)2 * m->nf * sizeof(uint16_t)));
+  TRY(dev_alloc(s, (void**)&s->eM, (size_t)2 * m->nf * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->derr, sizeof(int)));
   cudaMemset(s->derr, 0, sizeof(int));
   TRY(dev_alloc(s, (void**)&s->P, (size_t)m->ne * s->Nst * sizeof(double)));
@@ -187,9 +190,12 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   for (size_t k = 0; k < ex.size(); ++k) mi.e[k] = (unsigned char)ex[k];
   cudaError_t ce = launch_face_blocks(d, t, s->p, s->N, r->nq_lin, r->nqf_lin, mi, s->Q, s->Mij, s->C, s->x0h, s->stream);
   if (ce == cudaSuccess) ce = launch_assemble(d, s->N, s->Q, s->Aoff, s->Bdiag, s->Bvisc, s->stream);
-  // pair blocks (DF32, and the mixed modes' outer and viscous operators), unless the pair kernel would
-  // run fewer than 6 warps per SM at this N, Ng: there the binary64 kernel is faster and serves instead
-  if (ce == cudaSuccess && s->opt.precision != STDG_PREC_FP64 && (!s->op_warp || warp_df_warps_per_sm(s) >= s->df_min_warps))
+  if (ce == cudaSuccess) ce = launch_block_exps(m->ne, (int)NN, s->Bdiag, s->eB, s->stream);
+  if (ce == cudaSuccess) ce = launch_block_exps(m->nf, (int)NN, s->Aoff, s->eA, s->stream);
+  if (ce == cudaSuccess) ce = launch_block_exps(2 * m->nf, (int)(3 * NN), s->Q, s->eQ, s->stream);
+  if (ce == cudaSuccess) ce = launch_block_exps(2 * m->nf, (int)NN, s->Mij, s->eM, s->stream);
+  // binary32-pair copies of the blocks, for the comparison kernels that STDG_OP_KERNEL selects
+  if (ce == cudaSuccess && s->opt.precision != STDG_PREC_FP64 && s->op_pairs)
     ce = s->op_warp ? warp_prepare(s, STDG_PREC_DF32) : df_build_blocks(s);
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(s->stream);
   if (ce != cudaSuccess) {
@@ -301,11 +307,10 @@ extern "C" stdg_status stdg_pressure_apply_factored(stdg_solver* s, const double
   }
   // gradient and inverse momentum block per dual cell: v_j = -M_j^-1 (Q_lj x_l + Q_rj x_r) (boundary cells 0)
   cudaMemsetAsync(s->fac_v, 0, nv * sizeof(double), s->stream);
-  cudaError_t ce = launch_update((int)s->nf, s->N, s->Ng, s->dm.left, s->dm.right, s->Q, s->fac_v, xin, s->dt,
-                                 s->tm.Kinv, s->fac_v, s->stream);
+  cudaError_t ce = launch_update(face_ops(s), s->fac_v, xin, s->dt, s->tm.Kinv, s->fac_v, s->stream);
   if (ce != cudaSuccess) { set_error("update launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   // divergence back into each tet: y_i = -Sum_j D_ij v_j = Sum_j D_ij M_j^-1 Q_j x
-  ce = launch_rhs((int)s->ne, s->N, s->Ng, s->dm.t2f, s->dm.left, s->Q, s->fac_v, s->dt, pinned ? 1 : 0, y, s->stream);
+  ce = launch_rhs(face_ops(s), s->fac_v, s->dt, pinned ? 1 : 0, y, s->stream);
   if (ce != cudaSuccess) { set_error("rhs launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   s->nlaunch += 2;
   if (pinned) {
@@ -320,7 +325,7 @@ extern "C" stdg_status stdg_pressure_rhs(stdg_solver* s, const double* F, double
   if (e != STDG_OK) return e;
   if (!F || !b) { set_error("stdg_pressure_rhs: NULL buffer"); return STDG_EINVAL; }
   ++s->nlaunch;
-  cudaError_t ce = launch_rhs((int)s->ne, s->N, s->Ng, s->dm.t2f, s->dm.left, s->Q, F, -s->dt, pinned ? 1 : 0, b, s->stream);
+  cudaError_t ce = launch_rhs(face_ops(s), F, -s->dt, pinned ? 1 : 0, b, s->stream);
   if (ce != cudaSuccess) { set_error("rhs launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   return STDG_OK;
 }
@@ -330,8 +335,7 @@ extern "C" stdg_status stdg_velocity_update(stdg_solver* s, const double* F, con
   if (e != STDG_OK) return e;
   if (!F || !dp || !V) { set_error("stdg_velocity_update: NULL buffer"); return STDG_EINVAL; }
   ++s->nlaunch;
-  cudaError_t ce = launch_update((int)s->nf, s->N, s->Ng, s->dm.left, s->dm.right, s->Q, F, dp, s->dt,
-                                 s->tm.Kinv, V, s->stream);
+  cudaError_t ce = launch_update(face_ops(s), F, dp, s->dt, s->tm.Kinv, V, s->stream);
   if (ce != cudaSuccess) { set_error("update launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   return STDG_OK;
 }

@@ -75,39 +75,44 @@ cudaError_t launch_block_inverse(int ne, int N, const double* Bdiag, double* Bin
 namespace stdg {
 
 // Generic five-point block operator on tets (pressure operator of Eq. CS_19, or the viscous
-// operator of Eq. A1_mod which shares its spatial blocks):
-//   acc_i = (Bdiag_i + extra_coef Bextra_i) x_i + Sum_{f: interior} A_{i,p(i,f)} x_p
+// operator of Eq. A1_mod which shares its face blocks):
+//   acc_i = B_i x_i + Sum_{f: interior} A_{i,p(i,f)} x_p
 //   y_i[a][k] = scale Sum_b Tacc[a][b] acc_i[b][k] + mass_coef detJ_i Sum_b Kmass[a][b] x_i[b][k]
 // with Tacc = identity when tacc_identity.  pinned: x at (tet 0, mode 0, every a) read as 0,
-// y there = pin_diag * x.
+// y there = pin_diag * x.  eB, eA: the largest exponent of every block (launch_block_exps).
 struct ApplyArgs {
   int ne, N, Ng;
-  const int *t2f, *t2n, *left;
-  const double *Bdiag, *Aoff, *Bextra, *detJ;
-  double extra_coef, scale, mass_coef, pin_diag;
+  const int *gface, *gnbr;
+  const double *B, *Aoff, *detJ;
+  const uint16_t *eB, *eA;
+  double scale, mass_coef, pin_diag;
   int tacc_identity, pinned;
   double Tacc[kMaxNg * kMaxNg];
   double Kmass[kMaxNg * kMaxNg];
 };
 cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st);
 
+// The per-face blocks Q[nf][2][3][N][N], Mij[nf][2][N][N], the exponents of the largest entries of each
+// (face, side) and the face tables: what the products below read (fxops.cu).
+struct FaceOps {
+  int ne, nf, N, Ng;
+  const int *t2f, *left, *right;
+  const double *Q, *Mij;
+  const uint16_t *eQ, *eM;
+};
+// exponent of the largest entry of each of nblk blocks of len entries (0: all zero, 2047: not finite)
+cudaError_t launch_block_exps(int64_t nblk, int len, const double* blocks, uint16_t* exps, cudaStream_t st);
 // b_i[a][l] = coef Sum_{f} Sum_c Sum_m Q^c_{s(i,j)}[m][l] F_j[c][a][m]   (D = -Q^T; coef = -dt)
-cudaError_t launch_rhs(int ne, int N, int Ng, const int* t2f, const int* left, const double* Q,
-                       const double* F, double coef, int pinned, double* b, cudaStream_t st);
+cudaError_t launch_rhs(const FaceOps& f, const double* F, double coef, int pinned, double* b, cudaStream_t st);
 // V_j = F_j - dt (I (x) K^-1) Sum_s Q_sj dp_s on interior faces, V_j = F_j on boundary faces.
-cudaError_t launch_update(int nf, int N, int Ng, const int* left, const int* right, const double* Q,
-                          const double* F, const double* dp, double dt, const double* Kinv,
-                          double* V, cudaStream_t st);
-// The support steps in pair arithmetic at the compile-time degrees (support.cu); cudaErrorNotSupported
-// at other (N, Ng), where the binary64 kernels serve.  support_fp64(): STDG_SUPPORT=fp64 in the
-// environment (read once per process) keeps the binary64 kernels everywhere.
-bool support_fp64();
-cudaError_t sup_average(cudaStream_t st, int ne, int N, int Ng, const int* t2f, const int* left, const double* detJ,
-                        const double* Mij, const double* in, double* out);
-cudaError_t sup_face_grad(cudaStream_t st, int nf, int N, int Ng, const int* left, const int* right, const double* Q,
-                          const double* Pp, double dt, const double* Kinv, double* G);
-cudaError_t sup_update(cudaStream_t st, int nf, int N, int Ng, const int* left, const int* right, const double* Q,
-                       const double* F, const double* dp, double dt, const double* Kinv, double* V);
+cudaError_t launch_update(const FaceOps& f, const double* F, const double* dp, double dt, const double* Kinv, double* V,
+                          cudaStream_t st);
+// G_j = dt (I (x) K^-1) Sum_s Q_sj p_s  (boundary: the volume part of the single side)
+cudaError_t launch_face_grad(const FaceOps& f, const double* P, double dt, const double* Kinv, double* G, cudaStream_t st);
+// out[c][i][a][k] = 1/|J_i| Sum_f Sum_l Mij[j][s][k][l] in[j][c][a][l]
+cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* in, double* out, cudaStream_t st);
+// F[j][c][a][m] = Sum_s Sum_k Mij[j][s][k][m] vbar[c][s][a][k]; boundary: F = Vbc
+cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st);
 // U_j[s][c][a][k] = dt Sum_l Mij_s[k][l] V_j[c][a][l]
 cudaError_t launch_moments(int nf, int N, int Ng, const double* Mij, const double* V, double dt,
                            double* U, cudaStream_t st);

@@ -533,16 +533,14 @@ void prof_fold(stdg_solver* s) {
   s->ev_used = 0;
 }
 
-// the binary64-accurate pair kernel serves this operator (the pressure operator; with the warp
-// kernels also the viscous operator of Eq. A1_mod) in every precision mode but plain FP64
+// the binary32-pair kernels serve this operator: the pressure operator of a solver with a precision
+// other than plain FP64, when STDG_OP_KERNEL selects them (op_pairs)
 static bool df_serves(const stdg_solver* s, const ApplyArgs& a) {
-  if (s->opt.precision == STDG_PREC_FP64) return false;     // DF32 and the mixed modes (outer and viscous)
-  if (a.Bextra == nullptr && a.mass_coef == 0.0) return s->dfB || s->wdB;
-  return s->wdBv && a.Bextra == s->Bvisc && a.extra_coef == -1.0 && a.tacc_identity && !a.pinned;
+  return a.B == s->Bdiag && a.mass_coef == 0.0 && (s->dfB || s->wdB);
 }
 
-// y = op x with the binary64-accurate kernel for this operator (the pair kernel where it serves,
-// else the binary64 kernel), or with the binary64 kernel alone when fp64_only
+// y = op x with the binary64-accurate kernel (fixed point, or the pair kernels where they serve and
+// fp64_only is not set)
 static stdg_status op_apply(stdg_solver* s, const ApplyArgs& a, const double* x, double* y, bool fp64_only = false) {
   const bool prof = s->prof && !s->ev.empty() && !s->capturing;
   const bool use_df = !fp64_only && df_serves(s, a);
@@ -553,10 +551,8 @@ static stdg_status op_apply(stdg_solver* s, const ApplyArgs& a, const double* x,
   }
   ++s->nlaunch;
   ++s->op_launches;
-  // binary64-accurate operator from binary32 pairs when requested (pressure operator only)
-  cudaError_t e = !use_df ? launch_apply(a, x, y, s->stream)
-                 : a.Bextra ? launch_apply_warp_df_visc(s, x, y, a.scale, a.mass_coef, a.Kmass)
-                            : launch_apply_df(s, x, y, a.pinned, a.tacc_identity, a.scale, a.pin_diag);
+  cudaError_t e = use_df ? launch_apply_df(s, x, y, a.pinned, a.tacc_identity, a.scale, a.pin_diag)
+                         : launch_apply(a, x, y, s->stream);
   if (prof) {
     cudaEventRecord(s->ev[2 * s->ev_used + 1], s->stream);
     ++s->ev_used;
@@ -568,9 +564,9 @@ static stdg_status op_apply(stdg_solver* s, const ApplyArgs& a, const double* x,
 static ApplyArgs pressure_op(stdg_solver* s, int pinned, int kron, double scale, double pin_diag) {
   ApplyArgs a{};
   a.ne = (int)s->ne; a.N = s->N; a.Ng = s->Ng;
-  a.t2f = s->dm.t2f; a.t2n = s->dm.t2n; a.left = s->dm.left;
-  a.Bdiag = s->Bdiag; a.Aoff = s->Aoff; a.Bextra = nullptr; a.detJ = s->dm.detJ;
-  a.extra_coef = 0.0; a.scale = scale; a.mass_coef = 0.0; a.pin_diag = pin_diag;
+  a.gface = s->gface; a.gnbr = s->gnbr;
+  a.B = s->Bdiag; a.Aoff = s->Aoff; a.eB = s->eB; a.eA = s->eA; a.detJ = s->dm.detJ;
+  a.scale = scale; a.mass_coef = 0.0; a.pin_diag = pin_diag;
   a.tacc_identity = kron; a.pinned = pinned;
   for (int q = 0; q < s->Ng * s->Ng; ++q) a.Tacc[q] = s->tm.Tp[q];
   return a;
@@ -1760,13 +1756,33 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
   return STDG_OK;
 }
 
+// the diagonal blocks B_i - Bvisc_i of the viscous operator, formed at the first viscous solve
+__global__ void k_sub(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out) {
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+    out[e] = a[e] - b[e];
+}
+static stdg_status ensure_visc_diag(stdg_solver* s) {
+  if (s->eBv) return STDG_OK;
+  const int64_t n = s->ne * (int64_t)s->N * s->N;
+  stdg_status e;
+  if (!s->Bv && (e = dev_alloc(s, (void**)&s->Bv, (size_t)n * sizeof(double))) != STDG_OK) return e;
+  if ((e = dev_alloc(s, (void**)&s->eBv, (size_t)s->ne * sizeof(uint16_t))) != STDG_OK) return e;
+  s->nlaunch += 2;
+  k_sub<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, s->Bdiag, s->Bvisc, s->Bv);
+  const cudaError_t ce = launch_block_exps(s->ne, s->N * s->N, s->Bv, s->eBv, s->stream);
+  if (ce != cudaSuccess) { set_error("viscous blocks: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
+  return STDG_OK;
+}
+
 stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu, double tol, int* iters,
                           double* res) {
   ApplyArgs a{};
   a.ne = (int)s->ne; a.N = s->N; a.Ng = s->Ng;
-  a.t2f = s->dm.t2f; a.t2n = s->dm.t2n; a.left = s->dm.left;
-  a.Bdiag = s->Bdiag; a.Aoff = s->Aoff; a.Bextra = s->Bvisc; a.detJ = s->dm.detJ;
-  a.extra_coef = -1.0; a.scale = -nu * s->dt; a.mass_coef = 1.0; a.pin_diag = 0.0;
+  a.gface = s->gface; a.gnbr = s->gnbr;
+  stdg_status eb = ensure_visc_diag(s);
+  if (eb != STDG_OK) return eb;
+  a.B = s->Bv; a.Aoff = s->Aoff; a.eB = s->eBv; a.eA = s->eA; a.detJ = s->dm.detJ;
+  a.scale = -nu * s->dt; a.mass_coef = 1.0; a.pin_diag = 0.0;
   a.tacc_identity = 1; a.pinned = 0;
   for (int q = 0; q < s->Ng * s->Ng; ++q) a.Kmass[q] = s->K[q];
   const int64_t n = s->ne * (int64_t)s->Nst;

@@ -51,15 +51,15 @@ struct stdg_solver {
   int *gface = nullptr, *gnbr = nullptr;      // per-tet gather tables (int4 each) for the TMA kernels
   void *wB = nullptr, *wA = nullptr;          // warp-kernel block copies (binary32 / bfloat16), padded rows
   void *wdB = nullptr, *wdA = nullptr;        // warp-kernel (hi, lo) binary32 planes of the FP64 blocks
-  void *wdBv = nullptr;                       // same for the viscous diagonal blocks B_i - Bvisc_i
+  double* Bv = nullptr;                       // the viscous diagonal blocks B_i - Bvisc_i (lazily built)
+  uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;   // largest exponents of the blocks
   void *wBv32 = nullptr;                      // the viscous diagonal blocks in binary32 (padded rows)
   int warp_grid[32] = {0}, warp_wpc[32] = {0};
   int op_warp = 1;                            // 1: warp-per-tet kernels, 0: block-staged TMA kernels
-  int op_cta = 1;                             // with op_warp: several warps share each staged tet
+  int op_pairs = 0;                           // the pair kernels serve the binary64-accurate pressure operator
   int mix_inner = 80;                         // binary32 CG iterations per outer step of the mixed solve
   int mix_inner_mg = 40;                      // the same with the coarse correction (converges faster)
   int mix_m = 16;                             // directions the outer flexible CG keeps
-  int df_min_warps = 3;                       // the pair kernel serves where this many warps fit per SM
   bool visc_inner64 = false;                  // mixed viscous refinement: binary64-vector inner COCG
   bool conv_generic = false;                  // convection: the runtime-degree kernel at every degree
   double *fcgP = nullptr, *fcgQ = nullptr;    // their P_j and Q_j = S P_j
@@ -136,6 +136,9 @@ struct stdg_solver {
 };
 
 namespace stdg {
+inline FaceOps face_ops(const stdg_solver* s) {
+  return FaceOps{(int)s->ne, (int)s->nf, s->N, s->Ng, s->dm.t2f, s->dm.left, s->dm.right, s->Q, s->Mij, s->eQ, s->eM};
+}
 // binary32 Krylov kernels (lowprec.cu), exposed as launch functions
 struct LpKernels {
   void (*coldot)(cudaStream_t, int64_t, int, int, const float*, const float*, double*);
@@ -157,7 +160,6 @@ cudaError_t lp_build_blocks(stdg_solver* s, int kind);
 cudaError_t launch_apply_lp(stdg_solver* s, const float* x, float* y, int pinned, int kron, float scale, float pin_diag,
                             double* dotpart = nullptr);
 cudaError_t warp_prepare(stdg_solver* s, int precision);   // block copies + launch shape, outside capture
-int warp_df_warps_per_sm(stdg_solver* s);                  // resident warps per SM of the pair kernel
 cudaError_t launch_apply_warp_lp(stdg_solver* s, const float* x, float* y, int pinned, int kron, float scale,
                                  float pin_diag, double* dotpart = nullptr);
 int warp_blocks_lp(stdg_solver* s);   // blocks of the binary32 operator launch (dot partials it writes)
@@ -166,8 +168,6 @@ cudaError_t warp_launch_f32_visc(stdg_solver* s, const float* x, float* y, doubl
                                  const double* Kmass);
 cudaError_t launch_apply_warp_df(stdg_solver* s, const double* x, double* y, int pinned, int kron, double scale,
                                  double pin_diag);
-cudaError_t launch_apply_warp_df_visc(stdg_solver* s, const double* x, double* y, double scale, double mass_coef,
-                                      const double* Kmass);
 cudaError_t launch_apply_df(stdg_solver* s, const double* x, double* y, int pinned, int kron, double scale,
                             double pin_diag);
 cudaError_t df_build_blocks(stdg_solver* s);

@@ -46,81 +46,6 @@ __device__ inline void psi_hat(int N, const MultiIdx& mi, const double* C, const
   }
 }
 
-// ---- averaging: out[c][i][a][k] = 1/|J_i| Sum_f Sum_l Mij[j][s][k][l] in[j][c][a][l]
-__global__ void k_average(int ne, int N, int Ng, const int* __restrict__ t2f, const int* __restrict__ left,
-                          const double* __restrict__ detJ, const double* __restrict__ Mij,
-                          const double* __restrict__ in, double* __restrict__ out) {
-  const int i = blockIdx.x, Nst = N * Ng;
-  const size_t NN = (size_t)N * N;
-  const double inv = 1.0 / detJ[i];
-  for (int o = threadIdx.x; o < 3 * Nst; o += blockDim.x) {
-    const int c = o / Nst, rem = o % Nst, a = rem / N, k = rem % N;
-    double s = 0.0;
-    for (int f = 0; f < 4; ++f) {
-      const int j = t2f[4 * i + f];
-      const int sd = left[j] == i ? 0 : 1;
-      const double* M = Mij + ((size_t)j * 2 + sd) * NN + (size_t)k * N;
-      const double* v = in + ((size_t)j * 3 + c) * Nst + a * N;
-      for (int l = 0; l < N; ++l) s = fma(M[l], v[l], s);
-    }
-    out[((size_t)c * ne + i) * Nst + rem] = s * inv;
-  }
-}
-
-// ---- g_j = dt (I (x) K^-1) Sum_s Q_sj p_s  (boundary: Q volume part of the single side)
-__global__ void k_face_grad(int N, int Ng, const int* __restrict__ left, const int* __restrict__ right,
-                            const double* __restrict__ Q, const double* __restrict__ Pp, double dt, MArg Ki,
-                            double* __restrict__ G) {
-  extern __shared__ double sm[];
-  const int j = blockIdx.x, Nst = N * Ng;
-  const size_t NN = (size_t)N * N;
-  const int l = left[j], r = right[j];
-  double* g = sm;   // 3 x Nst
-  for (int o = threadIdx.x; o < 3 * Nst; o += blockDim.x) {
-    const int c = o / Nst, rem = o % Nst, b = rem / N, m = rem % N;
-    double s = 0.0;
-    if (r >= 0) {
-      for (int sd = 0; sd < 2; ++sd) {
-        const double* q = Q + ((size_t)j * 6 + sd * 3 + c) * NN + (size_t)m * N;
-        const double* pp = Pp + (size_t)(sd ? r : l) * Nst + b * N;
-        for (int ll = 0; ll < N; ++ll) s = fma(q[ll], pp[ll], s);
-      }
-    } else {
-      const double* q = Q + ((size_t)j * 6 + 3 + c) * NN + (size_t)m * N;
-      const double* pp = Pp + (size_t)l * Nst + b * N;
-      for (int ll = 0; ll < N; ++ll) s = fma(q[ll], pp[ll], s);
-    }
-    g[o] = s;
-  }
-  __syncthreads();
-  for (int o = threadIdx.x; o < 3 * Nst; o += blockDim.x) {
-    const int c = o / Nst, rem = o % Nst, a = rem / N, m = rem % N;
-    double s = 0.0;
-    for (int b = 0; b < Ng; ++b) s = fma(Ki.v[a * Ng + b], g[c * Nst + b * N + m], s);
-    G[(size_t)j * 3 * Nst + o] = dt * s;
-  }
-}
-
-// ---- goback: F[j][c][a][m] = Sum_s Sum_k Mij[j][s][k][m] vbar[c][s][a][k]; boundary: F = Vbc
-__global__ void k_goback(int ne, int N, int Ng, const int* __restrict__ left, const int* __restrict__ right,
-                         const double* __restrict__ Mij, const double* __restrict__ vbar,
-                         const double* __restrict__ Vbc, double* __restrict__ F) {
-  const int j = blockIdx.x, Nst = N * Ng;
-  const size_t NN = (size_t)N * N;
-  const int l = left[j], r = right[j];
-  for (int o = threadIdx.x; o < 3 * Nst; o += blockDim.x) {
-    if (r < 0) { F[(size_t)j * 3 * Nst + o] = Vbc[(size_t)j * 3 * Nst + o]; continue; }
-    const int c = o / Nst, rem = o % Nst, a = rem / N, m = rem % N;
-    double s = 0.0;
-    for (int sd = 0; sd < 2; ++sd) {
-      const double* M = Mij + ((size_t)j * 2 + sd) * NN + m;
-      const double* v = vbar + ((size_t)c * ne + (sd ? r : l)) * Nst + a * N;
-      for (int k = 0; k < N; ++k) s = fma(M[(size_t)k * N], v[k], s);
-    }
-    F[(size_t)j * 3 * Nst + o] = s;
-  }
-}
-
 // ---- start of a step: V[j][c][0][m] = Sum_a g1[a] Vn[j][c][a][m], other modes 0; boundary = Vbc
 __global__ void k_trace(int nf, int N, int Ng, const int* __restrict__ right, GArg g1, const double* __restrict__ Vn,
                         const double* __restrict__ Vbc, double* __restrict__ V) {
@@ -1185,23 +1110,6 @@ static stdg_status convection(stdg_solver* s, const double* vbar, double* ups) {
   return STDG_OK;
 }
 
-// averaging and face gradient: the pair-arithmetic kernels (support.cu) at the compile-time degrees,
-// the binary64 ones above otherwise (the go back and the pressure right-hand side stay binary64)
-static void step_average(stdg_solver* s, const double* in, double* out) {
-  const int ne = (int)s->ne, N = s->N, Ng = s->Ng;
-  if (!support_fp64() &&
-      sup_average(s->stream, ne, N, Ng, s->dm.t2f, s->dm.left, s->dm.detJ, s->Mij, in, out) != cudaErrorNotSupported)
-    return;
-  k_average<<<ne, 128, 0, s->stream>>>(ne, N, Ng, s->dm.t2f, s->dm.left, s->dm.detJ, s->Mij, in, out);
-}
-static void step_face_grad(stdg_solver* s, const double* P, MArg Ki, double* G) {
-  const int nf = (int)s->nf, N = s->N, Ng = s->Ng, Nst = s->Nst;
-  if (!support_fp64() && sup_face_grad(s->stream, nf, N, Ng, s->dm.left, s->dm.right, s->Q, P, s->dt, s->Kinv.data(),
-                                       G) != cudaErrorNotSupported)
-    return;
-  k_face_grad<<<nf, 128, 3 * Nst * sizeof(double), s->stream>>>(N, Ng, s->dm.left, s->dm.right, s->Q, P, s->dt, Ki, G);
-}
-
 extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int method, double tol,
                                  stdg_step_stats* stats) {
   if (!s || n_picard < 1 || n_picard > 8 || !(tol > 0.0) || nu < 0.0) { set_error("stdg_step: invalid argument"); return STDG_EINVAL; }
@@ -1214,15 +1122,15 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   const int64_t np = (int64_t)ne * Nst;
   cudaStream_t st = s->stream;
   GArg g0{}, g1{};
-  MArg K{}, Ki{};
+  MArg K{};
   for (int a = 0; a < Ng; ++a) { g0.v[a] = s->g0[a]; g1.v[a] = s->g1[a]; }
-  for (int q = 0; q < Ng * Ng; ++q) { K.v[q] = s->K[q]; Ki.v[q] = s->Kinv[q]; }
+  for (int q = 0; q < Ng * Ng; ++q) K.v[q] = s->K[q];
   stdg_step_stats local{};
   s->phase_of.clear();
   phase_mark(s, -1);
   // previous slab average and new-slab boundary data
   ++s->nlaunch;
-  step_average(s, s->V, s->Vbar_n);
+  launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar_n, st);
   if ((e = boundary_data(s, s->t)) != STDG_OK) return e;
   // step 0: v^{n+1,0}(x, tau) = v^n(x, 1), p^{n+1,0} = 0
   ++s->nlaunch;
@@ -1239,7 +1147,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   for (int k = 0; k < n_picard; ++k) {
     // 1. averaging and previous-Picard pressure gradient
     ++s->nlaunch;
-    step_average(s, s->V, s->Vbar);
+    launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar, st);
     // Lambda of Eq. prevpress, of p^{n+theta,k} = theta p^{n+1,k} + (1 - theta) p^n (Eq. CS_16_theta)
     const double* Plam = s->P;
     if (th != 1.0) {
@@ -1248,9 +1156,9 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
       Plam = s->Pth;
     }
     ++s->nlaunch;
-    step_face_grad(s, Plam, Ki, s->F);
+    launch_face_grad(face_ops(s), Plam, s->dt, s->Kinv.data(), s->F, st);
     ++s->nlaunch;
-    step_average(s, s->F, s->Lam);
+    launch_average(face_ops(s), s->dm.detJ, s->F, s->Lam, st);
     phase_mark(s, 1);
     // 2. convection
     ++s->nlaunch;
@@ -1272,10 +1180,10 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     phase_mark(s, 3);
     // 4. goback
     ++s->nlaunch;
-    k_goback<<<nf, 128, 0, st>>>(ne, N, Ng, s->dm.left, s->dm.right, s->Mij, s->Vbar, s->Vbc, s->F);
+    launch_goback(face_ops(s), s->Vbar, s->Vbc, s->F, st);
     // 5. pressure correction (Eq. A2_mod)
     ++s->nlaunch;
-    if (launch_rhs(ne, N, Ng, s->dm.t2f, s->dm.left, s->Q, s->F, -s->dt, 1, s->bvec, st) != cudaSuccess) {
+    if (launch_rhs(face_ops(s), s->F, -s->dt, 1, s->bvec, st) != cudaSuccess) {
       set_error("rhs launch failed"); return STDG_ECUDA;
     }
     if (s->gnn && s->ah_nsnap > 0) {
@@ -1292,7 +1200,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     k_axpy<<<1216, 256, 0, st>>>(np, 1.0 / th, s->dp, s->P);     // dp is the increment of p^{n+theta}
     // 6. velocity update (Eq. A3_mod)
     ++s->nlaunch;
-    if (launch_update(nf, N, Ng, s->dm.left, s->dm.right, s->Q, s->F, s->dp, s->dt, s->Kinv.data(), s->V, st) != cudaSuccess) {
+    if (launch_update(face_ops(s), s->F, s->dp, s->dt, s->Kinv.data(), s->V, st) != cudaSuccess) {
       set_error("update launch failed"); return STDG_ECUDA;
     }
     phase_mark(s, 6);
@@ -1304,7 +1212,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   }
   // diagnostics: discrete divergence Sum_j D_ij v_j on unpinned tets
   ++s->nlaunch;
-  launch_rhs(ne, N, Ng, s->dm.t2f, s->dm.left, s->Q, s->V, -s->dt, 0, s->bvec, st);
+  launch_rhs(face_ops(s), s->V, -s->dt, 0, s->bvec, st);
   ++s->nlaunch;
   k_maxabs<<<256, 256, 0, st>>>(np, Nst, s->bvec, s->part);
   std::vector<double> part(256);
