@@ -2,6 +2,7 @@
 #include <chrono>
 #include <cmath>
 #include <cstdlib>
+#include <algorithm>
 #include <cstring>
 #include <new>
 
@@ -115,15 +116,17 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   TRY(upload_i32(s, &d.t2code, m->t2code.data(), 4 * m->ne));
   {
     // gather tables: per tet and local face, (face id << 1 | tet is r(j)) or -1 on the boundary
-    std::vector<int> gf(4 * m->ne), gn(4 * m->ne);
+    std::vector<int> gf(4 * m->ne), gn(4 * m->ne), tf(4 * m->ne);
     for (int64_t i = 0; i < m->ne; ++i)
       for (int f = 0; f < 4; ++f) {
         const int64_t j = m->t2f[4 * i + f], nb = m->t2n[4 * i + f];
-        gf[4 * i + f] = nb >= 0 ? (int)((j << 1) | (m->left[j] == i ? 0 : 1)) : -1;
+        tf[4 * i + f] = (int)((j << 1) | (m->left[j] == i ? 0 : 1));
+        gf[4 * i + f] = nb >= 0 ? tf[4 * i + f] : -1;
         gn[4 * i + f] = (int)nb;
       }
     TRY(upload(s, &s->gface, gf.data(), gf.size()));
     TRY(upload(s, &s->gnbr, gn.data(), gn.size()));
+    TRY(upload(s, &s->tface, tf.data(), tf.size()));
     // compact boundary index of every face (-1: interior), for data given at boundary points
     std::vector<int> bi(m->nf);
     int nb = 0;
@@ -174,11 +177,15 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   TRY(dev_alloc(s, (void**)&s->x0h, (size_t)m->nf * 4 * sizeof(double)));
   TRY(dev_alloc(s, (void**)&s->Aoff, (size_t)m->nf * NN * sizeof(double)));
   TRY(dev_alloc(s, (void**)&s->Bdiag, (size_t)m->ne * NN * sizeof(double)));
-  TRY(dev_alloc(s, (void**)&s->Bvisc, (size_t)m->ne * NN * sizeof(double)));
+  TRY(dev_alloc(s, (void**)&s->Bv, (size_t)m->ne * NN * sizeof(double)));
   TRY(dev_alloc(s, (void**)&s->eB, (size_t)m->ne * sizeof(uint16_t)));
+  TRY(dev_alloc(s, (void**)&s->eBv, (size_t)m->ne * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eA, (size_t)m->nf * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eQ, (size_t)2 * m->nf * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eM, (size_t)2 * m->nf * sizeof(uint16_t)));
+  s->fxws.nvec = 3 * m->nf;                          // nf >= ne (four faces per tet, shared by two)
+  TRY(dev_alloc(s, &s->fxws.w, (size_t)s->fxws.nvec * s->Nst * sizeof(int2)));
+  TRY(dev_alloc(s, (void**)&s->fxws.e, (size_t)s->fxws.nvec * s->Ng * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->derr, sizeof(int)));
   cudaMemset(s->derr, 0, sizeof(int));
   TRY(dev_alloc(s, (void**)&s->P, (size_t)m->ne * s->Nst * sizeof(double)));
@@ -189,11 +196,18 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   std::vector<int> ex = multi_indices(s->p);
   for (size_t k = 0; k < ex.size(); ++k) mi.e[k] = (unsigned char)ex[k];
   cudaError_t ce = launch_face_blocks(d, t, s->p, s->N, r->nq_lin, r->nqf_lin, mi, s->Q, s->Mij, s->C, s->x0h, s->stream);
-  if (ce == cudaSuccess) ce = launch_assemble(d, s->N, s->Q, s->Aoff, s->Bdiag, s->Bvisc, s->stream);
-  if (ce == cudaSuccess) ce = launch_block_exps(m->ne, (int)NN, s->Bdiag, s->eB, s->stream);
-  if (ce == cudaSuccess) ce = launch_block_exps(m->nf, (int)NN, s->Aoff, s->eA, s->stream);
-  if (ce == cudaSuccess) ce = launch_block_exps(2 * m->nf, (int)(3 * NN), s->Q, s->eQ, s->stream);
-  if (ce == cudaSuccess) ce = launch_block_exps(2 * m->nf, (int)NN, s->Mij, s->eM, s->stream);
+  if (ce == cudaSuccess) ce = launch_assemble(d, s->N, s->Q, s->Aoff, s->Bdiag, s->Bv, s->stream);
+  // the blocks to fixed point, in place (fixed.cuh): what every product below reads
+  if (ce == cudaSuccess)
+    ce = fx_scales(m->ne, 6 * m->nf, s->N, s->Bdiag, s->Q, static_cast<int*>(s->fxws.w), &s->fxs, &s->fxt, s->stream);
+  auto encode = [&](int64_t nblk, int len, double* blocks, uint16_t* exps, const FxScale& sr, const FxScale& sc) {
+    if (ce == cudaSuccess) ce = launch_fx_encode(nblk, len, s->N, blocks, exps, sr, sc, s->stream);
+  };
+  encode(m->ne, (int)NN, s->Bdiag, s->eB, s->fxs, s->fxs);
+  encode(m->ne, (int)NN, s->Bv, s->eBv, s->fxs, s->fxs);
+  encode(m->nf, (int)NN, s->Aoff, s->eA, s->fxs, s->fxs);
+  encode(2 * m->nf, (int)(3 * NN), s->Q, s->eQ, s->fxt, s->fxs);
+  encode(2 * m->nf, (int)NN, s->Mij, s->eM, FxScale{}, FxScale{});
   // binary32-pair copies of the blocks, for the comparison kernels that STDG_OP_KERNEL selects
   if (ce == cudaSuccess && s->opt.precision != STDG_PREC_FP64 && s->op_pairs)
     ce = s->op_warp ? warp_prepare(s, STDG_PREC_DF32) : df_build_blocks(s);
@@ -360,7 +374,7 @@ extern "C" stdg_status stdg_velocity_moments(stdg_solver* s, const double* V, do
   stdg_status e = check(s);
   if (e != STDG_OK) return e;
   ++s->nlaunch;
-  cudaError_t ce = launch_moments((int)s->nf, s->N, s->Ng, s->Mij, V, s->dt, U, s->stream);
+  cudaError_t ce = launch_moments((int)s->nf, s->N, s->Ng, blocks_M(s), V, s->dt, U, s->stream);
   if (ce != cudaSuccess) { set_error("moments launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   return STDG_OK;
 }
@@ -369,11 +383,27 @@ extern "C" stdg_status stdg_get_blocks(const stdg_solver* s, double* Q, double* 
   if (!s) { set_error("NULL solver"); return STDG_EINVAL; }
   cudaSetDevice(s->device);
   cudaStreamSynchronize(s->stream);
-  const size_t NN = (size_t)s->N * s->N;
-  if (Q) STDG_CUDA(cudaMemcpy(Q, s->Q, s->nf * 6 * NN * sizeof(double), cudaMemcpyDeviceToHost));
-  if (Mij) STDG_CUDA(cudaMemcpy(Mij, s->Mij, s->nf * 2 * NN * sizeof(double), cudaMemcpyDeviceToHost));
-  if (Aoff) STDG_CUDA(cudaMemcpy(Aoff, s->Aoff, s->nf * NN * sizeof(double), cudaMemcpyDeviceToHost));
-  if (Bdiag) STDG_CUDA(cudaMemcpy(Bdiag, s->Bdiag, s->ne * NN * sizeof(double), cudaMemcpyDeviceToHost));
+  // decoded to binary64 in pieces of at most 64 MB (stream-ordered memory, returned below)
+  const int NN = s->N * s->N;
+  const struct { double* host; FxBlocks b; int64_t nblk; int len; } all[4] = {
+      {Q, blocks_Q(s), 2 * s->nf, 3 * NN}, {Mij, blocks_M(s), 2 * s->nf, NN},
+      {Aoff, blocks_A(s), s->nf, NN}, {Bdiag, blocks_B(s), s->ne, NN}};
+  for (const auto& a : all) {
+    if (!a.host || a.nblk == 0) continue;
+    const int64_t step = std::max<int64_t>(1, std::min<int64_t>(a.nblk, (8 << 20) / a.len));
+    double* tmp = nullptr;
+    STDG_CUDA(cudaMallocAsync((void**)&tmp, (size_t)step * a.len * sizeof(double), s->stream));
+    cudaError_t ce = cudaSuccess;
+    for (int64_t b = 0; b < a.nblk && ce == cudaSuccess; b += step) {
+      const int64_t n = std::min(step, a.nblk - b);
+      ce = launch_fx_decode(b, n, a.len, s->N, a.b, tmp, s->stream);
+      if (ce == cudaSuccess)
+        ce = cudaMemcpyAsync(a.host + b * a.len, tmp, (size_t)n * a.len * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
+      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s->stream);
+    }
+    cudaFreeAsync(tmp, s->stream);
+    STDG_CUDA(ce);
+  }
   return STDG_OK;
 }
 

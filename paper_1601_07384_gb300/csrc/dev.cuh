@@ -4,6 +4,7 @@
 
 #include <cstdint>
 
+#include "fixed.cuh"
 #include "internal.h"
 
 #define STDG_CUDA(call)                                                                  \
@@ -67,8 +68,8 @@ cudaError_t launch_face_blocks(const DevMesh& m, const DevRef& r, int p, int N, 
                                const MultiIdx& mi, double* Q, double* Mij, double* C, double* x0h,
                                cudaStream_t st);
 cudaError_t launch_assemble(const DevMesh& m, int N, const double* Q, double* Aoff, double* Bdiag,
-                            double* Bvisc, cudaStream_t st);
-cudaError_t launch_block_inverse(int ne, int N, const double* Bdiag, double* Binv, cudaStream_t st);
+                            double* Bv, cudaStream_t st);
+cudaError_t launch_block_inverse(int ne, int N, const FxBlocks& Bdiag, double* Binv, cudaStream_t st);
 
 }  // namespace stdg
 
@@ -79,12 +80,15 @@ namespace stdg {
 //   acc_i = B_i x_i + Sum_{f: interior} A_{i,p(i,f)} x_p
 //   y_i[a][k] = scale Sum_b Tacc[a][b] acc_i[b][k] + mass_coef detJ_i Sum_b Kmass[a][b] x_i[b][k]
 // with Tacc = identity when tacc_identity.  pinned: x at (tet 0, mode 0, every a) read as 0,
-// y there = pin_diag * x.  eB, eA: the largest exponent of every block (launch_block_exps).
+// y there = pin_diag * x.
+// Room for the limbs and exponents of the products' input vectors (up to nvec vectors of Ng columns of N).
+struct FxWork { void* w; uint16_t* e; int64_t nvec; };
 struct ApplyArgs {
+  FxWork ws;
   int ne, N, Ng;
   const int *gface, *gnbr;
-  const double *B, *Aoff, *detJ;
-  const uint16_t *eB, *eA;
+  FxBlocks B, A;
+  const double* detJ;
   double scale, mass_coef, pin_diag;
   int tacc_identity, pinned;
   double Tacc[kMaxNg * kMaxNg];
@@ -92,16 +96,23 @@ struct ApplyArgs {
 };
 cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st);
 
-// The per-face blocks Q[nf][2][3][N][N], Mij[nf][2][N][N], the exponents of the largest entries of each
-// (face, side) and the face tables: what the products below read (fxops.cu).
+// The per-face blocks Q[nf][2][3][N][N] (one exponent per face and side), Mij[nf][2][N][N] and the face
+// tables: what the products below read (fxops.cu).
 struct FaceOps {
+  FxWork ws;
   int ne, nf, N, Ng;
-  const int *t2f, *left, *right;
-  const double *Q, *Mij;
-  const uint16_t *eQ, *eM;
+  const int *tface, *left, *right;            // tface[4 i + f]: face << 1 | the tet is r(face)
+  FxBlocks Q, Mij;
 };
-// exponent of the largest entry of each of nblk blocks of len entries (0: all zero, 2047: not finite)
-cudaError_t launch_block_exps(int64_t nblk, int len, const double* blocks, uint16_t* exps, cudaStream_t st);
+// nblk blocks of len binary64 entries (rows of N) to fixed point in place (exps: their exponents), scaled
+// by r and c, and back (blocks first .. first + nblk - 1)
+cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint16_t* exps, const FxScale& r,
+                             const FxScale& c, cudaStream_t st);
+cudaError_t launch_fx_decode(int64_t first, int64_t nblk, int len, int N, const FxBlocks& in, double* out, cudaStream_t st);
+// The scaling of the tet modes by the diagonals of the blocks B, and of the rows of the (not yet encoded)
+// blocks Q to match; top: room for 2 N words on the device.  Waits for the stream.
+cudaError_t fx_scales(int64_t ne, int64_t nq, int N, const double* B, const double* Q, int* top, FxScale* s, FxScale* t,
+                      cudaStream_t st);
 // b_i[a][l] = coef Sum_{f} Sum_c Sum_m Q^c_{s(i,j)}[m][l] F_j[c][a][m]   (D = -Q^T; coef = -dt)
 cudaError_t launch_rhs(const FaceOps& f, const double* F, double coef, int pinned, double* b, cudaStream_t st);
 // V_j = F_j - dt (I (x) K^-1) Sum_s Q_sj dp_s on interior faces, V_j = F_j on boundary faces.
@@ -114,7 +125,7 @@ cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* i
 // F[j][c][a][m] = Sum_s Sum_k Mij[j][s][k][m] vbar[c][s][a][k]; boundary: F = Vbc
 cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st);
 // U_j[s][c][a][k] = dt Sum_l Mij_s[k][l] V_j[c][a][l]
-cudaError_t launch_moments(int nf, int N, int Ng, const double* Mij, const double* V, double dt,
+cudaError_t launch_moments(int nf, int N, int Ng, const FxBlocks& Mij, const double* V, double dt,
                            double* U, cudaStream_t st);
 
 }  // namespace stdg

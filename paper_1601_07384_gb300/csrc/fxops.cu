@@ -3,16 +3,23 @@
 // the face gradient and velocity update (Eq. prevpress, A3_mod), averaging and the go back (Eq. average,
 // goback).  All are one shape: a unit (tet or face) has SLOTS blocks of N x N; thread (unit, slot, row)
 // multiplies its row of its block with the NCOL columns of the slot's vector, and the slots of an output
-// group are added in 128-bit integers.
+// group are added in 96-bit integers.
 //
-// What bounds them: the binary64 kernels they replace were bound by sm_103a's binary64 pipe (64 cycles
-// per warp FMA, every block entry used for up to 15 columns).  Here an entry costs about 20 integer
-// instructions to scale and split, once, and 3 IMAD.WIDE (2 cycles each) per column, so the integer
-// pipe binds at many columns and the block traffic from HBM at one or two.  Layout: vectors as limbs in
-// shared memory, [set][column][row], two rows per 16-byte broadcast load; blocks read by rows are staged
-// through shared memory in rows of odd stride (64-bit accesses at odd strides hit every bank once)
-// by 8-byte cp.async, blocks read by columns (the transposed products) come straight from global
-// memory, coalesced over the threads of a slot.
+// What bounds them: binary64 kernels of this shape are bound by sm_103a's binary64 pipe (64 cycles per
+// warp FMA, every block entry used for up to 15 columns).  Here a product costs 3 IMAD.WIDE (4 cycles
+// each), with two of the integer ALU's additions per product, and the operands come through shared memory,
+// which returns 128 bytes a cycle to an SM (8 cycles of each scheduler per 64-bit operand, also when all
+// lanes read the same word).  Thread tiles of 2 or 3 rows save such reads and were slower: the
+// blocks of a CTA fill the shared memory, so fewer threads per CTA are fewer warps per SM (N = 35, NG = 5
+// at 24,576 tets: 479 us with one row, 671 with two, 849 with three).
+//
+// Two launches: k_fx_vec scales the vector to limbs once, with one exponent per column of every tet (face,
+// component), and applies the time matrix to it where the operation has one; k_fx starts at the same time
+// (programmatic dependent launch) and first copies its blocks, which do not depend on the vector, into
+// shared memory (8-byte cp.async; rows of odd stride, as 64-bit accesses at odd strides hit every bank
+// once).  Blocks read by columns only (rhs, go back) come straight from global memory instead, coalesced
+// over the threads of a slot.  Scaling the vectors inside k_fx instead, every one in all the units that
+// use it, took as many instructions as the products (N = 35, NG = 5).
 #include <algorithm>
 #include <cmath>
 
@@ -24,50 +31,49 @@ namespace stdg {
 namespace {
 
 // ---- the operations.  For unit u: mat() the block of a slot (nullptr: absent), its exponent and
-// whether it is read by columns; vec() the column-0 pointer of a vector set and the distance between
-// columns; store() one output.
-struct FxSlot { const double* m; int e; bool col; };
-struct FxVec { const double* p; int64_t stride_c, stride_q; };   // column (c, q) at p + c stride_c + q stride_q
+// whether it is read by columns; vec() the index of the vector (NG columns of N) of a set and component
+// in the operation's input (-1: absent); store() one output.
+struct FxSlot { const int2* m; int e; bool col; };
 
 // y_i = scale Sum over the diagonal and the four face blocks (T x)_nbr (+ mass term)
 struct FxApply {
   static constexpr int SLOTS = 5, SETS = 5, GROUPS = 1, C = 1;
-  static constexpr bool STAGED = true, MIX = true;
+  static constexpr bool STAGED = true;
   int n;                                    // units
   const int4 *gface, *gnbr;
-  const double *B, *A, *x, *detJ;
-  const uint16_t *eB, *eA;
+  FxBlocks B, A;
+  const double *x, *detJ;
   double* y;
   double scale, mass_coef, pin_diag;
-  int pinned;
+  int unscaled, mass, pinned;               // scale is 1 (1) or -1 (-1), else 0; mass_coef is not 0 (comparing
+                                            // them in the kernel would take the binary64 pipe)
   double K[kMaxNg * kMaxNg];
   __device__ int4 pick(const int4* t, int u) const { return t[u]; }
   __device__ static int at(const int4& v, int f) { return f == 0 ? v.x : f == 1 ? v.y : f == 2 ? v.z : v.w; }
   template <int N>
   __device__ FxSlot mat(int u, int sl) const {
-    if (sl == 0) return {B + (size_t)u * N * N, eB[u], true};        // symmetric: its columns are its rows
+    if (sl == 0) return {B.w + (size_t)u * N * N, B.e[u], true};        // symmetric: its columns are its rows
     const int g = at(gface[u], sl - 1);
     if (g < 0) return {nullptr, 0, false};
-    return {A + (size_t)(g >> 1) * N * N, eA[g >> 1], (g & 1) != 0};  // A_rl = A_lr^T
+    return {A.w + (size_t)(g >> 1) * N * N, A.e[g >> 1], (g & 1) != 0};  // A_rl = A_lr^T
   }
-  template <int N, int NG>
-  __device__ FxVec vec(int u, int set) const {
-    const int nb = set == 0 ? u : at(gnbr[u], set - 1);
-    if (nb < 0) return {nullptr, 0, 0};
-    return {x + (size_t)nb * N * NG, 0, N};
+  __device__ int vec(int u, int set, int) const { return set == 0 ? u : at(gnbr[u], set - 1); }
+  template <int N>
+  __device__ double entry(int u, int sl, int idx) const {
+    return sl == 0 ? fx_entry(B, N * N, u, idx, N) : fx_entry(A, N * N, at(gface[u], sl - 1) >> 1, idx, N);
   }
-  // pinned entries (constant mode of tet 0, every time column) read as 0
-  __device__ bool zero(int u, int set, int k) const {
-    return pinned && k == 0 && (set == 0 ? u : at(gnbr[u], set - 1)) == 0;
-  }
+  __device__ const FxScale& out_scale() const { return B.r; }
   __device__ static int set_of(int sl) { return sl; }
   __device__ static int group_of(int) { return 0; }
-  __device__ double unit_scale(int u) const { return mass_coef != 0.0 ? mass_coef * detJ[u] : 0.0; }
+  __device__ static int slot_of(int, int j) { return j; }
+  __device__ static bool copies(int) { return true; }
+  __device__ double unit_scale(int u) const { return mass ? mass_coef * detJ[u] : 0.0; }
   template <int N, int NG>
   __device__ void store(int u, int, int, int q, int k, double v, double us) const {
     const double* xu = x + (size_t)u * N * NG + k;
-    if (scale != 1.0) v *= scale;
-    if (mass_coef != 0.0) {
+    if (unscaled == 0) v *= scale;
+    else if (unscaled < 0) v = -v;
+    if (mass) {
       double m = 0.0;
       for (int b = 0; b < NG; ++b) m = fma(K[q * NG + b], xu[b * N], m);
       v = fma(us, m, v);
@@ -80,27 +86,28 @@ struct FxApply {
 // b_i = coef Sum_f Sum_c Q^c_f(i)^T F_f^c
 struct FxRhs {
   static constexpr int SLOTS = 12, SETS = 12, GROUPS = 1, C = 1;
-  static constexpr bool STAGED = false, MIX = false;
+  static constexpr bool STAGED = false;
   int n;
-  const int *t2f, *left;
-  const double *Q, *F;
-  const uint16_t* eQ;
+  const int4* tface;                        // per tet: its faces, (face << 1 | the tet is r)
+  FxBlocks Q;
   double* b;
   double coef;
   int pinned;
   template <int N>
   __device__ FxSlot mat(int u, int sl) const {
-    const int f = sl / 3, c = sl - 3 * f, j = t2f[4 * u + f], s = left[j] == u ? 0 : 1;
-    return {Q + ((size_t)j * 6 + 3 * s + c) * N * N, eQ[2 * j + s], true};
+    const int f = sl / 3, g = FxApply::at(tface[u], f);
+    return {Q.w + ((size_t)g * 3 + sl - 3 * f) * N * N, Q.e[g], true};
   }
-  template <int N, int NG>
-  __device__ FxVec vec(int u, int set) const {
-    const int f = set / 3, c = set - 3 * f;
-    return {F + ((size_t)t2f[4 * u + f] * 3 + c) * N * NG, 0, N};
+  __device__ int vec(int u, int set, int) const { return 3 * (FxApply::at(tface[u], set / 3) >> 1) + set % 3; }
+  template <int N>
+  __device__ double entry(int u, int sl, int idx) const {
+    return fx_entry(Q, 3 * N * N, FxApply::at(tface[u], sl / 3), (sl % 3) * N * N + idx, N);
   }
-  __device__ bool zero(int, int, int) const { return false; }
+  __device__ const FxScale& out_scale() const { return Q.c; }
   __device__ static int set_of(int sl) { return sl; }
   __device__ static int group_of(int) { return 0; }
+  __device__ static int slot_of(int, int j) { return j; }
+  __device__ static bool copies(int) { return true; }
   __device__ double unit_scale(int) const { return 0.0; }
   template <int N, int NG>
   __device__ void store(int u, int, int, int q, int k, double v, double) const {
@@ -113,11 +120,11 @@ struct FxRhs {
 // with the left tet)
 struct FxFace {
   static constexpr int SLOTS = 6, SETS = 2, GROUPS = 3, C = 1;
-  static constexpr bool STAGED = true, MIX = true;
+  static constexpr bool STAGED = true;
   int n;
   const int *left, *right;
-  const double *Q, *p, *in;
-  const uint16_t* eQ;
+  FxBlocks Q;
+  const double* in;
   double* out;
   double dt;
   int grad;
@@ -125,18 +132,22 @@ struct FxFace {
   __device__ FxSlot mat(int u, int sl) const {
     const int s = sl / 3, c = sl - 3 * s;
     if (right[u] < 0 && !(grad && s == 1)) return {nullptr, 0, false};
-    return {Q + ((size_t)u * 6 + 3 * s + c) * N * N, eQ[2 * u + s], false};
+    return {Q.w + ((size_t)u * 6 + 3 * s + c) * N * N, Q.e[2 * u + s], false};
   }
-  template <int N, int NG>
-  __device__ FxVec vec(int u, int set) const {
+  __device__ int vec(int u, int set, int) const {
     const int r = right[u];
-    if (r < 0 && !(grad && set == 1)) return {nullptr, 0, 0};
-    const int tet = set == 1 && r >= 0 ? r : left[u];
-    return {p + (size_t)tet * N * NG, 0, N};
+    if (r < 0 && !(grad && set == 1)) return -1;
+    return set == 1 && r >= 0 ? r : left[u];
   }
-  __device__ bool zero(int, int, int) const { return false; }
+  template <int N>
+  __device__ double entry(int u, int sl, int idx) const {
+    return fx_entry(Q, 3 * N * N, 2 * (size_t)u + sl / 3, (sl % 3) * N * N + idx, N);
+  }
+  __device__ const FxScale& out_scale() const { return Q.r; }
   __device__ static int set_of(int sl) { return sl / 3; }
   __device__ static int group_of(int sl) { return sl % 3; }
+  __device__ static int slot_of(int g, int j) { return 3 * j + g; }
+  __device__ static bool copies(int sl) { return sl % 3 == 0; }
   __device__ double unit_scale(int) const { return 0.0; }
   template <int N, int NG>
   __device__ void store(int u, int g, int, int q, int k, double v, double) const {
@@ -148,24 +159,25 @@ struct FxFace {
 // out^c_i = 1/|J_i| Sum_f M_f(i) in_f^c
 struct FxAverage {
   static constexpr int SLOTS = 4, SETS = 4, GROUPS = 1, C = 3;
-  static constexpr bool STAGED = true, MIX = false;
+  static constexpr bool STAGED = true;
   int n;
-  const int *t2f, *left;
-  const double *M, *in, *detJ;
-  const uint16_t* eM;
+  const int4* tface;
+  FxBlocks M;
+  const double* detJ;
   double* out;
   template <int N>
   __device__ FxSlot mat(int u, int f) const {
-    const int j = t2f[4 * u + f], s = left[j] == u ? 0 : 1;
-    return {M + ((size_t)j * 2 + s) * N * N, eM[2 * j + s], false};
+    const int g = FxApply::at(tface[u], f);
+    return {M.w + (size_t)g * N * N, M.e[g], false};
   }
-  template <int N, int NG>
-  __device__ FxVec vec(int u, int f) const {
-    return {in + (size_t)t2f[4 * u + f] * 3 * N * NG, N * NG, N};
-  }
-  __device__ bool zero(int, int, int) const { return false; }
+  __device__ int vec(int u, int f, int c) const { return 3 * (FxApply::at(tface[u], f) >> 1) + c; }
+  template <int N>
+  __device__ double entry(int u, int f, int idx) const { return fx_entry(M, N * N, FxApply::at(tface[u], f), idx, N); }
+  __device__ const FxScale& out_scale() const { return M.r; }
   __device__ static int set_of(int sl) { return sl; }
   __device__ static int group_of(int) { return 0; }
+  __device__ static int slot_of(int, int j) { return j; }
+  __device__ static bool copies(int) { return true; }
   __device__ double unit_scale(int u) const { return 1.0 / detJ[u]; }
   template <int N, int NG>
   __device__ void store(int u, int, int c, int q, int k, double v, double us) const {
@@ -176,27 +188,28 @@ struct FxAverage {
 // F_j^c = Sum_s M_s^T vbar_s^c, boundary faces the prescribed velocity
 struct FxGoback {
   static constexpr int SLOTS = 2, SETS = 2, GROUPS = 1, C = 3;
-  static constexpr bool STAGED = false, MIX = false;
-  int n;
-  int64_t ne;
+  static constexpr bool STAGED = false;
+  int n, ne;
   const int *left, *right;
-  const double *M, *vbar, *Vbc;
-  const uint16_t* eM;
+  FxBlocks M;
+  const double* Vbc;
   double* F;
   template <int N>
   __device__ FxSlot mat(int u, int s) const {
     if (right[u] < 0) return {nullptr, 0, false};
-    return {M + ((size_t)u * 2 + s) * N * N, eM[2 * u + s], true};
+    return {M.w + ((size_t)u * 2 + s) * N * N, M.e[2 * u + s], true};
   }
-  template <int N, int NG>
-  __device__ FxVec vec(int u, int s) const {
+  __device__ int vec(int u, int s, int c) const {
     const int r = right[u];
-    if (r < 0) return {nullptr, 0, 0};
-    return {vbar + (size_t)(s ? r : left[u]) * N * NG, ne * N * NG, N};
+    return r < 0 ? -1 : c * ne + (s ? r : left[u]);
   }
-  __device__ bool zero(int, int, int) const { return false; }
+  template <int N>
+  __device__ double entry(int u, int s, int idx) const { return fx_entry(M, N * N, 2 * (size_t)u + s, idx, N); }
+  __device__ const FxScale& out_scale() const { return M.c; }
   __device__ static int set_of(int sl) { return sl; }
   __device__ static int group_of(int) { return 0; }
+  __device__ static int slot_of(int, int j) { return j; }
+  __device__ static bool copies(int) { return true; }
   __device__ double unit_scale(int) const { return 0.0; }
   template <int N, int NG>
   __device__ void store(int u, int, int c, int q, int k, double v, double) const {
@@ -205,173 +218,231 @@ struct FxGoback {
   }
 };
 
-// units per CTA: about 200 to 320 threads, most lanes of the last warp used
-template <class P, int N>
-struct FxTile {
-  static constexpr int per = P::SLOTS * N;
-  static constexpr int TB = per >= 160 ? 1 : 256 / per;
-  static constexpr int threads = (TB * per + 31) / 32 * 32;
-};
 template <class P, int N, int NG>
-struct FxSmem {
-  static constexpr int TB = FxTile<P, N>::TB, NC = P::C * NG, NS = N | 1, NX = (N + 1) & ~1;
-  static constexpr size_t stage = P::STAGED ? (size_t)TB * P::SLOTS * N * NS * 8 : 0;
-  static constexpr size_t red = (size_t)TB * P::SLOTS * NC * N * 16;
-  static constexpr size_t xs = (size_t)TB * P::SETS * NC * NX * 8;
-  // the partial sums take the place of the staged blocks and the vectors
-  static constexpr size_t bytes = ((stage + xs > red ? stage + xs : red) + 15) / 16 * 16;
+struct FxTile {
+  static constexpr int NC = P::C * NG, NS = N | 1, NX = (N + 1) & ~1;
+  static constexpr int per = P::SLOTS * P::C * N;                // threads per unit
+  // shared memory of TB units: the vectors and the staged blocks, whose place the partial sums take
+  static constexpr size_t bytes(int TB) {
+    const size_t in = (size_t)TB * (P::SETS * NC * NX * 8 + (P::STAGED ? P::SLOTS * N * NS * 8 : 0));
+    const size_t red = (size_t)TB * P::SLOTS * NC * N * 12;
+    return ((in > red ? in : red) + 15) / 16 * 16;
+  }
+  // units per CTA: the fewest idle lanes with at most 256 threads and 40 KB
+  static constexpr int units() {
+    int best = 1;
+    for (int b = 2; b <= 32; ++b) {
+      const int nt = (b * per + 31) / 32 * 32, ot = (best * per + 31) / 32 * 32;
+      if (nt <= 256 && bytes(b) <= 40 * 1024 && b * per * ot > best * per * nt) best = b;
+    }
+    return best;
+  }
+  static constexpr int TB = units();
+  static constexpr int threads = (TB * per + 31) / 32 * 32;
+  // CTAs per SM to compile for: 6 NG accumulators and 28 more registers per thread where the blocks are read
+  // straight from global memory (loads in flight come from many warps), 48 where they are staged, as
+  // far as the shared memory goes
+  static constexpr int regs = 6 * NG + (P::STAGED ? 48 : 28), fit = 65536 / (threads * regs);
+  static constexpr int room = (int)(227 * 1024 / (bytes(TB) + 2048));
+  static constexpr int blocks = fit < 1 ? 1 : fit < room ? fit : room;
+  static constexpr size_t xs = (size_t)TB * P::SETS * NC * NX * 8, smem = bytes(TB);
 };
 
+// The input vector x as limbs: vector v (n of them, NG columns of N), column q, row k at w[(v NG + q) N + k],
+// the (scaled) column's exponent in e[v NG + q]; with mix.on the columns of (mix x), all with the vector's one
+// exponent.  pinned: row 0 of vector 0 reads as 0.
+struct FxInput {
+  FxScale sc;                                 // row k times 2^sc.s[k], the scaling of the blocks' columns
+  const double* x;
+  int2* w;
+  uint16_t* e;
+  int n, pinned;
+};
+__device__ __forceinline__ double fx_in(const FxInput& in, int v, size_t o, int k) {
+  return in.pinned && v == 0 && k == 0 ? 0.0 : in.x[o];
+}
+
+template <int N>
+struct FxLanes {                              // lanes per vector: a power of two that holds N rows, at most 32
+  static constexpr int G = N <= 1 ? 1 : N <= 4 ? 4 : N <= 16 ? 16 : 32, K = (N + G - 1) / G;
+};
+template <int N, int NG>
+__global__ void __launch_bounds__(256) k_fx_vec(const __grid_constant__ FxInput in, const __grid_constant__ FxMat mix) {
+  constexpr int G = FxLanes<N>::G, K = FxLanes<N>::K;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int t = blockIdx.x * 256 + threadIdx.x, v = t / G, k0 = t % G;
+  if ((t - (int)(threadIdx.x & 31)) / G >= in.n) return;      // whole warps past the end
+  const bool have = v < in.n;
+  double x[K][NG];
+  int e[NG], sc[K];
+#pragma unroll
+  for (int q = 0; q < NG; ++q) e[q] = 0;
+#pragma unroll
+  for (int j = 0; j < K; ++j) sc[j] = k0 + j * G < N ? in.sc.s[k0 + j * G] : 0;
+#pragma unroll
+  for (int j = 0; j < K; ++j) {
+    const int k = k0 + j * G;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      x[j][q] = have && k < N ? fx_in(in, v, ((size_t)v * NG + q) * N + k, k) : 0.0;
+      const int ek = fx_exp(x[j][q]);
+      e[q] = max(e[q], ek == 0 || ek == 2047 ? ek : min(max(ek + sc[j], 1), 2046));
+    }
+  }
+  if (mix.on) {
+#pragma unroll
+    for (int q = 1; q < NG; ++q) e[0] = max(e[0], e[q]);
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) e[0] = max(e[0], __shfl_xor_sync(0xffffffffu, e[0], o));
+    if (!have) return;
+    // exponents: of the columns before mixing where that takes the binary64 path (2047), else mixed
+    const bool ok = fx_ok(e[0]) && fx_ok(mix.e);
+    if (k0 < NG) in.e[v * NG + k0] = (uint16_t)(e[0] == 0 ? 0 : ok ? e[0] : 2047);
+#pragma unroll
+    for (int j = 0; j < K; ++j) {
+      const int k = k0 + j * G;
+      if (k >= N) continue;
+      int2 w[NG];
+#pragma unroll
+      for (int q = 0; q < NG; ++q) w[q] = fx_limbs_x(x[j][q], (e[0] ? e[0] : kFxMinExp) - sc[j]);
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {          // (T x)_q, below 5 2^122: its leading bits fit in 61
+        FxAcc T{};
+#pragma unroll
+        for (int b = 0; b < NG; ++b) fx_mad1(make_int2(mix.h[q * NG + b], mix.l[q * NG + b]), w[b], T);
+        const FxSum u = fx_sum(T, NG);        // 2^-37 of the sum of the products: 27 bits less are 2^-64
+        in.w[((size_t)v * NG + q) * N + k] =
+            fx_split((long long)((unsigned long long)__funnelshift_r(u.b, u.c, 27) << 32 | __funnelshift_r(u.a, u.b, 27)));
+      }
+    }
+  } else {
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+#pragma unroll
+      for (int o = G / 2; o > 0; o >>= 1) e[q] = max(e[q], __shfl_xor_sync(0xffffffffu, e[q], o));
+    }
+    if (!have) return;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      if (k0 == q % G) in.e[v * NG + q] = (uint16_t)(fx_ok(e[q]) ? e[q] : 2047);
+#pragma unroll
+      for (int j = 0; j < K; ++j) {
+        const int k = k0 + j * G;
+        if (k < N) in.w[((size_t)v * NG + q) * N + k] = fx_limbs_x(x[j][q], (e[q] ? e[q] : kFxMinExp) - sc[j]);
+      }
+    }
+  }
+}
+
 template <class P, int N, int NG>
-__global__ void __launch_bounds__(FxTile<P, N>::threads) k_fx(P a, FxMat mix) {
-  using T = FxTile<P, N>;
-  using S = FxSmem<P, N, NG>;
-  constexpr int TB = T::TB, NC = S::NC, NS = S::NS, NX = S::NX, NT = T::threads;
+__global__ void __launch_bounds__(FxTile<P, N, NG>::threads, FxTile<P, N, NG>::blocks) k_fx(const __grid_constant__ P a,
+                                                                                         const __grid_constant__ FxInput in,
+                                                                                         const __grid_constant__ FxMat mix) {
+  using T = FxTile<P, N, NG>;
+  constexpr int TB = T::TB, NC = T::NC, NS = T::NS, NX = T::NX, NT = T::threads, C = P::C;
   extern __shared__ __align__(16) unsigned char fxs[];
   int2* xs = reinterpret_cast<int2*>(fxs);                        // [unit][set][column][NX]
-  double* stage = reinterpret_cast<double*>(fxs + S::xs);         // [unit][slot][N][NS]
-  longlong2* red = reinterpret_cast<longlong2*>(fxs);             // [unit][slot][column][N]
+  int2* stage = reinterpret_cast<int2*>(fxs + T::xs);             // [unit][slot][N][NS]
+  constexpr int kRed = TB * P::SLOTS * NC * N;
+  long long* redl = reinterpret_cast<long long*>(fxs);            // [unit][slot][column][N]: low 64 bits of the sums
+  int* redh = reinterpret_cast<int*>(redl + kRed);                // and the high 32
   __shared__ int ex[TB][P::SETS][NC];                             // exponents of the vector columns
   __shared__ int slow[TB];                                        // the unit takes the binary64 path
-  __shared__ int es[TB][P::SLOTS];                                // exponents of the blocks (-1: absent)
+  __shared__ int es[TB][P::SLOTS];                                // exponents of the blocks (0: absent or zero)
   __shared__ double us[TB];
   const int t = threadIdx.x, u0 = blockIdx.x * TB;
-  for (int o = t; o < TB * P::SETS * NC; o += NT) (&ex[0][0][0])[o] = 0;
   if (t < TB) slow[t] = 0;
-  const int tl = t / T::per, sk = t - tl * T::per, sl = sk / N, k = sk - sl * N, u = u0 + tl;
+  const int tl = t / T::per, sk = t - tl * T::per, sl = sk / (C * N), ck = sk - sl * C * N, cg = ck / N, k0 = ck - cg * N;
+  const int u = u0 + tl;
   const bool act = tl < TB && u < a.n;
   FxSlot m{nullptr, 0, false};
   if (act) m = a.template mat<N>(u, sl);
   const bool have = m.m != nullptr;
   if constexpr (P::STAGED) {
+    // the threads of a slot copy its block: column k0, the rows dealt to the components
     if (have) {
-      double* st = stage + (size_t)(tl * P::SLOTS + sl) * N * NS + k;
+      int2* st = stage + (size_t)(tl * P::SLOTS + sl) * N * NS + k0;
 #pragma unroll 5
-      for (int j = 0; j < N; ++j) cp_async<8>(st + j * NS, m.m + j * N + k);
+      for (int j = cg; j < N; j += C) cp_async<8>(st + j * NS, m.m + j * N + k0);
     }
   }
-  __syncthreads();
-  // vectors: thread (unit, set, row) loads its columns; their largest exponents (with mixing one per
-  // set, as the columns are combined)
-  constexpr int XP = P::SETS * N, XR = (TB * XP + NT - 1) / NT;
-  double xv[XR][NC];
-#pragma unroll
-  for (int r = 0; r < XR; ++r) {
-    const int o = t + r * NT, xl = o / XP, xr = o - xl * XP, set = xr / N, xk = xr - set * N;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) xv[r][c] = 0.0;
-    if (xl >= TB || u0 + xl >= a.n) continue;
-    const FxVec v = a.template vec<N, NG>(u0 + xl, set);
-    if (v.p && !a.zero(u0 + xl, set, xk)) {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) xv[r][c] = v.p[(c / NG) * v.stride_c + (c % NG) * v.stride_q + xk];
-    }
-    if (P::MIX && mix.on) {
-      int e = 0;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) e = max(e, fx_exp(xv[r][c]));
-      if (e) atomicMax(&ex[xl][set][0], e);
-    } else {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int e = fx_exp(xv[r][c]);
-        if (e) atomicMax(&ex[xl][set][c], e);
-      }
-    }
-  }
-  if (act && k == 0) {
-    es[tl][sl] = have ? m.e : -1;
-    if (have && !fx_ok(m.e)) slow[tl] = 1;
+  if (act && ck == 0) {
+    es[tl][sl] = have ? m.e : 0;
     if (sl == 0) us[tl] = a.unit_scale(u);
   }
-  __syncthreads();
+  __syncthreads();                                     // slow is clear
+  if (have && ck == 0 && !fx_ok(m.e)) slow[tl] = 1;
+  asm volatile("griddepcontrol.wait;" ::: "memory");   // the limbs are complete
+  // the vectors: a thread copies its row of its component's NG columns (one slot of each set)
+  if (act && P::copies(sl)) {
+    const int set = P::set_of(sl), v = a.vec(u, set, cg);
+    int2* xd = xs + ((size_t)(tl * P::SETS + set) * NC + cg * NG) * NX;
+    if (v >= 0) {
+      const int2* src = in.w + (size_t)v * NG * N;
 #pragma unroll
-  for (int r = 0; r < XR; ++r) {
-    const int o = t + r * NT, xl = o / XP, xr = o - xl * XP, set = xr / N, xk = xr - set * N;
-    if (xl >= TB) continue;
-    int2* xd = xs + (size_t)(xl * P::SETS + set) * NC * NX + xk;
-    if (P::MIX && mix.on) {
-      const int e = ex[xl][set][0];
-      if (!fx_ok(e) || !fx_ok(mix.e)) slow[xl] = 1;
-      int h[NC], l[NC];
+      for (int q = 0; q < NG; ++q) cp_async<8>(xd + q * NX + k0, src + q * N + k0);
+    }
+    if (k0 == 0) {
 #pragma unroll
-      for (int c = 0; c < NC; ++c) fx_limbs<kFxX>(xv[r][c], e, h[c], l[c]);
-#pragma unroll 1
-      for (int c = 0; c < NC; ++c) {          // (T x)_c: |S0| < 5 2^55, kept to 2^-56 of the full scale
-        long long S0 = 0, S1 = 0;
-#pragma unroll
-        for (int b = 0; b < NC; ++b) fx_mad(mix.h[c * NC + b], mix.l[c * NC + b], h[b], l[b], S0, S1);
-        const long long V = (S0 + ((S1 + (1 << 28)) >> kFxL) + 2) >> 2;
-        xd[c * NX] = e ? fx_limbs_int(V) : make_int2(0, 0);
-      }
-    } else {
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int e = ex[xl][set][c];
-        if (!fx_ok(e)) slow[xl] = 1;
-        int2 v = make_int2(0, 0);
-        if (e) fx_limbs<kFxX>(xv[r][c], e, v.x, v.y);
-        xd[c * NX] = v;
+      for (int q = 0; q < NG; ++q) {
+        const int e = v >= 0 ? in.e[v * NG + q] : 0;
+        ex[tl][set][cg * NG + q] = e;
+        if (e == 2047) slow[tl] = 1;
       }
     }
   }
-  if constexpr (P::STAGED) cp_async_wait_all();
+  cp_async_wait_all();
   __syncthreads();
-  // products: row k of the slot's block with every column of the slot's vector
+  // products: row k of the slot's block with the NG columns of one component of the slot's vector
   const bool dbl = act && slow[tl] != 0;
-  long long S0[NC], S1[NC];
+  FxAcc acc[NG];
 #pragma unroll
-  for (int c = 0; c < NC; ++c) S0[c] = S1[c] = 0;
+  for (int q = 0; q < NG; ++q) acc[q] = FxAcc{};
   if (have && !dbl) {
-    const int2* xr = xs + (size_t)(tl * P::SETS + P::set_of(sl)) * NC * NX;
-    const double* mp = P::STAGED ? stage + (size_t)(tl * P::SLOTS + sl) * N * NS + (m.col ? k : k * NS) : m.m + k;
-    const int step = P::STAGED ? (m.col ? NS : 1) : N;
-    const int e = m.e ? m.e : kFxMinExp;
-#pragma unroll (NC > 5 ? 2 : N <= 10 ? 5 : 4)
+    const int2* xr = xs + ((size_t)(tl * P::SETS + P::set_of(sl)) * NC + cg * NG) * NX;
+    const int2* mr = P::STAGED ? stage + (size_t)(tl * P::SLOTS + sl) * N * NS + k0 * (m.col ? 1 : NS) : m.m + k0;
+    const int step = P::STAGED ? (m.col ? NS : 1) : N;           // along the sum
+#pragma unroll (NG >= 4 ? 2 : 5)
     for (int l = 0; l + 1 < N; l += 2) {
-      int h0, l0, h1, l1;
-      fx_limbs<kFxA>(mp[l * step], e, h0, l0);
-      fx_limbs<kFxA>(mp[(l + 1) * step], e, h1, l1);
+      const int2 m0 = mr[l * step], m1 = mr[(l + 1) * step];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int4 v = *reinterpret_cast<const int4*>(xr + c * NX + l);
-        fx_mad(h0, l0, v.x, v.y, S0[c], S1[c]);
-        fx_mad(h1, l1, v.z, v.w, S0[c], S1[c]);
+      for (int q = 0; q < NG; ++q) {
+        const int4 v = *reinterpret_cast<const int4*>(xr + q * NX + l);
+        fx_mad2(m0, make_int2(v.x, v.y), m1, make_int2(v.z, v.w), acc[q]);
       }
     }
     if constexpr (N & 1) {
-      int h0, l0;
-      fx_limbs<kFxA>(mp[(N - 1) * step], e, h0, l0);
+      const int2 m0 = mr[(N - 1) * step];
 #pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const int2 v = xr[c * NX + N - 1];
-        fx_mad(h0, l0, v.x, v.y, S0[c], S1[c]);
-      }
+      for (int q = 0; q < NG; ++q) fx_mad1(m0, xr[q * NX + N - 1], acc[q]);
     }
   }
   __syncthreads();                                     // the stage and the vectors are free
+  const int rbase = ((tl * P::SLOTS + sl) * NC + cg * NG) * N;
   if (have && dbl) {                                   // binary64 multiply-adds (non-finite or tiny operands)
-    const FxVec v = a.template vec<N, NG>(u, P::set_of(sl));
+    const int v = a.vec(u, P::set_of(sl), cg);
 #pragma unroll 1
-    for (int c = 0; c < NC; ++c) {
+    for (int q = 0; q < NG; ++q) {
       double s = 0.0;
 #pragma unroll 1
       for (int l = 0; l < N; ++l) {
-        const double* p = v.p + (c / NG) * v.stride_c + l;
         double xc = 0.0;
-        if (!a.zero(u, P::set_of(sl), l)) {
-          if (P::MIX && mix.on)
-            for (int b = 0; b < NG; ++b) xc = fma(mix.v[(c % NG) * NG + b], p[b * v.stride_q], xc);
-          else
-            xc = p[(c % NG) * v.stride_q];
+        if (mix.on) {
+          for (int b = 0; b < NG; ++b) xc = fma(mix.v[q * NG + b], fx_in(in, v, ((size_t)v * NG + b) * N + l, l), xc);
+        } else {
+          xc = fx_in(in, v, ((size_t)v * NG + q) * N + l, l);
         }
-        s = fma(m.m[m.col ? l * N + k : k * N + l], xc, s);
+        s = fma(a.template entry<N>(u, sl, m.col ? l * N + k0 : k0 * N + l), xc, s);
       }
-      red[((size_t)(tl * P::SLOTS + sl) * NC + c) * N + k] = make_longlong2(__double_as_longlong(s), 0);
+      redl[rbase + q * N + k0] = __double_as_longlong(s);
     }
   } else if (have) {
 #pragma unroll
-    for (int c = 0; c < NC; ++c) red[((size_t)(tl * P::SLOTS + sl) * NC + c) * N + k] = make_longlong2(S0[c], S1[c]);
+    for (int q = 0; q < NG; ++q) {
+      const FxSum w = fx_sum(acc[q], (N + 1) / 2);
+      redl[rbase + q * N + k0] = (long long)((unsigned long long)w.b << 32 | w.a);
+      redh[rbase + q * N + k0] = (int)w.c;
+    }
   }
   __syncthreads();
   // outputs: the slots of each group added with aligned exponents
@@ -380,77 +451,134 @@ __global__ void __launch_bounds__(FxTile<P, N>::threads) k_fx(P a, FxMat mix) {
     const int ol = o / per_out, rem = o - ol * per_out, g = rem / (NC * N), c = rem / N % NC, ok = rem % N;
     const int ou = u0 + ol;
     if (ou >= a.n) continue;
-    const longlong2* rp = red + ((size_t)ol * P::SLOTS * NC + c) * N + ok;
+    const int rp = (ol * P::SLOTS * NC + c) * N + ok;
     double v;
     if (slow[ol]) {
       v = 0.0;
       for (int s = 0; s < P::SLOTS; ++s)
-        if (P::group_of(s) == g && es[ol][s] >= 0) v += __longlong_as_double(rp[(size_t)s * NC * N].x);
+        if (P::group_of(s) == g && es[ol][s] > 0) v += __longlong_as_double(redl[rp + s * NC * N]);
     } else {
-      int top = 0;
-      for (int s = 0; s < P::SLOTS; ++s) {
-        if (P::group_of(s) != g || es[ol][s] <= 0) continue;
-        const int xe = ex[ol][P::set_of(s)][P::MIX && mix.on ? 0 : c];
-        if (xe > 0) top = max(top, es[ol][s] + xe);
+      // the exponent of each slot's sum, -1 where it is absent or zero
+      constexpr int SG = P::SLOTS / P::GROUPS;
+      int se[SG], top = 0;
+#pragma unroll
+      for (int j = 0; j < SG; ++j) {
+        const int s = P::slot_of(g, j), be = es[ol][s], xe = ex[ol][P::set_of(s)][c];
+        se[j] = be > 0 && xe > 0 ? be + xe : -1;
+        top = max(top, se[j]);
       }
-      __int128 sum = 0;
-      for (int s = 0; s < P::SLOTS; ++s) {
-        if (P::group_of(s) != g || es[ol][s] <= 0) continue;
-        const int xe = ex[ol][P::set_of(s)][P::MIX && mix.on ? 0 : c];
-        if (xe <= 0) continue;
-        const longlong2 r = rp[(size_t)s * NC * N];
-        sum += (((__int128)r.x << kFxL) + r.y) >> min(top - es[ol][s] - xe, 127);
+      FxSum sum{0, 0, 0};
+#pragma unroll
+      for (int j = 0; j < SG; ++j) {
+        if (se[j] < 0) continue;
+        const int p = rp + P::slot_of(g, j) * NC * N;
+        const unsigned long long lo = (unsigned long long)redl[p];
+        fx_add(sum, FxSum{(uint32_t)lo, (uint32_t)(lo >> 32), (uint32_t)redh[p]}, top - se[j]);
       }
-      v = fx_value(sum, fx_unit(top, P::MIX && mix.on ? mix.e - 1019 : 0));
+      v = fx_value(sum, fx_unit(top, (mix.on ? mix.e - 1019 : 0) + a.out_scale().s[ok]));
     }
     a.template store<N, NG>(ou, g, c / NG, c % NG, ok, v, us[ol]);
   }
 }
 
 template <class P, int N, int NG>
-cudaError_t fx_launch_t(const P& a, const FxMat& mix, cudaStream_t st) {
-  constexpr int smem = (int)FxSmem<P, N, NG>::bytes;
-  if (smem > 48 * 1024) {
-    const cudaError_t e = cudaFuncSetAttribute(k_fx<P, N, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+cudaError_t fx_launch_t(const P& a, const FxInput& in, const FxMat& mix, cudaStream_t st) {
+  using T = FxTile<P, N, NG>;
+  if (a.n <= 0) return cudaSuccess;
+  if (T::smem > 48 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k_fx<P, N, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
     if (e != cudaSuccess) return e;
   }
-  constexpr int TB = FxTile<P, N>::TB;
-  if (a.n > 0) k_fx<P, N, NG><<<(a.n + TB - 1) / TB, FxTile<P, N>::threads, smem, st>>>(a, mix);
-  return cudaGetLastError();
+  k_fx_vec<N, NG><<<(int)(((int64_t)in.n * FxLanes<N>::G + 255) / 256), 256, 0, st>>>(in, mix);
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((a.n + T::TB - 1) / T::TB);
+  cfg.blockDim = dim3(T::threads);
+  cfg.dynamicSmemBytes = T::smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_fx<P, N, NG>, a, in, mix);
+  return e != cudaSuccess ? e : cudaGetLastError();
 }
 template <class P, int N>
-cudaError_t fx_launch_n(int Ng, const P& a, const FxMat& mix, cudaStream_t st) {
+cudaError_t fx_launch_n(int Ng, const P& a, const FxInput& in, const FxMat& mix, cudaStream_t st) {
   switch (Ng) {
-    case 1: return fx_launch_t<P, N, 1>(a, mix, st);
-    case 2: return fx_launch_t<P, N, 2>(a, mix, st);
-    case 3: return fx_launch_t<P, N, 3>(a, mix, st);
-    case 4: return fx_launch_t<P, N, 4>(a, mix, st);
-    case 5: return fx_launch_t<P, N, 5>(a, mix, st);
+    case 1: return fx_launch_t<P, N, 1>(a, in, mix, st);
+    case 2: return fx_launch_t<P, N, 2>(a, in, mix, st);
+    case 3: return fx_launch_t<P, N, 3>(a, in, mix, st);
+    case 4: return fx_launch_t<P, N, 4>(a, in, mix, st);
+    case 5: return fx_launch_t<P, N, 5>(a, in, mix, st);
   }
   return cudaErrorInvalidValue;
 }
+// x: the input, nvec vectors, sc the scaling of its rows; ws: room for its limbs and exponents
 template <class P>
-cudaError_t fx_launch(int N, int Ng, const P& a, const FxMat& mix, cudaStream_t st) {
+cudaError_t fx_launch(int N, int Ng, const P& a, const double* x, int nvec, const FxScale& sc, const FxWork& ws, int pinned,
+                      const FxMat& mix, cudaStream_t st) {
+  const FxInput in{sc, x, static_cast<int2*>(ws.w), ws.e, nvec, pinned};
+  if (!in.w || !in.e || (int64_t)nvec > ws.nvec) return cudaErrorInvalidValue;
   switch (N) {
-    case 1: return fx_launch_n<P, 1>(Ng, a, mix, st);
-    case 4: return fx_launch_n<P, 4>(Ng, a, mix, st);
-    case 10: return fx_launch_n<P, 10>(Ng, a, mix, st);
-    case 20: return fx_launch_n<P, 20>(Ng, a, mix, st);
-    case 35: return fx_launch_n<P, 35>(Ng, a, mix, st);
+    case 1: return fx_launch_n<P, 1>(Ng, a, in, mix, st);
+    case 4: return fx_launch_n<P, 4>(Ng, a, in, mix, st);
+    case 10: return fx_launch_n<P, 10>(Ng, a, in, mix, st);
+    case 20: return fx_launch_n<P, 20>(Ng, a, in, mix, st);
+    case 35: return fx_launch_n<P, 35>(Ng, a, in, mix, st);
   }
   return cudaErrorInvalidValue;
 }
 
-// exponent of the largest entry of each block of `len` entries (fx_exp), one warp per block
-__global__ void k_fx_exps(int64_t nblk, int len, const double* __restrict__ in, uint16_t* __restrict__ out) {
+// blocks of `len` binary64 entries to limbs in place, with their exponents; one warp per block
+__global__ void __launch_bounds__(256) k_fx_encode(int64_t nblk, int len, int N, double* __restrict__ blocks,
+                                                   uint16_t* __restrict__ exps, FxScale r, FxScale c) {
   const int lane = threadIdx.x & 31;
   for (int64_t b = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; b < nblk;
        b += ((int64_t)gridDim.x * blockDim.x) >> 5) {
+    double* p = blocks + b * len;
     int e = 0;
-    for (int o = lane; o < len; o += 32) e = max(e, fx_exp(in[b * len + o]));
+    for (int o = lane; o < len; o += 32) {
+      p[o] = scalbn(p[o], -(r.s[o / N % N] + c.s[o % N]));
+      e = max(e, fx_exp(p[o]));
+    }
     e = __reduce_max_sync(0xffffffffu, e);
-    if (lane == 0) out[b] = (uint16_t)e;
+    if (lane == 0) exps[b] = (uint16_t)e;
+    for (int o = lane; o < len; o += 32) reinterpret_cast<int2*>(p)[o] = fx_encode(p[o], e);
   }
+}
+__global__ void __launch_bounds__(256) k_fx_decode(int64_t first, int64_t nblk, int len, int N, FxBlocks in,
+                                                   double* __restrict__ out) {
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < nblk * len; o += (int64_t)gridDim.x * blockDim.x)
+    out[o] = fx_entry(in, len, first + o / len, (int)(o % len), N);
+}
+// top[l]: largest exponent of the diagonal entries (l, l) of the blocks B
+__global__ void __launch_bounds__(256) k_fx_diag(int64_t ne, int N, const double* __restrict__ B, int* top) {
+  __shared__ int m[kMaxN];
+  if (threadIdx.x < kMaxN) m[threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < ne * N; o += (int64_t)gridDim.x * blockDim.x) {
+    const int l = (int)(o % N);
+    atomicMax(&m[l], fx_exp(B[o / N * N * N + l * N + l]));
+  }
+  __syncthreads();
+  if (threadIdx.x < N) atomicMax(&top[threadIdx.x], m[threadIdx.x]);
+}
+// top[m]: largest exponent in row m of the nq blocks Q with their columns scaled by c
+__global__ void __launch_bounds__(256) k_fx_rows(int64_t nq, int N, const double* __restrict__ Q, FxScale c, int* top) {
+  __shared__ int m[kMaxN];
+  if (threadIdx.x < kMaxN) m[threadIdx.x] = 0;
+  __syncthreads();
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < nq * N; o += (int64_t)gridDim.x * blockDim.x) {
+    int e = 0;
+    for (int l = 0; l < N; ++l) {
+      const int el = fx_exp(Q[o * N + l]);
+      if (el != 0 && el != 2047) e = max(e, el - c.s[l]);
+    }
+    atomicMax(&m[o % N], e);
+  }
+  __syncthreads();
+  if (threadIdx.x < N) atomicMax(&top[threadIdx.x], m[threadIdx.x]);
 }
 
 // host: an n x n matrix in limbs
@@ -468,8 +596,8 @@ FxMat fx_mat(const double* v, int n) {
   m.e = big > 0.0 ? std::max(E + 1022, 1) : 0;
   if (m.e < kFxMinExp) return m;
   for (int q = 0; q < n * n; ++q) {
-    const long long w = (long long)std::ldexp(v[q], kFxA - E);        // |w| < 2^kFxA
-    const long long h = (w + (1 << (kFxL - 1))) >> kFxL;
+    const long long w = std::llrint(std::ldexp(v[q], kFx - E));        // |w| <= 2^kFx
+    const long long h = (w + (1LL << (kFxL - 1))) >> kFxL;
     m.h[q] = (int)h;
     m.l[q] = (int)(w - h * (1LL << kFxL));
   }
@@ -478,54 +606,81 @@ FxMat fx_mat(const double* v, int n) {
 
 }  // namespace
 
-cudaError_t launch_block_exps(int64_t nblk, int len, const double* blocks, uint16_t* exps, cudaStream_t st) {
-  if (nblk > 0) k_fx_exps<<<1216, 256, 0, st>>>(nblk, len, blocks, exps);
+cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint16_t* exps, const FxScale& r,
+                             const FxScale& c, cudaStream_t st) {
+  if (nblk > 0) k_fx_encode<<<1216, 256, 0, st>>>(nblk, len, N, blocks, exps, r, c);
   return cudaGetLastError();
+}
+cudaError_t launch_fx_decode(int64_t first, int64_t nblk, int len, int N, const FxBlocks& in, double* out, cudaStream_t st) {
+  if (nblk > 0) k_fx_decode<<<1216, 256, 0, st>>>(first, nblk, len, N, in, out);
+  return cudaGetLastError();
+}
+
+cudaError_t fx_scales(int64_t ne, int64_t nq, int N, const double* B, const double* Q, int* top, FxScale* s, FxScale* t,
+                      cudaStream_t st) {
+  int h[kMaxN];
+  // exponents relative to the largest, halved for the diagonal (a diagonal entry is a sum of squares)
+  auto fetch = [&](const int* from, int div, FxScale* out) {
+    cudaError_t e = cudaMemcpyAsync(h, from, N * sizeof(int), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+    if (e != cudaSuccess) return e;
+    int big = 0;
+    for (int l = 0; l < N; ++l)
+      if (h[l] < 2047) big = std::max(big, h[l]);
+    *out = FxScale{};
+    for (int l = 0; l < N; ++l)
+      if (h[l] > 0 && h[l] < 2047) out->s[l] = (signed char)std::max(-60, (h[l] - big) / div);
+    return e;
+  };
+  cudaError_t e = cudaMemsetAsync(top, 0, 2 * N * sizeof(int), st);
+  if (e != cudaSuccess) return e;
+  k_fx_diag<<<304, 256, 0, st>>>(ne, N, B, top);
+  if ((e = cudaGetLastError()) != cudaSuccess || (e = fetch(top, 2, s)) != cudaSuccess) return e;
+  k_fx_rows<<<1216, 256, 0, st>>>(nq, N, Q, *s, top + N);
+  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  return fetch(top + N, 1, t);
 }
 
 cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st) {
   FxApply p{};
   p.n = a.ne;
   p.gface = reinterpret_cast<const int4*>(a.gface); p.gnbr = reinterpret_cast<const int4*>(a.gnbr);
-  p.B = a.B; p.A = a.Aoff; p.eB = a.eB; p.eA = a.eA; p.detJ = a.detJ;
+  p.B = a.B; p.A = a.A; p.detJ = a.detJ;
   p.x = x; p.y = y;
   p.scale = a.scale; p.mass_coef = a.mass_coef; p.pin_diag = a.pin_diag; p.pinned = a.pinned;
+  p.unscaled = a.scale == 1.0 ? 1 : a.scale == -1.0 ? -1 : 0;
+  p.mass = a.mass_coef != 0.0;
   for (int q = 0; q < a.Ng * a.Ng; ++q) p.K[q] = a.Kmass[q];
-  return fx_launch(a.N, a.Ng, p, a.tacc_identity ? FxMat{} : fx_mat(a.Tacc, a.Ng), st);
+  return fx_launch(a.N, a.Ng, p, x, a.ne, a.B.c, a.ws, a.pinned, a.tacc_identity ? FxMat{} : fx_mat(a.Tacc, a.Ng), st);
 }
 
 cudaError_t launch_rhs(const FaceOps& f, const double* F, double coef, int pinned, double* b, cudaStream_t st) {
   FxRhs p{};
-  p.n = f.ne; p.t2f = f.t2f; p.left = f.left; p.Q = f.Q; p.eQ = f.eQ; p.F = F; p.b = b; p.coef = coef; p.pinned = pinned;
-  return fx_launch(f.N, f.Ng, p, FxMat{}, st);
+  p.n = f.ne; p.tface = reinterpret_cast<const int4*>(f.tface); p.Q = f.Q; p.b = b; p.coef = coef; p.pinned = pinned;
+  return fx_launch(f.N, f.Ng, p, F, 3 * f.nf, f.Q.r, f.ws, 0, FxMat{}, st);
 }
 
-static FxFace fx_face(const FaceOps& f, const double* x, double dt) {
-  FxFace p{};
-  p.n = f.nf; p.left = f.left; p.right = f.right; p.Q = f.Q; p.eQ = f.eQ; p.p = x; p.dt = dt;
-  return p;
-}
 cudaError_t launch_update(const FaceOps& f, const double* F, const double* dp, double dt, const double* Kinv, double* V,
                           cudaStream_t st) {
-  FxFace p = fx_face(f, dp, dt);
-  p.in = F; p.out = V;
-  return fx_launch(f.N, f.Ng, p, fx_mat(Kinv, f.Ng), st);
+  FxFace p{};
+  p.n = f.nf; p.left = f.left; p.right = f.right; p.Q = f.Q; p.dt = dt; p.in = F; p.out = V;
+  return fx_launch(f.N, f.Ng, p, dp, f.ne, f.Q.c, f.ws, 0, fx_mat(Kinv, f.Ng), st);
 }
 cudaError_t launch_face_grad(const FaceOps& f, const double* P, double dt, const double* Kinv, double* G, cudaStream_t st) {
-  FxFace p = fx_face(f, P, dt);
-  p.grad = 1; p.out = G;
-  return fx_launch(f.N, f.Ng, p, fx_mat(Kinv, f.Ng), st);
+  FxFace p{};
+  p.n = f.nf; p.left = f.left; p.right = f.right; p.Q = f.Q; p.dt = dt; p.grad = 1; p.out = G;
+  return fx_launch(f.N, f.Ng, p, P, f.ne, f.Q.c, f.ws, 0, fx_mat(Kinv, f.Ng), st);
 }
 
 cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* in, double* out, cudaStream_t st) {
   FxAverage p{};
-  p.n = f.ne; p.t2f = f.t2f; p.left = f.left; p.M = f.Mij; p.eM = f.eM; p.in = in; p.detJ = detJ; p.out = out;
-  return fx_launch(f.N, f.Ng, p, FxMat{}, st);
+  p.n = f.ne; p.tface = reinterpret_cast<const int4*>(f.tface); p.M = f.Mij; p.detJ = detJ; p.out = out;
+  return fx_launch(f.N, f.Ng, p, in, 3 * f.nf, f.Mij.c, f.ws, 0, FxMat{}, st);
 }
 cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st) {
   FxGoback p{};
-  p.n = f.nf; p.ne = f.ne; p.left = f.left; p.right = f.right; p.M = f.Mij; p.eM = f.eM; p.vbar = vbar; p.Vbc = Vbc; p.F = F;
-  return fx_launch(f.N, f.Ng, p, FxMat{}, st);
+  p.n = f.nf; p.ne = f.ne; p.left = f.left; p.right = f.right; p.M = f.Mij; p.Vbc = Vbc; p.F = F;
+  return fx_launch(f.N, f.Ng, p, vbar, 3 * f.ne, f.Mij.r, f.ws, 0, FxMat{}, st);
 }
 
 }  // namespace stdg

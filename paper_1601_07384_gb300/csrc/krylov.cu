@@ -536,7 +536,7 @@ void prof_fold(stdg_solver* s) {
 // the binary32-pair kernels serve this operator: the pressure operator of a solver with a precision
 // other than plain FP64, when STDG_OP_KERNEL selects them (op_pairs)
 static bool df_serves(const stdg_solver* s, const ApplyArgs& a) {
-  return a.B == s->Bdiag && a.mass_coef == 0.0 && (s->dfB || s->wdB);
+  return a.mass_coef == 0.0 && (s->dfB || s->wdB);
 }
 
 // y = op x with the binary64-accurate kernel (fixed point, or the pair kernels where they serve and
@@ -565,7 +565,8 @@ static ApplyArgs pressure_op(stdg_solver* s, int pinned, int kron, double scale,
   ApplyArgs a{};
   a.ne = (int)s->ne; a.N = s->N; a.Ng = s->Ng;
   a.gface = s->gface; a.gnbr = s->gnbr;
-  a.B = s->Bdiag; a.Aoff = s->Aoff; a.eB = s->eB; a.eA = s->eA; a.detJ = s->dm.detJ;
+  a.ws = s->fxws;
+  a.B = blocks_B(s); a.A = blocks_A(s); a.detJ = s->dm.detJ;
   a.scale = scale; a.mass_coef = 0.0; a.pin_diag = pin_diag;
   a.tacc_identity = kron; a.pinned = pinned;
   for (int q = 0; q < s->Ng * s->Ng; ++q) a.Tacc[q] = s->tm.Tp[q];
@@ -747,7 +748,7 @@ static stdg_status ensure_block_inverse(stdg_solver* s) {
   if (e != STDG_OK) return e;
   if ((e = dev_alloc(s, (void**)&s->lpBinv, cnt * sizeof(float))) != STDG_OK) return e;
   s->nlaunch += 2;
-  cudaError_t ce = launch_block_inverse((int)s->ne, s->N, s->Bdiag, s->Binv, s->stream);
+  cudaError_t ce = launch_block_inverse((int)s->ne, s->N, blocks_B(s), s->Binv, s->stream);
   if (ce == cudaSuccess) { lp_kernels().f32(s->stream, (int64_t)cnt, s->Binv, s->lpBinv); ce = cudaGetLastError(); }
   if (ce != cudaSuccess) { set_error("block inverse launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   return STDG_OK;
@@ -1756,32 +1757,13 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
   return STDG_OK;
 }
 
-// the diagonal blocks B_i - Bvisc_i of the viscous operator, formed at the first viscous solve
-__global__ void k_sub(int64_t n, const double* __restrict__ a, const double* __restrict__ b, double* __restrict__ out) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    out[e] = a[e] - b[e];
-}
-static stdg_status ensure_visc_diag(stdg_solver* s) {
-  if (s->eBv) return STDG_OK;
-  const int64_t n = s->ne * (int64_t)s->N * s->N;
-  stdg_status e;
-  if (!s->Bv && (e = dev_alloc(s, (void**)&s->Bv, (size_t)n * sizeof(double))) != STDG_OK) return e;
-  if ((e = dev_alloc(s, (void**)&s->eBv, (size_t)s->ne * sizeof(uint16_t))) != STDG_OK) return e;
-  s->nlaunch += 2;
-  k_sub<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, s->Bdiag, s->Bvisc, s->Bv);
-  const cudaError_t ce = launch_block_exps(s->ne, s->N * s->N, s->Bv, s->eBv, s->stream);
-  if (ce != cudaSuccess) { set_error("viscous blocks: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
-  return STDG_OK;
-}
-
 stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu, double tol, int* iters,
                           double* res) {
   ApplyArgs a{};
   a.ne = (int)s->ne; a.N = s->N; a.Ng = s->Ng;
   a.gface = s->gface; a.gnbr = s->gnbr;
-  stdg_status eb = ensure_visc_diag(s);
-  if (eb != STDG_OK) return eb;
-  a.B = s->Bv; a.Aoff = s->Aoff; a.eB = s->eBv; a.eA = s->eA; a.detJ = s->dm.detJ;
+  a.ws = s->fxws;
+  a.B = blocks_Bv(s); a.A = blocks_A(s); a.detJ = s->dm.detJ;
   a.scale = -nu * s->dt; a.mass_coef = 1.0; a.pin_diag = 0.0;
   a.tacc_identity = 1; a.pinned = 0;
   for (int q = 0; q < s->Ng * s->Ng; ++q) a.Kmass[q] = s->K[q];

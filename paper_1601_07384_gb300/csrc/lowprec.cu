@@ -303,27 +303,27 @@ __global__ void __launch_bounds__(416) k_apply_tma(TmaArgs<Pol> a, const typenam
 
 // ------------------------------------------------------------------ block copies and vectors
 template <typename TB>
-__global__ void k_to_lp(int64_t nblk, int NN, int SB, const double* __restrict__ src, TB* __restrict__ dst);
+__global__ void k_to_lp(int64_t nblk, int N, int SB, FxBlocks src, TB* __restrict__ dst);
 template <>
-__global__ void k_to_lp<float>(int64_t nblk, int NN, int SB, const double* __restrict__ src, float* __restrict__ dst) {
+__global__ void k_to_lp<float>(int64_t nblk, int N, int SB, FxBlocks src, float* __restrict__ dst) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * SB; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = e / SB;
-    const int o = (int)(e % SB);
-    dst[e] = o < NN ? (float)src[b * NN + o] : 0.0f;
+    const int o = (int)(e % SB), NN = N * N;
+    dst[e] = o < NN ? (float)fx_entry(src, NN, b, o, N) : 0.0f;
   }
 }
 template <>
-__global__ void k_to_lp<__nv_bfloat16>(int64_t nblk, int NN, int SB, const double* __restrict__ src,
+__global__ void k_to_lp<__nv_bfloat16>(int64_t nblk, int N, int SB, FxBlocks src,
                                        __nv_bfloat16* __restrict__ dst) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * SB; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = e / SB;
-    const int o = (int)(e % SB);
-    dst[e] = __float2bfloat16_rn(o < NN ? (float)src[b * NN + o] : 0.0f);
+    const int o = (int)(e % SB), NN = N * N;
+    dst[e] = __float2bfloat16_rn(o < NN ? (float)fx_entry(src, NN, b, o, N) : 0.0f);
   }
 }
 
 template <typename TB>
-static cudaError_t build_lp(stdg_solver* s, int64_t ne, int64_t nf, int N, const double* Bdiag, const double* Aoff,
+static cudaError_t build_lp(stdg_solver* s, int64_t ne, int64_t nf, int N, const FxBlocks& Bdiag, const FxBlocks& Aoff,
                             void** Bd, void** Ao, int* SB, cudaStream_t st) {
   const int align = 16 / (int)sizeof(TB);
   const int sb = ((N * N + align - 1) / align) * align;
@@ -331,8 +331,8 @@ static cudaError_t build_lp(stdg_solver* s, int64_t ne, int64_t nf, int N, const
   if (e != cudaSuccess) return e;
   e = dev_alloc_cuda(s, Ao, (size_t)nf * sb * sizeof(TB));
   if (e != cudaSuccess) return e;
-  k_to_lp<TB><<<1216, 256, 0, st>>>(ne, N * N, sb, Bdiag, static_cast<TB*>(*Bd));
-  k_to_lp<TB><<<1216, 256, 0, st>>>(nf, N * N, sb, Aoff, static_cast<TB*>(*Ao));
+  k_to_lp<TB><<<1216, 256, 0, st>>>(ne, N, sb, Bdiag, static_cast<TB*>(*Bd));
+  k_to_lp<TB><<<1216, 256, 0, st>>>(nf, N, sb, Aoff, static_cast<TB*>(*Ao));
   *SB = sb;
   return cudaGetLastError();
 }
@@ -340,19 +340,19 @@ static cudaError_t build_lp(stdg_solver* s, int64_t ne, int64_t nf, int N, const
 cudaError_t lp_build_blocks(stdg_solver* s, int kind) {
   cudaError_t e;
   if (kind == STDG_PREC_MIXED_BF16)
-    e = build_lp<__nv_bfloat16>(s, s->ne, s->nf, s->N, s->Bdiag, s->Aoff, &s->lpB, &s->lpA, &s->lpSB, s->stream);
+    e = build_lp<__nv_bfloat16>(s, s->ne, s->nf, s->N, blocks_B(s), blocks_A(s), &s->lpB, &s->lpA, &s->lpSB, s->stream);
   else
-    e = build_lp<float>(s, s->ne, s->nf, s->N, s->Bdiag, s->Aoff, &s->lpB, &s->lpA, &s->lpSB, s->stream);
+    e = build_lp<float>(s, s->ne, s->nf, s->N, blocks_B(s), blocks_A(s), &s->lpB, &s->lpA, &s->lpSB, s->stream);
   if (e == cudaSuccess) s->lpkind = kind;
   return e;
 }
 
 // (hi, lo) binary32 pairs of the FP64 blocks, stride padded to a multiple of 2 pairs (16 bytes)
-__global__ void k_to_df(int64_t nblk, int NN, int SB, const double* __restrict__ src, float2* __restrict__ dst) {
+__global__ void k_to_df(int64_t nblk, int N, int SB, FxBlocks src, float2* __restrict__ dst) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * SB; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = e / SB;
-    const int o = (int)(e % SB);
-    const double v = o < NN ? src[b * NN + o] : 0.0;
+    const int o = (int)(e % SB), NN = N * N;
+    const double v = o < NN ? fx_entry(src, NN, b, o, N) : 0.0;
     const float hi = (float)v;
     dst[e] = make_float2(hi, (float)(v - (double)hi));
   }
@@ -364,8 +364,8 @@ cudaError_t df_build_blocks(stdg_solver* s) {
   if (e != cudaSuccess) return e;
   e = dev_alloc_cuda(s, &s->dfA, (size_t)s->nf * sb * sizeof(float2));
   if (e != cudaSuccess) return e;
-  k_to_df<<<1216, 256, 0, s->stream>>>(s->ne, s->N * s->N, sb, s->Bdiag, static_cast<float2*>(s->dfB));
-  k_to_df<<<1216, 256, 0, s->stream>>>(s->nf, s->N * s->N, sb, s->Aoff, static_cast<float2*>(s->dfA));
+  k_to_df<<<1216, 256, 0, s->stream>>>(s->ne, s->N, sb, blocks_B(s), static_cast<float2*>(s->dfB));
+  k_to_df<<<1216, 256, 0, s->stream>>>(s->nf, s->N, sb, blocks_A(s), static_cast<float2*>(s->dfA));
   s->dfSB = sb;
   return cudaGetLastError();
 }

@@ -352,10 +352,14 @@ stdg_status mg_ensure(stdg_solver* s) {
   std::vector<int> t2n(4 * (size_t)ne), t2f(4 * (size_t)ne);
   cudaStream_t st = s->stream;
   // the (0,0) entry of every diagonal block and of every face block
+  // (stored in fixed point; decoded below, once the copies are complete)
+  std::vector<uint16_t> eb(ne), ea(nf);
   STDG_CUDA(cudaMemcpy2DAsync(bd.data(), sizeof(double), s->Bdiag, NN * sizeof(double), sizeof(double), ne,
                               cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaMemcpy2DAsync(ao.data(), sizeof(double), s->Aoff, NN * sizeof(double), sizeof(double), nf,
                               cudaMemcpyDeviceToHost, st));
+  STDG_CUDA(cudaMemcpyAsync(eb.data(), s->eB, eb.size() * sizeof(uint16_t), cudaMemcpyDeviceToHost, st));
+  STDG_CUDA(cudaMemcpyAsync(ea.data(), s->eA, ea.size() * sizeof(uint16_t), cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaMemcpyAsync(t2n.data(), s->dm.t2n, t2n.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaMemcpyAsync(t2f.data(), s->dm.t2f, t2f.size() * sizeof(int), cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaMemcpyAsync(X0.data(), s->dm.X0, X0.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
@@ -363,6 +367,8 @@ stdg_status mg_ensure(stdg_solver* s) {
   STDG_CUDA(cudaMemcpyAsync(bary.data(), s->dm.bary, bary.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaMemcpyAsync(detJ.data(), s->dm.detJ, detJ.size() * sizeof(double), cudaMemcpyDeviceToHost, st));
   STDG_CUDA(cudaStreamSynchronize(st));
+  for (int i = 0; i < ne; ++i) bd[i] = fx_entry_host(bd[i], eb[i], 2 * s->fxs.s[0]);
+  for (int i = 0; i < nf; ++i) ao[i] = fx_entry_host(ao[i], ea[i], 2 * s->fxs.s[0]);
   const double omega = mg_omega();
 
   // level 0: constant-mode coefficients of the pinned S = -A_sp (tet 0 pinned: unit diagonal, no coupling)

@@ -459,8 +459,7 @@ __global__ void __launch_bounds__(128, 1) k_apply_warp(WarpArgs a, const typenam
 
 // padded block copies: dst block b = planes x NR x NP, zero outside N x N
 template <typename TB, int PLANES>
-__global__ void k_to_padded(int64_t nblk, int N, int NR, int NP, const double* __restrict__ src, TB* __restrict__ dst,
-                            const double* __restrict__ src2 = nullptr, double c2 = 0.0) {
+__global__ void k_to_padded(int64_t nblk, int N, int NR, int NP, FxBlocks src, TB* __restrict__ dst) {
   const int64_t per = (int64_t)PLANES * NR * NP;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * per; e += (int64_t)gridDim.x * blockDim.x) {
     const int64_t b = e / per;
@@ -468,8 +467,7 @@ __global__ void k_to_padded(int64_t nblk, int N, int NR, int NP, const double* _
     const int plane = rem / (NR * NP);
     const int rc = rem - plane * NR * NP;
     const int r = rc / NP, c = rc - r * NP;
-    double v = (r < N && c < N) ? src[b * N * N + r * N + c] : 0.0;
-    if (src2 && r < N && c < N) v += c2 * src2[b * N * N + r * N + c];
+    const double v = (r < N && c < N) ? fx_entry(src, (size_t)N * N, b, r * N + c, N) : 0.0;
     if constexpr (sizeof(TB) == 2) {
       dst[e] = __float2bfloat16_rn((float)v);
     } else if constexpr (PLANES == 2) {
@@ -495,21 +493,21 @@ static cudaError_t ensure_warp_blocks(stdg_solver* s, void** Bd, void** Ao) {
   if (e != cudaSuccess) return e;
   e = dev_alloc_cuda(s, Ao, (size_t)s->nf * per * sizeof(TB));
   if (e != cudaSuccess) return e;
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, s->Bdiag, static_cast<TB*>(*Bd));
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->nf, N, NR, NP, s->Aoff, static_cast<TB*>(*Ao));
+  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, blocks_B(s), static_cast<TB*>(*Bd));
+  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->nf, N, NR, NP, blocks_A(s), static_cast<TB*>(*Ao));
   s->nlaunch += 2;
   return cudaGetLastError();
 }
 
-// padded copy of the viscous diagonal blocks B_i - Bvisc_i (Eq. A1_mod, with the face blocks A_lr)
+// padded copy of the viscous diagonal blocks (Eq. A1_mod, with the face blocks A_lr)
 template <typename W>
 static cudaError_t ensure_warp_visc_diag(stdg_solver* s, void** Bv) {
-  if (*Bv || !s->Bvisc) return cudaSuccess;
+  if (*Bv) return cudaSuccess;
   using TB = typename W::TB;
   const int N = s->N, NR = warp_nr(N), NP = warp_np(N);
   cudaError_t e = dev_alloc_cuda(s, Bv, (size_t)s->ne * W::kPlanes * NR * NP * sizeof(TB));
   if (e != cudaSuccess) return e;
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, s->Bdiag, static_cast<TB*>(*Bv), s->Bvisc, -1.0);
+  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, blocks_Bv(s), static_cast<TB*>(*Bv));
   ++s->nlaunch;
   return cudaGetLastError();
 }

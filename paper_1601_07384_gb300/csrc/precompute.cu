@@ -8,7 +8,7 @@
 // and the assembled spatial five-point blocks of Sum_j D_ij M_j^-1 Q (Eq. CS_19) with
 // D = -Q^T and orthonormal psi (M_j^sp = I):
 //   A_lr = -Sum_c Q_l^cT Q_r^c,  B_i = -Sum_{j in S_i interior} Sum_c Q_ij^cT Q_ij^c,
-//   Bvisc_i = +Sum_{j in S_i boundary} Sum_c Q_ij^cT Q_ij^c (Dirichlet ghost, viscous only).
+//   Bv_i = B_i - Sum_{j in S_i boundary} Sum_c Q_ij^cT Q_ij^c (Dirichlet ghost, viscous only).
 #include "dev.cuh"
 
 namespace stdg {
@@ -229,9 +229,10 @@ __global__ void k_offdiag(int nf, int N, const int* right, const double* Q, doub
   }
 }
 
-// B_i = -Sum_{interior j in S_i} Sum_c Q_ij^cT Q_ij^c;  Bvisc_i = +Sum_{boundary j in S_i} (same, slot 0).
+// B_i = -Sum_{interior j in S_i} Sum_c Q_ij^cT Q_ij^c;  Bv_i = -Sum over all j in S_i (boundary: slot 0), the
+// diagonal blocks of the viscous operator.
 __global__ void k_diag(int ne, int N, const int* t2f, const int* t2n, const int* left,
-                       const double* Q, double* Bdiag, double* Bvisc) {
+                       const double* Q, double* Bdiag, double* Bv) {
   const int i = blockIdx.x;
   const size_t NN = (size_t)N * N;
   for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
@@ -247,14 +248,14 @@ __global__ void k_diag(int ne, int N, const int* t2f, const int* t2n, const int*
       if (t2n[4 * i + f] >= 0) sb -= acc; else sv += acc;
     }
     Bdiag[i * NN + idx] = sb;
-    Bvisc[i * NN + idx] = sv;
+    Bv[i * NN + idx] = sb - sv;
   }
 }
 
 // Binv_i = S_ii^-1 for the symmetric positive definite diagonal block S_ii = -B_i of the pinned
 // operator -A (tet 0: the pinned constant mode becomes an identity row and column).  Cholesky in
 // shared memory: S = L L^T, S^-1 = L^-T L^-1.
-__global__ void __launch_bounds__(128) k_block_inverse(int N, const double* __restrict__ Bdiag, double* __restrict__ Binv) {
+__global__ void __launch_bounds__(128) k_block_inverse(int N, FxBlocks Bdiag, double* __restrict__ Binv) {
   extern __shared__ double sm[];
   const int i = blockIdx.x;
   const size_t NN = (size_t)N * N;
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(128) k_block_inverse(int N, const double* __re
   double* Ci = sm + NN;
   for (int idx = threadIdx.x; idx < N * N; idx += blockDim.x) {
     int r = idx / N, c = idx % N;
-    double v = -Bdiag[i * NN + idx];
+    double v = -fx_entry(Bdiag, NN, i, idx, N);
     if (i == 0 && (r == 0 || c == 0)) v = (r == c) ? 1.0 : 0.0;
     G[idx] = v;
   }
@@ -276,7 +277,7 @@ __global__ void __launch_bounds__(128) k_block_inverse(int N, const double* __re
   }
 }
 
-cudaError_t launch_block_inverse(int ne, int N, const double* Bdiag, double* Binv, cudaStream_t st) {
+cudaError_t launch_block_inverse(int ne, int N, const FxBlocks& Bdiag, double* Binv, cudaStream_t st) {
   size_t smem = 2 * (size_t)N * N * sizeof(double);
   cudaError_t e = cudaFuncSetAttribute(k_block_inverse, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -285,9 +286,9 @@ cudaError_t launch_block_inverse(int ne, int N, const double* Bdiag, double* Bin
 }
 
 cudaError_t launch_assemble(const DevMesh& m, int N, const double* Q, double* Aoff, double* Bdiag,
-                            double* Bvisc, cudaStream_t st) {
+                            double* Bv, cudaStream_t st) {
   if (m.nf > 0) k_offdiag<<<m.nf, 128, 0, st>>>(m.nf, N, m.right, Q, Aoff);
-  if (m.ne > 0) k_diag<<<m.ne, 128, 0, st>>>(m.ne, N, m.t2f, m.t2n, m.left, Q, Bdiag, Bvisc);
+  if (m.ne > 0) k_diag<<<m.ne, 128, 0, st>>>(m.ne, N, m.t2f, m.t2n, m.left, Q, Bdiag, Bv);
   return cudaGetLastError();
 }
 

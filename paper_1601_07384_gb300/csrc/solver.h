@@ -39,7 +39,12 @@ struct stdg_solver {
   double *d_ttau = nullptr, *d_tw = nullptr, *d_tg = nullptr;   // device copies
   // per-face / per-tet blocks
   double *Q = nullptr, *Mij = nullptr, *C = nullptr, *x0h = nullptr;
-  double *Aoff = nullptr, *Bdiag = nullptr, *Bvisc = nullptr;
+  double *Aoff = nullptr, *Bdiag = nullptr, *Bv = nullptr;   // Bv: diagonal blocks of the viscous operator
+  // after stdg_solver_create Q, Mij, Aoff, Bdiag and Bv hold fixed-point entries (fixed.cuh, blocks_*
+  // below) with these exponents, one per block (Q: one per face and side)
+  uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;
+  stdg::FxScale fxs{}, fxt{};                 // scaling of the tet modes, and of the dual modes of Q
+  stdg::FxWork fxws{};                        // the products' input vectors in limbs (3 nf vectors fit)
   double *Binv = nullptr;                     // block-Jacobi: (-B_i)^-1, pinned (lazily built)
   double *kz = nullptr;                       // preconditioned residual
   // low-precision copies for the mixed-precision inner solve
@@ -48,11 +53,10 @@ struct stdg_solver {
   void *dfB = nullptr, *dfA = nullptr;        // (hi, lo) binary32 pairs of the FP64 blocks
   int dfSB = 0;
   int tma_grid[16] = {0};                     // persistent grid size per block element size
-  int *gface = nullptr, *gnbr = nullptr;      // per-tet gather tables (int4 each) for the TMA kernels
+  int *gface = nullptr, *gnbr = nullptr;      // per-tet gather tables (int4 each): interior faces, neighbours
+  int *tface = nullptr;                       // the same for all four faces
   void *wB = nullptr, *wA = nullptr;          // warp-kernel block copies (binary32 / bfloat16), padded rows
   void *wdB = nullptr, *wdA = nullptr;        // warp-kernel (hi, lo) binary32 planes of the FP64 blocks
-  double* Bv = nullptr;                       // the viscous diagonal blocks B_i - Bvisc_i (lazily built)
-  uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;   // largest exponents of the blocks
   void *wBv32 = nullptr;                      // the viscous diagonal blocks in binary32 (padded rows)
   int warp_grid[32] = {0}, warp_wpc[32] = {0};
   int op_warp = 1;                            // 1: warp-per-tet kernels, 0: block-staged TMA kernels
@@ -136,8 +140,16 @@ struct stdg_solver {
 };
 
 namespace stdg {
+inline FxBlocks fx_blocks(const double* b, const uint16_t* e, const FxScale& r, const FxScale& c) {
+  return FxBlocks{reinterpret_cast<const int2*>(b), e, r, c};
+}
+inline FxBlocks blocks_B(const stdg_solver* s) { return fx_blocks(s->Bdiag, s->eB, s->fxs, s->fxs); }
+inline FxBlocks blocks_Bv(const stdg_solver* s) { return fx_blocks(s->Bv, s->eBv, s->fxs, s->fxs); }
+inline FxBlocks blocks_A(const stdg_solver* s) { return fx_blocks(s->Aoff, s->eA, s->fxs, s->fxs); }
+inline FxBlocks blocks_Q(const stdg_solver* s) { return fx_blocks(s->Q, s->eQ, s->fxt, s->fxs); }
+inline FxBlocks blocks_M(const stdg_solver* s) { return fx_blocks(s->Mij, s->eM, FxScale{}, FxScale{}); }
 inline FaceOps face_ops(const stdg_solver* s) {
-  return FaceOps{(int)s->ne, (int)s->nf, s->N, s->Ng, s->dm.t2f, s->dm.left, s->dm.right, s->Q, s->Mij, s->eQ, s->eM};
+  return FaceOps{s->fxws, (int)s->ne, (int)s->nf, s->N, s->Ng, s->tface, s->dm.left, s->dm.right, blocks_Q(s), blocks_M(s)};
 }
 // binary32 Krylov kernels (lowprec.cu), exposed as launch functions
 struct LpKernels {

@@ -7,7 +7,7 @@
 //             g_j = dt (I (x) K^-1) Sum_s Q^sp_sj p_s  (boundary: volume part only)  (Eq. prevpress)
 //   convection Upsilon^c_i (Eq. convdg, Rusanov flux, s_max = 2 max(|v+|, |v-|) pointwise)
 //   goback    F_j = Sum_s M^sp_sj^T vbar_s                                       (Eq. goback)
-//   viscous   |J_i| K-mixing + nu dt (-(A_sp x)_i + Bvisc_i x_i) = rhs          (Eq. A1_mod)
+//   viscous   |J_i| K-mixing + nu dt (-(A_off x)_i - Bv_i x_i) = rhs          (Eq. A1_mod)
 #include <chrono>
 #include <cmath>
 #include <cstring>
@@ -66,7 +66,7 @@ __global__ void k_trace(int nf, int N, int Ng, const int* __restrict__ right, GA
 // rhs[c][i][a][k] = |J| g0[a] Sum_b g1[b] vbar_n[c][i][b][k] - Ups[c][i][a][k] - |J| Sum_b K[a][b] Lam[c][i][b][k]
 //                   - nu Sum_{boundary f} Sum_d Sum_m Q^{bd,d}[m][k] G[j][c][d][a][m]
 __global__ void k_visc_rhs(int ne, int N, int Ng, const int* __restrict__ t2f, const int* __restrict__ t2n,
-                           const double* __restrict__ detJ, const double* __restrict__ Q, GArg g0, GArg g1, MArg K,
+                           const double* __restrict__ detJ, FxBlocks Q, GArg g0, GArg g1, MArg K,
                            double nu, const double* __restrict__ vbar_n, const double* __restrict__ Ups,
                            const double* __restrict__ Lam, const double* __restrict__ Gbc, double* __restrict__ rhs) {
   const int i = blockIdx.x, Nst = N * Ng;
@@ -86,9 +86,8 @@ __global__ void k_visc_rhs(int ne, int N, int Ng, const int* __restrict__ t2f, c
       const int j = t2f[4 * i + f];
       double bsum = 0.0;
       for (int d = 0; d < 3; ++d) {
-        const double* q = Q + ((size_t)j * 6 + d) * NN + k;
         const double* gg = Gbc + (((size_t)j * 3 + c) * 3 + d) * Nst + a * N;
-        for (int m = 0; m < N; ++m) bsum = fma(q[(size_t)m * N], gg[m], bsum);
+        for (int m = 0; m < N; ++m) bsum = fma(fx_entry(Q, 3 * NN, 2 * (size_t)j, d * (int)NN + m * N + k, N), gg[m], bsum);
       }
       s -= nu * bsum;
     }
@@ -1166,7 +1165,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     phase_mark(s, 2);
     // 3. viscous systems (Eq. A1_mod), one per component, initial guess vbar^{n+1,k}
     ++s->nlaunch;
-    k_visc_rhs<<<ne, 128, 0, st>>>(ne, N, Ng, s->dm.t2f, s->dm.t2n, s->dm.detJ, s->Q, g0, g1, K, nu, s->Vbar_n,
+    k_visc_rhs<<<ne, 128, 0, st>>>(ne, N, Ng, s->dm.t2f, s->dm.t2n, s->dm.detJ, blocks_Q(s), g0, g1, K, nu, s->Vbar_n,
                                    s->Ups, s->Lam, s->Gbc, s->rhsv);
     if (cudaGetLastError() != cudaSuccess) { set_error("step kernels failed to launch"); return STDG_ECUDA; }
     int vits = 0;

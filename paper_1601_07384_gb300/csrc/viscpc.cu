@@ -31,11 +31,10 @@ constexpr int kEigWarps = 4;                 // tets per block of the eigensolve
 constexpr int kEigSweeps = 16;               // cyclic sweeps (each annihilates every pair once)
 constexpr int kEigLd = kMaxN + 1;
 
-// G_i = Bvisc_i - B_i; eigenvectors (columns of U) and eigenvalues, one warp per tet.  Binary32: the
+// G_i = -Bv_i (Bv_i: the diagonal blocks of the viscous operator); eigenvectors (columns of U) and eigenvalues, one warp per tet.  Binary32: the
 // preconditioner needs a fixed approximate inverse, and binary64 rotations on sm_103a's FP64 pipe
 // made this setup ~200 ms at 10,368 tets, p = 4.
-__global__ void __launch_bounds__(32 * kEigWarps) k_visc_eig(int ne, int N, const double* __restrict__ Bdiag,
-                                                             const double* __restrict__ Bvisc, float* __restrict__ Uout,
+__global__ void __launch_bounds__(32 * kEigWarps) k_visc_eig(int ne, int N, FxBlocks Bv, float* __restrict__ Uout,
                                                              float* __restrict__ lam) {
   extern __shared__ float sm[];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -46,7 +45,7 @@ __global__ void __launch_bounds__(32 * kEigWarps) k_visc_eig(int ne, int N, cons
   for (int i = blockIdx.x * kEigWarps + w; i < ne; i += gridDim.x * kEigWarps) {
     for (int e = lane; e < N * N; e += 32) {
       const int r = e / N, c = e - r * N;
-      A[r * kEigLd + c] = (float)(Bvisc[(size_t)i * NN + e] - Bdiag[(size_t)i * NN + e]);
+      A[r * kEigLd + c] = (float)-fx_entry(Bv, NN, i, e, N);
       V[r * kEigLd + c] = r == c ? 1.0f : 0.0f;
     }
     __syncwarp();
@@ -511,7 +510,7 @@ stdg_status visc_pc_ensure(stdg_solver* s) {
   STDG_CUDA(cudaFuncSetAttribute(k_visc_eig, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   const int blocks = (int)std::min<int64_t>((s->ne + kEigWarps - 1) / kEigWarps, 152 * 16);
   ++s->nlaunch;
-  k_visc_eig<<<blocks, 32 * kEigWarps, smem, s->stream>>>((int)s->ne, s->N, s->Bdiag, s->Bvisc, s->vpcU, s->vpcLam);
+  k_visc_eig<<<blocks, 32 * kEigWarps, smem, s->stream>>>((int)s->ne, s->N, blocks_Bv(s), s->vpcU, s->vpcLam);
   STDG_LAUNCH_CHECK();
   return STDG_OK;
 }
