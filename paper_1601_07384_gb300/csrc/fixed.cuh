@@ -55,6 +55,15 @@ __device__ __forceinline__ double fx_entry(const FxBlocks& B, size_t len, size_t
   if (!fx_ok(e)) return scalbn(__hiloint2double(w.y, w.x), sc);
   return e ? scalbn((double)((long long)w.x * (1LL << kFxL) + w.y), e - 1022 - kFx + sc) : 0.0;
 }
+// rounded to binary32 (sc: the scaling of its row and column): of the 61 bits at once and without the binary64
+// pipe, where the value is certain to be in the normal range
+__device__ __forceinline__ float fx_entry_f32(const FxBlocks& B, size_t len, size_t b, int idx, int sc) {
+  const int2 w = B.w[b * len + idx];
+  const int e = B.e[b], k = e - 1022 - kFx + sc;
+  if (fx_ok(e) && k >= -120 && k <= 60) return __ll2float_rn((long long)w.x * (1LL << kFxL) + w.y) * __int_as_float((k + 127) << 23);
+  if (!fx_ok(e)) return (float)scalbn(__hiloint2double(w.y, w.x), sc);
+  return e ? (float)scalbn((double)((long long)w.x * (1LL << kFxL) + w.y), k) : 0.0f;
+}
 // the same on the host, for an entry copied as the 8 bytes that it is stored in
 inline double fx_entry_host(double raw, int e, int sc) {
   if (e != 0 && (e < kFxMinExp || e > 2046)) return std::ldexp(raw, sc);

@@ -297,7 +297,9 @@ __global__ void __launch_bounds__(256) k_fx_vec(const __grid_constant__ FxInput 
     if (!have) return;
     // exponents: of the columns before mixing where that takes the binary64 path (2047), else mixed
     const bool ok = fx_ok(e[0]) && fx_ok(mix.e);
-    if (k0 < NG) in.e[v * NG + k0] = (uint16_t)(e[0] == 0 ? 0 : ok ? e[0] : 2047);
+#pragma unroll
+    for (int q = 0; q < NG; ++q)
+      if (k0 == q % G) in.e[v * NG + q] = (uint16_t)(e[0] == 0 ? 0 : ok ? e[0] : 2047);
 #pragma unroll
     for (int j = 0; j < K; ++j) {
       const int k = k0 + j * G;
@@ -485,7 +487,7 @@ template <class P, int N, int NG>
 cudaError_t fx_launch_t(const P& a, const FxInput& in, const FxMat& mix, cudaStream_t st) {
   using T = FxTile<P, N, NG>;
   if (a.n <= 0) return cudaSuccess;
-  if (T::smem > 48 * 1024) {
+  if (T::smem > 40 * 1024) {                  // with the static part above the 48 KB that need no opt-in
     const cudaError_t e = cudaFuncSetAttribute(k_fx<P, N, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
     if (e != cudaSuccess) return e;
   }

@@ -457,46 +457,63 @@ __global__ void __launch_bounds__(128, 1) k_apply_warp(WarpArgs a, const typenam
   }
 }
 
-// padded block copies: dst block b = planes x NR x NP, zero outside N x N
-template <typename TB, int PLANES>
-__global__ void k_to_padded(int64_t nblk, int N, int NR, int NP, FxBlocks src, TB* __restrict__ dst) {
-  const int64_t per = (int64_t)PLANES * NR * NP;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / per;
-    const int rem = (int)(e - b * per);
-    const int plane = rem / (NR * NP);
-    const int rc = rem - plane * NR * NP;
-    const int r = rc / NP, c = rc - r * NP;
-    const double v = (r < N && c < N) ? fx_entry(src, (size_t)N * N, b, r * N + c, N) : 0.0;
-    if constexpr (sizeof(TB) == 2) {
-      dst[e] = __float2bfloat16_rn((float)v);
-    } else if constexpr (PLANES == 2) {
-      const float hi = (float)v;
-      dst[e] = plane == 0 ? hi : (float)(v - (double)hi);
-    } else {
-      dst[e] = (float)v;
+// padded block copies: dst block b = planes x NR x NP, zero outside N x N.  A CTA takes whole blocks, about 4,096
+// entries at a time, indices by divisions with constants and the scaling from shared memory (a constant-bank read
+// with an index per thread is repeated for each value); one plane is rounded to binary32 without the binary64
+// pipe.  Bound by memory: 82,944 tets, p = 3, 8 bytes read and 4 written per entry, both copies.
+template <typename TB, int PLANES, int N>
+__global__ void __launch_bounds__(256) k_to_padded(int64_t nblk, const __grid_constant__ FxBlocks src, TB* __restrict__ dst) {
+  constexpr int NR = warp_nr_c(N), NP = warp_np_c(N), pl = NR * NP, per = PLANES * pl, cta = per < 4096 ? 4096 / per : 1;
+  __shared__ signed char rs[NR], cs[NP];
+  if (threadIdx.x < NR) rs[threadIdx.x] = threadIdx.x < N ? src.r.s[threadIdx.x] : 0;
+  if (threadIdx.x < NP) cs[threadIdx.x] = threadIdx.x < N ? src.c.s[threadIdx.x] : 0;
+  __syncthreads();
+  for (int64_t b0 = (int64_t)blockIdx.x * cta; b0 < nblk; b0 += (int64_t)gridDim.x * cta) {
+    const int cnt = (nblk - b0 < cta ? (int)(nblk - b0) : cta) * per;
+#pragma unroll 4
+    for (int e = threadIdx.x; e < cnt; e += 256) {
+      const int b = e / per, rem = e - b * per, plane = rem / pl, rc = rem - plane * pl, r = rc / NP, c = rc - r * NP;
+      const bool in = r < N && c < N;
+      TB* out = dst + b0 * per + e;
+      if constexpr (PLANES == 2) {
+        const double v = in ? fx_entry(src, (size_t)N * N, b0 + b, r * N + c, N) : 0.0;
+        const float hi = (float)v;
+        *out = plane == 0 ? hi : (float)(v - (double)hi);
+      } else {
+        *out = (TB)(in ? fx_entry_f32(src, (size_t)N * N, b0 + b, r * N + c, rs[r] + cs[c]) : 0.0f);
+      }
     }
   }
 }
+template <typename TB, int PLANES>
+static cudaError_t to_padded(stdg_solver* s, int64_t nblk, const FxBlocks& src, void* dst) {
+  TB* d = static_cast<TB*>(dst);
+  switch (s->N) {
+    case 1: k_to_padded<TB, PLANES, 1><<<1216, 256, 0, s->stream>>>(nblk, src, d); break;
+    case 4: k_to_padded<TB, PLANES, 4><<<1216, 256, 0, s->stream>>>(nblk, src, d); break;
+    case 10: k_to_padded<TB, PLANES, 10><<<1216, 256, 0, s->stream>>>(nblk, src, d); break;
+    case 20: k_to_padded<TB, PLANES, 20><<<1216, 256, 0, s->stream>>>(nblk, src, d); break;
+    case 35: k_to_padded<TB, PLANES, 35><<<1216, 256, 0, s->stream>>>(nblk, src, d); break;
+    default: return cudaErrorInvalidValue;
+  }
+  ++s->nlaunch;
+  return cudaGetLastError();
+}
 
-static int warp_np(int N) { int np = N; while (np % 8 != 4) ++np; return np; }
-static int warp_nr(int N) { return (N + 3) / 4 * 4; }
 static uint32_t a16(size_t b) { return (uint32_t)((b + 15) & ~(size_t)15); }
 
 template <typename W>
 static cudaError_t ensure_warp_blocks(stdg_solver* s, void** Bd, void** Ao) {
   if (*Bd) return cudaSuccess;
   using TB = typename W::TB;
-  const int N = s->N, NR = warp_nr(N), NP = warp_np(N);
+  const int N = s->N, NR = warp_nr_c(N), NP = warp_np_c(N);
   const size_t per = (size_t)W::kPlanes * NR * NP;
   cudaError_t e = dev_alloc_cuda(s, Bd, (size_t)s->ne * per * sizeof(TB));
   if (e != cudaSuccess) return e;
   e = dev_alloc_cuda(s, Ao, (size_t)s->nf * per * sizeof(TB));
   if (e != cudaSuccess) return e;
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, blocks_B(s), static_cast<TB*>(*Bd));
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->nf, N, NR, NP, blocks_A(s), static_cast<TB*>(*Ao));
-  s->nlaunch += 2;
-  return cudaGetLastError();
+  e = to_padded<TB, W::kPlanes>(s, s->ne, blocks_B(s), *Bd);
+  return e != cudaSuccess ? e : to_padded<TB, W::kPlanes>(s, s->nf, blocks_A(s), *Ao);
 }
 
 // padded copy of the viscous diagonal blocks (Eq. A1_mod, with the face blocks A_lr)
@@ -504,19 +521,17 @@ template <typename W>
 static cudaError_t ensure_warp_visc_diag(stdg_solver* s, void** Bv) {
   if (*Bv) return cudaSuccess;
   using TB = typename W::TB;
-  const int N = s->N, NR = warp_nr(N), NP = warp_np(N);
+  const int N = s->N, NR = warp_nr_c(N), NP = warp_np_c(N);
   cudaError_t e = dev_alloc_cuda(s, Bv, (size_t)s->ne * W::kPlanes * NR * NP * sizeof(TB));
   if (e != cudaSuccess) return e;
-  k_to_padded<TB, W::kPlanes><<<1216, 256, 0, s->stream>>>(s->ne, N, NR, NP, blocks_Bv(s), static_cast<TB*>(*Bv));
-  ++s->nlaunch;
-  return cudaGetLastError();
+  return to_padded<TB, W::kPlanes>(s, s->ne, blocks_Bv(s), *Bv);
 }
 
 // Per warp: S stages of [5 blocks | x], then (pair policy only) the (hi, lo) z planes, then the S
 // mbarriers.  binary32 x is staged in rows of NR entries per time column, binary64 x as it is.
 static WarpArgs warp_layout(const stdg_solver* s, size_t tb, int planes, size_t xin, int S) {
   WarpArgs a{};
-  a.ne = (int)s->ne; a.N = s->N; a.NR = warp_nr(s->N); a.NP = warp_np(s->N); a.Nst = s->Nst; a.S = S;
+  a.ne = (int)s->ne; a.N = s->N; a.NR = warp_nr_c(s->N); a.NP = warp_np_c(s->N); a.Nst = s->Nst; a.S = S;
   a.plane_elems = (uint32_t)(a.NR * a.NP);
   a.blk_bytes = (uint32_t)(planes * a.plane_elems * tb);
   a.xraw_off = 5 * a.blk_bytes;
