@@ -14,7 +14,6 @@
 namespace stdg {
 namespace {
 
-constexpr int kC32Blocks = 1216;    // 8 x 152 SMs
 constexpr int kC32Threads = 256;
 
 // warp sum in binary32 (binary64 shuffle-adds would cost FP64-pipe time per thread on sm_103a)
@@ -31,7 +30,7 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_mix_to32(int ne, int N, Mix
   const int64_t total = (int64_t)ne * N;
   const int Nst = N * NG;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     float v[NG];
 #pragma unroll
@@ -53,7 +52,7 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_mix_acc64(int ne, int N, Mi
   const int64_t total = (int64_t)ne * N;
   const int Nst = N * NG;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     float v[NG];
 #pragma unroll
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_cross(int ne, int N, const 
   const int64_t total = (int64_t)ne * N;
   const int Nst = N * NG;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     float uu[NG], vv[NG];
 #pragma unroll
@@ -150,7 +149,7 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_update(int ne, int N, const
   const int Nst = N * NG;
   float acc = 0.0f;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     float pp[NG], qq[NG], rn[NG];
 #pragma unroll
@@ -192,7 +191,7 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_dir(int ne, int N, const do
   const int64_t total = (int64_t)ne * N;
   const int Nst = N * NG;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     float pp[NG];
 #pragma unroll
@@ -213,21 +212,21 @@ __global__ void __launch_bounds__(kC32Threads) k_c32_dir(int ne, int N, const do
     default: { constexpr int G = 5; CALL; } break; \
   }
 
-void c32_mix_to32(cudaStream_t st, int ne, int N, int Ng, const Mix32& M, const double* in, float* out) {
-  STDG_C32_NG_SWITCH(Ng, (k_c32_mix_to32<G><<<kC32Blocks, kC32Threads, 0, st>>>(ne, N, M, in, out)));
+void c32_mix_to32(cudaStream_t st, int grid, int ne, int N, int Ng, const Mix32& M, const double* in, float* out) {
+  STDG_C32_NG_SWITCH(Ng, (k_c32_mix_to32<G><<<grid, kC32Threads, 0, st>>>(ne, N, M, in, out)));
 }
-void c32_mix_acc64(cudaStream_t st, int ne, int N, int Ng, const Mix32& M, const float* y, double* x) {
-  STDG_C32_NG_SWITCH(Ng, (k_c32_mix_acc64<G><<<kC32Blocks, kC32Threads, 0, st>>>(ne, N, M, y, x)));
+void c32_mix_acc64(cudaStream_t st, int grid, int ne, int N, int Ng, const Mix32& M, const float* y, double* x) {
+  STDG_C32_NG_SWITCH(Ng, (k_c32_mix_acc64<G><<<grid, kC32Threads, 0, st>>>(ne, N, M, y, x)));
 }
-void c32_cross(cudaStream_t st, int ne, int N, int Ng, const float* u, const float* v, double* part) {
-  STDG_C32_NG_SWITCH(Ng, (k_c32_cross<G><<<kC32Blocks, kC32Threads, 0, st>>>(ne, N, u, v, part)));
+void c32_cross(cudaStream_t st, int grid, int ne, int N, int Ng, const float* u, const float* v, double* part) {
+  STDG_C32_NG_SWITCH(Ng, (k_c32_cross<G><<<grid, kC32Threads, 0, st>>>(ne, N, u, v, part)));
 }
-void c32_update(cudaStream_t st, int ne, int N, int Ng, const double* M, float* y, float* r, const float* p,
+void c32_update(cudaStream_t st, int grid, int ne, int N, int Ng, const double* M, float* y, float* r, const float* p,
                 const float* q, const Mix32& W, double* part, int want) {
-  STDG_C32_NG_SWITCH(Ng, (k_c32_update<G><<<kC32Blocks, kC32Threads, 0, st>>>(ne, N, M, y, r, p, q, W, part, want)));
+  STDG_C32_NG_SWITCH(Ng, (k_c32_update<G><<<grid, kC32Threads, 0, st>>>(ne, N, M, y, r, p, q, W, part, want)));
 }
-void c32_dir(cudaStream_t st, int ne, int N, int Ng, const double* M, const float* z, float* p) {
-  STDG_C32_NG_SWITCH(Ng, (k_c32_dir<G><<<kC32Blocks, kC32Threads, 0, st>>>(ne, N, M, z, p)));
+void c32_dir(cudaStream_t st, int grid, int ne, int N, int Ng, const double* M, const float* z, float* p) {
+  STDG_C32_NG_SWITCH(Ng, (k_c32_dir<G><<<grid, kC32Threads, 0, st>>>(ne, N, M, z, p)));
 }
 
 }  // namespace stdg

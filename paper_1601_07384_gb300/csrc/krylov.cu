@@ -16,7 +16,6 @@ namespace stdg {
 constexpr int kRedBlocks = 1216;   // 8 x 152 SMs
 constexpr int kRedThreads = 256;
 constexpr int kMaxCols = 64;
-constexpr int kLpBlocksK = 1216;   // partial rows the binary32 block-Jacobi kernels write (lowprec.cu)
 
 __device__ inline double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -39,50 +38,87 @@ __device__ inline void block_reduce_store(double* v, int cnt, double* part, int 
   }
 }
 
-// per-time-column dot products: part[b][a] = Sum over this block's elements of column a
-__global__ void __launch_bounds__(kRedThreads) k_coldot(int64_t n, int N, int Ng, const double* __restrict__ x,
-                                                       const double* __restrict__ y, double* part) {
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    int a = (int)((e / N) % Ng);
-    acc[a] = fma(x[e], y[e], acc[a]);
+// Blocks of the vector kernels and reductions over `items` (tet, row) pairs: one thread per pair up to
+// kRedBlocks blocks.  (Every block ends with a reduction on the binary64 pipe, so blocks without work are not
+// free: 1,216 blocks for 30,720 pairs took 6.2 us per dot product.)
+static int red_grid(int64_t items) {
+  const int64_t b = (items + kRedThreads - 1) / kRedThreads;
+  return (int)(b < 1 ? 1 : b > kRedBlocks ? kRedBlocks : b);
+}
+
+// Block-reduce CNT per-thread values into part[blockIdx.x * CNT + c]
+template <int CNT>
+__device__ inline void block_sums_store(const double (&v)[CNT], double* part) {
+  __shared__ double red[8][kRedThreads / 32];
+  int col;
+  const double t = warp_sums<CNT>(v, col);
+  red[col][threadIdx.x >> 5] = t;                  // the lanes that share a column write the same value
+  __syncthreads();
+  if (threadIdx.x < CNT) {
+    double s = 0.0;
+    for (int k = 0; k < kRedThreads / 32; ++k) s += red[threadIdx.x][k];
+    part[(size_t)blockIdx.x * CNT + threadIdx.x] = s;
   }
-  block_reduce_store(acc, Ng, part, Ng);
+}
+// per-time-column dot products: part[b][a] = Sum over this block's elements of column a
+template <int NG>
+__global__ void __launch_bounds__(kRedThreads) k_coldot(int64_t npairs, int N, const double* __restrict__ x,
+                                                       const double* __restrict__ y, double* part) {
+  double acc[NG];
+#pragma unroll
+  for (int a = 0; a < NG; ++a) acc[a] = 0.0;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+#pragma unroll
+    for (int a = 0; a < NG; ++a) acc[a] = fma(x[o + a * N], y[o + a * N], acc[a]);
+  }
+  block_sums_store<NG>(acc, part);
+}
+static void coldot(cudaStream_t st, int rb, int64_t npairs, int N, int Ng, const double* x, const double* y, double* part) {
+  STDG_NG_SWITCH(Ng, (k_coldot<G><<<rb, kRedThreads, 0, st>>>(npairs, N, x, y, part)));
 }
 
 // x += alpha_a p; r -= alpha_a q; partials of r.r per column (slot a) and of ||(I (x) Tp) r||^2 (slot Ng)
 struct TpArg { double v[kMaxNg * kMaxNg]; };
 // want = 0 (block-Jacobi PCG between convergence checks): only the x and r updates; the binary64
 // pipe is 1/64 of the binary32 rate on sm_103a, so the norms are not formed when nobody reads them.
-__global__ void __launch_bounds__(kRedThreads) k_cg_update(int64_t ne, int N, int Ng, const double* __restrict__ alpha,
+template <int NG>
+__global__ void __launch_bounds__(kRedThreads) k_cg_update(int64_t npairs, int N, const double* __restrict__ alpha,
                                                           double* __restrict__ x, double* __restrict__ r,
                                                           const double* __restrict__ p, const double* __restrict__ q,
-                                                          TpArg Tp, double* part, int want = 1) {
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  double al[kMaxNg];
-  for (int a = 0; a < Ng; ++a) al[a] = alpha[a];
-  const int64_t npairs = ne * N;
-  const int Nst = N * Ng;
+                                                          TpArg Tp, double* part, int want) {
+  double acc[NG + 1], al[NG];
+#pragma unroll
+  for (int a = 0; a < NG; ++a) al[a] = alpha[a];
+#pragma unroll
+  for (int a = 0; a <= NG; ++a) acc[a] = 0.0;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
-    const int k = (int)(e % N);
-    double rv[kMaxNg];
-    for (int a = 0; a < Ng; ++a) {
-      const int64_t o = i * Nst + a * N + k;
-      x[o] = fma(al[a], p[o], x[o]);
-      double rn = fma(-al[a], q[o], r[o]);
-      r[o] = rn;
-      rv[a] = rn;
-      if (want) acc[a] = fma(rn, rn, acc[a]);
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+    double rv[NG];
+#pragma unroll
+    for (int a = 0; a < NG; ++a) {
+      x[o + a * N] = fma(al[a], p[o + a * N], x[o + a * N]);
+      rv[a] = fma(-al[a], q[o + a * N], r[o + a * N]);
+      r[o + a * N] = rv[a];
+      if (want) acc[a] = fma(rv[a], rv[a], acc[a]);
     }
-    if (want)
-      for (int a = 0; a < Ng; ++a) {
+    if (want) {
+#pragma unroll
+      for (int a = 0; a < NG; ++a) {
         double w = 0.0;
-        for (int b = 0; b < Ng; ++b) w = fma(Tp.v[a * Ng + b], rv[b], w);
-        acc[Ng] = fma(w, w, acc[Ng]);
+#pragma unroll
+        for (int b = 0; b < NG; ++b) w = fma(Tp.v[a * NG + b], rv[b], w);
+        acc[NG] = fma(w, w, acc[NG]);
       }
+    }
   }
-  if (want) block_reduce_store(acc, Ng + 1, part, Ng + 1);
+  if (want) block_sums_store<NG + 1>(acc, part);
+}
+static void cg_update(cudaStream_t st, int rb, int64_t npairs, int N, int Ng, const double* alpha, double* x, double* r,
+                      const double* p, const double* q, const TpArg& Tp, double* part, int want = 1) {
+  STDG_NG_SWITCH(Ng, (k_cg_update<G><<<rb, kRedThreads, 0, st>>>(npairs, N, alpha, x, r, p, q, Tp, part, want)));
 }
 
 // z_i[a][k] = Sum_l Binv_i[k][l] r_i[a][l]  (block Jacobi); partials of r.z per column a.
@@ -164,23 +200,44 @@ __global__ void __launch_bounds__(256) k_bjacobi32(int ne, int N, int Ng, const 
   }
 }
 
-// beta_a = rznew_a / rz_a; rz <- rznew; res = sqrt(mix2)
-__global__ void k_cg_beta2(int Ng, double* rz, const double* rznew, double* beta, double* res, const double* mix2) {
-  int a = threadIdx.x;
-  if (a < Ng) {
-    beta[a] = (rz[a] != 0.0) ? rznew[a] / rz[a] : 0.0;
-    rz[a] = rznew[a];
+// The end of a plain CG iteration, one block per slot of the Ng + 1 partial sums (k_cg_update): rznew_a, then
+// beta_a = rznew_a / rz_a, rz_a <- rznew_a; slot Ng: res = sqrt
+__global__ void k_final_beta_res(int nparts, int Ng, const double* __restrict__ part, double* rz, double* beta, double* res) {
+  __shared__ double red[kRedThreads / 32];
+  const int a = blockIdx.x;
+  double s = 0.0;
+  for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += part[(size_t)b * (Ng + 1) + a];
+  s = warp_sum(s);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int k = 0; k < kRedThreads / 32; ++k) t += red[k];
+    if (a == Ng) {
+      res[0] = sqrt(t);
+    } else {
+      beta[a] = rz[a] != 0.0 ? t / rz[a] : 0.0;
+      rz[a] = t;
+    }
   }
-  if (a == 0) res[0] = sqrt(mix2[0]);
 }
 
 // p = r + beta_a p
-__global__ void k_cg_dir(int64_t n, int N, int Ng, const double* __restrict__ beta, const double* __restrict__ r,
-                         double* __restrict__ p) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    int a = (int)((e / N) % Ng);
-    p[e] = fma(beta[a], p[e], r[e]);
+template <int NG>
+__global__ void __launch_bounds__(kRedThreads) k_cg_dir(int64_t npairs, int N, const double* __restrict__ beta,
+                                                       const double* __restrict__ r, double* __restrict__ p) {
+  double be[NG];
+#pragma unroll
+  for (int a = 0; a < NG; ++a) be[a] = beta[a];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+#pragma unroll
+    for (int a = 0; a < NG; ++a) p[o + a * N] = fma(be[a], p[o + a * N], r[o + a * N]);
   }
+}
+static void cg_dir(cudaStream_t st, int rb, int64_t npairs, int N, int Ng, const double* beta, const double* r, double* p) {
+  STDG_NG_SWITCH(Ng, (k_cg_dir<G><<<rb, kRedThreads, 0, st>>>(npairs, N, beta, r, p)));
 }
 
 // out[c] = Sum_b part[b * width + c] in fixed order (one block per column)
@@ -224,27 +281,36 @@ __global__ void k_cg_alpha_guard(int Ng, const double* rr, const double* pq, dou
   if (a < Ng) alpha[a] = bad ? 0.0 : al;
   if (a == 0 && bad) flag[0] = 1.0;
 }
-// One block: reduce the per-block p.q partials of every column in a fixed order, then the guarded
-// step length of k_cg_alpha_guard (one launch instead of two per binary32 iteration).
-__global__ void k_final_alpha_guard(int nparts, int Ng, const double* __restrict__ part, const double* rz,
-                                    double* alpha, double* flag) {
-  __shared__ double red[kMaxNg][kRedThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int a = 0; a < Ng; ++a) {
-    double s = 0.0;
-    for (int b = threadIdx.x; b < nparts; b += blockDim.x) s += part[(size_t)b * Ng + a];
-    s = warp_sum(s);
-    if (lane == 0) red[a][w] = s;
+// Sums of `width` columns of partials by one block of T = 1024 / width * width threads, in a fixed order:
+// thread t adds entries t, t + T, ... (all of column t % width), warp c the threads' sums of column c, c + 32, ...
+// out: shared, [width].  (One column after another with 256 threads took 11 us for 5 columns.)
+__device__ inline void block_column_sums(int nparts, int width, const double* __restrict__ part, double* scratch, double* out) {
+  const int T = 1024 / width * width, t = threadIdx.x;
+  double s = 0.0;
+  if (t < T)
+    for (int e = t; e < nparts * width; e += T) s += part[e];
+  scratch[t] = s;
+  __syncthreads();
+  for (int c = t >> 5; c < width; c += 32) {
+    double v = 0.0;
+    for (int k = c + (t & 31) * width; k < T; k += 32 * width) v += scratch[k];
+    v = warp_sum(v);
+    if ((t & 31) == 0) out[c] = v;
   }
   __syncthreads();
+}
+// One block: reduce the per-block p.q partials of every column, then the guarded step length of
+// k_cg_alpha_guard (one launch instead of two per binary32 iteration).
+__global__ void __launch_bounds__(1024) k_final_alpha_guard(int nparts, int Ng, const double* __restrict__ part,
+                                                            const double* rz, double* alpha, double* flag) {
+  __shared__ double scratch[1024], pq[kMaxNg];
+  block_column_sums(nparts, Ng, part, scratch, pq);
   if (threadIdx.x == 0) {
     double al[kMaxNg];
     bool bad = flag[0] != 0.0;
     for (int a = 0; a < Ng; ++a) {
-      double pq = 0.0;
-      for (int q = 0; q < (int)(blockDim.x >> 5); ++q) pq += red[a][q];
-      al[a] = rz[a] / pq;
-      if (!(pq > 0.0) || !isfinite(al[a])) bad = true;
+      al[a] = rz[a] / pq[a];
+      if (!(pq[a] > 0.0) || !isfinite(al[a])) bad = true;
     }
     for (int a = 0; a < Ng; ++a) alpha[a] = bad ? 0.0 : al[a];
     if (bad) flag[0] = 1.0;
@@ -269,8 +335,8 @@ __global__ void __launch_bounds__(kRedThreads) k_visc_mass_inv(int64_t ne, int N
   double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   const int Nst = N * Ng;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
-    const int k = (int)(e % N);
+    const int64_t i = (uint32_t)e / (uint32_t)N;
+    const int k = (int)(e - i * N);
     const double c = 1.0 / (mass * detJ[i]);
     double rv[kMaxNg];
     for (int b = 0; b < Ng; ++b) rv[b] = r[i * Nst + b * N + k];
@@ -342,24 +408,29 @@ __global__ void k_final_res(int nparts, int width, int slot, const double* __res
   }
 }
 // flexible CG with m stored directions: per direction j (blockIdx.y) and column a, partials of z.Q_j
-__global__ void __launch_bounds__(kRedThreads) k_fcg_dots(int64_t n, int N, int Ng, int m, const double* __restrict__ Qb,
+template <int NG>
+__global__ void __launch_bounds__(kRedThreads) k_fcg_dots(int64_t npairs, int N, int m, const double* __restrict__ Qb,
                                                          const double* __restrict__ z, double* part) {
   const int j = blockIdx.y;
-  const double* Q = Qb + (size_t)j * n;
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    acc[(e / N) % Ng] = fma(z[e], Q[e], acc[(e / N) % Ng]);
-  __shared__ double red[8][kRedThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int c = 0; c < Ng; ++c) {
-    double s = warp_sum(acc[c]);
-    if (lane == 0) red[c][w] = s;
+  const double* Q = Qb + (size_t)j * npairs * NG;
+  double acc[NG];
+#pragma unroll
+  for (int a = 0; a < NG; ++a) acc[a] = 0.0;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+#pragma unroll
+    for (int a = 0; a < NG; ++a) acc[a] = fma(z[o + a * N], Q[o + a * N], acc[a]);
   }
+  __shared__ double red[8][kRedThreads / 32];
+  int col;
+  const double t = warp_sums<NG>(acc, col);
+  red[col][threadIdx.x >> 5] = t;
   __syncthreads();
-  if (threadIdx.x < Ng) {
+  if (threadIdx.x < NG) {
     double s = 0.0;
     for (int q = 0; q < kRedThreads / 32; ++q) s += red[threadIdx.x][q];
-    part[(size_t)blockIdx.x * m * Ng + j * Ng + threadIdx.x] = s;
+    part[((size_t)blockIdx.x * m + j) * NG + threadIdx.x] = s;
   }
 }
 // c[j][a] = -(z.Q_j)_a / (P_j.Q_j)_a
@@ -367,13 +438,23 @@ __global__ void k_fcg_coef(int cnt, const double* zq, const double* pq, double* 
   for (int t = threadIdx.x; t < cnt; t += blockDim.x) c[t] = pq[t] != 0.0 ? -zq[t] / pq[t] : 0.0;
 }
 // p = z + Sum_j c[j][a] P_j  (column a of each entry)
-__global__ void k_fcg_dir(int64_t n, int N, int Ng, int m, const double* __restrict__ c, const double* __restrict__ Pb,
-                          const double* __restrict__ z, double* __restrict__ p) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int a = (int)((e / N) % Ng);
-    double v = z[e];
-    for (int j = 0; j < m; ++j) v = fma(c[j * Ng + a], Pb[(size_t)j * n + e], v);
-    p[e] = v;
+template <int NG>
+__global__ void __launch_bounds__(kRedThreads) k_fcg_dir(int64_t npairs, int N, int m, const double* __restrict__ c,
+                                                        const double* __restrict__ Pb, const double* __restrict__ z,
+                                                        double* __restrict__ p) {
+  const int64_t n = npairs * NG;
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+    double v[NG];
+#pragma unroll
+    for (int a = 0; a < NG; ++a) v[a] = z[o + a * N];
+    for (int j = 0; j < m; ++j) {
+#pragma unroll
+      for (int a = 0; a < NG; ++a) v[a] = fma(c[j * NG + a], Pb[(size_t)j * n + o + a * N], v[a]);
+    }
+#pragma unroll
+    for (int a = 0; a < NG; ++a) p[o + a * N] = v[a];
   }
 }
 // beta_a = rrnew_a / rr_a; rr <- rrnew; res = sqrt(tp2)
@@ -391,8 +472,8 @@ __global__ void k_timemix(int64_t ne, int N, int Ng, TpArg M, double coef, const
                           double* __restrict__ out) {
   const int Nst = N * Ng;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
-    const int k = (int)(e % N);
+    const int64_t i = (uint32_t)e / (uint32_t)N;
+    const int k = (int)(e - i * N);
     double v[kMaxNg];
     for (int b = 0; b < Ng; ++b) v[b] = in[i * Nst + b * N + k];
     for (int a = 0; a < Ng; ++a) {
@@ -511,10 +592,11 @@ static stdg_status ensure_basis(stdg_solver* s, int cols) {
 }
 
 static double host_norm(stdg_solver* s, const double* v, int64_t n) {
+  const int rb = red_grid(s->ne * (int64_t)s->N);
   ++s->nlaunch;
-  k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, v, s->part);
+  k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, v, s->part);
   ++s->nlaunch;
-  k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, s->part, s->scal + 900);
+  k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, s->part, s->scal + 900);
   cudaMemcpyAsync(s->hostbuf + 900, s->scal + 900, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   cudaStreamSynchronize(s->stream);
   return std::sqrt(s->hostbuf[900]);
@@ -722,14 +804,12 @@ static stdg_status run_batched(stdg_solver* s, int B, int kernels_per_iter, int 
         s->kind_n[kind] += 1;
       }
     }
-    bool done = false;
-    for (int j = last_only ? B - 1 : 0; j < B; ++j) {
-      rabs = s->hostbuf[j];
-      if (!std::isfinite(rabs)) { set_error("Krylov: non-finite residual"); st = STDG_ENAN; break; }
-      if (rabs <= tol_abs) { done = true; }
-    }
+    for (int j = last_only ? B - 1 : 0; j < B; ++j)
+      if (!std::isfinite(s->hostbuf[j])) { set_error("Krylov: non-finite residual"); st = STDG_ENAN; break; }
+    // the iterate returned is the batch's last: the residual norms are not monotone, and an earlier one of the
+    // batch that met the tolerance does not count
     rabs = s->hostbuf[B - 1];
-    if (done) break;
+    if (rabs <= tol_abs) break;
   }
   if (exec) cudaGraphExecDestroy(exec);
   if (graph) cudaGraphDestroy(graph);
@@ -761,10 +841,11 @@ static stdg_status ensure_block_inverse(stdg_solver* s) {
 static stdg_status cg_block(stdg_solver* s, const ApplyArgs& op, const double* rhs, double* x, bool zero_x0,
                             const TpArg& mix, double tol_abs, int* iters, double* res_abs, int precond = 0) {
   const int N = s->N, Ng = s->Ng;
-  const int64_t n = s->ne * (int64_t)s->Nst;
+  const int64_t n = s->ne * (int64_t)s->Nst, npairs = s->ne * (int64_t)N;
+  const int rb = red_grid(npairs);
   double* r = s->kr; double* p = s->kp; double* q = s->kq; double* z = s->kz;
-  double* rz = s->scal; double* pq = s->scal + 8; double* alpha = s->scal + 16; double* beta = s->scal + 24;
-  double* rrnew = s->scal + 32; double* res = s->scal + 48; double* rznew = s->scal + 56;
+  double* rz = s->scal; double* alpha = s->scal + 16; double* beta = s->scal + 24;
+  double* res = s->scal + 48;
   const int bj_tb = s->Nst > 256 ? 1 : 256 / s->Nst;
   const int bj_threads = bj_tb * s->Nst > 256 ? s->Nst : 256;
   const size_t bj_smem = (size_t)bj_tb * s->Nst * sizeof(float);
@@ -773,10 +854,10 @@ static stdg_status cg_block(stdg_solver* s, const ApplyArgs& op, const double* r
     if (e == STDG_OK && precond == 2) e = mg_ensure(s);
     if (e != STDG_OK) return e;
   }
-  // block Jacobi writes kRedBlocks rows of r.z partials, the coarse correction its own rows after them
+  // block Jacobi writes rb rows of r.z partials, the coarse correction its own rows after them
   const bool mg = precond == 2;
-  const int nrz = kRedBlocks + (mg ? mg_partial_blocks() : 0);
-  double* mgpart = s->part + (size_t)kRedBlocks * Ng;
+  const int nrz = rb + (mg ? mg_partial_blocks(s) : 0);
+  double* mgpart = s->part + (size_t)rb * Ng;
   if (zero_x0) {
     cudaMemsetAsync(x, 0, n * sizeof(double), s->stream);
     cudaMemcpyAsync(r, rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
@@ -784,20 +865,20 @@ static stdg_status cg_block(stdg_solver* s, const ApplyArgs& op, const double* r
     stdg_status e = op_apply(s, op, x, r);
     if (e != STDG_OK) return e;
     ++s->nlaunch;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, rhs, nullptr, 1, r);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, rhs, nullptr, 1, r);
   }
   if (precond) {
     ++s->nlaunch;
-    k_bjacobi32<<<kRedBlocks, bj_threads, bj_smem, s->stream>>>((int)s->ne, N, Ng, s->lpBinv, r, z, s->part);
+    k_bjacobi32<<<rb, bj_threads, bj_smem, s->stream>>>((int)s->ne, N, Ng, s->lpBinv, r, z, s->part);
     if (mg) { mg_apply_f64(s, r, z, mgpart); s->nlaunch += mg_launches(s); }
     cudaMemcpyAsync(p, z, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
   } else {
     cudaMemcpyAsync(p, r, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
     ++s->nlaunch;
-    k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, r, r, s->part);
+    coldot(s->stream, rb, npairs, N, Ng, r, r, s->part);
   }
   ++s->nlaunch;
-  k_final<<<Ng, kRedThreads, 0, s->stream>>>(precond ? nrz : kRedBlocks, Ng, s->part, rz);
+  k_final<<<Ng, kRedThreads, 0, s->stream>>>(precond ? nrz : rb, Ng, s->part, rz);
   // one CG iteration; ends by copying the full-system residual norm to the host.  With the
   // preconditioner, inside a captured batch only the batch's last iteration forms the norm (the
   // host reads only that one), and the step length / beta come from fused reduction kernels.
@@ -807,29 +888,27 @@ static stdg_status cg_block(stdg_solver* s, const ApplyArgs& op, const double* r
     stdg_status e = op_apply(s, op, p, q);
     if (evs) cudaEventRecordWithFlags(evs[1], s->stream, cudaEventRecordExternal);
     if (e != STDG_OK) return e;
-    k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, p, q, s->part);
+    coldot(s->stream, rb, npairs, N, Ng, p, q, s->part);
     if (precond) {
       const int want = slot == Bb - 1;
-      k_final_alpha<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, s->part, rz, alpha);
-      k_cg_update<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, alpha, x, r, p, q, mix, s->part, want);
-      if (want) k_final_res<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng + 1, Ng, s->part, res);
-      k_bjacobi32<<<kRedBlocks, bj_threads, bj_smem, s->stream>>>((int)s->ne, N, Ng, s->lpBinv, r, z, s->part);
+      k_final_alpha<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, s->part, rz, alpha);
+      cg_update(s->stream, rb, npairs, N, Ng, alpha, x, r, p, q, mix, s->part, want);
+      if (want) k_final_res<<<1, kRedThreads, 0, s->stream>>>(rb, Ng + 1, Ng, s->part, res);
+      k_bjacobi32<<<rb, bj_threads, bj_smem, s->stream>>>((int)s->ne, N, Ng, s->lpBinv, r, z, s->part);
       if (mg) mg_apply_f64(s, r, z, mgpart);
       k_final_beta<<<Ng, kRedThreads, 0, s->stream>>>(nrz, Ng, s->part, rz, beta);
-      k_cg_dir<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, beta, z, p);
+      cg_dir(s->stream, rb, npairs, N, Ng, beta, z, p);
       if (want) cudaMemcpyAsync(s->hostbuf + slot, res, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
       return STDG_OK;
     }
-    k_final<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, s->part, pq);
-    k_cg_alpha<<<1, 32, 0, s->stream>>>(Ng, rz, pq, alpha);
-    k_cg_update<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, alpha, x, r, p, q, mix, s->part);
-    k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng + 1, s->part, rrnew);
-    k_cg_beta2<<<1, 32, 0, s->stream>>>(Ng, rz, rrnew, beta, res, rrnew + Ng);
-    k_cg_dir<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, beta, r, p);
+    k_final_alpha<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, s->part, rz, alpha);
+    cg_update(s->stream, rb, npairs, N, Ng, alpha, x, r, p, q, mix, s->part);
+    k_final_beta_res<<<Ng + 1, kRedThreads, 0, s->stream>>>(rb, Ng, s->part, rz, beta, res);
+    cg_dir(s->stream, rb, npairs, N, Ng, beta, r, p);
     cudaMemcpyAsync(s->hostbuf + slot, res, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     return STDG_OK;
   };
-  const int kpi = precond ? 7 + mg_launches(s) : 8;
+  const int kpi = precond ? 7 + mg_launches(s) : 6;
   int it = 0;
   double rabs = INFINITY;
   const int maxit = s->opt.max_iters;
@@ -866,6 +945,7 @@ static stdg_status gmres(stdg_solver* s, const ApplyArgs& op, const double* b, d
                          double tol_abs, int* iters, int* nrestarts, double* res_abs, int restart = 0,
                          double pc_nu = -1.0) {
   const int m = restart > 0 ? restart : s->opt.restart;
+  const int rb = red_grid(s->ne * (int64_t)s->N);
   const int64_t n = s->ne * (int64_t)s->Nst;
   const bool pc = pc_nu >= 0.0;
   stdg_status e = ensure_basis(s, m + 1);
@@ -881,14 +961,14 @@ static stdg_status gmres(stdg_solver* s, const ApplyArgs& op, const double* b, d
     e = op_apply(s, op, x, s->kq);
     if (e != STDG_OK) return e;
     ++s->nlaunch;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
     beta = host_norm(s, s->kq, n);
     if (!std::isfinite(beta)) { set_error("GMRES: non-finite residual"); return STDG_ENAN; }
     if (beta <= tol_abs || it >= maxit) break;
     s->hostbuf[901] = beta * beta;
     cudaMemcpyAsync(s->scal + 901, s->hostbuf + 901, sizeof(double), cudaMemcpyHostToDevice, s->stream);
     ++s->nlaunch;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, s->kq, s->scal + 901, 0, s->basis);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, s->kq, s->scal + 901, 0, s->basis);
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int k = 0;
@@ -902,23 +982,23 @@ static stdg_status gmres(stdg_solver* s, const ApplyArgs& op, const double* b, d
       }
       if (e != STDG_OK) return e;
       // classical Gram-Schmidt, second pass only when the first cancelled (gate at hd[260])
-      k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, s->part);
-      k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, s->part, hd + 258);
+      k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, w, s->part);
+      k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, s->part, hd + 258);
       for (int pass = 0; pass < 2; ++pass) {
         double* hp = hd + pass * 128;
         const double* gate = pass == 0 ? nullptr : hd + 260;
         if (pass == 1) k_reorth_gate<<<1, 32, 0, s->stream>>>(k + 1, hd, hd + 258, hd + 260);
-        k_multidot<<<dim3(kRedBlocks, k + 1), kRedThreads, 0, s->stream>>>(n, s->basis, w, s->part, gate);
-        k_final<<<k + 1, kRedThreads, 0, s->stream>>>(kRedBlocks, k + 1, s->part, hp, gate);
-        k_multiaxpy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, k + 1, s->basis, hp, -1.0, w, gate);
+        k_multidot<<<dim3(rb, k + 1), kRedThreads, 0, s->stream>>>(n, s->basis, w, s->part, gate);
+        k_final<<<k + 1, kRedThreads, 0, s->stream>>>(rb, k + 1, s->part, hp, gate);
+        k_multiaxpy<<<rb, kRedThreads, 0, s->stream>>>(n, k + 1, s->basis, hp, -1.0, w, gate);
       }
       s->nlaunch += 9;
       ++s->nlaunch;
-      k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, s->part);
+      k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, w, s->part);
       ++s->nlaunch;
-      k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, s->part, hd + 256);
+      k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, s->part, hd + 256);
       ++s->nlaunch;
-      k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, hd + 256, 0, w);
+      k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, w, hd + 256, 0, w);
       cudaMemcpyAsync(s->hostbuf, hd, 257 * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
       if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("GMRES: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
       for (int i = 0; i <= k; ++i) H[(size_t)i * m + k] = s->hostbuf[i] + s->hostbuf[128 + i];
@@ -950,10 +1030,10 @@ static stdg_status gmres(stdg_solver* s, const ApplyArgs& op, const double* b, d
     ++s->nlaunch;
     if (pc) {
       cudaMemsetAsync(s->kp, 0, n * sizeof(double), s->stream);
-      k_multiaxpy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, k, s->basis, hd, 1.0, s->kp);
+      k_multiaxpy<<<rb, kRedThreads, 0, s->stream>>>(n, k, s->basis, hd, 1.0, s->kp);
       if ((e = visc_pc_apply(s, pc_nu, s->kp, x, 1)) != STDG_OK) return e;
     } else {
-      k_multiaxpy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, k, s->basis, hd, 1.0, x);
+      k_multiaxpy<<<rb, kRedThreads, 0, s->stream>>>(n, k, s->basis, hd, 1.0, x);
     }
     ++restarts;
   }
@@ -974,6 +1054,7 @@ static stdg_status fgmres(stdg_solver* s, const ApplyArgs& op, const double* b, 
   TpArg Kinv{};
   for (int c = 0; c < s->Ng * s->Ng; ++c) Kinv.v[c] = s->Kinv[c];
   const int m0 = s->opt.restart;
+  const int rb = red_grid(s->ne * (int64_t)s->N);
   const int m = m0 + (use_gnn ? 1 : 0);            // directions per cycle
   const int64_t n = s->ne * (int64_t)s->Nst;
   stdg_status e = ensure_basis(s, m + 1);
@@ -989,14 +1070,14 @@ static stdg_status fgmres(stdg_solver* s, const ApplyArgs& op, const double* b, 
     e = op_apply(s, op, x, s->kq);
     if (e != STDG_OK) return e;
     ++s->nlaunch;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
     beta = host_norm(s, s->kq, n);
     if (!std::isfinite(beta)) { set_error("GMRES: non-finite residual"); return STDG_ENAN; }
     if (beta <= tol_abs || it >= maxit) break;
     s->hostbuf[901] = beta * beta;
     cudaMemcpyAsync(s->scal + 901, s->hostbuf + 901, sizeof(double), cudaMemcpyHostToDevice, s->stream);
     ++s->nlaunch;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, s->kq, s->scal + 901, 0, s->basis);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, s->kq, s->scal + 901, 0, s->basis);
     std::fill(g.begin(), g.end(), 0.0);
     g[0] = beta;
     int k = 0;
@@ -1004,7 +1085,7 @@ static stdg_status fgmres(stdg_solver* s, const ApplyArgs& op, const double* b, 
       double* w = s->basis + (size_t)(k + 1) * n;
       double* zk = s->kzz + (size_t)k * n;
       if (visc) {                                 // viscous systems: inverse of the mass part
-        k_visc_mass_inv<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, s->N, s->Ng, Kinv, op.mass_coef, op.detJ,
+        k_visc_mass_inv<<<rb, kRedThreads, 0, s->stream>>>(s->ne, s->N, s->Ng, Kinv, op.mass_coef, op.detJ,
                                                                     s->basis + (size_t)k * n, zk, nullptr);
         ++s->nlaunch;
         e = STDG_OK;
@@ -1015,23 +1096,23 @@ static stdg_status fgmres(stdg_solver* s, const ApplyArgs& op, const double* b, 
       e = op_apply(s, op, zk, w);
       if (e != STDG_OK) return e;
       // classical Gram-Schmidt, second pass only when the first cancelled (gate at hd[260])
-      k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, s->part);
-      k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, s->part, hd + 258);
+      k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, w, s->part);
+      k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, s->part, hd + 258);
       for (int pass = 0; pass < 2; ++pass) {
         double* hp = hd + pass * 128;
         const double* gate = pass == 0 ? nullptr : hd + 260;
         if (pass == 1) k_reorth_gate<<<1, 32, 0, s->stream>>>(k + 1, hd, hd + 258, hd + 260);
-        k_multidot<<<dim3(kRedBlocks, k + 1), kRedThreads, 0, s->stream>>>(n, s->basis, w, s->part, gate);
-        k_final<<<k + 1, kRedThreads, 0, s->stream>>>(kRedBlocks, k + 1, s->part, hp, gate);
-        k_multiaxpy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, k + 1, s->basis, hp, -1.0, w, gate);
+        k_multidot<<<dim3(rb, k + 1), kRedThreads, 0, s->stream>>>(n, s->basis, w, s->part, gate);
+        k_final<<<k + 1, kRedThreads, 0, s->stream>>>(rb, k + 1, s->part, hp, gate);
+        k_multiaxpy<<<rb, kRedThreads, 0, s->stream>>>(n, k + 1, s->basis, hp, -1.0, w, gate);
       }
       s->nlaunch += 9;
       ++s->nlaunch;
-      k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, s->part);
+      k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, w, s->part);
       ++s->nlaunch;
-      k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, s->part, hd + 256);
+      k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, s->part, hd + 256);
       ++s->nlaunch;
-      k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, w, hd + 256, 0, w);
+      k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, w, hd + 256, 0, w);
       cudaMemcpyAsync(s->hostbuf, hd, 257 * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
       if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("GMRES: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
       for (int i = 0; i <= k; ++i) H[(size_t)i * m + k] = s->hostbuf[i] + s->hostbuf[128 + i];
@@ -1061,7 +1142,7 @@ static stdg_status fgmres(stdg_solver* s, const ApplyArgs& op, const double* b, 
     std::memcpy(s->hostbuf, y.data(), k * sizeof(double));
     cudaMemcpyAsync(hd, s->hostbuf, k * sizeof(double), cudaMemcpyHostToDevice, s->stream);
     ++s->nlaunch;
-    k_multiaxpy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, k, s->kzz, hd, 1.0, x);
+    k_multiaxpy<<<rb, kRedThreads, 0, s->stream>>>(n, k, s->kzz, hd, 1.0, x);
     ++restarts;
   }
   *iters = it; *nrestarts = restarts; *res_abs = beta;
@@ -1103,10 +1184,12 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
   stdg_status e = ensure_lowprec(s);
   if (e == STDG_OK && mg) e = mg_ensure(s);
   if (e != STDG_OK) return e;
-  const int nrz = kLpBlocksK + (mg ? mg_partial_blocks() : 0);   // r.z partial rows: block Jacobi, coarse
+  const int lpb = lp_partial_blocks((int)s->ne, s->N);           // r.z partial rows: block Jacobi, then coarse
+  const int nrz = lpb + (mg ? mg_partial_blocks(s) : 0);
   const int mgl = mg ? mg_launches(s) : 0;
   const int N = s->N, Ng = s->Ng, m = s->mix_m;
-  const int64_t n = s->ne * (int64_t)s->Nst;
+  const int64_t n = s->ne * (int64_t)s->Nst, npairs = s->ne * (int64_t)N;
+  const int rb = red_grid(npairs);
   if (!s->fcgP && (e = dev_alloc(s, (void**)&s->fcgP, (size_t)m * n * sizeof(double))) != STDG_OK) return e;
   if (!s->fcgQ && (e = dev_alloc(s, (void**)&s->fcgQ, (size_t)m * n * sizeof(double))) != STDG_OK) return e;
   LpKernels lk = lp_kernels();
@@ -1115,8 +1198,7 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
   const double idt2 = 1.0 / (s->dt * s->dt);
   for (int c = 0; c < Ng * Ng; ++c) { Tpd[c] = Tp.v[c] = s->tm.Tp[c]; Tpinv.v[c] = s->tm.K[c] * idt2; }
   // inner (binary32) scalars
-  double* rz = s->scal; double* pq = s->scal + 8; double* alpha = s->scal + 16; double* beta = s->scal + 24;
-  double* rrnew = s->scal + 32; double* res = s->scal + 48; double* rznew = s->scal + 56;
+  double* rz = s->scal; double* alpha = s->scal + 16; double* beta = s->scal + 24;
   double* flag = s->scal + 96;                            // breakdown of the binary32 recurrence
   // outer (binary64) scalars: m x Ng dots z.Q_j, P_j.Q_j, coefficients; Ng-wide rest
   double* o_rp = s->scal + 400; double* o_al = s->scal + 408; double* o_rr = s->scal + 416;
@@ -1124,7 +1206,7 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
   double* r = s->kr; double* z = s->kz; double* rhs = s->kb;
   const ApplyArgs S = pressure_op(s, 1, 1, -1.0, 1.0);
   ++s->nlaunch;
-  k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, b, rhs);
+  k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, b, rhs);
   cudaMemsetAsync(x, 0, n * sizeof(double), s->stream);
   cudaMemcpyAsync(r, rhs, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
   double rdec = host_norm(s, r, n);                       // ||r|| of the decoupled system
@@ -1138,9 +1220,9 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     cudaError_t ce = launch_apply_lp(s, s->fp, s->fq, 1, 1, -1.0f, 1.0f, s->opdot);
     if (evs) cudaEventRecordWithFlags(evs[1], s->stream, cudaEventRecordExternal);
     if (ce != cudaSuccess) { set_error("low-precision operator launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
-    k_final_alpha_guard<<<1, kRedThreads, 0, s->stream>>>(npq, Ng, s->opdot, rz, alpha, flag);
+    k_final_alpha_guard<<<1, 1024, 0, s->stream>>>(npq, Ng, s->opdot, rz, alpha, flag);
     lp_update_bjacobi(s->stream, (int)s->ne, N, Ng, alpha, s->fx, s->fr, s->fp, s->fq, s->lpBinv, s->fz, s->part);
-    if (mg) mg_apply_f32(s, s->fr, s->fz, s->part + (size_t)kLpBlocksK * Ng);
+    if (mg) mg_apply_f32(s, s->fr, s->fz, s->part + (size_t)lpb * Ng);
     k_final_beta<<<Ng, kRedThreads, 0, s->stream>>>(nrz, Ng, s->part, rz, beta);
     lk.dir(s->stream, n, N, Ng, beta, s->fz, s->fp);
     return STDG_OK;
@@ -1177,7 +1259,7 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     cudaMemsetAsync(s->fx, 0, n * sizeof(float), s->stream);
     cudaMemsetAsync(flag, 0, sizeof(double), s->stream);
     lk.bjacobi(s->stream, (int)s->ne, N, Ng, s->lpBinv, s->fr, s->fz, s->part);
-    if (mg) mg_apply_f32(s, s->fr, s->fz, s->part + (size_t)kLpBlocksK * Ng);
+    if (mg) mg_apply_f32(s, s->fr, s->fz, s->part + (size_t)lpb * Ng);
     k_final<<<Ng, kRedThreads, 0, s->stream>>>(nrz, Ng, s->part, rz);
     cudaMemcpyAsync(s->fp, s->fz, n * sizeof(float), cudaMemcpyDeviceToDevice, s->stream);
     s->nlaunch += 3 + mgl;
@@ -1201,24 +1283,24 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     if (used == 0) {
       cudaMemcpyAsync(p, z, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
     } else {
-      k_fcg_dots<<<dim3(kRedBlocks, used), kRedThreads, 0, s->stream>>>(n, N, Ng, used, s->fcgQ, z, s->part);
-      k_final<<<used * Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, used * Ng, s->part, o_zq);
+      STDG_NG_SWITCH(Ng, (k_fcg_dots<G><<<dim3(rb, used), kRedThreads, 0, s->stream>>>(npairs, N, used, s->fcgQ, z, s->part)));
+      k_final<<<used * Ng, kRedThreads, 0, s->stream>>>(rb, used * Ng, s->part, o_zq);
       k_fcg_coef<<<1, 64, 0, s->stream>>>(used * Ng, o_zq, o_pqs, o_c);
       // the slot being overwritten is excluded: when the ring is full its coefficient is set to 0
       if (used == m) cudaMemsetAsync(o_c + slot * Ng, 0, Ng * sizeof(double), s->stream);
-      k_fcg_dir<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, used, o_c, s->fcgP, z, s->kp);
+      STDG_NG_SWITCH(Ng, (k_fcg_dir<G><<<rb, kRedThreads, 0, s->stream>>>(npairs, N, used, o_c, s->fcgP, z, s->kp)));
       cudaMemcpyAsync(p, s->kp, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
       s->nlaunch += 4;
     }
     e = op_apply(s, S, p, q);
     if (e != STDG_OK) return e;
-    k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, p, q, s->part);
-    k_final<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, s->part, o_pqs + slot * Ng);
-    k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, r, p, s->part);
-    k_final<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, s->part, o_rp);
+    coldot(s->stream, rb, npairs, N, Ng, p, q, s->part);
+    k_final<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, s->part, o_pqs + slot * Ng);
+    coldot(s->stream, rb, npairs, N, Ng, r, p, s->part);
+    k_final<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, s->part, o_rp);
     k_cg_alpha<<<1, 32, 0, s->stream>>>(Ng, o_rp, o_pqs + slot * Ng, o_al);
-    k_cg_update<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, o_al, x, r, p, q, Tp, s->part);
-    k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng + 1, s->part, o_rr);
+    cg_update(s->stream, rb, npairs, N, Ng, o_al, x, r, p, q, Tp, s->part);
+    k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(rb, Ng + 1, s->part, o_rr);
     cudaMemcpyAsync(s->hostbuf + 880, o_rr, (Ng + 1) * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     s->nlaunch += 9;
     if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("mixed solve: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
@@ -1233,12 +1315,12 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
       // rounding, ~1e-14 of |A| |x|, can exceed tol |b|); if it misses the tolerance, continue from
       // that residual with a fresh set of directions (at most 3 times)
       if ((e = op_apply(s, pressure_op(s, 1, 0, 1.0, -1.0), x, s->kq, true)) != STDG_OK) return e;
-      k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);   // kq = b - A x
+      k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);   // kq = b - A x
       ++s->nlaunch;
       rfull = host_norm(s, s->kq, n);
       if (rfull <= tol * bn || rdec == 0.0 || refresh >= 3) break;
       ++refresh;
-      k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, s->kq, r);   // r = -(I (x) Tp^-1)(b - A x)
+      k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, s->kq, r);   // r = -(I (x) Tp^-1)(b - A x)
       ++s->nlaunch;
       rdec = host_norm(s, r, n);
       ring = 0;
@@ -1265,6 +1347,7 @@ stdg_status solve_pressure(stdg_solver* s, const double* b, double* x, double to
     return STDG_EINVAL;
   }
   const int64_t n = s->ne * (int64_t)s->Nst;
+  const int rb = red_grid(s->ne * (int64_t)s->N);
   const double bn = host_norm(s, b, n);
   if (!std::isfinite(bn)) { set_error("stdg_solve: non-finite right-hand side"); return STDG_ENAN; }
   int it = 0, rs = 0;
@@ -1313,7 +1396,7 @@ stdg_status solve_pressure(stdg_solver* s, const double* b, double* x, double to
     const double idt2 = 1.0 / (s->dt * s->dt);
     for (int q = 0; q < s->Ng * s->Ng; ++q) { Tp.v[q] = s->tm.Tp[q]; Tpinv.v[q] = s->tm.K[q] * idt2; }
     ++s->nlaunch;
-    k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, s->N, s->Ng, Tpinv, -1.0, b, s->kb);
+    k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, s->N, s->Ng, Tpinv, -1.0, b, s->kb);
     r = cg_block(s, pressure_op(s, 1, 1, -1.0, 1.0), s->kb, x, true, Tp, tol * bn, &it, &rabs,
                  method == STDG_SOLVER_KRON_PCG ? 1 : method == STDG_SOLVER_KRON_MG ? 2 : 0);
   } else {
@@ -1332,7 +1415,7 @@ stdg_status solve_pressure(stdg_solver* s, const double* b, double* x, double to
       stdg_status e2 = op_apply(s, pressure_op(s, 1, 0, 1.0, -1.0), x, s->kq, true);
       if (e2 != STDG_OK) return e2;
       ++s->nlaunch;
-      k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
+      k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);
       rn = host_norm(s, s->kq, n);
     }
     st->iterations = it;
@@ -1395,38 +1478,40 @@ __global__ void __launch_bounds__(kRedThreads) k_crossdot(int ne, int N, const d
 
 struct PairArg { int p[kMaxNg]; };
 
-// The complex scalars of every block of R, from the cross products C (Ng x Ng).  The bilinear form of
-// a 2 x 2 block (columns a, a+1 = real, imaginary part) is (C_aa - C_a+1,a+1) + i (C_a,a+1 + C_a+1,a);
-// of a 1 x 1 block C_aa.  rho[2a], rho[2a+1]: r^T z of the block led by column a.
+// The complex scalars of every block of R, from the cross products C (Ng x Ng), which one block first
+// reduces from the partials.  The bilinear form of a 2 x 2 block (columns a, a+1 = real, imaginary part) is
+// (C_aa - C_a+1,a+1) + i (C_a,a+1 + C_a+1,a); of a 1 x 1 block C_aa.  rho[2a], rho[2a+1]: r^T z of the
+// block led by column a.
 //  mode 0: alpha = rho / (p^T q)  -> M (Ng x Ng real form of the multiplier), flag on breakdown
 //  mode 1: beta = (r^T z)_new / rho, rho <- (r^T z)_new  -> M
 //  mode 2: rho <- r^T z
-__global__ void k_cocg_scalars(int Ng, PairArg pr, int mode, const double* __restrict__ C, double* rho, double* M,
-                               double* flag) {
-  if (threadIdx.x != 0) return;
-  for (int q = 0; q < Ng * Ng; ++q) M[q] = 0.0;
-  for (int a = 0; a < Ng; ++a) {
-    const bool two = pr.p[a] == 1;
-    double br, bi;
-    if (two) { br = C[a * Ng + a] - C[(a + 1) * Ng + a + 1]; bi = C[a * Ng + a + 1] + C[(a + 1) * Ng + a]; }
-    else { br = C[a * Ng + a]; bi = 0.0; }
-    double zr = 0.0, zi = 0.0;
-    if (mode == 2) { rho[2 * a] = br; rho[2 * a + 1] = bi; }
-    else {
-      // z = num / den (complex)
-      const double nr = mode == 0 ? rho[2 * a] : br, ni = mode == 0 ? rho[2 * a + 1] : bi;
-      const double dr = mode == 0 ? br : rho[2 * a], di = mode == 0 ? bi : rho[2 * a + 1];
-      const double dd = dr * dr + di * di;
-      if (dd > 0.0 && isfinite(dd)) { zr = (nr * dr + ni * di) / dd; zi = (ni * dr - nr * di) / dd; }
-      else if (nr != 0.0 || ni != 0.0) flag[0] = 1.0;
-      if (mode == 1) { rho[2 * a] = br; rho[2 * a + 1] = bi; }
-    }
-    M[a * Ng + a] = zr;
-    if (two) {
-      M[a * Ng + a + 1] = -zi; M[(a + 1) * Ng + a] = zi; M[(a + 1) * Ng + a + 1] = zr;
-      ++a;
-    }
+__global__ void __launch_bounds__(1024) k_cocg_scalars(int nparts, int Ng, PairArg pr, int mode,
+                                                       const double* __restrict__ part, double* rho, double* M,
+                                                       double* flag) {
+  __shared__ double scratch[1024], C[kMaxNg * kMaxNg];
+  block_column_sums(nparts, Ng * Ng, part, scratch, C);
+  const int a = threadIdx.x;                      // thread a: the block led by column a
+  if (a >= Ng || (a > 0 && pr.p[a - 1] == 1 && pr.p[a] == 0)) return;
+  for (int q = 0; q < Ng; ++q) M[a * Ng + q] = 0.0;
+  const bool two = pr.p[a] == 1;
+  if (two)
+    for (int q = 0; q < Ng; ++q) M[(a + 1) * Ng + q] = 0.0;
+  double br, bi;
+  if (two) { br = C[a * Ng + a] - C[(a + 1) * Ng + a + 1]; bi = C[a * Ng + a + 1] + C[(a + 1) * Ng + a]; }
+  else { br = C[a * Ng + a]; bi = 0.0; }
+  double zr = 0.0, zi = 0.0;
+  if (mode == 2) { rho[2 * a] = br; rho[2 * a + 1] = bi; }
+  else {
+    // z = num / den (complex)
+    const double nr = mode == 0 ? rho[2 * a] : br, ni = mode == 0 ? rho[2 * a + 1] : bi;
+    const double dr = mode == 0 ? br : rho[2 * a], di = mode == 0 ? bi : rho[2 * a + 1];
+    const double dd = dr * dr + di * di;
+    if (dd > 0.0 && isfinite(dd)) { zr = (nr * dr + ni * di) / dd; zi = (ni * dr - nr * di) / dd; }
+    else if (nr != 0.0 || ni != 0.0) flag[0] = 1.0;
+    if (mode == 1) { rho[2 * a] = br; rho[2 * a + 1] = bi; }
   }
+  M[a * Ng + a] = zr;
+  if (two) { M[a * Ng + a + 1] = -zi; M[(a + 1) * Ng + a] = zi; M[(a + 1) * Ng + a + 1] = zr; }
 }
 
 // x += M p, r -= M q (M from the device, Ng x Ng); with want, partials of ||(I (x) W) r||^2
@@ -1494,33 +1579,33 @@ __global__ void __launch_bounds__(kRedThreads) k_cocg_dir(int ne, int N, const d
 
 // launches of the three vector kernels above for the solver's Ng
 struct CocgLaunch {
-  int Ng;
+  int Ng, rb;
   void cross(cudaStream_t st, int ne, int N, const double* u, const double* v, double* part) const {
     switch (Ng) {
-      case 1: k_crossdot<1><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
-      case 2: k_crossdot<2><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
-      case 3: k_crossdot<3><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
-      case 4: k_crossdot<4><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
-      default: k_crossdot<5><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
+      case 1: k_crossdot<1><<<rb, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
+      case 2: k_crossdot<2><<<rb, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
+      case 3: k_crossdot<3><<<rb, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
+      case 4: k_crossdot<4><<<rb, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
+      default: k_crossdot<5><<<rb, kRedThreads, 0, st>>>(ne, N, u, v, part); break;
     }
   }
   void update(cudaStream_t st, int ne, int N, const double* M, double* x, double* r, const double* p, const double* q,
               const TpArg& W, double* part, int want) const {
     switch (Ng) {
-      case 1: k_cocg_update<1><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
-      case 2: k_cocg_update<2><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
-      case 3: k_cocg_update<3><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
-      case 4: k_cocg_update<4><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
-      default: k_cocg_update<5><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
+      case 1: k_cocg_update<1><<<rb, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
+      case 2: k_cocg_update<2><<<rb, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
+      case 3: k_cocg_update<3><<<rb, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
+      case 4: k_cocg_update<4><<<rb, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
+      default: k_cocg_update<5><<<rb, kRedThreads, 0, st>>>(ne, N, M, x, r, p, q, W, part, want); break;
     }
   }
   void dir(cudaStream_t st, int ne, int N, const double* M, const double* z, double* p) const {
     switch (Ng) {
-      case 1: k_cocg_dir<1><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
-      case 2: k_cocg_dir<2><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
-      case 3: k_cocg_dir<3><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
-      case 4: k_cocg_dir<4><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
-      default: k_cocg_dir<5><<<kRedBlocks, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
+      case 1: k_cocg_dir<1><<<rb, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
+      case 2: k_cocg_dir<2><<<rb, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
+      case 3: k_cocg_dir<3><<<rb, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
+      case 4: k_cocg_dir<4><<<rb, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
+      default: k_cocg_dir<5><<<rb, kRedThreads, 0, st>>>(ne, N, M, z, p); break;
     }
   }
 };
@@ -1556,7 +1641,7 @@ __global__ void k_add(int64_t n, const double* __restrict__ d, double* __restric
 static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, const double* b, double* x,
                                 double tol_abs, int* iters, double* res, bool zero_x0 = false,
                                 bool lowprec = false) {
-  const int Ng = s->Ng, N = s->N;
+  const int Ng = s->Ng, N = s->N, rb = red_grid(s->ne * (int64_t)N);
   const int64_t n = s->ne * (int64_t)s->Nst;
   if (s->vbd < 0) s->vbd = time_blockdiag(s->K.data(), Ng, s->vW, s->vWinv, s->vR, s->vpair) ? 1 : 0;
   if (!s->vbd) return STDG_EUNSUPPORTED;
@@ -1575,42 +1660,39 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
   for (int q = 0; q < Ng * Ng; ++q) at.Kmass[q] = s->vR[q];
   double* y = s->kx; double* r = s->kr; double* z = s->kz; double* p = s->kp; double* q = s->kq;
   double* bt = s->kb;
-  double* C = s->scal + 300;                          // Ng^2 cross products
   double* rho = s->scal + 330;                        // 2 Ng
   double* Ma = s->scal + 340; double* Mb = s->scal + 370;   // Ng^2 each
   double* flag = s->scal + 398; double* resd = s->scal + 399;
-  const int G2 = Ng * Ng;
   const LpKernels lk = lp_kernels();
   auto apply = [&](const double* in, double* out) -> stdg_status {
     if (!lowprec) return op_apply(s, at, in, out);
     lk.f32(s->stream, n, in, s->fp);
     const cudaError_t ce = warp_launch_f32_visc(s, s->fp, s->fq, at.scale, at.mass_coef, at.Kmass);
     if (ce != cudaSuccess) { set_error("binary32 viscous operator: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
-    k_f64_from_f32<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, s->fq, out);
+    k_f64_from_f32<<<rb, kRedThreads, 0, s->stream>>>(n, s->fq, out);
     s->nlaunch += 3;
     ++s->op_launches;
     return STDG_OK;
   };
   s->nlaunch += 1;
-  k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Wi, 1.0, b, bt);
+  k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Wi, 1.0, b, bt);
   if (zero_x0) {
     cudaMemsetAsync(y, 0, n * sizeof(double), s->stream);
     cudaMemcpyAsync(r, bt, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
   } else {
     s->nlaunch += 2;
-    k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Wi, 1.0, x, y);
+    k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Wi, 1.0, x, y);
     if ((e = apply(y, r)) != STDG_OK) return e;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, bt, nullptr, 1, r);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, bt, nullptr, 1, r);
   }
   if ((e = visc_pc_apply(s, nu, r, z, 0, s->vR)) != STDG_OK) return e;
   cudaMemcpyAsync(p, z, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
   cudaMemsetAsync(flag, 0, sizeof(double), s->stream);
   s->nlaunch += 3;
-  const CocgLaunch cl{Ng};
+  const CocgLaunch cl{Ng, rb};
   const int ne = (int)s->ne;
   cl.cross(s->stream, ne, N, r, z, s->part);
-  k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-  k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 2, C, rho, Ma, flag);
+  k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 2, s->part, rho, Ma, flag);
   // a few tens of iterations per solve: batches of at most 4 between host checks
   const int B = s->opt.graph_batch > 1 ? std::min(4, s->opt.graph_batch) : 1;
   auto body = [&](int slot, cudaEvent_t* evs) -> stdg_status {
@@ -1620,24 +1702,22 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
     if (e2 != STDG_OK) return e2;
     const int want = slot == B - 1;
     cl.cross(s->stream, ne, N, p, q, s->part);
-    k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-    k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 0, C, rho, Ma, flag);
+    k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 0, s->part, rho, Ma, flag);
     cl.update(s->stream, ne, N, Ma, y, r, p, q, W, s->part, want);
     if (want) {
-      k_final_norm<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, s->part, resd);
+      k_final_norm<<<1, kRedThreads, 0, s->stream>>>(rb, s->part, resd);
       cudaMemcpyAsync(s->hostbuf + slot, resd, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     }
     if ((e2 = visc_pc_apply(s, nu, r, z, 0, s->vR)) != STDG_OK) return e2;
     cl.cross(s->stream, ne, N, r, z, s->part);
-    k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-    k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 1, C, rho, Mb, flag);
+    k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 1, s->part, rho, Mb, flag);
     cl.dir(s->stream, ne, N, Mb, z, p);
     return STDG_OK;
   };
   int it = 0;
   double rabs = INFINITY;
   const int kind = lowprec ? 2 : df_serves(s, at) ? 1 : 0;
-  const int kpi = 11 + (lowprec ? 2 : 0);
+  const int kpi = 9 + (lowprec ? 2 : 0);
   if (B > 1) {
     e = run_batched(s, B, kpi, s->opt.max_iters, tol_abs, body, &it, &rabs, kind, true);
   } else {
@@ -1655,7 +1735,7 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
   double hflag = 0.0;
   cudaMemcpyAsync(&hflag, flag, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
   ++s->nlaunch;
-  k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, W, 1.0, y, x);
+  k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, W, 1.0, y, x);
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("viscous COCG: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
   *iters = it;
   *res = rabs;
@@ -1672,7 +1752,7 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
 // binary64; x is left unchanged unless the solve reaches tol_abs.
 static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu, const double* b, double* x,
                                   double tol_abs, int* iters, double* res) {
-  const int Ng = s->Ng, N = s->N, ne = (int)s->ne;
+  const int Ng = s->Ng, N = s->N, ne = (int)s->ne, rb = red_grid(s->ne * (int64_t)N);
   const int64_t n = s->ne * (int64_t)s->Nst;
   if (s->vbd < 0) s->vbd = time_blockdiag(s->K.data(), Ng, s->vW, s->vWinv, s->vR, s->vpair) ? 1 : 0;
   if (!s->vbd) return STDG_EUNSUPPORTED;
@@ -1688,19 +1768,16 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
   ApplyArgs at = a;                                   // the decoupled operator: time matrix R
   for (int q = 0; q < Ng * Ng; ++q) at.Kmass[q] = s->vR[q];
   float* y = s->fx; float* r = s->fr; float* z = s->fz; float* p = s->fp; float* q = s->fq;
-  double* C = s->scal + 300;                          // Ng^2 cross products
   double* rho = s->scal + 330;                        // 2 Ng
   double* Ma = s->scal + 340; double* Mb = s->scal + 370;   // Ng^2 each
   double* flag = s->scal + 398; double* resd = s->scal + 399;
-  const int G2 = Ng * Ng;
-  c32_mix_to32(s->stream, ne, N, Ng, Wi, b, r);      // r = (I (x) W^-1) b, y = 0
+  c32_mix_to32(s->stream, rb, ne, N, Ng, Wi, b, r);      // r = (I (x) W^-1) b, y = 0
   cudaMemsetAsync(y, 0, n * sizeof(float), s->stream);
   if ((e = visc_pc_apply32(s, nu, r, z, s->vR)) != STDG_OK) return e;
   cudaMemcpyAsync(p, z, n * sizeof(float), cudaMemcpyDeviceToDevice, s->stream);
   cudaMemsetAsync(flag, 0, sizeof(double), s->stream);
-  c32_cross(s->stream, ne, N, Ng, r, z, s->part);
-  k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-  k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 2, C, rho, Ma, flag);
+  c32_cross(s->stream, rb, ne, N, Ng, r, z, s->part);
+  k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 2, s->part, rho, Ma, flag);
   s->nlaunch += 4;
   const int B = s->opt.graph_batch > 1 ? std::min(4, s->opt.graph_batch) : 1;
   auto body = [&](int slot, cudaEvent_t* evs) -> stdg_status {
@@ -1709,25 +1786,23 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
     if (evs) cudaEventRecordWithFlags(evs[1], s->stream, cudaEventRecordExternal);
     if (ae != cudaSuccess) { set_error("binary32 viscous operator: %s", cudaGetErrorString(ae)); return STDG_ECUDA; }
     const int want = slot == B - 1;
-    c32_cross(s->stream, ne, N, Ng, p, q, s->part);
-    k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-    k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 0, C, rho, Ma, flag);
-    c32_update(s->stream, ne, N, Ng, Ma, y, r, p, q, W, s->part, want);
+    c32_cross(s->stream, rb, ne, N, Ng, p, q, s->part);
+    k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 0, s->part, rho, Ma, flag);
+    c32_update(s->stream, rb, ne, N, Ng, Ma, y, r, p, q, W, s->part, want);
     if (want) {
-      k_final_norm<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, s->part, resd);
+      k_final_norm<<<1, kRedThreads, 0, s->stream>>>(rb, s->part, resd);
       cudaMemcpyAsync(s->hostbuf + slot, resd, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     }
     stdg_status e2 = visc_pc_apply32(s, nu, r, z, s->vR);
     if (e2 != STDG_OK) return e2;
-    c32_cross(s->stream, ne, N, Ng, r, z, s->part);
-    k_final<<<G2, kRedThreads, 0, s->stream>>>(kRedBlocks, G2, s->part, C);
-    k_cocg_scalars<<<1, 32, 0, s->stream>>>(Ng, pr, 1, C, rho, Mb, flag);
-    c32_dir(s->stream, ne, N, Ng, Mb, z, p);
+    c32_cross(s->stream, rb, ne, N, Ng, r, z, s->part);
+    k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 1, s->part, rho, Mb, flag);
+    c32_dir(s->stream, rb, ne, N, Ng, Mb, z, p);
     return STDG_OK;
   };
   int it = 0;
   double rabs = INFINITY;
-  constexpr int kpi = 10;                             // kernels per iteration (+1 norm per check)
+  constexpr int kpi = 8;                              // kernels per iteration (+1 norm per check)
   if (B > 1) {
     e = run_batched(s, B, kpi, s->opt.max_iters, tol_abs, body, &it, &rabs, 2, true);
     s->nlaunch += it / B;
@@ -1753,7 +1828,7 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
   if (hflag != 0.0) { set_error("viscous COCG: breakdown (p^T A p = 0)"); return STDG_ENOCONV; }
   if (!(rabs <= tol_abs)) { set_error("viscous COCG reached max_iters (%d)", it); return STDG_ENOCONV; }
   ++s->nlaunch;
-  c32_mix_acc64(s->stream, ne, N, Ng, W, y, x);     // x += (I (x) W) y
+  c32_mix_acc64(s->stream, rb, ne, N, Ng, W, y, x);     // x += (I (x) W) y
   return STDG_OK;
 }
 
@@ -1768,6 +1843,7 @@ stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu,
   a.tacc_identity = 1; a.pinned = 0;
   for (int q = 0; q < s->Ng * s->Ng; ++q) a.Kmass[q] = s->K[q];
   const int64_t n = s->ne * (int64_t)s->Nst;
+  const int rb = red_grid(s->ne * (int64_t)s->N);
   const double bn = host_norm(s, b, n);
   if (!std::isfinite(bn)) { set_error("viscous solve: non-finite right-hand side"); return STDG_ENAN; }
   if (bn == 0.0) { cudaMemsetAsync(x, 0, n * sizeof(double), s->stream); *iters = 0; *res = 0; return STDG_OK; }
@@ -1797,7 +1873,7 @@ stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu,
     for (int outer = 0; outer < 8; ++outer) {
       if ((e0 = op_apply(s, a, x, ro)) != STDG_OK) return e0;
       ++s->nlaunch;
-      k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(nn, b, nullptr, 1, ro);
+      k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(nn, b, nullptr, 1, ro);
       const double nr = host_norm(s, ro, nn);
       if (!std::isfinite(nr)) { set_error("viscous solve: non-finite residual"); return STDG_ENAN; }
       if (nr <= tol * bn) { *iters = it1; *res = nr; return STDG_OK; }
@@ -1811,7 +1887,7 @@ stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu,
       if (e0 != STDG_OK) return e0;
       if (s->visc_inner64) {
         ++s->nlaunch;
-        k_add<<<kRedBlocks, kRedThreads, 0, s->stream>>>(nn, s->basis + nn, x);
+        k_add<<<rb, kRedThreads, 0, s->stream>>>(nn, s->basis + nn, x);
       }
     }
   }
@@ -1869,8 +1945,9 @@ static stdg_status noalloc_fetch(stdg_solver* s, const double* dev_src, double* 
 }
 
 static stdg_status noalloc_norm(stdg_solver* s, const double* v, int64_t n, double* part, double* dst, double* out) {
-  k_sumsq<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, v, part);
-  k_final<<<1, kRedThreads, 0, s->stream>>>(kRedBlocks, 1, part, dst);
+  const int rb = red_grid(s->ne * (int64_t)s->N);
+  k_sumsq<<<rb, kRedThreads, 0, s->stream>>>(n, v, part);
+  k_final<<<1, kRedThreads, 0, s->stream>>>(rb, 1, part, dst);
   s->nlaunch += 2;
   double h = 0.0;
   stdg_status e = noalloc_fetch(s, dst, &h);
@@ -1881,7 +1958,8 @@ static stdg_status noalloc_norm(stdg_solver* s, const double* v, int64_t n, doub
 stdg_status solve_pressure_noalloc(stdg_solver* s, const double* b, double* x, double tol, stdg_solve_stats* st) {
   auto t0 = std::chrono::steady_clock::now();
   const int N = s->N, Ng = s->Ng;
-  const int64_t n = s->ne * (int64_t)s->Nst;
+  const int64_t n = s->ne * (int64_t)s->Nst, npairs = s->ne * (int64_t)N;
+  const int rb = red_grid(npairs);
   if (n > kNoAllocMaxDofs) {
     set_error("stdg_solve_noalloc: %lld pressure unknowns exceed the allocation-free limit of %lld "
               "(use stdg_solve)", (long long)n, (long long)kNoAllocMaxDofs);
@@ -1910,23 +1988,23 @@ stdg_status solve_pressure_noalloc(stdg_solver* s, const double* b, double* x, d
     const double idt2 = 1.0 / (s->dt * s->dt);
     for (int c = 0; c < Ng * Ng; ++c) { Tp.v[c] = s->tm.Tp[c]; Tpinv.v[c] = s->tm.K[c] * idt2; }
     const ApplyArgs op = pressure_op(s, 1, 1, -1.0, 1.0);
-    k_timemix<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, b, bt);
+    k_timemix<<<rb, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, Tpinv, -1.0, b, bt);
     cudaMemcpyAsync(r, bt, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
     cudaMemcpyAsync(p, bt, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
-    k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, r, r, part);
-    k_final<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, part, rr);
+    coldot(s->stream, rb, npairs, N, Ng, r, r, part);
+    k_final<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, part, rr);
     s->nlaunch += 3;
     const double tol_abs = tol * bn;
     rabs = INFINITY;
     while (it < s->opt.max_iters) {
       if ((e = op_apply(s, op, p, q)) != STDG_OK) return e;
-      k_coldot<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, p, q, part);
-      k_final<<<Ng, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng, part, pq);
+      coldot(s->stream, rb, npairs, N, Ng, p, q, part);
+      k_final<<<Ng, kRedThreads, 0, s->stream>>>(rb, Ng, part, pq);
       k_cg_alpha<<<1, 32, 0, s->stream>>>(Ng, rr, pq, alpha);
-      k_cg_update<<<kRedBlocks, kRedThreads, 0, s->stream>>>(s->ne, N, Ng, alpha, x, r, p, q, Tp, part);
-      k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(kRedBlocks, Ng + 1, part, rrnew);
+      cg_update(s->stream, rb, npairs, N, Ng, alpha, x, r, p, q, Tp, part);
+      k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(rb, Ng + 1, part, rrnew);
       k_cg_beta<<<1, 32, 0, s->stream>>>(Ng, rr, rrnew, beta, res);
-      k_cg_dir<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, N, Ng, beta, r, p);
+      cg_dir(s->stream, rb, npairs, N, Ng, beta, r, p);
       s->nlaunch += 7;
       ++it;
       if ((e = noalloc_fetch(s, res, &rabs)) != STDG_OK) return e;
@@ -1937,7 +2015,7 @@ stdg_status solve_pressure_noalloc(stdg_solver* s, const double* b, double* x, d
   if (st) {
     double rn = 0.0;
     if ((e = op_apply(s, pressure_op(s, 1, 0, 1.0, -1.0), x, q)) != STDG_OK) return e;
-    k_scale_copy<<<kRedBlocks, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, q);
+    k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, q);
     ++s->nlaunch;
     if ((e = noalloc_norm(s, q, n, part, nrm, &rn)) != STDG_OK) return e;
     st->iterations = it;

@@ -14,6 +14,8 @@
 // Every mbarrier wait is bounded; on timeout the kernel records an error word and returns.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+
 #include "lp_ptx.cuh"
 #include "solver.h"
 
@@ -302,23 +304,18 @@ __global__ void __launch_bounds__(416) k_apply_tma(TmaArgs<Pol> a, const typenam
 }
 
 // ------------------------------------------------------------------ block copies and vectors
+// Low-precision copies of the blocks, padded to SB entries.  A CTA takes whole blocks, about 1,024 entries at a
+// time (indices inside them in 32 bits).
 template <typename TB>
-__global__ void k_to_lp(int64_t nblk, int N, int SB, FxBlocks src, TB* __restrict__ dst);
-template <>
-__global__ void k_to_lp<float>(int64_t nblk, int N, int SB, FxBlocks src, float* __restrict__ dst) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * SB; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / SB;
-    const int o = (int)(e % SB), NN = N * N;
-    dst[e] = o < NN ? (float)fx_entry(src, NN, b, o, N) : 0.0f;
-  }
-}
-template <>
-__global__ void k_to_lp<__nv_bfloat16>(int64_t nblk, int N, int SB, FxBlocks src,
-                                       __nv_bfloat16* __restrict__ dst) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nblk * SB; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t b = e / SB;
-    const int o = (int)(e % SB), NN = N * N;
-    dst[e] = __float2bfloat16_rn(o < NN ? (float)fx_entry(src, NN, b, o, N) : 0.0f);
+__global__ void __launch_bounds__(256) k_to_lp(int64_t nblk, int N, int SB, const __grid_constant__ FxBlocks src,
+                                               TB* __restrict__ dst) {
+  const int NN = N * N, per = SB < 1024 ? 1024 / SB : 1;
+  for (int64_t b0 = (int64_t)blockIdx.x * per; b0 < nblk; b0 += (int64_t)gridDim.x * per) {
+    const int cnt = (nblk - b0 < per ? (int)(nblk - b0) : per) * SB;
+    for (int e = threadIdx.x; e < cnt; e += 256) {
+      const int b = e / SB, o = e - b * SB, r = o / N;
+      dst[b0 * SB + e] = (TB)(o < NN ? fx_entry_f32(src, NN, b0 + b, o, src.r.s[r] + src.c.s[o - r * N]) : 0.0f);
+    }
   }
 }
 
@@ -485,7 +482,7 @@ __global__ void __launch_bounds__(256) k_lp_coldot(int64_t ne, int N, int Ng, co
   float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   const int Nst = N * Ng;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o = i * Nst + (e - i * N);
     for (int a = 0; a < Ng; ++a) acc[a] = fmaf(x[o + a * N], y[o + a * N], acc[a]);
   }
@@ -502,7 +499,7 @@ __global__ void __launch_bounds__(256) k_lp_cg_update(int64_t ne, int N, int Ng,
   for (int a = 0; a < Ng; ++a) al[a] = (float)alpha[a];
   const int Nst = N * Ng;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
+    const int64_t i = (uint32_t)e / (uint32_t)N;
     const int64_t o0 = i * Nst + (e - i * N);
     float rv[kMaxNg];
     for (int a = 0; a < Ng; ++a) {
@@ -523,15 +520,17 @@ __global__ void __launch_bounds__(256) k_lp_cg_update(int64_t ne, int N, int Ng,
   if (!want) return;
   lp_block_store(acc, Ng + 1, part, Ng + 1);
 }
-__global__ void k_lp_cg_dir(int64_t ne, int N, int Ng, const double* __restrict__ beta, const float* __restrict__ z,
-                            float* __restrict__ p) {
-  float be[kMaxNg];
-  for (int a = 0; a < Ng; ++a) be[a] = (float)beta[a];
-  const int Nst = N * Ng;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
-    const int64_t o = i * Nst + (e - i * N);
-    for (int a = 0; a < Ng; ++a) p[o + a * N] = fmaf(be[a], p[o + a * N], z[o + a * N]);
+template <int NG>
+__global__ void __launch_bounds__(256) k_lp_cg_dir(int64_t npairs, int N, const double* __restrict__ beta,
+                                                  const float* __restrict__ z, float* __restrict__ p) {
+  float be[NG];
+#pragma unroll
+  for (int a = 0; a < NG; ++a) be[a] = (float)beta[a];
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < npairs; e += (int64_t)gridDim.x * blockDim.x) {
+    const uint32_t i = (uint32_t)e / (uint32_t)N;
+    const int64_t o = (int64_t)i * N * NG + (e - (int64_t)i * N);
+#pragma unroll
+    for (int a = 0; a < NG; ++a) p[o + a * N] = fmaf(be[a], p[o + a * N], z[o + a * N]);
   }
 }
 // z_i = Binv_i r_i per time column: thread per (tet, row k) covering all Ng columns, so each entry of
@@ -582,28 +581,30 @@ __global__ void __launch_bounds__(256) k_lp_bjacobi(int ne, int Nrt, int Ng, con
 // memory (thread per (tet, row), all columns), and partials of r.z per column.  With N and Ng at
 // compile time (NC, NGC != 0) a thread's N column loads of Binv are all issued before its first
 // multiply-add, so each warp keeps N loads in flight.
-template <int NC, int NGC>
-__global__ void __launch_bounds__(256) k_lp_update_bj(int ne, int Nrt, int Ngrt, const double* __restrict__ alpha,
-                                                     float* __restrict__ x, float* __restrict__ r,
-                                                     const float* __restrict__ p, const float* __restrict__ q,
-                                                     const float* __restrict__ Binv, float* __restrict__ z,
-                                                     double* part) {
-  constexpr int NGM = NGC ? NGC : kMaxNg;
-  extern __shared__ float rs[];
-  __shared__ float s_al[kMaxNg];
-  const int Ng = NGC ? NGC : Ngrt;
-  if (threadIdx.x < Ng) s_al[threadIdx.x] = (float)alpha[threadIdx.x];
-  const int N = NC ? NC : Nrt;
-  const int Nst = N * Ng;
-  const int TB = blockDim.x / N;
-  const size_t NN = (size_t)N * N;
-  float acc[NGM];
+template <int N, int NG>
+__global__ void __launch_bounds__(256) k_lp_update_bj(int ne, const double* __restrict__ alpha, float* __restrict__ x,
+                                                     float* __restrict__ r, const float* __restrict__ p,
+                                                     const float* __restrict__ q, const float* __restrict__ Binv,
+                                                     float* __restrict__ z, double* part) {
+  constexpr int Nst = N * NG, TB = 256 / N, NN = N * N;
+  __shared__ float rs[TB * Nst];
+  __shared__ float s_al[NG];
+  if (threadIdx.x < NG) s_al[threadIdx.x] = (float)alpha[threadIdx.x];
+  float acc[NG];
 #pragma unroll
-  for (int a = 0; a < NGM; ++a) acc[a] = 0.0f;
+  for (int a = 0; a < NG; ++a) acc[a] = 0.0f;
   const int tl = threadIdx.x / N, k = threadIdx.x - tl * N;
   for (int i0 = blockIdx.x * TB; i0 < ne; i0 += gridDim.x * TB) {
+    const int i = i0 + tl;
+    const bool act = tl < TB && i < ne;
+    float bv[N];                                  // the inverse's loads overlap the vector updates
+    if (act) {
+      const float* B = Binv + (size_t)i * NN + k;
+#pragma unroll
+      for (int l2 = 0; l2 < N; ++l2) bv[l2] = __ldg(B + l2 * N);
+    }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < TB * Nst; idx += blockDim.x) {
+    for (int idx = threadIdx.x; idx < TB * Nst; idx += 256) {
       if (i0 + idx / Nst >= ne) continue;
       const size_t g = (size_t)i0 * Nst + idx;
       const float al = s_al[(idx % Nst) / N];
@@ -613,53 +614,54 @@ __global__ void __launch_bounds__(256) k_lp_update_bj(int ne, int Nrt, int Ngrt,
       rs[idx] = rn;
     }
     __syncthreads();
-    const int i = i0 + tl;
-    if (tl < TB && i < ne) {
-      const float* B = Binv + (size_t)i * NN + k;
+    if (act) {
       const float* rr = rs + tl * Nst;
-      float sa[NGM];
+      float sa[NG];
 #pragma unroll
-      for (int a = 0; a < NGM; ++a) sa[a] = 0.0f;
-      if constexpr (NC > 0) {
-        float bv[NC];
+      for (int a = 0; a < NG; ++a) sa[a] = 0.0f;
 #pragma unroll
-        for (int l2 = 0; l2 < NC; ++l2) bv[l2] = __ldg(B + (size_t)l2 * NC);
+      for (int l2 = 0; l2 < N; ++l2)
 #pragma unroll
-        for (int l2 = 0; l2 < NC; ++l2)
+        for (int a = 0; a < NG; ++a) sa[a] = fmaf(bv[l2], rr[a * N + l2], sa[a]);
 #pragma unroll
-          for (int a = 0; a < NGM; ++a)
-            if (NGC || a < Ng) sa[a] = fmaf(bv[l2], rr[a * NC + l2], sa[a]);
-      } else {
-#pragma unroll 4
-        for (int l2 = 0; l2 < N; ++l2) {
-          const float b = B[(size_t)l2 * N];
-#pragma unroll
-          for (int a = 0; a < NGM; ++a)
-            if (a < Ng) sa[a] = fmaf(b, rr[a * N + l2], sa[a]);
-        }
+      for (int a = 0; a < NG; ++a) {
+        z[(size_t)i * Nst + a * N + k] = sa[a];
+        acc[a] = fmaf(sa[a], rr[a * N + k], acc[a]);
       }
-#pragma unroll
-      for (int a = 0; a < NGM; ++a)
-        if (NGC || a < Ng) {
-          z[(size_t)i * Nst + a * N + k] = sa[a];
-          acc[a] = fmaf(sa[a], rr[a * N + k], acc[a]);
-        }
     }
   }
   __syncthreads();
-  lp_block_store(acc, Ng, part, Ng);
+  lp_block_store(acc, NG, part, NG);
 }
 
+// Blocks of the block-Jacobi kernels: one pass of 256 / N tets each up to 4,096 blocks, then equal numbers of
+// passes (a fixed 1,216 blocks at 10,368 tets of N = 35 left 266 of them with a second pass, all others idle).
+int lp_partial_blocks(int ne, int N) {
+  const int tb = 256 / N, passes = (ne + tb - 1) / tb, rounds = (passes + 4095) / 4096;
+  return passes < 1 ? 1 : (passes + rounds - 1) / rounds;
+}
+
+template <int NC>
+static void lp_update_bj_n(cudaStream_t st, int grid, int ne, int Ng, const double* alpha, float* x,
+                           float* r, const float* p, const float* q, const float* Binv, float* z, double* part) {
+  switch (Ng) {
+    case 1: k_lp_update_bj<NC, 1><<<grid, 256, 0, st>>>(ne, alpha, x, r, p, q, Binv, z, part); break;
+    case 2: k_lp_update_bj<NC, 2><<<grid, 256, 0, st>>>(ne, alpha, x, r, p, q, Binv, z, part); break;
+    case 3: k_lp_update_bj<NC, 3><<<grid, 256, 0, st>>>(ne, alpha, x, r, p, q, Binv, z, part); break;
+    case 4: k_lp_update_bj<NC, 4><<<grid, 256, 0, st>>>(ne, alpha, x, r, p, q, Binv, z, part); break;
+    default: k_lp_update_bj<NC, 5><<<grid, 256, 0, st>>>(ne, alpha, x, r, p, q, Binv, z, part); break;
+  }
+}
 void lp_update_bjacobi(cudaStream_t st, int ne, int N, int Ng, const double* alpha, float* x, float* r, const float* p,
                        const float* q, const float* Binv, float* z, double* part) {
-  const int TB = 256 / N;
-  const size_t smem = (size_t)TB * N * Ng * sizeof(float);
-  if (N == 35 && Ng == 5) k_lp_update_bj<35, 5><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
-  else if (N == 20 && Ng == 2) k_lp_update_bj<20, 2><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
-  else if (N == 35) k_lp_update_bj<35, 0><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
-  else if (N == 20) k_lp_update_bj<20, 0><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
-  else if (N == 10) k_lp_update_bj<10, 0><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
-  else k_lp_update_bj<0, 0><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, alpha, x, r, p, q, Binv, z, part);
+  const int grid = lp_partial_blocks(ne, N);
+  switch (N) {
+    case 1: lp_update_bj_n<1>(st, grid, ne, Ng, alpha, x, r, p, q, Binv, z, part); break;
+    case 4: lp_update_bj_n<4>(st, grid, ne, Ng, alpha, x, r, p, q, Binv, z, part); break;
+    case 10: lp_update_bj_n<10>(st, grid, ne, Ng, alpha, x, r, p, q, Binv, z, part); break;
+    case 20: lp_update_bj_n<20>(st, grid, ne, Ng, alpha, x, r, p, q, Binv, z, part); break;
+    default: lp_update_bj_n<35>(st, grid, ne, Ng, alpha, x, r, p, q, Binv, z, part); break;
+  }
 }
 
 // out = float(coef * Sum_b M[a][b] in[b])   (time mixing + conversion)
@@ -667,8 +669,8 @@ __global__ void k_lp_from64(int64_t ne, int N, int Ng, const double* __restrict_
                             const double* __restrict__ in, float* __restrict__ out) {
   const int Nst = N * Ng;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = e / N;
-    const int k = (int)(e % N);
+    const int64_t i = (uint32_t)e / (uint32_t)N;
+    const int k = (int)(e - i * N);
     for (int a = 0; a < Ng; ++a) {
       double s = 0.0;
       for (int b = 0; b < Ng; ++b) s = fma(M[a * Ng + b], in[i * Nst + b * N + k], s);
@@ -705,16 +707,24 @@ LpKernels lp_kernels() {
     k_lp_cg_update<<<kLpBlocks, 256, 0, st>>>(ne, N, Ng, alpha, x, r, p, q, t, part, want);
   };
   k.dir = [](cudaStream_t st, int64_t n, int N, int Ng, const double* beta, const float* z, float* p) {
-    k_lp_cg_dir<<<kLpBlocks, 256, 0, st>>>(n / ((int64_t)N * Ng), N, Ng, beta, z, p);
+    const int64_t np = n / Ng;
+    const int grid = (int)std::min<int64_t>(kLpBlocks, (np + 255) / 256);
+    switch (Ng) {
+      case 1: k_lp_cg_dir<1><<<grid, 256, 0, st>>>(np, N, beta, z, p); break;
+      case 2: k_lp_cg_dir<2><<<grid, 256, 0, st>>>(np, N, beta, z, p); break;
+      case 3: k_lp_cg_dir<3><<<grid, 256, 0, st>>>(np, N, beta, z, p); break;
+      case 4: k_lp_cg_dir<4><<<grid, 256, 0, st>>>(np, N, beta, z, p); break;
+      default: k_lp_cg_dir<5><<<grid, 256, 0, st>>>(np, N, beta, z, p); break;
+    }
   };
   k.bjacobi = [](cudaStream_t st, int ne, int N, int Ng, const float* Binv, const float* r, float* z, double* part) {
     const int TB = 256 / N;                         // one thread per (tet, row)
     const size_t smem = (size_t)TB * N * Ng * sizeof(float);
     switch (N) {
-      case 20: k_lp_bjacobi<20><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
-      case 35: k_lp_bjacobi<35><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
-      case 10: k_lp_bjacobi<10><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
-      default: k_lp_bjacobi<0><<<kLpBlocks, 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
+      case 20: k_lp_bjacobi<20><<<lp_partial_blocks(ne, N), 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
+      case 35: k_lp_bjacobi<35><<<lp_partial_blocks(ne, N), 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
+      case 10: k_lp_bjacobi<10><<<lp_partial_blocks(ne, N), 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
+      default: k_lp_bjacobi<0><<<lp_partial_blocks(ne, N), 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
     }
   };
   k.from64 = [](cudaStream_t st, int64_t ne, int N, int Ng, const double* Mdev, double coef, const double* in, float* out) {

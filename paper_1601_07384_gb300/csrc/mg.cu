@@ -31,7 +31,7 @@ namespace stdg {
 
 constexpr int kCoarseMax = 512;       // the coarsest level is solved with a dense inverse
 constexpr int kMgThreads = 256;
-constexpr int kMgUp0Blocks = 304;     // 2 x 152 SMs: the blocks that write r.z partials
+constexpr int kMgUp0Blocks = 304;     // 2 x 152 SMs: at most so many blocks write r.z partials
 constexpr int kMgMaxLevels = 16;
 
 struct MgLevel {
@@ -54,19 +54,17 @@ struct MgState {
 
 namespace {
 
-__device__ inline void mg_block_store(double* v, int cnt, double* part) {
-  __shared__ double red[kMaxNg][kMgThreads / 32];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int c = 0; c < cnt; ++c) {
-    double t = v[c];
-    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    if (lane == 0) red[c][w] = t;
-  }
+template <int NG>
+__device__ inline void mg_block_store(const double (&v)[NG], double* part) {
+  __shared__ double red[8][kMgThreads / 32];
+  int col;
+  const double t = warp_sums<NG>(v, col);
+  red[col][threadIdx.x >> 5] = t;                  // the lanes that share a column write the same value
   __syncthreads();
-  if (threadIdx.x < cnt) {
-    double t = 0.0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += red[threadIdx.x][k];
-    part[(size_t)blockIdx.x * cnt + threadIdx.x] = t;
+  if (threadIdx.x < NG) {
+    double u = 0.0;
+    for (int k = 0; k < kMgThreads / 32; ++k) u += red[threadIdx.x][k];
+    part[(size_t)blockIdx.x * NG + threadIdx.x] = u;
   }
 }
 
@@ -211,47 +209,49 @@ __global__ void __launch_bounds__(kMgThreads) k_mg_up(int n, int Ng, const int* 
 
 // Tets <- level 1, added to the preconditioned residual's constant modes: z_i0 += x_i, with the
 // partials of r.(R^T x) per column (the coarse part of r.z).  The pinned coefficient is left alone.
-template <typename T>
-__global__ void __launch_bounds__(kMgThreads) k_mg_up0(int ne, int Ng, int N, int Nst, const int* __restrict__ t2n,
+template <typename T, int NG>
+__global__ void __launch_bounds__(kMgThreads) k_mg_up0(int ne, int N, const int4* __restrict__ t2n,
                                                        const float* __restrict__ a0, const float* __restrict__ d0,
                                                        const int* __restrict__ par0, const T* __restrict__ r,
                                                        const float* __restrict__ x1, T* __restrict__ z,
                                                        double* __restrict__ part) {
-  double dot[kMaxNg] = {0, 0, 0, 0, 0};
+  const int Nst = N * NG;
+  double dot[NG];
+#pragma unroll
+  for (int q = 0; q < NG; ++q) dot[q] = 0.0;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < ne; i += gridDim.x * blockDim.x) {
     if (i == 0) continue;
     const float* a = a0 + (size_t)i * 5;
     const float di = d0[i];
     const int pi = par0[i];
-    T ri[kMaxNg];
-    float s[kMaxNg], ei[kMaxNg];
+    const int4 t4 = t2n[i];
+    const int nbs[4] = {t4.x, t4.y, t4.z, t4.w};
+    T ri[NG];
+    float s[NG], ei[NG];
 #pragma unroll
-    for (int q = 0; q < kMaxNg; ++q)
-      if (q < Ng) {
-        ri[q] = r[(size_t)i * Nst + q * N];
-        ei[q] = di * (float)ri[q] + x1[(size_t)pi * Ng + q];
-        s[q] = (float)ri[q] - a[0] * ei[q];
-      }
+    for (int q = 0; q < NG; ++q) {
+      ri[q] = r[(size_t)i * Nst + q * N];
+      ei[q] = di * (float)ri[q] + x1[(size_t)pi * NG + q];
+      s[q] = (float)ri[q] - a[0] * ei[q];
+    }
 #pragma unroll
     for (int f = 0; f < 4; ++f) {
-      const int nb = t2n[4 * i + f];
+      const int nb = nbs[f];
       if (nb <= 0) continue;
       const float w = a[1 + f], dj = d0[nb];
       const int pj = par0[nb];
 #pragma unroll
-      for (int q = 0; q < kMaxNg; ++q)
-        if (q < Ng) s[q] -= w * (dj * (float)r[(size_t)nb * Nst + q * N] + x1[(size_t)pj * Ng + q]);
+      for (int q = 0; q < NG; ++q) s[q] -= w * (dj * (float)r[(size_t)nb * Nst + q * N] + x1[(size_t)pj * NG + q]);
     }
 #pragma unroll
-    for (int q = 0; q < kMaxNg; ++q)
-      if (q < Ng) {
-        const float xi = ei[q] + di * s[q];
-        const size_t o = (size_t)i * Nst + q * N;
-        z[o] = z[o] + (T)xi;
-        dot[q] += (double)ri[q] * (double)xi;
-      }
+    for (int q = 0; q < NG; ++q) {
+      const float xi = ei[q] + di * s[q];
+      const size_t o = (size_t)i * Nst + q * N;
+      z[o] = z[o] + (T)xi;
+      dot[q] += (double)ri[q] * (double)xi;
+    }
   }
-  mg_block_store(dot, Ng, part);
+  mg_block_store<NG>(dot, part);
 }
 
 inline int mg_grid(int n) { return std::max(1, std::min((n + kMgThreads - 1) / kMgThreads, 1216)); }
@@ -503,7 +503,9 @@ stdg_status mg_ensure(stdg_solver* s) {
 }
 
 int mg_launches(const stdg_solver* s) { return s->mg ? 2 * s->mg->L + 1 : 0; }
-int mg_partial_blocks() { return kMgUp0Blocks; }
+int mg_partial_blocks(const stdg_solver* s) {
+  return std::max(1, std::min(((int)s->ne + kMgThreads - 1) / kMgThreads, kMgUp0Blocks));
+}
 int mg_levels(const stdg_solver* s, int* sizes, int cap) {
   if (!s->mg) return 0;
   const int n = (int)s->mg->sizes.size();
@@ -526,8 +528,8 @@ static void mg_apply_t(stdg_solver* s, const T* r, T* z, double* part) {
   for (int l = L - 1; l >= 1; --l)
     k_mg_up<<<mg_grid(lv[l].n), kMgThreads, 0, st>>>(lv[l].n, Ng, lv[l].rp, lv[l].ci, lv[l].va, lv[l].dl, lv[l].par,
                                                      lv[l].r, lv[l + 1].x, lv[l].x);
-  k_mg_up0<T><<<kMgUp0Blocks, kMgThreads, 0, st>>>(ne, Ng, N, Nst, s->dm.t2n, mg->a0, mg->d0, mg->par0, r, lv[1].x, z,
-                                                   part);
+STDG_NG_SWITCH(Ng, (k_mg_up0<T, G><<<mg_partial_blocks(s), kMgThreads, 0, st>>>(
+      ne, N, reinterpret_cast<const int4*>(s->dm.t2n), mg->a0, mg->d0, mg->par0, r, lv[1].x, z, part)));
 }
 
 void mg_apply_f32(stdg_solver* s, const float* r, float* z, double* part) { mg_apply_t<float>(s, r, z, part); }

@@ -165,7 +165,8 @@ struct LpKernels {
   void (*f32s)(cudaStream_t, int64_t, double, const double*, float*);
 };
 LpKernels lp_kernels();
-// x += alpha p; r -= alpha q; z = Binv r; partials of r.z per column (kLpBlocks partials)
+// x += alpha p; r -= alpha q; z = Binv r; partials of r.z per column (lp_partial_blocks rows)
+int lp_partial_blocks(int ne, int N);
 void lp_update_bjacobi(cudaStream_t st, int ne, int N, int Ng, const double* alpha, float* x, float* r, const float* p,
                        const float* q, const float* Binv, float* z, double* part);
 cudaError_t lp_build_blocks(stdg_solver* s, int kind);
@@ -206,7 +207,7 @@ stdg_status mg_ensure(stdg_solver* s);       // host + device setup, outside str
 void mg_apply_f32(stdg_solver* s, const float* r, float* z, double* part);
 void mg_apply_f64(stdg_solver* s, const double* r, double* z, double* part);
 int mg_launches(const stdg_solver* s);       // kernel launches per application
-int mg_partial_blocks();
+int mg_partial_blocks(const stdg_solver* s);
 int mg_levels(const stdg_solver* s, int* sizes, int cap);
 void mg_free(stdg_solver* s);
 // Dense layer products on the tensor cores (tcgemm.cu): D = A B^T (+ A2 B2^T) with bfloat16 operands
@@ -233,16 +234,16 @@ stdg_status visc_pc_apply(stdg_solver* s, double nu, const double* r, double* z,
                           const double* Kt = nullptr);
 stdg_status visc_pc_apply32(stdg_solver* s, double nu, const float* r, float* z, const double* Kt);
 
-// Binary32 vector kernels of the inner COCG solves (cocg32.cu).  Vectors are [tet][time column][N];
+// Binary32 vector kernels of the inner COCG solves (cocg32.cu), on `grid` blocks (as many rows of partials).  Vectors are [tet][time column][N];
 // the multipliers M (Ng x Ng, binary64 on the device) are block diagonal with blocks of size 1 or 2,
 // so only M[a][a-1..a+1] is read.  mix holds an Ng x Ng matrix applied to every tet's time columns.
 struct Mix32 { float v[kMaxNg * kMaxNg]; };
-void c32_mix_to32(cudaStream_t st, int ne, int N, int Ng, const Mix32& M, const double* in, float* out);
-void c32_mix_acc64(cudaStream_t st, int ne, int N, int Ng, const Mix32& M, const float* y, double* x);
-void c32_cross(cudaStream_t st, int ne, int N, int Ng, const float* u, const float* v, double* part);
-void c32_update(cudaStream_t st, int ne, int N, int Ng, const double* M, float* y, float* r, const float* p,
+void c32_mix_to32(cudaStream_t st, int grid, int ne, int N, int Ng, const Mix32& M, const double* in, float* out);
+void c32_mix_acc64(cudaStream_t st, int grid, int ne, int N, int Ng, const Mix32& M, const float* y, double* x);
+void c32_cross(cudaStream_t st, int grid, int ne, int N, int Ng, const float* u, const float* v, double* part);
+void c32_update(cudaStream_t st, int grid, int ne, int N, int Ng, const double* M, float* y, float* r, const float* p,
                 const float* q, const Mix32& W, double* part, int want);
-void c32_dir(cudaStream_t st, int ne, int N, int Ng, const double* M, const float* z, float* p);
+void c32_dir(cudaStream_t st, int grid, int ne, int N, int Ng, const double* M, const float* z, float* p);
 bool time_blockdiag(const double* K, int Ng, double* W, double* Winv, double* R, int* pair);
 void prof_fold(stdg_solver* s);
 }  // namespace stdg
