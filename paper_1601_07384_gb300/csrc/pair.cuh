@@ -1,7 +1,7 @@
 // Binary64-accurate arithmetic on unevaluated pairs of binary32 numbers (hi, lo), value hi + lo:
 // products split exactly by fused multiply-adds, sums kept error-free (TwoSum), so a sum of products
 // is accurate to about 2^-48 of the sum of |terms| at a few binary32 operations per term, on a pipe
-// 64 times faster than sm_103a's binary64 pipe.  Shared by the convection and support kernels.
+// 64 times faster than sm_103a's binary64 pipe.  Shared by the convection kernels.
 #pragma once
 #include "lp_ptx.cuh"
 
@@ -10,6 +10,19 @@ namespace stdg {
 __device__ __forceinline__ float2 pair_split(double a) {
   const float h = (float)a;
   return make_float2(h, (float)(a - (double)h));
+}
+// the same pair (ties in hi aside) by integer operations where both parts are normal numbers: conversions and
+// subtractions in binary64 take 64 cycles per warp each
+__device__ __forceinline__ float2 pair_split_int(double a) {
+  const unsigned h = (unsigned)__double2hiint(a), l = (unsigned)__double2loint(a);
+  const int e = (int)(h >> 20 & 0x7FF) - 1023;
+  if (e < -60 || e > 120) return a == 0.0 ? make_float2(0.0f, 0.0f) : pair_split(a);
+  // the 53 bits m as hm 2^29 + lm, hm rounded to nearest
+  const unsigned hm = ((h & 0xFFFFFu | 0x100000u) << 3 | l >> 29) + (l >> 28 & 1);
+  const int lm = (int)(l << 3) >> 3;
+  const unsigned sg = h & 0x80000000u;
+  return make_float2((float)hm * __uint_as_float((unsigned)(e + 104) << 23 | sg),
+                     (float)lm * __uint_as_float((unsigned)(e + 75) << 23 | sg));
 }
 // The rounded products below are formed with __fmul_rn, which is never fused into a multiply-add:
 // with the compiler's default contraction a plain product feeding the sum s + p may become
@@ -44,6 +57,13 @@ __device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
   const float bb = s - a.x;
   const float e = ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y);
   return pair_norm(s, e);
+}
+// sqrt(a) for a >= 0: one Newton step in the residual doubles the 24 bits of the binary32 root
+__device__ __forceinline__ float2 pair_sqrt(float2 a) {
+  const float s = __fsqrt_rn(a.x);
+  if (!(s > 0.0f) || s > 3.4e38f) return make_float2(s, 0.0f);
+  const float r = fmaf(-s, s, a.x) + a.y;
+  return pair_norm(s, __fdividef(r, s + s));
 }
 __device__ __forceinline__ float2 pair_neg(float2 a) { return make_float2(-a.x, -a.y); }
 

@@ -91,7 +91,7 @@ struct stdg_solver {
   double theta = 1.0;                          // semi-implicit pressure weight (p_t = 0 only)
   double *Pn = nullptr, *Pth = nullptr;        // p^n and theta p^{n+1,k} + (1 - theta) p^n (theta < 1)
   float2 *cphiP = nullptr, *cdphiP = nullptr, *cfphiP = nullptr;   // convection tables as (hi, lo) pairs
-  float2 *cphiT = nullptr, *cfphiT = nullptr;                        // the value tables transposed
+  float2* conv_tab = nullptr;                                         // tables of the modal kernels (conv.cu)
   float2 *ctgP = nullptr, *ctwP = nullptr;                            // time basis and weights, as pairs
   // device allocations: through the caller's allocator when one was given (stdg_solver_create_alloc),
   // else cudaMalloc; released in reverse order by stdg_solver_destroy
@@ -198,6 +198,7 @@ void gnn_mg_harvest_snap(stdg_solver* s, int k, const double* r, const double* x
 void gnn_mg_harvest_finish(stdg_solver* s, int got, const double* x);
 stdg_status solve_viscous(stdg_solver* s, const double* b, double* x, double nu, double tol, int* iters,
                           double* res);
+stdg_status convection_modal(stdg_solver* s, const FieldArg& fld, const double* vbar, double* ups);   // conv.cu
 stdg_status dev_alloc(stdg_solver* s, void** p, size_t bytes);
 cudaError_t dev_alloc_cuda(stdg_solver* s, void** p, size_t bytes);   // the same, as a CUDA error code
 void dev_free(stdg_solver* s, void* p);                                 // early release of one array
