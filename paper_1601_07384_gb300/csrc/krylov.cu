@@ -1752,7 +1752,11 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
 // binary64; x is left unchanged unless the solve reaches tol_abs.
 static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu, const double* b, double* x,
                                   double tol_abs, int* iters, double* res) {
-  const int Ng = s->Ng, N = s->N, ne = (int)s->ne, rb = red_grid(s->ne * (int64_t)N);
+  const int Ng = s->Ng, N = s->N, ne = (int)s->ne;
+  // three blocks per SM: every block ends with binary64 reductions of up to 3 Ng - 2 sums, and one block sums
+  // the rows that they leave (1,216 rows at 10,368 tets, p = p_t = 4: 14.7 us an iteration for that alone)
+  const int64_t want = red_grid(s->ne * (int64_t)N);
+  const int rb = want < 456 ? (int)want : 456;
   const int64_t n = s->ne * (int64_t)s->Nst;
   if (s->vbd < 0) s->vbd = time_blockdiag(s->K.data(), Ng, s->vW, s->vWinv, s->vR, s->vpair) ? 1 : 0;
   if (!s->vbd) return STDG_EUNSUPPORTED;

@@ -457,6 +457,203 @@ __global__ void __launch_bounds__(128, 1) k_apply_warp(WarpArgs a, const typenam
   }
 }
 
+// Five warps per tet, one per block, for the blocks of p = 4 in binary32 or bfloat16: a CTA runs a
+// strided stream of tets with two stages, warp w staging and multiplying block w (0: the diagonal one).  The
+// kernel with a warp per tet needs a stage of all five blocks per warp: 7 warps per SM at p = 4, too few to
+// cover their own shared-memory latency and loads; here 15 at p = 4 with the next tet's blocks always in flight,
+// and a fifth of the work between two waits.  One barrier per tet: after it the stage is free and the five
+// partial rows are complete (two buffers of these, so that the sums of one tet and the products of the next
+// overlap).
+template <typename W, int NG, int N>
+struct CtaDim {
+  static constexpr int NR = warp_nr_c(N), NP = warp_np_c(N), T = 160;
+  static_assert(N > 32 && N <= 35, "rows: one per lane and the rest in groups of 8 lanes");
+  static constexpr uint32_t blk = (uint32_t)(NR * NP * sizeof(typename W::TB));
+  static constexpr uint32_t xrow = (uint32_t)(NG * NR * sizeof(float));             // one slot's x
+  static constexpr uint32_t stage = 5 * blk + 5 * xrow, red = 5 * NG * NR * sizeof(float);
+  static constexpr uint32_t smem = 2 * stage + 2 * red + 16;
+  static_assert(blk % 16 == 0 && xrow % 16 == 0 && red % 16 == 0, "bulk copies and vector loads");
+};
+template <typename W, int NG, int N>
+__global__ void __launch_bounds__(160, 3) k_apply_cta(const __grid_constant__ WarpArgs a,
+                                                                   const float* __restrict__ x, float* __restrict__ y) {
+  using TB = typename W::TB;
+  using D = CtaDim<W, NG, N>;
+  constexpr int NR = D::NR, NP = D::NP, Nst = N * NG;
+  extern __shared__ __align__(128) unsigned char wsm[];
+  const int lane = threadIdx.x & 31, slot = threadIdx.x >> 5, G = gridDim.x;
+  float* red = reinterpret_cast<float*>(wsm + 2 * D::stage);                       // [2][slot][q][NR]
+  uint64_t* bar = reinterpret_cast<uint64_t*>(wsm + 2 * D::stage + 2 * D::red);
+  for (int st = 0; st < 2; ++st) {
+    float* xz = reinterpret_cast<float*>(wsm + st * D::stage + 5 * D::blk);
+    for (int e = threadIdx.x; e < 5 * NG * NR; e += D::T) xz[e] = 0.0f;             // padding entries stay 0
+  }
+  // parameters in binary32, converted once (every binary64 conversion or compare takes 64 cycles per warp)
+  __shared__ float tacc[NG * NG], kmass[NG * NG];
+  const float scale = (float)a.scale;
+  const bool has_mass = a.mass_coef != 0.0;
+  if (threadIdx.x < NG * NG) {
+    tacc[threadIdx.x] = (float)a.Tacc[threadIdx.x];
+    kmass[threadIdx.x] = (float)a.Kmass[threadIdx.x];
+  }
+  if (threadIdx.x == 0) {
+    for (int st = 0; st < 2; ++st) mbar_init(&bar[st], 5 + D::T);                   // five expect_tx, all cp.async arrivals
+    fence_async_smem();
+  }
+  __syncthreads();
+  // this warp's block of tet i: f = index << 1 | transposed, or -1; nb the tet whose x it multiplies
+  auto fetch = [&](int i, int& f, int& nb) {
+    f = -1; nb = -1;
+    if (i >= a.ne) return;
+    if (slot == 0) { f = i << 1; nb = i; return; }
+    f = reinterpret_cast<const int*>(a.gface)[4 * (size_t)i + slot - 1];
+    nb = reinterpret_cast<const int*>(a.gnbr)[4 * (size_t)i + slot - 1];
+  };
+  auto issue = [&](int st, int f, int nb) {
+    unsigned char* sb = wsm + st * D::stage;
+    if (lane == 0) {
+      fence_async_smem();                         // earlier generic reads of this stage before the copy
+      mbar_expect_tx(&bar[st], f >= 0 ? D::blk : 0);
+      if (f >= 0)
+        tma_load_1d(sb + slot * D::blk, static_cast<const unsigned char*>(slot == 0 ? a.Bd : a.Ao) + (size_t)(f >> 1) * D::blk,
+                    D::blk, &bar[st]);
+    }
+    if (f >= 0) {
+      float* xr = reinterpret_cast<float*>(sb + 5 * D::blk + slot * D::xrow);
+      const float* src = x + (size_t)nb * Nst;
+#pragma unroll
+      for (int q = 0; q < NG; ++q)
+        for (int l = lane; l < N; l += 32) cp_async<4>(xr + q * NR + l, src + q * N + l);
+    }
+    cp_async_mbar_arrive_noinc(&bar[st]);
+  };
+  float dacc[NG];
+#pragma unroll
+  for (int q = 0; q < NG; ++q) dacc[q] = 0.0f;
+  int i = blockIdx.x, it = 0, f0, n0, f1, n1, f2, n2;
+  bool abort = false;
+  fetch(i, f0, n0);
+  fetch(i + G, f1, n1);
+  fetch(i + 2 * G, f2, n2);
+  if (i < a.ne) issue(0, f0, n0);
+  if (i + G < a.ne) issue(1, f1, n1);
+  for (; i < a.ne; i += G, ++it) {
+    const int st = it & 1;
+    long spins = 0;
+    while (!mbar_wait_hint(&bar[st], (uint32_t)(it >> 1) & 1))
+      if (++spins > kWarpSpin) { abort = true; break; }
+    __syncwarp();
+    float* rd = red + (st * 5 + slot) * NG * NR;
+    if (!abort) {
+      const TB* B = reinterpret_cast<const TB*>(wsm + st * D::stage + slot * D::blk);
+      float* z = reinterpret_cast<float*>(wsm + st * D::stage + 5 * D::blk + slot * D::xrow);
+      if (a.pinned && n0 == 0) {                  // the constant mode of tet 0 reads as 0
+        if (lane < NG) z[lane * NR] = 0.0f;
+        __syncwarp();
+      }
+      float2 c0[NG], c1[NG];
+#pragma unroll
+      for (int q = 0; q < NG; ++q) c0[q] = c1[q] = make_float2(0.0f, 0.0f);
+      if (f0 >= 0) {                              // row `lane`
+        if (f0 & 1) {                             // column: A_rl = A_lr^T
+#pragma unroll
+          for (int l = 0; l < NR; l += 8) {
+            warp_chunk2<NG>(B + l * NP + lane, NP, z + l, NR, c0);
+            if (l + 4 < NR) warp_chunk2<NG>(B + (l + 4) * NP + lane, NP, z + l + 4, NR, c1);
+          }
+        } else {
+#pragma unroll
+          for (int l = 0; l < NR; l += 8) {
+            warp_chunk2<NG>(B + lane * NP + l, 1, z + l, NR, c0);
+            if (l + 4 < NR) warp_chunk2<NG>(B + lane * NP + l + 4, 1, z + l + 4, NR, c1);
+          }
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NG; ++q) rd[q * NR + lane] = (c0[q].x + c0[q].y) + (c1[q].x + c1[q].y);
+      const int g = lane >> 3, c = lane & 7, r = 32 + g;   // rows 32 .. 34: 8 lanes per row, chunks split
+      float2 ec[NG];
+#pragma unroll
+      for (int q = 0; q < NG; ++q) ec[q] = make_float2(0.0f, 0.0f);
+      if (f0 >= 0 && r < N) {
+        for (int l = 4 * c; l < NR; l += 32) {
+          if (f0 & 1) warp_chunk2<NG>(B + l * NP + r, NP, z + l, NR, ec);
+          else warp_chunk2<NG>(B + r * NP + l, 1, z + l, NR, ec);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        float h = ec[q].x + ec[q].y;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+        if (c == 0 && r < N) rd[q * NR + r] = h;
+      }
+    }
+    if (__syncthreads_or(abort)) { abort = true; break; }
+    // the stage is free: the tet after the next one
+    if (i + 2 * G < a.ne) issue(st, f2, n2);
+    f0 = f1; n0 = n1; f1 = f2; n1 = n2;
+    fetch(i + 3 * G, f2, n2);
+    const int k = threadIdx.x;
+    if (k < N) {                                  // row k: the five sums, time mixing, scale, mass term, pin
+      const float* rk = red + st * 5 * NG * NR + k;
+      float v[NG];
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        v[q] = 0.0f;
+#pragma unroll
+        for (int sl = 0; sl < 5; ++sl) v[q] += rk[(sl * NG + q) * NR];
+      }
+      const float* xi = x + (size_t)i * Nst + k;
+      const float mj = has_mass ? (float)(a.mass_coef * a.detJ[i]) : 0.0f;
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        float o = v[q];
+        if (!a.kron) {
+          o = 0.0f;
+#pragma unroll
+          for (int b = 0; b < NG; ++b) o += tacc[q * NG + b] * v[b];
+        }
+        o *= scale;
+        if (has_mass) {
+          float m = 0.0f;
+#pragma unroll
+          for (int b = 0; b < NG; ++b) m += kmass[q * NG + b] * xi[b * N];
+          o += mj * m;
+        }
+        if (a.pinned && i == 0 && k == 0) o = (float)a.pin_diag * x[q * N];
+        y[(size_t)i * Nst + q * N + k] = o;
+        if (a.dotpart) dacc[q] += xi[q * N] * o;
+      }
+    }
+  }
+  if (a.dotpart) {                                // fixed order: lanes by shuffle, warps by index
+    __shared__ float wdot[5][NG];
+#pragma unroll
+    for (int q = 0; q < NG; ++q) {
+      float v = dacc[q];
+      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+      if (lane == 0) wdot[slot][q] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < NG) {
+      double t = 0.0;
+      for (int w = 0; w < 5; ++w) t += (double)wdot[w][threadIdx.x];
+      a.dotpart[(size_t)blockIdx.x * NG + threadIdx.x] = t;
+    }
+  }
+  if (abort) {
+    if (threadIdx.x == 0) atomicExch(a.err, 1);
+    // bounded wait for the copies in flight: those of tets it and, where there is one, it + 1
+    for (int j = it; j < it + 2; ++j) {
+      if (i + (j - it) * G >= a.ne) break;
+      long spins = 0;
+      while (!mbar_wait_hint(&bar[j & 1], (uint32_t)(j >> 1) & 1) && ++spins < kWarpSpin) {
+      }
+    }
+  }
+}
+
 // padded block copies: dst block b = planes x NR x NP, zero outside N x N.  A CTA takes whole blocks, about 4,096
 // entries at a time, indices by divisions with constants and the scaling from shared memory (a constant-bank read
 // with an index per thread is repeated for each value); one plane is rounded to binary32 without the binary64
@@ -557,10 +754,23 @@ static constexpr int warp_kind() { return W::kPlanes == 2 ? 2 : (sizeof(typename
 template <typename W>
 using WarpKernel = void (*)(WarpArgs, const typename W::XIn*, typename W::YOut*);
 
+// p = 4: k_apply_cta with binary32 blocks at every size (us per application, the warp-per-tet kernel -> this one, L2
+// flushed; p_t = 0: 750 tets 10.9 -> 10.9, 2,058 17.1 -> 15.0, 10,368 47.8 -> 45.7; p_t = 2: 13.0 -> 11.9, 21.2 -> 17.0,
+// 64.2 -> 51.9; p_t = 4: 13.0 -> 12.9, 21.2 -> 21.1, 66.2 -> 66.2), with bfloat16 blocks, of which twice as many warps
+// fit, only where few tets leave those without work (p_t = 2: 2,058 tets 21.2 -> 15.0, 4,374 29.3 -> 25.2; but p_t = 0:
+// 4,374 19.1 -> 19.1, 10,368 31.4 -> 33.4).  p = 3 keeps the warp per tet: 82,944 tets, p_t = 1, 99 us against 127.
+template <typename W>
+static bool cta_serves(const stdg_solver* s) {
+  return W::kPlanes == 1 && s->N == 35 && (sizeof(typename W::TB) == 4 || s->ne <= 32 * 152);
+}
+
 // the instantiation for this N: compile-time N for p = 2, 3, 4, runtime N otherwise
 template <typename W, int NG>
-static WarpKernel<W> warp_kernel(int N) {
-  switch (N) {
+static WarpKernel<W> warp_kernel(const stdg_solver* s) {
+  if constexpr (W::kPlanes == 1) {
+    if (cta_serves<W>(s)) return k_apply_cta<W, NG, 35>;
+  }
+  switch (s->N) {
     case 10: return k_apply_warp<W, NG, 10>;
     case 20: return k_apply_warp<W, NG, 20>;
     case 35: return k_apply_warp<W, NG, 35>;
@@ -573,12 +783,22 @@ static WarpKernel<W> warp_kernel(int N) {
 template <typename W, int NG>
 static cudaError_t warp_configure(stdg_solver* s) {
   const WarpArgs a = warp_args<W>(s);
-  const WarpKernel<W> kern = warp_kernel<W, NG>(s->N);
+  const WarpKernel<W> kern = warp_kernel<W, NG>(s);
   int& grid = s->warp_grid[warp_kind<W>() * 8 + NG];
   int& wpc = s->warp_wpc[warp_kind<W>() * 8 + NG];
   if (grid != 0) return cudaSuccess;
   int nsm = 152;
   cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, s->device);
+  if (cta_serves<W>(s)) {
+    const int smem = (int)CtaDim<W, NG, 35>::smem;
+    int per = 0;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, kern, 160, smem);
+    if (e != cudaSuccess || per == 0) return e != cudaSuccess ? e : cudaErrorInvalidConfiguration;
+    wpc = 5;
+    grid = nsm * (per < 8 ? per : 8);             // at most 1,216 rows of x . y partials
+    return cudaSuccess;
+  }
   int best = 0, bw = 1;
   for (int c : {4, 2, 1}) {
     const size_t smem = (size_t)c * a.warp_bytes;
@@ -612,8 +832,8 @@ template <typename W, int NG>
 static cudaError_t launch_warp_ng(stdg_solver* s, const WarpArgs& a, const typename W::XIn* x, typename W::YOut* y) {
   const int grid = s->warp_grid[warp_kind<W>() * 8 + NG], wpc = s->warp_wpc[warp_kind<W>() * 8 + NG];
   if (grid == 0) return cudaErrorNotReady;                  // warp_prepare has not run
-  const size_t smem = (size_t)wpc * a.warp_bytes;
-  warp_kernel<W, NG>(s->N)<<<grid, 32 * wpc, smem, s->stream>>>(a, x, y);
+  const size_t smem = cta_serves<W>(s) ? CtaDim<W, NG, 35>::smem : (size_t)wpc * a.warp_bytes;
+  warp_kernel<W, NG>(s)<<<grid, 32 * wpc, smem, s->stream>>>(a, x, y);
   return cudaGetLastError();
 }
 

@@ -155,3 +155,22 @@ def test_step_matches_oracle_at_other_degrees(p, pt):
             Uo[j, s] = (fb["Mij"][s] @ so.V[j].T).T
     assert rel(P.cpu().numpy(), so.P.ravel()) <= 1e-10
     assert rel(U, Uo) <= 1e-10
+
+
+@pytest.mark.parametrize("pt", range(5))
+@pytest.mark.parametrize("precision,tol", [("mixed_f32", 4e-6), ("mixed_bf16", 2e-2)])
+@pytest.mark.parametrize("n", [2, 5, 9, 10])
+def test_low_precision_operator_at_p4(n, pt, precision, tol):
+    """Five warps per tet: fewer tets than CTAs, a few per CTA (both stages reused), and sizes on either side of
+    the line above which bfloat16 blocks take the kernel with one warp per tet; against the binary64 product."""
+    import paper_1601_07384_gb300 as g
+    gs = g.Solver(g.Mesh(*kuhn_mesh(n, seed=0)), g.Reference(4, pt), 0.01, precision=precision)
+    x = torch.randn(gs.pressure_empty().numel(), generator=torch.Generator().manual_seed(n), dtype=torch.float32).cuda()
+    for pinned in (True, False):
+        y = gs.pressure_apply_f32(x, pinned=pinned).double()
+        yo = gs.pressure_apply(x.double(), pinned=pinned)
+        # the pinned row carries its own large diagonal entry: compare it apart
+        sel = torch.ones_like(yo, dtype=torch.bool)
+        if pinned:
+            sel.view(-1)[torch.arange(pt + 1, device="cuda") * 35] = False
+        assert float((y - yo)[sel].abs().max() / yo[sel].abs().max()) <= tol
