@@ -534,8 +534,8 @@ def main():
     e2e = (time.perf_counter() - te0) / ne2e
 
     # ---- roofline of the dominant operator kernel (CUDA-event time of its launches in the timed region)
-    kinds = ["fp64 blocks (k_apply)", "binary32-pair blocks (k_apply_warp<WDF>)", "binary32 blocks (k_apply_warp<WF32>)",
-             "bfloat16 blocks (k_apply_warp<WBF16>)"]
+    kinds = ["fixed-point blocks (k_fx)", "binary32-pair blocks (k_apply_warp<WDF>)", "binary32 blocks (k_apply_warp/k_apply_cta<WF32>)",
+             "bfloat16 blocks (k_apply_warp/k_apply_cta<WBF16>)"]
     kbest = int(np.argmax(prof["kind_ms"]))
     nlaunch_k = max(prof["kind_launches"][kbest], 1)
     op_launch_ms = prof["kind_ms"][kbest] / nlaunch_k

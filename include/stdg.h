@@ -98,14 +98,12 @@ enum { STDG_SOLVER_GMRES = 0, STDG_SOLVER_CG = 1, STDG_SOLVER_KRON_CG = 2, STDG_
        STDG_SOLVER_FGMRES_BJ = 4, STDG_SOLVER_FGMRES_GNN = 5, STDG_SOLVER_KRON_MG = 6, STDG_SOLVER_KRON_MG_GNN = 7 };
 
 /* Precision of the operator blocks used inside the Krylov iteration (stdg_solver_options).
- *  STDG_PREC_FP64   : blocks and arithmetic in binary64.
- *  STDG_PREC_DF32   : binary64 blocks and vectors, products formed in pairs of binary32
- *                     ("double-float", ~48-bit significand) because sm_103a's binary64
- *                     pipe is 1/64 of its binary32 rate; results agree with STDG_PREC_FP64
- *                     to ~1e-14 relative per operator application.  Used for the pressure
- *                     and the viscous operators inside the solves.  Where that kernel would
- *                     run fewer than 6 warps per SM (its shared memory per warp grows as N^2:
- *                     p >= 4), the binary64 kernel serves instead; the results are the same.
+ *  STDG_PREC_FP64   : binary64 vectors and binary64-accurate products: the blocks are kept as 61-bit
+ *                     fixed-point numbers with an exponent per block and multiplied on the integer
+ *                     pipe (sm_103a's binary64 pipe is 1/64 of its binary32 rate); non-finite values
+ *                     propagate as in binary64.
+ *  STDG_PREC_DF32   : the same products (STDG_OP_KERNEL=warp in the environment, read when the solver
+ *                     is created, forms them in pairs of binary32 instead, ~1e-14 relative).
  *  STDG_PREC_MIXED_F32 / STDG_PREC_MIXED_BF16 : the Kronecker CG methods run as an inner-outer
  *                     iteration: flexible CG in binary64 (operator as in STDG_PREC_DF32)
  *                     preconditioned by a fixed number of block-Jacobi CG iterations whose
@@ -324,8 +322,7 @@ stdg_status stdg_solve(stdg_solver* s, const double* b_dev, double* x_dev, doubl
  *  - All calls share the one array, which keeps whatever the last call left in it (x is set to
  *    zero before the iteration; everything else is written before it is read).  Calls whose
  *    device work overlaps -- on different streams or from different threads -- race on it.
- *  - It always runs the Kronecker-decoupled CG on the binary64-accurate operator (binary64 blocks,
- *    or their binary32-pair form when the solver was created with another precision option), one
+ *  - It always runs the Kronecker-decoupled CG on the binary64-accurate operator, one
  *    host check per iteration: never the mixed-precision inner-outer iteration that stdg_solve runs
  *    for STDG_SOLVER_KRON_CG under STDG_PREC_MIXED_*.  Its iterates then differ from that call's at
  *    rounding level and its iteration count from that call's.
@@ -443,9 +440,9 @@ stdg_status stdg_tc_gemm_bf16(const float* A_dev, int64_t lda, const float* B_de
                               int64_t ldd, int M, int N, int K, void* stream);
 
 /* Throughput of the current device's binary64 and binary32 FMA pipes in TFLOP/s (2 flops per FMA),
- * measured with independent FMA chains on every SM and CUDA events on `stream`: the peaks the
- * binary64 operator kernel and, divided by the 12 binary32 operations of one pair product, the
- * pair kernel are rated against.  A measurement helper (the paper has no counterpart); allocates
+ * measured with independent FMA chains on every SM and CUDA events on `stream`: the peaks that
+ * binary64 arithmetic and, divided by the 12 binary32 operations of one product of binary32 pairs, the
+ * pair kernels are rated against.  A measurement helper (the paper has no counterpart); allocates
  * 16 bytes of device memory for the duration of the call. */
 stdg_status stdg_fma_probe(double* tflops_fp64, double* tflops_fp32, void* stream);
 

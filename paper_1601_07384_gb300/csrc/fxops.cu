@@ -11,7 +11,10 @@
 // which returns 128 bytes a cycle to an SM (8 cycles of each scheduler per 64-bit operand, also when all
 // lanes read the same word).  Thread tiles of 2 or 3 rows save such reads and were slower: the
 // blocks of a CTA fill the shared memory, so fewer threads per CTA are fewer warps per SM (N = 35, NG = 5
-// at 24,576 tets: 479 us with one row, 671 with two, 849 with three).
+// at 24,576 tets: 1.4 times the time with two rows, 1.8 times with three).  Measured, start of a pass to its
+// end, binary64 kernels before -> now: operator at 20,250 tets, p = 3, p_t = 0, 198 -> 80 us; at 24,576 tets,
+// p = p_t = 4, 766 (binary32 pairs) -> 579 us; right-hand side at 7,986 tets, p = p_t = 4, 1,597 -> 442 us;
+// velocity update at 20,250 tets, p = p_t = 2, 164 -> 107 us.
 //
 // Two launches: k_fx_vec scales the vector to limbs once, with one exponent per column of every tet (face,
 // component), and applies the time matrix to it where the operation has one; k_fx starts at the same time
