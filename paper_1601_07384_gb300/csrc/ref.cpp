@@ -49,8 +49,9 @@ static void jacobi(int n, double a, double b, double x, double* P, double* dP) {
 
 void gauss_jacobi01(int n, int alpha, std::vector<double>& x, std::vector<double>& w) {
   x.clear(); w.clear();
-  // neighbouring roots are at least about 2 / n^2 apart: some 40 intervals between them
-  const int grid = n * n < 500 ? 40 * n * n + 40 : 20000;
+  // neighbouring roots are at least about 8 / (n + 2)^2 apart: some 30 intervals between them (20,000 at every n
+  // took about a millisecond a rule)
+  const int grid = 8 * n * n + 8;
   double prev_x = -1.0, prev_v, d;
   jacobi(n, alpha, 0.0, -1.0 + 1e-15, &prev_v, &d);
   std::vector<double> roots;
