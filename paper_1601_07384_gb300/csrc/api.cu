@@ -71,7 +71,7 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   if (opts) {
     s->opt = *opts;
     if (s->opt.restart <= 0) s->opt.restart = 50;
-    if (s->opt.restart > 60) { delete s; set_error("restart must be <= 60"); return STDG_EUNSUPPORTED; }
+    if (s->opt.restart > kMaxRestart) { delete s; set_error("restart must be <= %d", kMaxRestart); return STDG_EUNSUPPORTED; }
     if (s->opt.max_iters <= 0) s->opt.max_iters = 200000;
     if (s->opt.graph_batch <= 0) s->opt.graph_batch = 8;
     if (s->opt.graph_batch > 64) { delete s; set_error("graph_batch must be <= 64"); return STDG_EINVAL; }
@@ -87,7 +87,7 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
     const char* mi = std::getenv("STDG_MIXED_INNER");   // binary32 iterations per outer mixed step
     if (mi && std::atoi(mi) > 0 && std::atoi(mi) <= 1000) s->mix_inner = s->mix_inner_mg = std::atoi(mi);
     const char* mm = std::getenv("STDG_MIXED_M");       // directions kept by the outer flexible CG
-    if (mm && std::atoi(mm) > 0 && std::atoi(mm) <= 16) s->mix_m = std::atoi(mm);
+    if (mm && std::atoi(mm) > 0 && std::atoi(mm) <= kMaxDirs) s->mix_m = std::atoi(mm);
     const char* vi = std::getenv("STDG_VISC_INNER64");
     s->visc_inner64 = vi && std::atoi(vi) == 1;
     const char* ck = std::getenv("STDG_CONV_KERNEL");  // "generic": no compile-time-degree convection kernel

@@ -15,7 +15,14 @@ namespace stdg {
 
 constexpr int kRedBlocks = 1216;   // 8 x 152 SMs
 constexpr int kRedThreads = 256;
-constexpr int kMaxCols = 64;
+// Columns that a reduction leaves per block: partials are kRedBlocks x kMaxCols.  The widest are the dots with
+// every stored direction of the flexible CG, one per time column.
+constexpr int kMaxCols = 80;
+static_assert(kMaxCols >= kMaxDirs * kMaxNg, "dots of the flexible CG (k_fcg_dots)");
+static_assert(kMaxCols >= kMaxRestart + 1, "dots of a Gram-Schmidt pass (k_multidot)");
+static_assert(kMaxCols >= kMaxNg * kMaxNg, "cross products of the viscous solve (k_crossdot)");
+static_assert((kLpMaxBlocks + kMgUp0Blocks) * kMaxNg <= kRedBlocks * kMaxCols, "r.z of the binary32 preconditioners");
+static_assert((kRedBlocks + kMgUp0Blocks) * kMaxNg <= kRedBlocks * kMaxCols, "r.z of the binary64 preconditioners");
 
 __device__ inline double warp_sum(double v) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);

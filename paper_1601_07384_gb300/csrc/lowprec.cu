@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(256) k_lp_update_bj(int ne, const double* __re
 // Blocks of the block-Jacobi kernels: one pass of 256 / N tets each up to 4,096 blocks, then equal numbers of
 // passes (a fixed 1,216 blocks at 10,368 tets of N = 35 left 266 of them with a second pass, all others idle).
 int lp_partial_blocks(int ne, int N) {
-  const int tb = 256 / N, passes = (ne + tb - 1) / tb, rounds = (passes + 4095) / 4096;
+  const int tb = 256 / N, passes = (ne + tb - 1) / tb, rounds = (passes + kLpMaxBlocks - 1) / kLpMaxBlocks;
   return passes < 1 ? 1 : (passes + rounds - 1) / rounds;
 }
 

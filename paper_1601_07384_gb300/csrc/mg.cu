@@ -31,7 +31,6 @@ namespace stdg {
 
 constexpr int kCoarseMax = 512;       // the coarsest level is solved with a dense inverse
 constexpr int kMgThreads = 256;
-constexpr int kMgUp0Blocks = 304;     // 2 x 152 SMs: at most so many blocks write r.z partials
 constexpr int kMgMaxLevels = 16;
 
 struct MgLevel {

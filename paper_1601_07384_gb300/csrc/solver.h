@@ -5,6 +5,10 @@
 #include "dev.cuh"
 
 namespace stdg {
+constexpr int kMaxDirs = 16;       // directions kept by the outer flexible CG of the mixed solves, at most
+constexpr int kMaxRestart = 60;    // GMRES directions (stdg_solver_options.restart), one more with the network's
+constexpr int kLpMaxBlocks = 4096; // rows of partials of the binary32 block Jacobi (lp_partial_blocks), at most
+constexpr int kMgUp0Blocks = 304;  // 2 x 152 SMs: rows of partials of the coarse correction, at most
 struct MgState;                    // agglomeration coarse correction (mg.cu)
 // State of the learned preconditioner (gnn.cu)
 struct GnnState {
@@ -63,7 +67,7 @@ struct stdg_solver {
   int op_pairs = 0;                           // the pair kernels serve the binary64-accurate pressure operator
   int mix_inner = 80;                         // binary32 CG iterations per outer step of the mixed solve
   int mix_inner_mg = 40;                      // the same with the coarse correction (converges faster)
-  int mix_m = 16;                             // directions the outer flexible CG keeps
+  int mix_m = stdg::kMaxDirs;                 // directions the outer flexible CG keeps
   bool visc_inner64 = false;                  // mixed viscous refinement: binary64-vector inner COCG
   bool conv_generic = false;                  // convection: the runtime-degree kernel at every degree
   double *fcgP = nullptr, *fcgQ = nullptr;    // their P_j and Q_j = S P_j
