@@ -40,6 +40,16 @@ __device__ __forceinline__ bool mbar_wait_hint(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
+// A warp waits for a phase, every lane for at most tries + 1 of the above: true on all lanes when one of them gave
+// up.  Without the vote some lanes could leave while the others go on to the warp's next shuffle and wait for them
+// there without a limit.
+__device__ __forceinline__ bool warp_wait_gave_up(uint64_t* bar, uint32_t parity, long tries) {
+  bool gave_up = false;
+  long spins = 0;
+  while (!mbar_wait_hint(bar, parity))
+    if (++spins > tries) { gave_up = true; break; }
+  return __any_sync(0xffffffffu, gave_up) != 0;
+}
 __device__ __forceinline__ void mbar_expect_tx_only(uint64_t* bar, uint32_t bytes) {
   asm volatile("mbarrier.expect_tx.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(bytes) : "memory");
 }

@@ -226,13 +226,7 @@ __global__ void __launch_bounds__(128, 1) k_apply_warp(WarpArgs a, const typenam
       gf_c = gf_n; gn_c = gn_n;
       if (inx + nw < a.ne) { gf_n = a.gface[inx + nw]; gn_n = a.gnbr[inx + nw]; }
     }
-    {
-      long spins = 0;
-      const uint32_t par = (uint32_t)((it / S) & 1);
-      while (!mbar_wait_hint(&bar[st], par))
-        if (++spins > kWarpSpin) { abort = true; break; }
-    }
-    if (__any_sync(0xffffffffu, abort)) { abort = true; break; }
+    if (warp_wait_gave_up(&bar[st], (uint32_t)((it / S) & 1), kWarpSpin)) { abort = true; break; }
     __syncwarp();
     if (kPrefetch && lane == 0 && i + S * nw < a.ne) {   // the blocks after the next staged tet: towards L2
       const int ip = i + S * nw;
@@ -539,9 +533,7 @@ __global__ void __launch_bounds__(160, 3) k_apply_cta(const __grid_constant__ Wa
   if (i + G < a.ne) issue(1, f1, n1);
   for (; i < a.ne; i += G, ++it) {
     const int st = it & 1;
-    long spins = 0;
-    while (!mbar_wait_hint(&bar[st], (uint32_t)(it >> 1) & 1))
-      if (++spins > kWarpSpin) { abort = true; break; }
+    abort = warp_wait_gave_up(&bar[st], (uint32_t)(it >> 1) & 1, kWarpSpin);   // one path for the whole warp
     __syncwarp();
     float* rd = red + (st * 5 + slot) * NG * NR;
     if (!abort) {
