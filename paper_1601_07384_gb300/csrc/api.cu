@@ -181,7 +181,7 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   TRY(dev_alloc(s, (void**)&s->eB, (size_t)m->ne * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eBv, (size_t)m->ne * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eA, (size_t)m->nf * sizeof(uint16_t)));
-  TRY(dev_alloc(s, (void**)&s->eQ, (size_t)2 * m->nf * sizeof(uint16_t)));
+  TRY(dev_alloc(s, (void**)&s->eQ, (size_t)6 * m->nf * sizeof(uint16_t)));
   TRY(dev_alloc(s, (void**)&s->eM, (size_t)2 * m->nf * sizeof(uint16_t)));
   s->fxws.nvec = 3 * m->nf;                          // nf >= ne (four faces per tet, shared by two)
   TRY(dev_alloc(s, &s->fxws.w, (size_t)s->fxws.nvec * s->Nst * sizeof(int2)));
@@ -206,7 +206,7 @@ static stdg_status solver_create(const stdg_mesh* m, const stdg_ref* r, double d
   encode(m->ne, (int)NN, s->Bdiag, s->eB, s->fxs, s->fxs);
   encode(m->ne, (int)NN, s->Bv, s->eBv, s->fxs, s->fxs);
   encode(m->nf, (int)NN, s->Aoff, s->eA, s->fxs, s->fxs);
-  encode(2 * m->nf, (int)(3 * NN), s->Q, s->eQ, s->fxt, s->fxs);
+  encode(6 * m->nf, (int)NN, s->Q, s->eQ, s->fxt, s->fxs);
   encode(2 * m->nf, (int)NN, s->Mij, s->eM, FxScale{}, FxScale{});
   // binary32-pair copies of the blocks, for the comparison kernels that STDG_OP_KERNEL selects
   if (ce == cudaSuccess && s->opt.precision != STDG_PREC_FP64 && s->op_pairs)
@@ -386,7 +386,7 @@ extern "C" stdg_status stdg_get_blocks(const stdg_solver* s, double* Q, double* 
   // decoded to binary64 in pieces of at most 64 MB (stream-ordered memory, returned below)
   const int NN = s->N * s->N;
   const struct { double* host; FxBlocks b; int64_t nblk; int len; } all[4] = {
-      {Q, blocks_Q(s), 2 * s->nf, 3 * NN}, {Mij, blocks_M(s), 2 * s->nf, NN},
+      {Q, blocks_Q(s), 6 * s->nf, NN}, {Mij, blocks_M(s), 2 * s->nf, NN},
       {Aoff, blocks_A(s), s->nf, NN}, {Bdiag, blocks_B(s), s->ne, NN}};
   for (const auto& a : all) {
     if (!a.host || a.nblk == 0) continue;

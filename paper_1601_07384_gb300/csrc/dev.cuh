@@ -132,8 +132,9 @@ struct ApplyArgs {
 };
 cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st);
 
-// The per-face blocks Q[nf][2][3][N][N] (one exponent per face and side), Mij[nf][2][N][N] and the face
-// tables: what the products below read (fxops.cu).
+// The per-face blocks Q[nf][2][3][N][N] (one exponent per face, side and component: on a mesh stretched in one
+// direction the components differ by the ratio of the elements' sides), Mij[nf][2][N][N] and the face tables:
+// what the products below read (fxops.cu).
 struct FaceOps {
   FxWork ws;
   int ne, nf, N, Ng;

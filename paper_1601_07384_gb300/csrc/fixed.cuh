@@ -45,7 +45,7 @@ __device__ __forceinline__ bool fx_ok(int e) { return e == 0 || (e >= kFxMinExp 
 
 // exponents by which the rows or columns of the blocks of an operator are scaled, one per mode
 struct FxScale { signed char s[40]; };
-// The blocks of an operator (len entries each, N x N or several N x N after one another): entry idx of
+// The blocks of an operator (len entries each): entry idx of
 // block b at w[b * len + idx], divided by 2^(r.s[row] + c.s[column]), as limbs (h, l), or as binary64 where
 // the block's exponent e[b] is outside the range.
 struct FxBlocks { const int2* w; const uint16_t* e; FxScale r, c; };

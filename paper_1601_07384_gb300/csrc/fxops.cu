@@ -99,12 +99,13 @@ struct FxRhs {
   template <int N>
   __device__ FxSlot mat(int u, int sl) const {
     const int f = sl / 3, g = FxApply::at(tface[u], f);
-    return {Q.w + ((size_t)g * 3 + sl - 3 * f) * N * N, Q.e[g], true};
+    const size_t b = (size_t)g * 3 + sl - 3 * f;
+    return {Q.w + b * N * N, Q.e[b], true};
   }
   __device__ int vec(int u, int set, int) const { return 3 * (FxApply::at(tface[u], set / 3) >> 1) + set % 3; }
   template <int N>
   __device__ double entry(int u, int sl, int idx) const {
-    return fx_entry(Q, 3 * N * N, FxApply::at(tface[u], sl / 3), (sl % 3) * N * N + idx, N);
+    return fx_entry(Q, N * N, (size_t)FxApply::at(tface[u], sl / 3) * 3 + sl % 3, idx, N);
   }
   __device__ const FxScale& out_scale() const { return Q.c; }
   __device__ static int set_of(int sl) { return sl; }
@@ -135,7 +136,8 @@ struct FxFace {
   __device__ FxSlot mat(int u, int sl) const {
     const int s = sl / 3, c = sl - 3 * s;
     if (right[u] < 0 && !(grad && s == 1)) return {nullptr, 0, false};
-    return {Q.w + ((size_t)u * 6 + 3 * s + c) * N * N, Q.e[2 * u + s], false};
+    const size_t b = (size_t)u * 6 + 3 * s + c;
+    return {Q.w + b * N * N, Q.e[b], false};
   }
   __device__ int vec(int u, int set, int) const {
     const int r = right[u];
@@ -144,7 +146,7 @@ struct FxFace {
   }
   template <int N>
   __device__ double entry(int u, int sl, int idx) const {
-    return fx_entry(Q, 3 * N * N, 2 * (size_t)u + sl / 3, (sl % 3) * N * N + idx, N);
+    return fx_entry(Q, N * N, 6 * (size_t)u + sl, idx, N);
   }
   __device__ const FxScale& out_scale() const { return Q.r; }
   __device__ static int set_of(int sl) { return sl / 3; }

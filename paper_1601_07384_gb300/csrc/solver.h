@@ -45,7 +45,7 @@ struct stdg_solver {
   double *Q = nullptr, *Mij = nullptr, *C = nullptr, *x0h = nullptr;
   double *Aoff = nullptr, *Bdiag = nullptr, *Bv = nullptr;   // Bv: diagonal blocks of the viscous operator
   // after stdg_solver_create Q, Mij, Aoff, Bdiag and Bv hold fixed-point entries (fixed.cuh, blocks_*
-  // below) with these exponents, one per block (Q: one per face and side)
+  // below) with these exponents, one per block of N x N
   uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;
   stdg::FxScale fxs{}, fxt{};                 // scaling of the tet modes, and of the dual modes of Q
   stdg::FxWork fxws{};                        // the products' input vectors in limbs (3 nf vectors fit)

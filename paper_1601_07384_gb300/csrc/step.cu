@@ -87,7 +87,7 @@ __global__ void k_visc_rhs(int ne, int N, int Ng, const int* __restrict__ t2f, c
       double bsum = 0.0;
       for (int d = 0; d < 3; ++d) {
         const double* gg = Gbc + (((size_t)j * 3 + c) * 3 + d) * Nst + a * N;
-        for (int m = 0; m < N; ++m) bsum = fma(fx_entry(Q, 3 * NN, 2 * (size_t)j, d * (int)NN + m * N + k, N), gg[m], bsum);
+        for (int m = 0; m < N; ++m) bsum = fma(fx_entry(Q, NN, 6 * (size_t)j + d, m * N + k, N), gg[m], bsum);
       }
       s -= nu * bsum;
     }
