@@ -31,49 +31,60 @@
 namespace stdg {
 namespace {
 
-// S[m] = Sum_k tab[k * stride] V[m * N + k] for the NA coefficient rows of V, as normalised pairs
-template <int N, int NA>
-__device__ __forceinline__ void conv_contract(const float2* __restrict__ tab, int stride, const float2* V,
-                                              float2 (&S)[NA]) {
-  constexpr int NA2 = (NA + 1) / 2;
-  float2 sm[NA2], cm[NA2];
+// n sums of products of pairs, two at a time: s + c, with FINE s - c - d (pair_fma2)
+template <int n, bool FINE = false>
+struct ConvSum {
+  static constexpr int H = (n + 1) / 2;
+  float2 s[H], c[H], d[FINE ? H : 1];
+  __device__ __forceinline__ void zero() {
 #pragma unroll
-  for (int m = 0; m < NA2; ++m) sm[m] = cm[m] = make_float2(0.0f, 0.0f);
-#pragma unroll 2
-  for (int k = 0; k < N; ++k) {
-    const float2 pk = __ldg(tab + (size_t)k * stride);
-    const float2 ah2 = make_float2(pk.x, pk.x), nah2 = make_float2(-pk.x, -pk.x), al2 = make_float2(pk.y, pk.y);
+    for (int m = 0; m < H; ++m) s[m] = c[m] = make_float2(0.0f, 0.0f);
 #pragma unroll
-    for (int m = 0; m < NA2; ++m) {
-      const float2 v0 = V[(2 * m) * N + k];
-      const float2 v1 = 2 * m + 1 < NA ? V[(2 * m + 1) * N + k] : make_float2(0.0f, 0.0f);
-      pair_fma2(ah2, nah2, al2, make_float2(v0.x, v1.x), make_float2(v0.y, v1.y), sm[m], cm[m]);
+    for (int m = 0; m < (FINE ? H : 1); ++m) d[m] = make_float2(0.0f, 0.0f);
+  }
+  // += a x[m * stride]
+  __device__ __forceinline__ void axpy(float2 a, const float2* x, int stride = 1) {
+    const float2 ah2 = make_float2(a.x, a.x), nah2 = make_float2(-a.x, -a.x), al2 = make_float2(a.y, a.y);
+#pragma unroll
+    for (int m = 0; m < H; ++m) {
+      const float2 x0 = x[2 * m * stride], x1 = 2 * m + 1 < n ? x[(2 * m + 1) * stride] : make_float2(0.0f, 0.0f);
+      const float2 xh = make_float2(x0.x, x1.x), xl = make_float2(x0.y, x1.y);
+      if constexpr (FINE) pair_fma2(ah2, nah2, al2, xh, xl, s[m], c[m], d[m]);
+      else pair_fma2(ah2, nah2, al2, xh, xl, s[m], c[m]);
     }
   }
+  // += the sums t
+  __device__ __forceinline__ void add(const ConvSum& t) {
+    static_assert(!FINE, "fine sums are added up term by term");
 #pragma unroll
-  for (int m = 0; m < NA2; ++m) {
-    S[2 * m] = pair_norm(sm[m].x, cm[m].x);
-    if (2 * m + 1 < NA) S[2 * m + 1] = pair_norm(sm[m].y, cm[m].y);
+    for (int m = 0; m < H; ++m) {
+      float2 s2, e;
+      df_two_diff2(s[m], make_float2(-t.s[m].x, -t.s[m].y), s2, e);
+      s[m] = s2;
+      c[m] = __fadd2_rn(__fadd2_rn(c[m], t.c[m]), e);
+    }
   }
-}
-// (s, c)[m] += a x[m] for n pairs x[m] (one after another), packed two at a time
-template <int n>
-__device__ __forceinline__ void conv_axpy(float2 a, const float2* x, float2 (&s)[(n + 1) / 2], float2 (&c)[(n + 1) / 2]) {
-  const float2 ah2 = make_float2(a.x, a.x), nah2 = make_float2(-a.x, -a.x), al2 = make_float2(a.y, a.y);
-#pragma unroll
-  for (int m = 0; m < (n + 1) / 2; ++m) {
-    const float2 x0 = x[2 * m], x1 = 2 * m + 1 < n ? x[2 * m + 1] : make_float2(0.0f, 0.0f);
-    pair_fma2(ah2, nah2, al2, make_float2(x0.x, x1.x), make_float2(x0.y, x1.y), s[m], c[m]);
+  __device__ __forceinline__ float2 get(int m) const {
+    const float sm = (m & 1) ? s[m >> 1].y : s[m >> 1].x, cm = (m & 1) ? c[m >> 1].y : c[m >> 1].x;
+    float2 v = pair_norm(sm, FINE ? -cm : cm);
+    if constexpr (FINE) v.y -= (m & 1) ? d[m >> 1].y : d[m >> 1].x;
+    return v;
   }
-}
-template <int n>
-__device__ __forceinline__ void conv_zero(float2 (&s)[n], float2 (&c)[n]) {
+  __device__ __forceinline__ double value(int m) const {
+    const float2 v = get(m);
+    return pair_value(v.x, v.y);
+  }
+};
+// S[m] = Sum_k tab[k * stride] V[m * N + k] for the NA coefficient rows of V, as normalised pairs
+template <int N, int NA, bool FINE = false>
+__device__ __forceinline__ void conv_contract(const float2* __restrict__ tab, int stride, const float2* V,
+                                              float2 (&S)[NA]) {
+  ConvSum<NA, FINE> sum;
+  sum.zero();
+#pragma unroll 2
+  for (int k = 0; k < N; ++k) sum.axpy(__ldg(tab + (size_t)k * stride), V + k, N);
 #pragma unroll
-  for (int m = 0; m < n; ++m) s[m] = c[m] = make_float2(0.0f, 0.0f);
-}
-template <int n>
-__device__ __forceinline__ float2 conv_get(const float2 (&s)[n], const float2 (&c)[n], int m) {
-  return (m & 1) ? pair_norm(s[m >> 1].y, c[m >> 1].y) : pair_norm(s[m >> 1].x, c[m >> 1].x);
+  for (int m = 0; m < NA; ++m) S[m] = sum.get(m);
 }
 
 template <int P, int NG>
@@ -83,6 +94,13 @@ struct ConvDim {
   static constexpr int NF1 = (3 * P + 3) / 2, NF = NF1 * NF1;          // face rule: that of all non-polynomial data
   static constexpr int NTV = (3 * (NG - 1) + 2) / 2, NTF = (3 * (NG - 1) + 3) / 2;   // time rules
   static constexpr int NA = 3 * NG, Nst = N * NG;
+  // Sums of few terms add more rounding than the shorter sums save: fine sums for the traces, moments and outputs at
+  // p = 1 and for the moments at p = 2.  Relative rms error against binary64 at p_t = 0, a kernel per tet that sums
+  // over the points -> plain sums here -> as built: p = 1 5.1e-15 -> 6.6e-15 -> 4.5e-15, p = 2 1.0e-14 -> 9.3e-15 ->
+  // 7.6e-15, p = 3 2.0e-14 -> 1.5e-14 -> 1.4e-14, p = 4 2.4e-14 -> 2.1e-14 -> 2.0e-14; with random coefficients of
+  // order 1, plain sums were also worse at p = 2 (8.0e-15 -> 8.2e-15 -> 6.5e-15).  Cost at p_t = 0: 82,944 tets,
+  // p = 1, 206 -> 228 us; 34,992 tets, p = 2, 256 -> 275 us; at p = 3 and 4 below 1 %.
+  static constexpr bool FINE = P == 1, FINE_M = P <= 2;
   // faces per CTA of 256 threads: all points of a face side by side
   static constexpr int kFT = 256, FB = kFT / NF;
   static constexpr int face_in = FB * 2 * NA * N, face_g = FB * NF * NA;
@@ -140,7 +158,7 @@ __global__ void __launch_bounds__(256, 2) k_conv_face(const __grid_constant__ Co
     const int code = (fs & 1) ? a.code_r[j] : a.code_l[j];
     if (code < 0) continue;                       // no tet at this side of a boundary face
     float2 S[NA];
-    conv_contract<N, NA>(t.Rt + (size_t)code * N * M + m, M, V + fs * NA * N, S);
+    conv_contract<N, NA, C::FINE>(t.Rt + (size_t)code * N * M + m, M, V + fs * NA * N, S);
 #pragma unroll
     for (int q = 0; q < NA; ++q) T[(fs * NA + q) * M + m] = S[q];
   }
@@ -159,9 +177,9 @@ __global__ void __launch_bounds__(256, 2) k_conv_face(const __grid_constant__ Co
       const double s0 = a.tri_st[2 * q], t0 = a.tri_st[2 * q + 1];
       for (int d = 0; d < 3; ++d) x[d] = fv[d] + s0 * (fv[3 + d] - fv[d]) + t0 * (fv[6 + d] - fv[d]);
     }
-    float2 gs[3][(NG + 1) / 2], gc[3][(NG + 1) / 2];
+    ConvSum<NG> gs[3];
 #pragma unroll
-    for (int c = 0; c < 3; ++c) conv_zero(gs[c], gc[c]);
+    for (int c = 0; c < 3; ++c) gs[c].zero();
     const float2 wq = pair_mul(pair_split(a.dt * 2.0 * a.area[j]), t.fw[q]);
     const float2 nP[3] = {pair_split_int(a.normal[3 * (size_t)j]), pair_split_int(a.normal[3 * (size_t)j + 1]),
                           pair_split_int(a.normal[3 * (size_t)j + 2])};
@@ -211,27 +229,27 @@ __global__ void __launch_bounds__(256, 2) k_conv_face(const __grid_constant__ Co
         // h = W (0.5 (v+_c un+ + v-_c un-) - 0.5 s_max (v+_c - v-_c))
         const float2 cen = pair_mul(Wh, pair_add(pair_mul(vp[c], unp), pair_mul(vm[c], unm)));
         const float2 h = pair_add(cen, pair_neg(pair_mul(hs, pair_add(vp[c], pair_neg(vm[c])))));
-        conv_axpy<NG>(h, g, gs[c], gc[c]);
+        gs[c].axpy(h, g);
       }
     }
     float2* Gu = G + (f * NF + q) * NA;           // V is used up (every thread passed the barrier after T)
 #pragma unroll
     for (int c = 0; c < 3; ++c)
 #pragma unroll
-      for (int b = 0; b < NG; ++b) Gu[c * NG + b] = conv_get(gs[c], gc[c], b);
+      for (int b = 0; b < NG; ++b) Gu[c * NG + b] = gs[c].get(b);
   }
   __syncthreads();
   // moments: thread (face, c, m)
   for (int o = th; o < FB * 3 * M; o += C::kFT) {
     const int ff = o / (3 * M), rem = o - ff * 3 * M, c = rem / M, m = rem - c * M;
     if (j0 + ff >= a.nf) break;
-    float2 s[(NG + 1) / 2], e[(NG + 1) / 2];
-    conv_zero(s, e);
+    ConvSum<NG, C::FINE_M> s;
+    s.zero();
 #pragma unroll 4
-    for (int v = 0; v < NF; ++v) conv_axpy<NG>(__ldg(t.chi + v * M + m), G + (ff * NF + v) * NA + c * NG, s, e);
+    for (int v = 0; v < NF; ++v) s.axpy(__ldg(t.chi + v * M + m), G + (ff * NF + v) * NA + c * NG);
     float2* out = a.hf + (((size_t)(j0 + ff) * 3 + c) * NG) * M + m;
 #pragma unroll
-    for (int b = 0; b < NG; ++b) out[b * M] = conv_get(s, e, b);
+    for (int b = 0; b < NG; ++b) out[b * M] = s.get(b);
   }
 }
 
@@ -261,9 +279,9 @@ __global__ void __launch_bounds__(ConvDim<P, NG>::kTT, P == 3 ? 4 : 2) k_conv_te
     if (tl < TB && i < a.ne) {
       float2 S[NA];
       conv_contract<N, NA>(t.vphi + q, NV, V + tl * NA * N, S);
-      float2 gs[6][(NG + 1) / 2], gc[6][(NG + 1) / 2];
+      ConvSum<NG> gs[6];
 #pragma unroll
-      for (int r = 0; r < 6; ++r) conv_zero(gs[r], gc[r]);
+      for (int r = 0; r < 6; ++r) gs[r].zero();
       const float2 wq = pair_mul(pair_split(a.dt * a.detJ[i]), t.vw[q]);
 #pragma unroll 1
       for (int ti = 0; ti < C::NTV; ++ti) {
@@ -282,14 +300,14 @@ __global__ void __launch_bounds__(ConvDim<P, NG>::kTT, P == 3 ? 4 : 2) k_conv_te
 #pragma unroll
         for (int r = 0; r < 6; ++r) {
           constexpr int rc[6] = {0, 0, 0, 1, 1, 2}, rd[6] = {0, 1, 2, 1, 2, 2};
-          conv_axpy<NG>(pair_mul(Wv[rc[r]], v[rd[r]]), g, gs[r], gc[r]);
+          gs[r].axpy(pair_mul(Wv[rc[r]], v[rd[r]]), g);
         }
       }
       float2* Gu = G + (tl * NV + q) * R6;
 #pragma unroll
       for (int b = 0; b < NG; ++b)
 #pragma unroll
-        for (int r = 0; r < 6; ++r) Gu[b * 6 + r] = conv_get(gs[r], gc[r], b);
+        for (int r = 0; r < 6; ++r) Gu[b * 6 + r] = gs[r].get(b);
     }
   }
   __syncthreads();
@@ -297,13 +315,13 @@ __global__ void __launch_bounds__(ConvDim<P, NG>::kTT, P == 3 ? 4 : 2) k_conv_te
     const int sh = th / (TB * N1 * NG), rem = th - sh * TB * N1 * NG, tl = rem / (N1 * NG), al = rem - tl * N1 * NG;
     const int b = al / N1, l = al - b * N1;
     if (sh < QS) {
-      float2 s[3], e[3];
-      conv_zero(s, e);
+      ConvSum<6> s;
+      s.zero();
 #pragma unroll 2
-      for (int v = sh; v < NV; v += QS) conv_axpy<6>(__ldg(t.vphi1 + v * N1 + l), G + (tl * NV + v) * R6 + b * 6, s, e);
+      for (int v = sh; v < NV; v += QS) s.axpy(__ldg(t.vphi1 + v * N1 + l), G + (tl * NV + v) * R6 + b * 6);
       float2* out = H + (sh * TB + tl) * HL + (l * NG + b) * 6;
 #pragma unroll
-      for (int r = 0; r < 6; ++r) out[r] = conv_get(s, e, r);
+      for (int r = 0; r < 6; ++r) out[r] = s.get(r);
     }
   }
   __syncthreads();                                // G is free
@@ -339,27 +357,31 @@ __global__ void __launch_bounds__(ConvDim<P, NG>::kTT, P == 3 ? 4 : 2) k_conv_te
   for (int o = th; o < TB * 3 * N; o += NT) {
     const int tl = o / (3 * N), rem = o - tl * 3 * N, c = rem / N, k = rem - c * N, i = i0 + tl;
     if (i >= a.ne) break;
-    float2 s[(NG + 1) / 2], r[(NG + 1) / 2];
-    conv_zero(s, r);
+    // plain sums: every derivative and face by itself first (the error part c of a sum grows with its length,
+    // and with it the rounding of c)
+    ConvSum<NG, C::FINE> s, part;
+    auto& sum = C::FINE ? s : part;
+    s.zero();
     const float2* u = U + (tl * 3 + c) * 3 * N1 * NG;
+#pragma unroll 1
+    for (int e = 0; e < 3; ++e) {
+      if constexpr (!C::FINE) part.zero();
 #pragma unroll 4
-    for (int el = 0; el < 3 * N1; ++el) conv_axpy<NG>(pair_neg(__ldg(t.D + el * N + k)), u + el * NG, s, r);
+      for (int l = 0; l < N1; ++l) sum.axpy(pair_neg(__ldg(t.D + (e * N1 + l) * N + k)), u + (e * N1 + l) * NG);
+      if constexpr (!C::FINE) s.add(part);
+    }
 #pragma unroll 1
     for (int f = 0; f < 4; ++f) {
       const float2* R = t.Rk + (size_t)a.t2code[4 * i + f] * M * N + k;
       const float2* h = F + ((tl * 4 + f) * 3 + c) * NG * M;
+      if constexpr (!C::FINE) part.zero();
 #pragma unroll 3
-      for (int m = 0; m < M; ++m) {
-        float2 hm[NG];
-#pragma unroll
-        for (int b = 0; b < NG; ++b) hm[b] = h[b * M + m];
-        conv_axpy<NG>(__ldg(R + m * N), hm, s, r);
-      }
+      for (int m = 0; m < M; ++m) sum.axpy(__ldg(R + m * N), h + m, M);
+      if constexpr (!C::FINE) s.add(part);
     }
     double* out = a.ups + ((size_t)c * a.ne + i) * Nst + k;
 #pragma unroll
-    for (int b = 0; b < NG; ++b)
-      out[b * N] = (b & 1) ? pair_value(s[b >> 1].y, r[b >> 1].y) : pair_value(s[b >> 1].x, r[b >> 1].x);
+    for (int b = 0; b < NG; ++b) out[b * N] = s.value(b);
   }
 }
 

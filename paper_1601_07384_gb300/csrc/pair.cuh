@@ -58,12 +58,15 @@ __device__ __forceinline__ float2 pair_add(float2 a, float2 b) {
   const float e = ((a.x - (s - bb)) + (b.x - bb)) + (a.y + b.y);
   return pair_norm(s, e);
 }
-// sqrt(a) for a >= 0: one Newton step in the residual doubles the 24 bits of the binary32 root
+// sqrt(a) for a >= 0: the binary32 root s, its residual (a.x - s s is exact) over 2 s, and the residual that this
+// leaves over 2 s again: to the rounding of the low part, as a binary64 root split into a pair
 __device__ __forceinline__ float2 pair_sqrt(float2 a) {
   const float s = __fsqrt_rn(a.x);
   if (!(s > 0.0f) || s > 3.4e38f) return make_float2(s, 0.0f);
-  const float r = fmaf(-s, s, a.x) + a.y;
-  return pair_norm(s, __fdividef(r, s + s));
+  float r, t;
+  df_two_sum(fmaf(-s, s, a.x), a.y, r, t);
+  const float inv = __fdividef(1.0f, s + s), q = r * inv;
+  return pair_norm(s, fmaf(fmaf(-q, q, fmaf(-(s + s), q, r)) + t, inv, q));
 }
 __device__ __forceinline__ float2 pair_neg(float2 a) { return make_float2(-a.x, -a.y); }
 
@@ -79,6 +82,23 @@ __device__ __forceinline__ void pair_fma2(float2 ah2, float2 nah2, float2 al2, f
   df_two_diff2(s, pn, s2, err);                   // s + a_hi b_hi, error-free
   c = __fadd2_rn(c, __fadd2_rn(err, e));
   s = s2;
+}
+
+// The same with the error part negated, nc, and the rounding errors of its additions collected in d: the sum
+// s - nc - d is accurate to the rounding of the single terms, at twice the operations
+__device__ __forceinline__ void pair_fma2(float2 ah2, float2 nah2, float2 al2, float2 bh2, float2 bl2, float2& s,
+                                          float2& nc, float2& d) {
+  const float2 pn = __fmul2_rn(nah2, bh2);
+  float2 e = __ffma2_rn(ah2, bh2, pn);
+  e = __ffma2_rn(al2, bh2, e);
+  e = __ffma2_rn(ah2, bl2, e);
+  float2 s2, err, n1, n2, d1, d2;
+  df_two_diff2(s, pn, s2, err);
+  df_two_diff2(nc, err, n1, d1);
+  df_two_diff2(n1, e, n2, d2);
+  d = __fadd2_rn(d, __fadd2_rn(d1, d2));
+  s = s2;
+  nc = n2;
 }
 
 }  // namespace stdg
