@@ -374,7 +374,7 @@ extern "C" stdg_status stdg_velocity_moments(stdg_solver* s, const double* V, do
   stdg_status e = check(s);
   if (e != STDG_OK) return e;
   ++s->nlaunch;
-  cudaError_t ce = launch_moments((int)s->nf, s->N, s->Ng, blocks_M(s), V, s->dt, U, s->stream);
+  cudaError_t ce = launch_moments(face_ops(s), V, s->dt, U, s->stream);
   if (ce != cudaSuccess) { set_error("moments launch failed: %s", cudaGetErrorString(ce)); return STDG_ECUDA; }
   return STDG_OK;
 }

@@ -162,8 +162,7 @@ cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* i
 // F[j][c][a][m] = Sum_s Sum_k Mij[j][s][k][m] vbar[c][s][a][k]; boundary: F = Vbc
 cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st);
 // U_j[s][c][a][k] = dt Sum_l Mij_s[k][l] V_j[c][a][l]
-cudaError_t launch_moments(int nf, int N, int Ng, const FxBlocks& Mij, const double* V, double dt,
-                           double* U, cudaStream_t st);
+cudaError_t launch_moments(const FaceOps& f, const double* V, double dt, double* U, cudaStream_t st);
 
 }  // namespace stdg
 

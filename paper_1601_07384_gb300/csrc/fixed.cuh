@@ -49,12 +49,6 @@ struct FxScale { signed char s[40]; };
 // block b at w[b * len + idx], divided by 2^(r.s[row] + c.s[column]), as limbs (h, l), or as binary64 where
 // the block's exponent e[b] is outside the range.
 struct FxBlocks { const int2* w; const uint16_t* e; FxScale r, c; };
-__device__ __forceinline__ double fx_entry(const FxBlocks& B, size_t len, size_t b, int idx, int N) {
-  const int2 w = B.w[b * len + idx];
-  const int e = B.e[b], sc = B.r.s[idx / N % N] + B.c.s[idx % N];
-  if (!fx_ok(e)) return scalbn(__hiloint2double(w.y, w.x), sc);
-  return e ? scalbn((double)((long long)w.x * (1LL << kFxL) + w.y), e - 1022 - kFx + sc) : 0.0;
-}
 // rounded to binary32 (sc: the scaling of its row and column): of the 61 bits at once and without the binary64
 // pipe, where the value is certain to be in the normal range
 __device__ __forceinline__ float fx_entry_f32(const FxBlocks& B, size_t len, size_t b, int idx, int sc) {
@@ -171,6 +165,15 @@ __device__ __forceinline__ double fx_value(const FxSum& T, int k) {
     return __longlong_as_double((long long)((f + ((unsigned long long)(k - 1) << 52)) | (unsigned long long)s << 63));
   const double d = scalbn(__longlong_as_double((long long)(f + (1022ull << 52))), k - 1023);
   return s ? -d : d;
+}
+
+// entry idx of block b rounded to binary64, without the binary64 pipe
+__device__ __forceinline__ double fx_entry(const FxBlocks& B, size_t len, size_t b, int idx, int N) {
+  const int2 w = B.w[b * len + idx];
+  const int e = B.e[b], sc = B.r.s[idx / N % N] + B.c.s[idx % N];
+  if (!fx_ok(e)) return scalbn(__hiloint2double(w.y, w.x), sc);
+  const long long m = (long long)w.x * (1LL << kFxL) + w.y;
+  return fx_value(FxSum{(uint32_t)m, (uint32_t)((unsigned long long)m >> 32), (uint32_t)(m >> 63)}, e - 1022 - kFx + sc);
 }
 
 // A small matrix (the time matrices) in limbs with one exponent; the entries as they are for the

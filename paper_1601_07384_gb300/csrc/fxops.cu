@@ -1,9 +1,9 @@
 // The products of per-tet and per-face binary64 blocks with space-time vectors, in 64-bit fixed point
 // (fixed.cuh): the five-point operator (Eq. CS_19 / A1_mod), the pressure right-hand side (Eq. A2_mod),
 // the face gradient and velocity update (Eq. prevpress, A3_mod), averaging and the go back (Eq. average,
-// goback).  All are one shape: a unit (tet or face) has SLOTS blocks of N x N; thread (unit, slot, row)
-// multiplies its row of its block with the NCOL columns of the slot's vector, and the slots of an output
-// group are added in 96-bit integers.
+// goback), the velocity moments (Eq. vis3).  All are one shape: a unit (tet or face) has SLOTS blocks of
+// N x N; thread (unit, slot, row) multiplies its row of its block with the NCOL columns of the slot's vector,
+// and the slots of an output group are added in 96-bit integers.
 //
 // What bounds them: binary64 kernels of this shape are bound by sm_103a's binary64 pipe (64 cycles per
 // warp FMA, every block entry used for up to 15 columns).  Here a product costs 3 IMAD.WIDE (4 cycles
@@ -220,6 +220,35 @@ struct FxGoback {
   __device__ void store(int u, int, int c, int q, int k, double v, double) const {
     const size_t o = (((size_t)u * 3 + c) * NG + q) * N + k;
     F[o] = right[u] < 0 ? Vbc[o] : v;
+  }
+};
+
+// U_j^(s)c = dt M_s V_j^c (boundary faces: 0 in the place of the absent side)
+struct FxMoments {
+  static constexpr int SLOTS = 2, SETS = 1, GROUPS = 2, C = 3;
+  static constexpr bool STAGED = true;
+  int n;
+  const int* right;
+  FxBlocks M;
+  double* U;
+  double dt;
+  template <int N>
+  __device__ FxSlot mat(int u, int s) const {
+    if (s == 1 && right[u] < 0) return {nullptr, 0, false};
+    return {M.w + ((size_t)u * 2 + s) * N * N, M.e[2 * u + s], false};
+  }
+  __device__ int vec(int u, int, int c) const { return 3 * u + c; }
+  template <int N>
+  __device__ double entry(int u, int s, int idx) const { return fx_entry(M, N * N, 2 * (size_t)u + s, idx, N); }
+  __device__ const FxScale& out_scale() const { return M.r; }
+  __device__ static int set_of(int) { return 0; }
+  __device__ static int group_of(int sl) { return sl; }
+  __device__ static int slot_of(int g, int) { return g; }
+  __device__ static bool copies(int sl) { return sl == 0; }
+  __device__ double unit_scale(int) const { return 0.0; }
+  template <int N, int NG>
+  __device__ void store(int u, int g, int c, int q, int k, double v, double) const {
+    U[((((size_t)u * 2 + g) * 3 + c) * NG + q) * N + k] = dt * v;
   }
 };
 
@@ -688,6 +717,32 @@ cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vb
   FxGoback p{};
   p.n = f.nf; p.ne = f.ne; p.left = f.left; p.right = f.right; p.M = f.Mij; p.Vbc = Vbc; p.F = F;
   return fx_launch(f.N, f.Ng, p, vbar, 3 * f.ne, f.Mij.r, f.ws, 0, FxMat{}, st);
+}
+
+// One launch for the blocks of p <= 1, where two launches are what k_fx costs (750 tets, p = 1, p_t = 0: 18.0 ->
+// 14.4 us); a block per face, binary64 multiply-adds, the face's blocks decoded to shared memory.
+__global__ void __launch_bounds__(128) k_moments_small(int N, int Ng, const __grid_constant__ FxBlocks M,
+                                                       const double* __restrict__ V, double dt, double* __restrict__ U) {
+  __shared__ double Ms[2 * 16];
+  const int j = blockIdx.x, Nst = N * Ng, NN = N * N;
+  for (int e = threadIdx.x; e < 2 * NN; e += 128) Ms[e] = fx_entry(M, NN, 2 * (size_t)j + e / NN, e % NN, N);
+  __syncthreads();
+  for (int o = threadIdx.x; o < 6 * Nst; o += 128) {
+    const int s = o / (3 * Nst), rem = o - s * 3 * Nst, k = rem % N;
+    const double* v = V + (size_t)j * 3 * Nst + rem - k;
+    double acc = 0.0;
+    for (int l = 0; l < N; ++l) acc = fma(Ms[s * NN + k * N + l], v[l], acc);
+    U[(size_t)j * 6 * Nst + o] = dt * acc;
+  }
+}
+cudaError_t launch_moments(const FaceOps& f, const double* V, double dt, double* U, cudaStream_t st) {
+  if (f.N <= 4) {
+    if (f.nf > 0) k_moments_small<<<f.nf, 128, 0, st>>>(f.N, f.Ng, f.Mij, V, dt, U);
+    return cudaGetLastError();
+  }
+  FxMoments p{};
+  p.n = f.nf; p.right = f.right; p.M = f.Mij; p.U = U; p.dt = dt;
+  return fx_launch(f.N, f.Ng, p, V, 3 * f.nf, f.Mij.c, f.ws, 0, FxMat{}, st);
 }
 
 }  // namespace stdg

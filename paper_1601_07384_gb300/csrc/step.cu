@@ -65,33 +65,69 @@ __global__ void k_trace(int nf, int N, int Ng, const int* __restrict__ right, GA
 // ---- viscous right-hand side (Eq. A1_mod):
 // rhs[c][i][a][k] = |J| g0[a] Sum_b g1[b] vbar_n[c][i][b][k] - Ups[c][i][a][k] - |J| Sum_b K[a][b] Lam[c][i][b][k]
 //                   - nu Sum_{boundary f} Sum_d Sum_m Q^{bd,d}[m][k] G[j][c][d][a][m]
-__global__ void k_visc_rhs(int ne, int N, int Ng, const int* __restrict__ t2f, const int* __restrict__ t2n,
-                           const double* __restrict__ detJ, FxBlocks Q, GArg g0, GArg g1, MArg K,
-                           double nu, const double* __restrict__ vbar_n, const double* __restrict__ Ups,
-                           const double* __restrict__ Lam, const double* __restrict__ Gbc, double* __restrict__ rhs) {
-  const int i = blockIdx.x, Nst = N * Ng;
-  const size_t NN = (size_t)N * N;
+// One block per tet.  The sums over a boundary face (binary64 multiply-adds, which bound the kernel) read the block
+// Q^{bd,d} from shared memory, where it is decoded once: at every use (3 Ng times per entry) the decoding took most
+// of the time (10,368 tets, p = p_t = 4: 1,613 us, now 375).
+constexpr int kVT = 192;            // three outputs a thread at N Ng = 175
+__global__ void __launch_bounds__(kVT) k_visc_rhs(int ne, int N, int Ng, const int* __restrict__ t2f,
+                                                  const int* __restrict__ t2n, const double* __restrict__ detJ,
+                                                  const __grid_constant__ FxBlocks Q, GArg g0, GArg g1, MArg K, double nu,
+                                                  const double* __restrict__ vbar_n, const double* __restrict__ Ups,
+                                                  const double* __restrict__ Lam, const double* __restrict__ Gbc,
+                                                  double* __restrict__ rhs) {
+  __shared__ double Qs[kMaxN * kMaxN];
+  constexpr int R = (3 * kMaxN * kMaxNg + kVT - 1) / kVT;   // outputs per thread, at most
+  const int i = blockIdx.x, Nst = N * Ng, NN = N * N;
+  const int D = 3 * NN <= kMaxN * kMaxN ? 3 : 1;        // components decoded at a time
   const double dj = detJ[i];
-  for (int o = threadIdx.x; o < 3 * Nst; o += blockDim.x) {
-    const int c = o / Nst, rem = o % Nst, a = rem / N, k = rem % N;
+  double s[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int o = threadIdx.x + kVT * r;
+    s[r] = 0.0;
+    if (o >= 3 * Nst) break;
+    const int c = o / Nst, rem = o - c * Nst, a = rem / N, k = rem - a * N;
     const size_t vb = ((size_t)c * ne + i) * Nst;
     double tr = 0.0, kl = 0.0;
     for (int b = 0; b < Ng; ++b) {
       tr = fma(g1.v[b], vbar_n[vb + b * N + k], tr);
       kl = fma(K.v[a * Ng + b], Lam[vb + b * N + k], kl);
     }
-    double s = dj * g0.v[a] * tr - Ups[vb + rem] - dj * kl;
-    for (int f = 0; f < 4; ++f) {
-      if (t2n[4 * i + f] >= 0) continue;
-      const int j = t2f[4 * i + f];
-      double bsum = 0.0;
-      for (int d = 0; d < 3; ++d) {
-        const double* gg = Gbc + (((size_t)j * 3 + c) * 3 + d) * Nst + a * N;
-        for (int m = 0; m < N; ++m) bsum = fma(fx_entry(Q, NN, 6 * (size_t)j + d, m * N + k, N), gg[m], bsum);
+    s[r] = dj * g0.v[a] * tr - Ups[vb + rem] - dj * kl;
+  }
+  for (int f = 0; f < 4; ++f) {
+    if (t2n[4 * i + f] >= 0) continue;                  // the same for the whole block
+    const int j = t2f[4 * i + f];
+    double bsum[R];
+#pragma unroll
+    for (int r = 0; r < R; ++r) bsum[r] = 0.0;
+    for (int d0 = 0; d0 < 3; d0 += D) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < D * NN; e += kVT) {
+        const int d = e / NN;
+        Qs[e] = fx_entry(Q, NN, 6 * (size_t)j + d0 + d, e - d * NN, N);
       }
-      s -= nu * bsum;
+      __syncthreads();
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int o = threadIdx.x + kVT * r;
+        if (o >= 3 * Nst) break;
+        const int c = o / Nst, rem = o - c * Nst, a = rem / N, k = rem - a * N;
+        for (int d = 0; d < D; ++d) {
+          const double* gg = Gbc + (((size_t)j * 3 + c) * 3 + d0 + d) * Nst + a * N;
+          for (int m = 0; m < N; ++m) bsum[r] = fma(Qs[d * NN + m * N + k], gg[m], bsum[r]);
+        }
+      }
     }
-    rhs[vb + rem] = s;
+#pragma unroll
+    for (int r = 0; r < R; ++r) s[r] -= nu * bsum[r];
+  }
+#pragma unroll
+  for (int r = 0; r < R; ++r) {
+    const int o = threadIdx.x + kVT * r;
+    if (o >= 3 * Nst) break;
+    const int c = o / Nst;
+    rhs[((size_t)c * ne + i) * Nst + o - c * Nst] = s[r];
   }
 }
 
@@ -840,7 +876,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     phase_mark(s, 2);
     // 3. viscous systems (Eq. A1_mod), one per component, initial guess vbar^{n+1,k}
     ++s->nlaunch;
-    k_visc_rhs<<<ne, 128, 0, st>>>(ne, N, Ng, s->dm.t2f, s->dm.t2n, s->dm.detJ, blocks_Q(s), g0, g1, K, nu, s->Vbar_n,
+    k_visc_rhs<<<ne, kVT, 0, st>>>(ne, N, Ng, s->dm.t2f, s->dm.t2n, s->dm.detJ, blocks_Q(s), g0, g1, K, nu, s->Vbar_n,
                                    s->Ups, s->Lam, s->Gbc, s->rhsv);
     if (cudaGetLastError() != cudaSuccess) { set_error("step kernels failed to launch"); return STDG_ECUDA; }
     int vits = 0;

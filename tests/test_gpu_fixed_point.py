@@ -60,3 +60,18 @@ def test_components_of_a_stretched_mesh_keep_their_accuracy(p, pt, axis):
             Uo[j, s] = (fb["Mij"][s] @ Vo[j].T).T
     for c in range(3):
         assert rel(U[:, :, c], Uo[:, :, c]) <= 1e-12, c
+
+
+@pytest.mark.parametrize("p,pt", [(p, pt) for p in range(5) for pt in range(5)])
+def test_velocity_moments_match_oracle_at_every_degree(p, pt):
+    """Velocities of order 1 on all faces, the boundary's with one side only."""
+    gs, d = setup(2, p, pt)
+    m = d.mesh
+    V = np.random.default_rng(10 * p + pt).standard_normal((m.nf, 3, d.Nst))
+    U = gs.velocity_moments(cuda(V.ravel())).cpu().numpy().reshape(m.nf, 2, 3, d.Nst)
+    for j in range(m.nf):
+        fb = d.face_blocks(j)
+        for s, Mij in enumerate(fb["Mij"]):
+            assert rel(U[j, s], (Mij @ V[j].T).T) <= 1e-12
+        if len(fb["Mij"]) == 1:
+            assert not U[j, 1].any()
