@@ -22,7 +22,7 @@
 // own quadrature points for the evaluation (all columns of a point in registers, the basis table
 // coalesced over the points), and outputs for the tests; all pair
 // products run two at a time in packed binary32 operations.
-#include <cmath>
+#include <algorithm>
 #include <vector>
 
 #include "pair.cuh"
@@ -397,107 +397,133 @@ cudaError_t conv_launch(const ConvIn& a, const ConvTab& t, cudaStream_t st) {
   return cudaGetLastError();
 }
 
+// ---- the tables, in binary64 on the device from the nonlinear-degree tables of the solver and the nodes of the
+// (smaller) volume rule: evaluated on the host and uploaded they were 2.4 ms of the first call at p = p_t = 4
+constexpr int kVNodes = 6, kTNodes = 7;           // points of the volume and time rules, at most
+struct ConvNodes {
+  int nv, mv;                                     // nodes per direction, in time
+  double x[3][kVNodes], w[3][kVNodes];            // Gauss-Jacobi (1 - x)^0, (1 - x)^1, (1 - x)^2
+  double tg[kTNodes * kMaxNg], tw[kTNodes];       // time basis at the time nodes
+  MultiIdx mi;
+};
+struct ConvSrc {                                  // [nq][N], [nq][3][N], [nq]; [64][nqf][N], [nqf][2], [nqf]; [nt][Ng], [nt]
+  const double *tet_phi, *tet_dphi, *tet_w, *face_phi, *tri_st, *tri_w, *tg, *tw;
+  int nq, nqf, nt;
+};
+struct ConvOff { int o[14]; };                    // where each table starts (ConvTab's order)
+
+// P_n of the Jacobi weight (al, 0)
+__device__ double conv_jacobi(int n, double al, double x) {
+  double a = 1.0, b = 0.5 * ((al + 2.0) * x + al);
+  if (n == 0) return a;
+  for (int k = 2; k <= n; ++k) {
+    const double q = 2.0 * k + al;
+    const double c = ((q - 1) * (q * (q - 2) * x + al * al) * b - 2 * (k + al - 1) * (k - 1) * q * a) / (2 * k * (k + al) * (q - 2));
+    a = b; b = c;
+  }
+  return b;
+}
+__device__ double conv_pow(double x, int n) {
+  double v = 1.0;
+  for (int k = 0; k < n; ++k) v *= x;
+  return v;
+}
+// orthonormal Dubiner basis function k of the tetrahedron at the collapsed coordinates (u, v, w)
+__device__ double conv_phi(const MultiIdx& mi, int k, double u, double v, double w) {
+  const int i = mi.e[3 * k], j = mi.e[3 * k + 1], l = mi.e[3 * k + 2];
+  return sqrt((2.0 * i + 1) * (2.0 * i + 2 * j + 2) * (2.0 * i + 2 * j + 2 * l + 3)) * conv_jacobi(i, 0, 2 * u - 1) *
+         conv_pow(1 - v, i) * conv_jacobi(j, 2.0 * i + 1, 2 * v - 1) * conv_pow(1 - w, i + j) *
+         conv_jacobi(l, 2.0 * i + 2 * j + 2, 2 * w - 1);
+}
 // orthonormal Dubiner basis of the reference triangle {s, t >= 0, s + t <= 1}, order "n = 0..p, i = 0..n, (i, n - i)"
-void tri_basis(int p, double s, double t, double* out) {
-  auto jac = [](int n, double al, double x) {     // P_n of the Jacobi weight (al, 0)
-    double a = 1.0, b = 0.5 * ((al + 2.0) * x + al);
-    if (n == 0) return a;
-    for (int k = 2; k <= n; ++k) {
-      const double q = 2.0 * k + al;
-      const double c = ((q - 1) * (q * (q - 2) * x + al * al) * b - 2 * (k + al - 1) * (k - 1) * q * a) / (2 * k * (k + al) * (q - 2));
-      a = b; b = c;
-    }
-    return b;
-  };
-  int m = 0;
-  for (int n = 0; n <= p; ++n)
-    for (int i = 0; i <= n; ++i) {
-      const int jj = n - i;
-      out[m++] = std::sqrt((2.0 * i + 1) * (2.0 * i + 2.0 * jj + 2)) * jac(i, 0.0, 2 * s / (1 - t) - 1) * std::pow(1 - t, i) *
-                 jac(jj, 2.0 * i + 1, 2 * t - 1);
-    }
+__device__ double conv_chi(int m, double s, double t) {
+  int n = 0;
+  while ((n + 1) * (n + 2) / 2 <= m) ++n;
+  const int i = m - n * (n + 1) / 2, j = n - i;
+  return sqrt((2.0 * i + 1) * (2.0 * i + 2.0 * j + 2)) * conv_jacobi(i, 0, 2 * s / (1 - t) - 1) * conv_pow(1 - t, i) *
+         conv_jacobi(j, 2.0 * i + 1, 2 * t - 1);
 }
 
-const double kVert[4][3] = {{0, 0, 0}, {1, 0, 0}, {0, 1, 0}, {0, 0, 1}};
+__global__ void __launch_bounds__(256) k_conv_tables(int N, int N1, int M, int Ng, const __grid_constant__ ConvNodes nd,
+                                                     const ConvSrc a, const ConvOff off, float2* __restrict__ out) {
+  __shared__ double chi[49 * 15];                 // at the face points
+  const int F = a.nqf, nv = nd.nv, V = nv * nv * nv;
+  for (int e = threadIdx.x; e < F * M; e += 256) chi[e] = conv_chi(e % M, a.tri_st[2 * (e / M)], a.tri_st[2 * (e / M) + 1]);
+  __syncthreads();
+  for (int g = blockIdx.x * 256 + threadIdx.x; g < off.o[13]; g += gridDim.x * 256) {
+    int t = 0;
+    while (g >= off.o[t + 1]) ++t;
+    const int e = g - off.o[t];
+    double v = 0.0;
+    if (t <= 2) {                                 // at point q of the volume rule: phi_k, and the weight
+      const int q = t == 0 ? e % V : t == 1 ? e / N1 : e, k = t == 0 ? e / V : e % N1;
+      const int qa = q / (nv * nv), qb = q / nv % nv, qc = q % nv;
+      v = t == 2 ? nd.w[0][qa] * nd.w[1][qb] * nd.w[2][qc] : conv_phi(nd.mi, k, nd.x[0][qa], nd.x[1][qb], nd.x[2][qc]);
+    } else if (t == 3) {
+      v = nd.tg[e];
+    } else if (t == 4) {
+      v = nd.tw[e];
+    } else if (t == 5) {                          // int phi_l d_e phi_k
+      const int d = e / (N1 * N), l = e / N % N1, k = e % N;
+      for (int q = 0; q < a.nq; ++q) v = fma(a.tet_w[q] * a.tet_phi[(size_t)q * N + l], a.tet_dphi[((size_t)q * 3 + d) * N + k], v);
+    } else if (t <= 7) {                          // int chi_m phi_k over the face with these vertices
+      const int code = e / (N * M), r = e % (N * M), k = t == 6 ? r / M : r % N, m = t == 6 ? r % M : r / N;
+      const int va = code >> 4, vb = code >> 2 & 3, vc = code & 3;
+      if (va != vb && vb != vc && va != vc)
+        for (int q = 0; q < F; ++q) v = fma(a.tri_w[q] * chi[q * M + m], a.face_phi[((size_t)code * F + q) * N + k], v);
+    } else if (t <= 9) {
+      v = t == 8 ? chi[e % F * M + e / F] : chi[e];
+    } else {
+      v = t == 10 ? a.tri_w[e] : t == 11 ? a.tg[e] : a.tw[e];
+    }
+    out[g] = pair_split(v);
+  }
+}
 
 }  // namespace
 
-// The tables of (p, p_t) on the device, built at the first call.
+// The tables of (p, p_t) on the device, built at the first call, in the solver's stream.
 static stdg_status conv_tables(stdg_solver* s, ConvTab* t) {
   const int p = s->p, pt = s->pt, N = s->N, Ng = s->Ng, N1 = p * (p + 1) * (p + 2) / 6, M = (p + 1) * (p + 2) / 2;
   // points of the rules: volume, face, and in time
   const int nv = (3 * p + 1) / 2, nf = (3 * p + 3) / 2, mv = (3 * pt + 2) / 2, mf = (3 * pt + 3) / 2;
-  const size_t V = (size_t)nv * nv * nv, F = (size_t)nf * nf;
-  const size_t len[13] = {N * V, V * N1, V, (size_t)mv * Ng, (size_t)mv, (size_t)3 * N1 * N, (size_t)64 * N * M,
-                          (size_t)64 * M * N, M * F, F * M, F, (size_t)mf * Ng, (size_t)mf};
-  size_t off[14] = {0};
-  for (int k = 0; k < 13; ++k) off[k + 1] = off[k] + len[k];
+  const int V = nv * nv * nv, F = nf * nf;
+  if (nv > kVNodes || mv > kTNodes || F != s->nqf_nl || mf != s->nt_nl || F * M > 49 * 15) {
+    set_error("convection: unexpected quadrature rules");
+    return STDG_EINVAL;
+  }
+  const int len[13] = {N * V, V * N1, V, mv * Ng, mv, 3 * N1 * N, 64 * N * M, 64 * M * N, M * F, F * M, F, mf * Ng, mf};
+  ConvOff off{};
+  for (int k = 0; k < 13; ++k) off.o[k + 1] = off.o[k] + len[k];
   if (!s->conv_tab) {
-    const Rule vr = tet_rule(nv), fr = tri_rule(nf), lr = tri_rule(p + 1), mr = tet_rule(p + 1);
-    const Rule vt = line_rule(mv), ft = line_rule(mf);
-    std::vector<double> h(off[13], 0.0), phi(N), dphi(3 * N), chi(M), g(Ng), dg(Ng);
-    for (int q = 0; q < vr.n; ++q) {
-      dubiner_eval(p, &vr.x[3 * q], phi.data(), dphi.data());
-      for (int k = 0; k < N; ++k) h[off[0] + (size_t)k * vr.n + q] = phi[k];
-      for (int l = 0; l < N1; ++l) h[off[1] + (size_t)q * N1 + l] = phi[l];   // the first N1 functions span P_{p-1}
-      h[off[2] + q] = vr.w[q];
+    ConvNodes nd{};
+    nd.nv = nv; nd.mv = mv;
+    std::vector<double> x, w, g(Ng), dg(Ng);
+    for (int al = 0; al < 3; ++al) {
+      gauss_jacobi01(nv, al, x, w);
+      for (int q = 0; q < nv; ++q) { nd.x[al][q] = x[q]; nd.w[al][q] = w[q]; }
     }
-    auto time_rule = [&](const Rule& r, size_t og, size_t ow) {
-      for (int q = 0; q < r.n; ++q) {
-        legendre01(pt, r.x[q], g.data(), dg.data());
-        for (int b = 0; b < Ng; ++b) h[og + (size_t)q * Ng + b] = g[b];
-        h[ow + q] = r.w[q];
-      }
-    };
-    time_rule(vt, off[3], off[4]);
-    time_rule(ft, off[11], off[12]);
-    for (int q = 0; q < mr.n; ++q) {
-      dubiner_eval(p, &mr.x[3 * q], phi.data(), dphi.data());
-      for (int e = 0; e < 3; ++e)
-        for (int l = 0; l < N1; ++l)
-          for (int k = 0; k < N; ++k) h[off[5] + ((size_t)e * N1 + l) * N + k] += mr.w[q] * phi[l] * dphi[e * N + k];
+    gauss_jacobi01(mv, 0, x, w);
+    for (int q = 0; q < mv; ++q) {
+      legendre01(pt, x[q], g.data(), dg.data());
+      for (int b = 0; b < Ng; ++b) nd.tg[q * Ng + b] = g[b];
+      nd.tw[q] = w[q];
     }
-    for (int a = 0; a < 4; ++a)
-      for (int b = 0; b < 4; ++b)
-        for (int c = 0; c < 4; ++c) {
-          if (a == b || b == c || a == c) continue;
-          const size_t code = (size_t)tri_code(a, b, c);
-          for (int q = 0; q < lr.n; ++q) {
-            const double u = lr.x[2 * q], v = lr.x[2 * q + 1];
-            double xi[3];
-            for (int d = 0; d < 3; ++d) xi[d] = kVert[a][d] + u * (kVert[b][d] - kVert[a][d]) + v * (kVert[c][d] - kVert[a][d]);
-            dubiner_eval(p, xi, phi.data(), dphi.data());
-            tri_basis(p, u, v, chi.data());
-            for (int k = 0; k < N; ++k)
-              for (int m = 0; m < M; ++m) {
-                h[off[6] + (code * N + k) * M + m] += lr.w[q] * chi[m] * phi[k];
-                h[off[7] + (code * M + m) * N + k] += lr.w[q] * chi[m] * phi[k];
-              }
-          }
-        }
-    for (int q = 0; q < fr.n; ++q) {
-      tri_basis(p, fr.x[2 * q], fr.x[2 * q + 1], chi.data());
-      for (int m = 0; m < M; ++m) h[off[8] + (size_t)m * fr.n + q] = h[off[9] + (size_t)q * M + m] = chi[m];
-      h[off[10] + q] = fr.w[q];
-    }
-    std::vector<float2> hp(off[13]);
-    for (size_t k = 0; k < hp.size(); ++k) {
-      const float hi = (float)h[k];
-      hp[k] = make_float2(hi, (float)(h[k] - (double)hi));
-    }
+    const std::vector<int> ex = multi_indices(p);
+    for (size_t k = 0; k < ex.size(); ++k) nd.mi.e[k] = (unsigned char)ex[k];
+    const ConvSrc src{s->dr.tet_nl_phi, s->dr.tet_nl_dphi, s->dr.tet_nl_w, s->dr.face_nl_phi, s->dr.tri_nl_st, s->dr.tri_nl_w,
+                      s->d_tg, s->d_tw, s->nq_nl, F, mf};
     float2* d = nullptr;
-    const stdg_status e = dev_alloc(s, (void**)&d, hp.size() * sizeof(float2));
+    const stdg_status e = dev_alloc(s, (void**)&d, (size_t)off.o[13] * sizeof(float2));
     if (e != STDG_OK) return e;
-    if (cudaMemcpyAsync(d, hp.data(), hp.size() * sizeof(float2), cudaMemcpyHostToDevice, s->stream) != cudaSuccess ||
-        cudaStreamSynchronize(s->stream) != cudaSuccess) {
-      set_error("convection tables: upload failed");
-      return STDG_ECUDA;
-    }
+    ++s->nlaunch;
+    k_conv_tables<<<std::min(304, (off.o[13] + 255) / 256), 256, 0, s->stream>>>(N, N1, M, Ng, nd, src, off, d);
+    STDG_LAUNCH_CHECK();
     s->conv_tab = d;
   }
   const float2* d = s->conv_tab;
-  *t = ConvTab{d + off[0], d + off[1], d + off[2], d + off[3], d + off[4], d + off[5], d + off[6],
-               d + off[7], d + off[8], d + off[9], d + off[10], d + off[11], d + off[12]};
+  *t = ConvTab{d + off.o[0], d + off.o[1], d + off.o[2], d + off.o[3], d + off.o[4], d + off.o[5], d + off.o[6],
+               d + off.o[7], d + off.o[8], d + off.o[9], d + off.o[10], d + off.o[11], d + off.o[12]};
   return STDG_OK;
 }
 

@@ -26,10 +26,10 @@ void set_error(const char* fmt, ...) {
 
 const char* last_error() { return g_err; }
 
-// P_n^(a,b)(x) and its derivative by the three-term recurrence.
-static void jacobi(int n, double a, double b, double x, double* P, double* dP) {
+// P_n^(a,b)(x) by the three-term recurrence
+static double jacobi_value(int n, double a, double b, double x) {
   double p0 = 1.0, p1 = 0.5 * (a - b + (a + b + 2.0) * x);
-  if (n == 0) { *P = 1.0; *dP = 0.0; return; }
+  if (n == 0) return 1.0;
   for (int k = 2; k <= n; ++k) {
     double c = 2.0 * k + a + b;
     double a1 = 2.0 * k * (k + a + b) * (c - 2.0);
@@ -39,12 +39,15 @@ static void jacobi(int n, double a, double b, double x, double* P, double* dP) {
     double p2 = ((a2 + a3 * x) * p1 - a4 * p0) / a1;
     p0 = p1; p1 = p2;
   }
-  *P = p1;
+  return p1;
+}
+// the same with its derivative
+static void jacobi(int n, double a, double b, double x, double* P, double* dP) {
+  *P = jacobi_value(n, a, b, x);
+  if (n == 0) { *dP = 0.0; return; }
   // d/dx P_n^(a,b) = (n + a + b + 1)/2 P_{n-1}^(a+1,b+1)
   if (n == 1) { *dP = 0.5 * (a + b + 2.0); return; }
-  double q, dq;
-  jacobi(n - 1, a + 1.0, b + 1.0, x, &q, &dq);
-  *dP = 0.5 * (n + a + b + 1.0) * q;
+  *dP = 0.5 * (n + a + b + 1.0) * jacobi_value(n - 1, a + 1.0, b + 1.0, x);
 }
 
 void gauss_jacobi01(int n, int alpha, std::vector<double>& x, std::vector<double>& w) {
@@ -52,19 +55,16 @@ void gauss_jacobi01(int n, int alpha, std::vector<double>& x, std::vector<double
   // neighbouring roots are at least about 8 / (n + 2)^2 apart: some 30 intervals between them (20,000 at every n
   // took about a millisecond a rule)
   const int grid = 8 * n * n + 8;
-  double prev_x = -1.0, prev_v, d;
-  jacobi(n, alpha, 0.0, -1.0 + 1e-15, &prev_v, &d);
+  double prev_x = -1.0, prev_v = jacobi_value(n, alpha, 0.0, -1.0 + 1e-15);
   std::vector<double> roots;
   for (int g = 1; g <= grid; ++g) {
     double xx = -1.0 + 2.0 * g / grid;
     if (g == grid) xx = 1.0 - 1e-15;
-    double v;
-    jacobi(n, alpha, 0.0, xx, &v, &d);
+    const double v = jacobi_value(n, alpha, 0.0, xx);
     if ((v < 0) != (prev_v < 0)) {
       double lo = prev_x, hi = xx, flo = prev_v;
       for (int it = 0; it < 200 && hi - lo > 1e-15; ++it) {
-        double mid = 0.5 * (lo + hi), fm;
-        jacobi(n, alpha, 0.0, mid, &fm, &d);
+        const double mid = 0.5 * (lo + hi), fm = jacobi_value(n, alpha, 0.0, mid);
         if ((fm < 0) == (flo < 0)) { lo = mid; flo = fm; } else { hi = mid; }
       }
       double r = 0.5 * (lo + hi);

@@ -1,6 +1,10 @@
-"""The convective term's rounding error against the binary64 oracle: the kernels with the degrees at compile time
+"""The convective term's rounding error and its first call.
+
+The rounding error against the binary64 oracle: the kernels with the degrees at compile time
 are at least as accurate as the general kernel (STDG_CONV_KERNEL=generic), which sums every test function over the
 points themselves, at every degree."""
+import time
+
 import numpy as np
 import pytest
 
@@ -47,3 +51,25 @@ def test_rounding_error_is_no_larger_than_the_general_kernels(p, pt, data, monke
             err[kernel] += np.square(out - exact).sum() / np.square(exact).sum()
     print(f"p={p} pt={pt} {data}: rms error {np.sqrt(err['default'] / 2):.2e}, general {np.sqrt(err['generic'] / 2):.2e}")
     assert err["default"] <= err["generic"]
+
+
+@pytest.mark.parametrize("p,pt", [(3, 1), (4, 4)])
+def test_first_call_of_a_solver_builds_its_tables_quickly(p, pt):
+    """The tables of the degrees are built in the first call, on the device: medians over five solvers, with room for
+    six later calls and half a millisecond (evaluated on the host they took 0.9 and 2.5 ms)."""
+    import paper_1601_07384_gb300 as g
+    first, later = [], []
+    for k in range(6):
+        s = g.Solver(g.Mesh(*kuhn_mesh(2, seed=k)), g.Reference(p, pt), 0.01)
+        s.set_boundary(g.zero())
+        vbar = torch.ones(3 * s.ne * s.Nst, dtype=torch.float64, device="cuda")
+        ups = torch.empty_like(vbar)
+        for out in (first, later):
+            torch.cuda.synchronize()
+            t0 = time.perf_counter()
+            s.convection(vbar, ups)
+            torch.cuda.synchronize()
+            out.append(time.perf_counter() - t0)
+    f, l = np.median(first[1:]), np.median(later[1:])
+    print(f"p={p} pt={pt}: first {f * 1e6:.0f} us, later {l * 1e6:.0f} us")
+    assert f <= 6 * l + 5e-4
