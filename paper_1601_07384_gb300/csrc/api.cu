@@ -383,26 +383,22 @@ extern "C" stdg_status stdg_get_blocks(const stdg_solver* s, double* Q, double* 
   if (!s) { set_error("NULL solver"); return STDG_EINVAL; }
   cudaSetDevice(s->device);
   cudaStreamSynchronize(s->stream);
-  // decoded to binary64 in pieces of at most 64 MB (stream-ordered memory, returned below)
+  // decoded to binary64 in pieces, in the room of the products' input vectors (free between products): the call
+  // needs no memory of its own
   const int NN = s->N * s->N;
+  double* const tmp = static_cast<double*>(s->fxws.w);
+  const int64_t room = s->fxws.nvec * s->Nst;
   const struct { double* host; FxBlocks b; int64_t nblk; int len; } all[4] = {
       {Q, blocks_Q(s), 6 * s->nf, NN}, {Mij, blocks_M(s), 2 * s->nf, NN},
       {Aoff, blocks_A(s), s->nf, NN}, {Bdiag, blocks_B(s), s->ne, NN}};
   for (const auto& a : all) {
-    if (!a.host || a.nblk == 0) continue;
-    const int64_t step = std::max<int64_t>(1, std::min<int64_t>(a.nblk, (8 << 20) / a.len));
-    double* tmp = nullptr;
-    STDG_CUDA(cudaMallocAsync((void**)&tmp, (size_t)step * a.len * sizeof(double), s->stream));
-    cudaError_t ce = cudaSuccess;
-    for (int64_t b = 0; b < a.nblk && ce == cudaSuccess; b += step) {
-      const int64_t n = std::min(step, a.nblk - b);
-      ce = launch_fx_decode(b, n, a.len, s->N, a.b, tmp, s->stream);
-      if (ce == cudaSuccess)
-        ce = cudaMemcpyAsync(a.host + b * a.len, tmp, (size_t)n * a.len * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-      if (ce == cudaSuccess) ce = cudaStreamSynchronize(s->stream);
+    const int64_t total = a.host ? a.nblk * a.len : 0;
+    for (int64_t o = 0; o < total; o += room) {
+      const int64_t n = std::min(room, total - o);
+      STDG_CUDA(launch_fx_decode(o, n, a.len, s->N, a.b, tmp, s->stream));
+      STDG_CUDA(cudaMemcpyAsync(a.host + o, tmp, (size_t)n * sizeof(double), cudaMemcpyDeviceToHost, s->stream));
+      STDG_CUDA(cudaStreamSynchronize(s->stream));
     }
-    cudaFreeAsync(tmp, s->stream);
-    STDG_CUDA(ce);
   }
   return STDG_OK;
 }

@@ -142,10 +142,10 @@ struct FaceOps {
   FxBlocks Q, Mij;
 };
 // nblk blocks of len binary64 entries (rows of N) to fixed point in place (exps: their exponents), scaled
-// by r and c, and back (blocks first .. first + nblk - 1)
+// by r and c, and back (n entries from entry first of the first block on)
 cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint16_t* exps, const FxScale& r,
                              const FxScale& c, cudaStream_t st);
-cudaError_t launch_fx_decode(int64_t first, int64_t nblk, int len, int N, const FxBlocks& in, double* out, cudaStream_t st);
+cudaError_t launch_fx_decode(int64_t first, int64_t n, int len, int N, const FxBlocks& in, double* out, cudaStream_t st);
 // The scaling of the tet modes by the diagonals of the blocks B, and of the rows of the (not yet encoded)
 // blocks Q to match; top: room for 2 N words on the device.  Waits for the stream.
 cudaError_t fx_scales(int64_t ne, int64_t nq, int N, const double* B, const double* Q, int* top, FxScale* s, FxScale* t,

@@ -583,10 +583,10 @@ __global__ void __launch_bounds__(256) k_fx_encode(int64_t nblk, int len, int N,
     for (int o = lane; o < len; o += 32) reinterpret_cast<int2*>(p)[o] = fx_encode(p[o], e);
   }
 }
-__global__ void __launch_bounds__(256) k_fx_decode(int64_t first, int64_t nblk, int len, int N, FxBlocks in,
+__global__ void __launch_bounds__(256) k_fx_decode(int64_t first, int64_t n, int len, int N, const __grid_constant__ FxBlocks in,
                                                    double* __restrict__ out) {
-  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < nblk * len; o += (int64_t)gridDim.x * blockDim.x)
-    out[o] = fx_entry(in, len, first + o / len, (int)(o % len), N);
+  for (int64_t o = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; o < n; o += (int64_t)gridDim.x * blockDim.x)
+    out[o] = fx_entry(in, len, (first + o) / len, (int)((first + o) % len), N);
 }
 // top[l]: largest exponent of the diagonal entries (l, l) of the blocks B
 __global__ void __launch_bounds__(256) k_fx_diag(int64_t ne, int N, const double* __restrict__ B, int* top) {
@@ -647,8 +647,8 @@ cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint1
   if (nblk > 0) k_fx_encode<<<1216, 256, 0, st>>>(nblk, len, N, blocks, exps, r, c);
   return cudaGetLastError();
 }
-cudaError_t launch_fx_decode(int64_t first, int64_t nblk, int len, int N, const FxBlocks& in, double* out, cudaStream_t st) {
-  if (nblk > 0) k_fx_decode<<<1216, 256, 0, st>>>(first, nblk, len, N, in, out);
+cudaError_t launch_fx_decode(int64_t first, int64_t n, int len, int N, const FxBlocks& in, double* out, cudaStream_t st) {
+  if (n > 0) k_fx_decode<<<1216, 256, 0, st>>>(first, n, len, N, in, out);
   return cudaGetLastError();
 }
 
