@@ -261,6 +261,14 @@ stdg_status stdg_solver_create_alloc(const stdg_mesh* mesh, const stdg_ref* ref,
                                      const stdg_solver_options* opts, void* cuda_stream, stdg_alloc_fn alloc_fn,
                                      stdg_free_fn free_fn, void* user, stdg_solver** out);
 void stdg_solver_destroy(stdg_solver* s);
+/* Threads and streams: stdg_pressure_apply, stdg_pressure_apply_factored, stdg_pressure_rhs,
+ * stdg_velocity_update, stdg_velocity_moments, stdg_convection and stdg_get_blocks prepare their
+ * input in one array of the solver, as do the solves and steps built on them.  Calls of these (but
+ * for _factored, which keeps two vectors more) on one solver from several threads enter its stream
+ * one after another, each as a whole.  Device work of one solver must not overlap otherwise: a call
+ * that the caller has captured into a CUDA graph and replays on another stream needs to be ordered
+ * with the solver's other work.  Solves, steps and the calls of the learned preconditioner keep
+ * further state and take one thread at a time; different solvers are independent. */
 /* Change the time step (rebuilds only the Ng x Ng time factor dt^2 K^-1). */
 stdg_status stdg_set_dt(stdg_solver* s, double dt);
 /* Change the cap on Krylov iterations per solve (stdg_solver_options.max_iters); STDG_EINVAL if < 1. */

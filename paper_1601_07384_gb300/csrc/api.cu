@@ -386,6 +386,7 @@ extern "C" stdg_status stdg_get_blocks(const stdg_solver* s, double* Q, double* 
   // decoded to binary64 in pieces, in the room of the products' input vectors (free between products): the call
   // needs no memory of its own
   const int NN = s->N * s->N;
+  std::lock_guard<std::mutex> lock(*s->fxws.order);
   double* const tmp = static_cast<double*>(s->fxws.w);
   const int64_t room = s->fxws.nvec * s->Nst;
   const struct { double* host; FxBlocks b; int64_t nblk; int len; } all[4] = {

@@ -531,6 +531,7 @@ static stdg_status conv_tables(stdg_solver* s, ConvTab* t) {
 stdg_status convection_modal(stdg_solver* s, const FieldArg& fld, const double* vbar, double* ups) {
   if (s->p < 1 || s->p > 4) return STDG_EUNSUPPORTED;
   ConvTab t{};
+  std::lock_guard<std::mutex> lock(*s->fxws.order);
   const stdg_status e = conv_tables(s, &t);
   if (e != STDG_OK) return e;
   const int M = (s->p + 1) * (s->p + 2) / 2;

@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <mutex>
 
 #include "fixed.cuh"
 #include "internal.h"
@@ -118,7 +119,9 @@ namespace stdg {
 // with Tacc = identity when tacc_identity.  pinned: x at (tet 0, mode 0, every a) read as 0,
 // y there = pin_diag * x.
 // Room for the limbs and exponents of the products' input vectors (up to nvec vectors of Ng columns of N).
-struct FxWork { void* w; uint16_t* e; int64_t nvec; };
+// A product writes them in one launch and reads them in the next: `order` is held from the first to the second, so
+// that products of several threads enter the solver's stream one after another.
+struct FxWork { void* w; uint16_t* e; int64_t nvec; std::mutex* order; };
 struct ApplyArgs {
   FxWork ws;
   int ne, N, Ng;

@@ -48,7 +48,8 @@ struct stdg_solver {
   // below) with these exponents, one per block of N x N
   uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;
   stdg::FxScale fxs{}, fxt{};                 // scaling of the tet modes, and of the dual modes of Q
-  stdg::FxWork fxws{};                        // the products' input vectors in limbs (3 nf vectors fit)
+  std::mutex fx_order;
+  stdg::FxWork fxws{nullptr, nullptr, 0, &fx_order};   // the products' input vectors in limbs (3 nf vectors fit)
   double *Binv = nullptr;                     // block-Jacobi: (-B_i)^-1, pinned (lazily built)
   double *kz = nullptr;                       // preconditioned residual
   // low-precision copies for the mixed-precision inner solve
