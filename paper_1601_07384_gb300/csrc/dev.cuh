@@ -101,12 +101,12 @@ struct TimeMats {
 };
 
 // Launchers (precompute.cu)
-cudaError_t launch_face_blocks(const DevMesh& m, const DevRef& r, int p, int N, int nq, int nqf,
+[[nodiscard]] cudaError_t launch_face_blocks(const DevMesh& m, const DevRef& r, int p, int N, int nq, int nqf,
                                const MultiIdx& mi, double* Q, double* Mij, double* C, double* x0h,
                                cudaStream_t st);
-cudaError_t launch_assemble(const DevMesh& m, int N, const double* Q, double* Aoff, double* Bdiag,
+[[nodiscard]] cudaError_t launch_assemble(const DevMesh& m, int N, const double* Q, double* Aoff, double* Bdiag,
                             double* Bv, cudaStream_t st);
-cudaError_t launch_block_inverse(int ne, int N, const FxBlocks& Bdiag, double* Binv, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_block_inverse(int ne, int N, const FxBlocks& Bdiag, double* Binv, cudaStream_t st);
 
 }  // namespace stdg
 
@@ -133,7 +133,7 @@ struct ApplyArgs {
   double Tacc[kMaxNg * kMaxNg];
   double Kmass[kMaxNg * kMaxNg];
 };
-cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_apply(const ApplyArgs& a, const double* x, double* y, cudaStream_t st);
 
 // The per-face blocks Q[nf][2][3][N][N] (one exponent per face, side and component: on a mesh stretched in one
 // direction the components differ by the ratio of the elements' sides), Mij[nf][2][N][N] and the face tables:
@@ -146,26 +146,26 @@ struct FaceOps {
 };
 // nblk blocks of len binary64 entries (rows of N) to fixed point in place (exps: their exponents), scaled
 // by r and c, and back (n entries from entry first of the first block on)
-cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint16_t* exps, const FxScale& r,
+[[nodiscard]] cudaError_t launch_fx_encode(int64_t nblk, int len, int N, double* blocks, uint16_t* exps, const FxScale& r,
                              const FxScale& c, cudaStream_t st);
-cudaError_t launch_fx_decode(int64_t first, int64_t n, int len, int N, const FxBlocks& in, double* out, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_fx_decode(int64_t first, int64_t n, int len, int N, const FxBlocks& in, double* out, cudaStream_t st);
 // The scaling of the tet modes by the diagonals of the blocks B, and of the rows of the (not yet encoded)
 // blocks Q to match; top: room for 2 N words on the device.  Waits for the stream.
-cudaError_t fx_scales(int64_t ne, int64_t nq, int N, const double* B, const double* Q, int* top, FxScale* s, FxScale* t,
+[[nodiscard]] cudaError_t fx_scales(int64_t ne, int64_t nq, int N, const double* B, const double* Q, int* top, FxScale* s, FxScale* t,
                       cudaStream_t st);
 // b_i[a][l] = coef Sum_{f} Sum_c Sum_m Q^c_{s(i,j)}[m][l] F_j[c][a][m]   (D = -Q^T; coef = -dt)
-cudaError_t launch_rhs(const FaceOps& f, const double* F, double coef, int pinned, double* b, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_rhs(const FaceOps& f, const double* F, double coef, int pinned, double* b, cudaStream_t st);
 // V_j = F_j - dt (I (x) K^-1) Sum_s Q_sj dp_s on interior faces, V_j = F_j on boundary faces.
-cudaError_t launch_update(const FaceOps& f, const double* F, const double* dp, double dt, const double* Kinv, double* V,
+[[nodiscard]] cudaError_t launch_update(const FaceOps& f, const double* F, const double* dp, double dt, const double* Kinv, double* V,
                           cudaStream_t st);
 // G_j = dt (I (x) K^-1) Sum_s Q_sj p_s  (boundary: the volume part of the single side)
-cudaError_t launch_face_grad(const FaceOps& f, const double* P, double dt, const double* Kinv, double* G, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_face_grad(const FaceOps& f, const double* P, double dt, const double* Kinv, double* G, cudaStream_t st);
 // out[c][i][a][k] = 1/|J_i| Sum_f Sum_l Mij[j][s][k][l] in[j][c][a][l]
-cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* in, double* out, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_average(const FaceOps& f, const double* detJ, const double* in, double* out, cudaStream_t st);
 // F[j][c][a][m] = Sum_s Sum_k Mij[j][s][k][m] vbar[c][s][a][k]; boundary: F = Vbc
-cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_goback(const FaceOps& f, const double* vbar, const double* Vbc, double* F, cudaStream_t st);
 // U_j[s][c][a][k] = dt Sum_l Mij_s[k][l] V_j[c][a][l]
-cudaError_t launch_moments(const FaceOps& f, const double* V, double dt, double* U, cudaStream_t st);
+[[nodiscard]] cudaError_t launch_moments(const FaceOps& f, const double* V, double dt, double* U, cudaStream_t st);
 
 }  // namespace stdg
 

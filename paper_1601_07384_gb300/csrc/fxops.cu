@@ -526,6 +526,8 @@ cudaError_t fx_launch_t(const P& a, const FxInput& in, const FxMat& mix, cudaStr
     if (e != cudaSuccess) return e;
   }
   k_fx_vec<N, NG><<<(int)(((int64_t)in.n * FxLanes<N>::G + 255) / 256), 256, 0, st>>>(in, mix);
+  const cudaError_t ev = cudaGetLastError();
+  if (ev != cudaSuccess) return ev;
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((a.n + T::TB - 1) / T::TB);
   cfg.blockDim = dim3(T::threads);

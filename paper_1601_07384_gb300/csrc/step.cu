@@ -840,7 +840,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   phase_mark(s, -1);
   // previous slab average and new-slab boundary data
   ++s->nlaunch;
-  launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar_n, st);
+  STDG_CUDA(launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar_n, st));
   if ((e = boundary_data(s, s->t)) != STDG_OK) return e;
   // step 0: v^{n+1,0}(x, tau) = v^n(x, 1), p^{n+1,0} = 0
   ++s->nlaunch;
@@ -857,7 +857,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   for (int k = 0; k < n_picard; ++k) {
     // 1. averaging and previous-Picard pressure gradient
     ++s->nlaunch;
-    launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar, st);
+    STDG_CUDA(launch_average(face_ops(s), s->dm.detJ, s->V, s->Vbar, st));
     // Lambda of Eq. prevpress, of p^{n+theta,k} = theta p^{n+1,k} + (1 - theta) p^n (Eq. CS_16_theta)
     const double* Plam = s->P;
     if (th != 1.0) {
@@ -866,9 +866,9 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
       Plam = s->Pth;
     }
     ++s->nlaunch;
-    launch_face_grad(face_ops(s), Plam, s->dt, s->Kinv.data(), s->F, st);
+    STDG_CUDA(launch_face_grad(face_ops(s), Plam, s->dt, s->Kinv.data(), s->F, st));
     ++s->nlaunch;
-    launch_average(face_ops(s), s->dm.detJ, s->F, s->Lam, st);
+    STDG_CUDA(launch_average(face_ops(s), s->dm.detJ, s->F, s->Lam, st));
     phase_mark(s, 1);
     // 2. convection
     ++s->nlaunch;
@@ -890,12 +890,10 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     phase_mark(s, 3);
     // 4. goback
     ++s->nlaunch;
-    launch_goback(face_ops(s), s->Vbar, s->Vbc, s->F, st);
+    STDG_CUDA(launch_goback(face_ops(s), s->Vbar, s->Vbc, s->F, st));
     // 5. pressure correction (Eq. A2_mod)
     ++s->nlaunch;
-    if (launch_rhs(face_ops(s), s->F, -s->dt, 1, s->bvec, st) != cudaSuccess) {
-      set_error("rhs launch failed"); return STDG_ECUDA;
-    }
+    STDG_CUDA(launch_rhs(face_ops(s), s->F, -s->dt, 1, s->bvec, st));
     if (s->gnn && s->ah_nsnap > 0) {
       int tot = 0;
       e = stdg_gnn_harvest(s, s->bvec, s->ah_nsnap, s->ah_every, s->ah_max, &tot);
@@ -910,9 +908,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
     k_axpy<<<1216, 256, 0, st>>>(np, 1.0 / th, s->dp, s->P);     // dp is the increment of p^{n+theta}
     // 6. velocity update (Eq. A3_mod)
     ++s->nlaunch;
-    if (launch_update(face_ops(s), s->F, s->dp, s->dt, s->Kinv.data(), s->V, st) != cudaSuccess) {
-      set_error("update launch failed"); return STDG_ECUDA;
-    }
+    STDG_CUDA(launch_update(face_ops(s), s->F, s->dp, s->dt, s->Kinv.data(), s->V, st));
     phase_mark(s, 6);
     local.press_iters[k] = ss.iterations;
     local.fallbacks += ss.fallback;
@@ -922,7 +918,7 @@ extern "C" stdg_status stdg_step(stdg_solver* s, double nu, int n_picard, int me
   }
   // diagnostics: discrete divergence Sum_j D_ij v_j on unpinned tets
   ++s->nlaunch;
-  launch_rhs(face_ops(s), s->V, -s->dt, 0, s->bvec, st);
+  STDG_CUDA(launch_rhs(face_ops(s), s->V, -s->dt, 0, s->bvec, st));
   ++s->nlaunch;
   k_maxabs<<<256, 256, 0, st>>>(np, Nst, s->bvec, s->part);
   std::vector<double> part(256);
