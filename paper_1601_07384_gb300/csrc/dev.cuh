@@ -121,7 +121,8 @@ namespace stdg {
 // Room for the limbs and exponents of the products' input vectors (up to nvec vectors of Ng columns of N).
 // A product writes them in one launch and reads them in the next: `order` is held from the first to the second, so
 // that products of several threads enter the solver's stream one after another.
-struct FxWork { void* w; uint16_t* e; int64_t nvec; std::mutex* order; };
+// launches: a product's launch beside the one that its caller counts is added here.
+struct FxWork { void* w; uint16_t* e; int64_t nvec; std::mutex* order; int64_t* launches; };
 struct ApplyArgs {
   FxWork ws;
   int ne, N, Ng;

@@ -559,6 +559,7 @@ cudaError_t fx_launch(int N, int Ng, const P& a, const double* x, int nvec, cons
   const FxInput in{sc, x, static_cast<int2*>(ws.w), ws.e, nvec, pinned};
   if (!in.w || !in.e || (int64_t)nvec > ws.nvec) return cudaErrorInvalidValue;
   std::lock_guard<std::mutex> lock(*ws.order);
+  ++*ws.launches;
   switch (N) {
     case 1: return fx_launch_n<P, 1>(Ng, a, in, mix, st);
     case 4: return fx_launch_n<P, 4>(Ng, a, in, mix, st);

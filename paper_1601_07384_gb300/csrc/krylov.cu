@@ -628,6 +628,8 @@ static bool df_serves(const stdg_solver* s, const ApplyArgs& a) {
   return a.mass_coef == 0.0 && (s->dfB || s->wdB);
 }
 
+static int op_kernels(const stdg_solver* s, const ApplyArgs& a) { return df_serves(s, a) ? 1 : 2; }
+
 // y = op x with the binary64-accurate kernel (fixed point, or the pair kernels where they serve and
 // fp64_only is not set)
 static stdg_status op_apply(stdg_solver* s, const ApplyArgs& a, const double* x, double* y, bool fp64_only = false) {
@@ -713,8 +715,10 @@ static stdg_status graph_capture(stdg_solver* s, int B, Body body, GraphLoop& g)
     set_error("stream capture failed to start");
     return STDG_ECUDA;
   }
+  const int64_t launched = s->nlaunch, applied = s->op_launches;
   for (int j = 0; j < B && st == STDG_OK; ++j) st = body(j, g.prof ? &s->gev[2 * j] : nullptr);
   cudaError_t ce = cudaStreamEndCapture(s->stream, &g.graph);
+  s->nlaunch = launched; s->op_launches = applied;      // recorded, not launched: counted with every replay
   s->capturing = false;
   s->stream = user;
   if (st != STDG_OK) return st;
@@ -784,8 +788,10 @@ static stdg_status run_batched(stdg_solver* s, int B, int kernels_per_iter, int 
     set_error("stream capture failed to start");
     return STDG_ECUDA;
   }
+  const int64_t launched = s->nlaunch, applied = s->op_launches;
   for (int j = 0; j < B && st == STDG_OK; ++j) st = body(j, prof ? &s->gev[2 * j] : nullptr);
   cudaError_t ce = cudaStreamEndCapture(s->stream, &graph);
+  s->nlaunch = launched; s->op_launches = applied;      // recorded, not launched: counted with every replay
   s->capturing = false;
   if (st == STDG_OK && (ce != cudaSuccess || cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)) {
     set_error("graph capture/instantiation failed: %s", cudaGetErrorString(ce));
@@ -915,19 +921,20 @@ static stdg_status cg_block(stdg_solver* s, const ApplyArgs& op, const double* r
     cudaMemcpyAsync(s->hostbuf + slot, res, sizeof(double), cudaMemcpyDeviceToHost, s->stream);
     return STDG_OK;
   };
-  const int kpi = precond ? 7 + mg_launches(s) : 6;
+  const int kpi = (precond ? 6 : 5) + (mg ? mg_launches(s) : 0);   // kernels of an iteration beside the operator's
   int it = 0;
   double rabs = INFINITY;
   const int maxit = s->opt.max_iters;
   if (s->opt.graph_batch > 1) {
     const int kind = df_serves(s, op) ? 1 : 0;
-    stdg_status e = run_batched(s, s->opt.graph_batch, kpi, maxit, tol_abs, body, &it, &rabs, kind, precond);
+    stdg_status e = run_batched(s, s->opt.graph_batch, kpi + op_kernels(s, op), maxit, tol_abs, body, &it, &rabs, kind, precond);
+    if (precond) s->nlaunch += it / s->opt.graph_batch;   // the norm of every batch
     if (e != STDG_OK) return e;
   } else {
     while (it < maxit) {
       stdg_status e = body(0, nullptr);
       if (e != STDG_OK) return e;
-      s->nlaunch += kpi;
+      s->nlaunch += kpi + (precond ? 1 : 0);            // op_apply counts its own
       ++it;
       if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("CG: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
       rabs = s->hostbuf[0];
@@ -1282,6 +1289,7 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     // z = ||r|| d in binary64
     cudaMemsetAsync(z, 0, n * sizeof(double), s->stream);
     lk.accum(s->stream, n, rdec, s->fx, z);
+    ++s->nlaunch;
     }
     // ---- flexible CG step: p = z - Sum_j (z.Q_j / P_j.Q_j) P_j over the stored directions
     const int slot = ring % m, used = ring < m ? ring : m;
@@ -1309,7 +1317,7 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     cg_update(s->stream, rb, npairs, N, Ng, o_al, x, r, p, q, Tp, s->part);
     k_final<<<Ng + 1, kRedThreads, 0, s->stream>>>(rb, Ng + 1, s->part, o_rr);
     cudaMemcpyAsync(s->hostbuf + 880, o_rr, (Ng + 1) * sizeof(double), cudaMemcpyDeviceToHost, s->stream);
-    s->nlaunch += 9;
+    s->nlaunch += 7;
     if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("mixed solve: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
     ++it; ++ring;
     double rr = 0.0;
@@ -1695,7 +1703,7 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
   if ((e = visc_pc_apply(s, nu, r, z, 0, s->vR)) != STDG_OK) return e;
   cudaMemcpyAsync(p, z, n * sizeof(double), cudaMemcpyDeviceToDevice, s->stream);
   cudaMemsetAsync(flag, 0, sizeof(double), s->stream);
-  s->nlaunch += 3;
+  s->nlaunch += 2;                                    // the two below
   const CocgLaunch cl{Ng, rb};
   const int ne = (int)s->ne;
   cl.cross(s->stream, ne, N, r, z, s->part);
@@ -1724,14 +1732,15 @@ static stdg_status cocg_viscous(stdg_solver* s, const ApplyArgs& a, double nu, c
   int it = 0;
   double rabs = INFINITY;
   const int kind = lowprec ? 2 : df_serves(s, at) ? 1 : 0;
-  const int kpi = 9 + (lowprec ? 2 : 0);
+  const int kpi = 6;                                  // kernels of an iteration beside operator and preconditioner
   if (B > 1) {
-    e = run_batched(s, B, kpi, s->opt.max_iters, tol_abs, body, &it, &rabs, kind, true);
+    e = run_batched(s, B, kpi + 1 + (lowprec ? 3 : op_kernels(s, at)), s->opt.max_iters, tol_abs, body, &it, &rabs, kind, true);
+    s->nlaunch += it / B;                             // the norm of every batch
   } else {
     e = STDG_OK;
     while (it < s->opt.max_iters) {
       if ((e = body(0, nullptr)) != STDG_OK) break;
-      s->nlaunch += kpi;
+      s->nlaunch += kpi + 1;                          // operator and preconditioner count their own
       ++it;
       if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("viscous COCG: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }
       rabs = s->hostbuf[0];
@@ -1789,7 +1798,7 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
   cudaMemsetAsync(flag, 0, sizeof(double), s->stream);
   c32_cross(s->stream, rb, ne, N, Ng, r, z, s->part);
   k_cocg_scalars<<<1, 1024, 0, s->stream>>>(rb, Ng, pr, 2, s->part, rho, Ma, flag);
-  s->nlaunch += 4;
+  s->nlaunch += 3;                                    // visc_pc_apply32 counts its own
   const int B = s->opt.graph_batch > 1 ? std::min(4, s->opt.graph_batch) : 1;
   auto body = [&](int slot, cudaEvent_t* evs) -> stdg_status {
     if (evs) cudaEventRecordWithFlags(evs[0], s->stream, cudaEventRecordExternal);
@@ -1821,7 +1830,7 @@ static stdg_status cocg_viscous32(stdg_solver* s, const ApplyArgs& a, double nu,
     e = STDG_OK;
     while (it < s->opt.max_iters) {
       if ((e = body(0, nullptr)) != STDG_OK) break;
-      s->nlaunch += kpi + 1;
+      s->nlaunch += kpi;                              // with the norm; the preconditioner counts its own
       ++s->op_launches;
       ++it;
       if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("viscous COCG: %s", cudaGetErrorString(cudaGetLastError())); return STDG_ECUDA; }

@@ -49,7 +49,7 @@ struct stdg_solver {
   uint16_t *eB = nullptr, *eA = nullptr, *eQ = nullptr, *eM = nullptr, *eBv = nullptr;
   stdg::FxScale fxs{}, fxt{};                 // scaling of the tet modes, and of the dual modes of Q
   std::mutex fx_order;
-  stdg::FxWork fxws{nullptr, nullptr, 0, &fx_order};   // the products' input vectors in limbs (3 nf vectors fit)
+  stdg::FxWork fxws{nullptr, nullptr, 0, &fx_order, &nlaunch};   // the products' input vectors in limbs (3 nf fit)
   double *Binv = nullptr;                     // block-Jacobi: (-B_i)^-1, pinned (lazily built)
   double *kz = nullptr;                       // preconditioned residual
   // low-precision copies for the mixed-precision inner solve
