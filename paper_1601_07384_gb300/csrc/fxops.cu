@@ -525,21 +525,23 @@ cudaError_t fx_launch_t(const P& a, const FxInput& in, const FxMat& mix, cudaStr
     const cudaError_t e = cudaFuncSetAttribute(k_fx<P, N, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)T::smem);
     if (e != cudaSuccess) return e;
   }
-  k_fx_vec<N, NG><<<(int)(((int64_t)in.n * FxLanes<N>::G + 255) / 256), 256, 0, st>>>(in, mix);
-  const cudaError_t ev = cudaGetLastError();
-  if (ev != cudaSuccess) return ev;
+  // (errors as the launches return them: asking for CUDA's last error between the two delayed the second by a
+  // microsecond)
   cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)(((int64_t)in.n * FxLanes<N>::G + 255) / 256));
+  cfg.blockDim = dim3(256);
+  cfg.stream = st;
+  const cudaError_t ev = cudaLaunchKernelEx(&cfg, k_fx_vec<N, NG>, in, mix);
+  if (ev != cudaSuccess) return ev;
   cfg.gridDim = dim3((a.n + T::TB - 1) / T::TB);
   cfg.blockDim = dim3(T::threads);
   cfg.dynamicSmemBytes = T::smem;
-  cfg.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  const cudaError_t e = cudaLaunchKernelEx(&cfg, k_fx<P, N, NG>, a, in, mix);
-  return e != cudaSuccess ? e : cudaGetLastError();
+  return cudaLaunchKernelEx(&cfg, k_fx<P, N, NG>, a, in, mix);
 }
 template <class P, int N>
 cudaError_t fx_launch_n(int Ng, const P& a, const FxInput& in, const FxMat& mix, cudaStream_t st) {

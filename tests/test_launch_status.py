@@ -33,5 +33,6 @@ def test_no_caller_drops_a_status():
 def test_the_first_launch_of_a_product_is_checked_before_the_second():
     code = open(os.path.join(CSRC, "fxops.cu")).read()
     body = code[code.index("cudaError_t fx_launch_t"):code.index("cudaError_t fx_launch_n")]
-    first, second = body.index("k_fx_vec<N, NG><<<"), body.index("cudaLaunchKernelEx")
-    assert "cudaGetLastError()" in body[first:second]
+    first = re.search(r"(\w+) = cudaLaunchKernelEx\(&cfg, k_fx_vec<N, NG>", body)
+    assert first and re.match(r"[^;]*;\s*if \(%s != cudaSuccess\) return %s;" % (first[1], first[1]), body[first.start():])
+    assert "return cudaLaunchKernelEx(&cfg, k_fx<P, N, NG>" in body
