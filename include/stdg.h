@@ -476,7 +476,8 @@ stdg_status stdg_profile_read(stdg_solver* s, stdg_profile_stats* out);
 /* Copy per-face spatial blocks to host arrays (any may be NULL):
  *  Q_host[nf][2][3][N][N]: Q^sp_{s,j}[c][m][l] = int_{T_sj} psi_m d_c phi_l - sigma n_c int_{Gamma_j} psi_m phi_l
  *     (Eq. MD_6 without the time factor); on a boundary face slot 1 holds the volume part.
- *  Mij_host[nf][2][N][N]: int_{T_sj} phi_k psi_l.   Aoff_host[nf][N][N], Bdiag_host[ne][N][N]. */
+ *  Mij_host[nf][2][N][N]: int_{T_sj} phi_k psi_l.   Aoff_host[nf][N][N], Bdiag_host[ne][N][N].
+ * Takes up to 64 MB from the solver's allocator for the duration of the call, or none where it refuses. */
 stdg_status stdg_get_blocks(const stdg_solver* s, double* Q_host, double* Mij_host,
                             double* Aoff_host, double* Bdiag_host);
 

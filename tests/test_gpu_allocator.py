@@ -1,4 +1,4 @@
-"""Device memory of a solver comes from its allocator alone: stdg_get_blocks copies the blocks out without any."""
+"""Device memory of a solver comes from its allocator alone, and stdg_get_blocks does without where that has none."""
 import ctypes as C
 
 import numpy as np
@@ -36,15 +36,26 @@ class PoolHigh:
 
 
 @pytest.mark.parametrize("n,p,pt", [(1, 4, 0), (2, 1, 1), (2, 4, 4), (3, 2, 0)])
-def test_get_blocks_allocates_nothing_and_matches_oracle(n, p, pt):
-    """(1, 4, 0): the room that the blocks are decoded in holds a block and a half, so most pieces end inside one."""
+def test_get_blocks_takes_memory_from_the_allocator_or_none_and_matches_oracle(n, p, pt, monkeypatch):
+    """Nothing from the runtime's pool, and the allocator gets back what it gave; once it gives no more, the same
+    values.  (1, 4, 0): the room that the blocks are then decoded in holds a block and a half, so that most pieces
+    end inside one."""
     import paper_1601_07384_gb300 as g
     s = g.Solver(g.Mesh(*kuhn_mesh(n, seed=0)), g.Reference(p, pt), 1.0)
     torch.cuda.synchronize()
-    high, free, calls = PoolHigh(), torch.cuda.mem_get_info()[0], s.alloc_stats()[1]
+    high, live = PoolHigh(), s.alloc_stats()[0]
     blk = s.blocks()
-    assert high.read() == 0
-    assert torch.cuda.mem_get_info()[0] == free and s.alloc_stats()[1] == calls
+    assert high.read() == 0 and s.alloc_stats()[0] == live
+
+    def none_left(*args, **kwargs):
+        raise torch.cuda.OutOfMemoryError("none left")
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", none_left)
+    torch.cuda.synchronize()
+    free, calls = torch.cuda.mem_get_info()[0], s.alloc_stats()[1]
+    again = s.blocks()
+    assert high.read() == 0 and torch.cuda.mem_get_info()[0] == free and s.alloc_stats()[1] == calls
+    assert all(np.array_equal(blk[k], again[k]) for k in blk)
     d = SpaceTimeDG(Mesh(*kuhn_mesh(n, seed=0)), p, 0, 1.0)
     B = np.zeros_like(blk["Bdiag"])
     close = lambda a, b: np.abs(a - b).max() <= 1e-12 * max(np.abs(b).max(), 1e-300)   # noqa: E731
