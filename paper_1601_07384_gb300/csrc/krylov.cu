@@ -128,45 +128,9 @@ static void cg_update(cudaStream_t st, int rb, int64_t npairs, int N, int Ng, co
   STDG_NG_SWITCH(Ng, (k_cg_update<G><<<rb, kRedThreads, 0, st>>>(npairs, N, alpha, x, r, p, q, Tp, part, want)));
 }
 
-// z_i[a][k] = Sum_l Binv_i[k][l] r_i[a][l]  (block Jacobi); partials of r.z per column a.
-// Fixed grid (kRedBlocks blocks striding over tets) so the partials stay deterministic.
-__global__ void __launch_bounds__(128) k_bjacobi(int ne, int N, int Ng, const double* __restrict__ Binv,
-                                                 const double* __restrict__ r, double* __restrict__ z,
-                                                 double* part) {
-  extern __shared__ double sm[];
-  const int Nst = N * Ng;
-  const size_t NN = (size_t)N * N;
-  double* rs = sm;
-  double acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  for (int i = blockIdx.x; i < ne; i += gridDim.x) {
-    __syncthreads();
-    for (int o = threadIdx.x; o < Nst; o += blockDim.x) rs[o] = r[(size_t)i * Nst + o];
-    __syncthreads();
-    for (int o = threadIdx.x; o < Nst; o += blockDim.x) {
-      const int a = o / N, k = o % N;
-      const double* B = Binv + (size_t)i * NN + k;     // symmetric: read column k (coalesced over k)
-      double s = 0.0;
-      for (int l = 0; l < N; ++l) s = fma(B[(size_t)l * N], rs[a * N + l], s);
-      z[(size_t)i * Nst + o] = s;
-      acc[a] = fma(s, rs[o], acc[a]);
-    }
-  }
-  __shared__ double red[8][4];
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  for (int a = 0; a < Ng; ++a) {
-    double v = warp_sum(acc[a]);
-    if (lane == 0) red[a][w] = v;
-  }
-  __syncthreads();
-  if (threadIdx.x < Ng) {
-    double s = 0.0;
-    for (int q = 0; q < (int)(blockDim.x >> 5); ++q) s += red[threadIdx.x][q];
-    part[(size_t)blockIdx.x * Ng + threadIdx.x] = s;
-  }
-}
-
-// Same with binary32 inverses and binary32 products (the preconditioner need not be FP64; the
-// CG iterates, residuals and scalars stay binary64).
+// z_i[a][k] = Sum_l Binv_i[k][l] r_i[a][l] (block Jacobi) with binary32 inverses and binary32 products (the
+// preconditioner need not be FP64; the CG iterates, residuals and scalars stay binary64); partials of r.z per
+// column a, one row per block.
 __global__ void __launch_bounds__(256) k_bjacobi32(int ne, int N, int Ng, const float* __restrict__ Binv,
                                                    const double* __restrict__ r, double* __restrict__ z,
                                                    double* part) {
@@ -273,21 +237,6 @@ __global__ void k_cg_alpha(int Ng, const double* rr, const double* pq, double* a
   int a = threadIdx.x;
   if (a < Ng) alpha[a] = (pq[a] != 0.0) ? rr[a] / pq[a] : 0.0;
 }
-// Guarded step length for the binary32 CG of the mixed-precision solve: a breakdown (p.Ap <= 0 or a
-// non-finite step in any column: the rounded operator has lost definiteness along p) freezes the
-// recurrence (alpha = 0) and raises flag[0] until the host restarts the direction.
-__global__ void k_cg_alpha_guard(int Ng, const double* rr, const double* pq, double* alpha, double* flag) {
-  const int a = threadIdx.x;
-  double al = 0.0;
-  bool bad = false;
-  if (a < Ng) {
-    al = rr[a] / pq[a];
-    bad = flag[0] != 0.0 || !(pq[a] > 0.0) || !isfinite(al);
-  }
-  bad = __any_sync(0xffffffffu, bad);
-  if (a < Ng) alpha[a] = bad ? 0.0 : al;
-  if (a == 0 && bad) flag[0] = 1.0;
-}
 // Sums of `width` columns of partials by one block of T = 1024 / width * width threads, in a fixed order:
 // thread t adds entries t, t + T, ... (all of column t % width), warp c the threads' sums of column c, c + 32, ...
 // out: shared, [width].  (One column after another with 256 threads took 11 us for 5 columns.)
@@ -306,8 +255,10 @@ __device__ inline void block_column_sums(int nparts, int width, const double* __
   }
   __syncthreads();
 }
-// One block: reduce the per-block p.q partials of every column, then the guarded step length of
-// k_cg_alpha_guard (one launch instead of two per binary32 iteration).
+// One block: reduce the per-block p.q partials of every column, then the guarded step length for the binary32 CG
+// of the mixed-precision solve: a breakdown (p.Ap <= 0 or a non-finite step in any column: the rounded operator
+// has lost definiteness along p) freezes the recurrence (alpha = 0) and raises flag[0] until the host restarts
+// the direction.
 __global__ void __launch_bounds__(1024) k_final_alpha_guard(int nparts, int Ng, const double* __restrict__ part,
                                                             const double* rz, double* alpha, double* flag) {
   __shared__ double scratch[1024], pq[kMaxNg];
@@ -322,16 +273,6 @@ __global__ void __launch_bounds__(1024) k_final_alpha_guard(int nparts, int Ng, 
     for (int a = 0; a < Ng; ++a) alpha[a] = bad ? 0.0 : al[a];
     if (bad) flag[0] = 1.0;
   }
-}
-// k_cg_beta2 for the mixed solve: the residual estimate reads -1 once the recurrence is frozen
-__global__ void k_cg_beta_guard(int Ng, double* rz, const double* rznew, double* beta, double* res, const double* mix2,
-                                const double* flag) {
-  int a = threadIdx.x;
-  if (a < Ng) {
-    beta[a] = (rz[a] != 0.0) ? rznew[a] / rz[a] : 0.0;
-    rz[a] = rznew[a];
-  }
-  if (a == 0) res[0] = flag[0] != 0.0 ? -1.0 : sqrt(mix2[0]);
 }
 // Preconditioner of the viscous systems (Eq. A1_mod): the inverse of their mass part,
 // z_i = (mass |J_i| K)^-1 (x) I r_i (K^-1 passed in Kinv), with partials of r.z per column.
@@ -1178,15 +1119,13 @@ static stdg_status ensure_lowprec(stdg_solver* s) {
   const size_t n = (size_t)s->ne * s->Nst;
   for (float** v : {&s->fr, &s->fp, &s->fq, &s->fz, &s->fx, &s->fb})
     if ((e = dev_alloc(s, (void**)v, n * sizeof(float))) != STDG_OK) return e;
-  if ((e = dev_alloc(s, (void**)&s->dmix, kMaxNg * kMaxNg * sizeof(double))) != STDG_OK) return e;
-  cudaMemcpyAsync(s->dmix, s->K.data(), s->Ng * s->Ng * sizeof(double), cudaMemcpyHostToDevice, s->stream);
   if (cudaStreamSynchronize(s->stream) != cudaSuccess) { set_error("low-precision setup failed"); return STDG_ECUDA; }
   return STDG_OK;
 }
 
 // Mixed precision, inner-outer.  Outer: flexible CG in binary64 on the Kronecker-decoupled system
 // S X = B' (S = -A_sp (x) I with the pin, B' = -(I (x) Tp^-1) b), operator applied by the
-// binary64-accurate pair kernel; each new direction is S-orthogonalised against the last m
+// binary64-accurate kernel (op_apply); each new direction is S-orthogonalised against the last m
 // directions (flexible CG, Notay 2000), and x, r and all scalars are binary64, so the binary32 parts
 // change how fast it converges, not the accuracy it reaches.  Preconditioner: a fixed number of
 // block-Jacobi CG iterations in binary32 (binary32 or bfloat16 operator, binary32 vectors) started

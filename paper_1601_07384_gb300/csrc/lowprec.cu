@@ -448,10 +448,6 @@ cudaError_t launch_apply_df(stdg_solver* s, const double* x, double* y, int pinn
 
 // ------------------------------------------------------------------ binary32 Krylov vectors
 constexpr int kLpBlocks = 1216;
-__device__ inline double lp_warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return v;
-}
 // Block-reduce `cnt` binary32 per-thread partials (cnt <= 8) into part[blockIdx.x * stride + c]: binary32
 // within a warp (five shuffle-adds; binary64 ones would cost 5 cnt FP64-pipe operations per thread, tens
 // of microseconds per launch on sm_103a), binary64 across the warps, in a fixed order.
@@ -474,52 +470,7 @@ __device__ inline void lp_block_store(const float (&v)[MAXC], int cnt, double* p
     part[blockIdx.x * stride + threadIdx.x] = t;
   }
 }
-// Column dots of binary32 vectors: one thread per (tet, row) pair covering all Ng columns, binary32
-// sums per thread (about ten pairs each), binary64 across threads (the binary64 pipe is 1/64 of
-// the binary32 rate on sm_103a, so no per-element binary64 work)
-__global__ void __launch_bounds__(256) k_lp_coldot(int64_t ne, int N, int Ng, const float* __restrict__ x,
-                                                  const float* __restrict__ y, double* part) {
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  const int Nst = N * Ng;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = (uint32_t)e / (uint32_t)N;
-    const int64_t o = i * Nst + (e - i * N);
-    for (int a = 0; a < Ng; ++a) acc[a] = fmaf(x[o + a * N], y[o + a * N], acc[a]);
-  }
-  lp_block_store(acc, Ng, part, Ng);
-}
-struct LpTp { float v[kMaxNg * kMaxNg]; };
-// x += alpha_a p; r -= alpha_a q; with want, partials of r.r per column and of ||(I (x) Tp) r||^2
-__global__ void __launch_bounds__(256) k_lp_cg_update(int64_t ne, int N, int Ng, const double* __restrict__ alpha,
-                                                     float* __restrict__ x, float* __restrict__ r,
-                                                     const float* __restrict__ p, const float* __restrict__ q,
-                                                     LpTp Tp, double* part, int want) {
-  float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  float al[kMaxNg];
-  for (int a = 0; a < Ng; ++a) al[a] = (float)alpha[a];
-  const int Nst = N * Ng;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = (uint32_t)e / (uint32_t)N;
-    const int64_t o0 = i * Nst + (e - i * N);
-    float rv[kMaxNg];
-    for (int a = 0; a < Ng; ++a) {
-      const int64_t o = o0 + a * N;
-      x[o] = fmaf(al[a], p[o], x[o]);
-      const float rn = fmaf(-al[a], q[o], r[o]);
-      r[o] = rn;
-      rv[a] = rn;
-      if (want) acc[a] = fmaf(rn, rn, acc[a]);
-    }
-    if (want)
-      for (int a = 0; a < Ng; ++a) {
-        float w = 0.0f;
-        for (int b = 0; b < Ng; ++b) w = fmaf(Tp.v[a * Ng + b], rv[b], w);
-        acc[Ng] = fmaf(w, w, acc[Ng]);
-      }
-  }
-  if (!want) return;
-  lp_block_store(acc, Ng + 1, part, Ng + 1);
-}
+// p = z + beta_a p
 template <int NG>
 __global__ void __launch_bounds__(256) k_lp_cg_dir(int64_t npairs, int N, const double* __restrict__ beta,
                                                   const float* __restrict__ z, float* __restrict__ p) {
@@ -664,27 +615,9 @@ void lp_update_bjacobi(cudaStream_t st, int ne, int N, int Ng, const double* alp
   }
 }
 
-// out = float(coef * Sum_b M[a][b] in[b])   (time mixing + conversion)
-__global__ void k_lp_from64(int64_t ne, int N, int Ng, const double* __restrict__ M, double coef,
-                            const double* __restrict__ in, float* __restrict__ out) {
-  const int Nst = N * Ng;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < ne * N; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = (uint32_t)e / (uint32_t)N;
-    const int k = (int)(e - i * N);
-    for (int a = 0; a < Ng; ++a) {
-      double s = 0.0;
-      for (int b = 0; b < Ng; ++b) s = fma(M[a * Ng + b], in[i * Nst + b * N + k], s);
-      out[i * Nst + a * N + k] = (float)(coef * s);
-    }
-  }
-}
 __global__ void k_lp_accum(int64_t n, double scale, const float* __restrict__ d, double* __restrict__ x) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
     x[e] = fma(scale, (double)d[e], x[e]);
-}
-__global__ void k_lp_scale(int64_t n, float s, float* __restrict__ p) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    p[e] *= s;
 }
 __global__ void k_lp_f32s(int64_t n, double sc, const double* __restrict__ in, float* __restrict__ out) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
@@ -697,15 +630,6 @@ __global__ void k_lp_f32(int64_t n, const double* __restrict__ in, float* __rest
 
 LpKernels lp_kernels() {
   LpKernels k;
-  k.coldot = [](cudaStream_t st, int64_t n, int N, int Ng, const float* x, const float* y, double* part) {
-    k_lp_coldot<<<kLpBlocks, 256, 0, st>>>(n / ((int64_t)N * Ng), N, Ng, x, y, part);
-  };
-  k.update = [](cudaStream_t st, int64_t ne, int N, int Ng, const double* alpha, float* x, float* r, const float* p,
-                const float* q, const double* Tp, double* part, int want) {
-    LpTp t{};
-    for (int c = 0; c < Ng * Ng; ++c) t.v[c] = (float)Tp[c];
-    k_lp_cg_update<<<kLpBlocks, 256, 0, st>>>(ne, N, Ng, alpha, x, r, p, q, t, part, want);
-  };
   k.dir = [](cudaStream_t st, int64_t n, int N, int Ng, const double* beta, const float* z, float* p) {
     const int64_t np = n / Ng;
     const int grid = (int)std::min<int64_t>(kLpBlocks, (np + 255) / 256);
@@ -727,14 +651,10 @@ LpKernels lp_kernels() {
       default: k_lp_bjacobi<0><<<lp_partial_blocks(ne, N), 256, smem, st>>>(ne, N, Ng, Binv, r, z, part); break;
     }
   };
-  k.from64 = [](cudaStream_t st, int64_t ne, int N, int Ng, const double* Mdev, double coef, const double* in, float* out) {
-    k_lp_from64<<<kLpBlocks, 256, 0, st>>>(ne, N, Ng, Mdev, coef, in, out);
-  };
   k.accum = [](cudaStream_t st, int64_t n, double scale, const float* d, double* x) {
     k_lp_accum<<<kLpBlocks, 256, 0, st>>>(n, scale, d, x);
   };
   k.f32 = [](cudaStream_t st, int64_t n, const double* in, float* out) { k_lp_f32<<<kLpBlocks, 256, 0, st>>>(n, in, out); };
-  k.scale = [](cudaStream_t st, int64_t n, float s, float* p) { k_lp_scale<<<kLpBlocks, 256, 0, st>>>(n, s, p); };
   k.f32s = [](cudaStream_t st, int64_t n, double sc, const double* in, float* out) {
     k_lp_f32s<<<kLpBlocks, 256, 0, st>>>(n, sc, in, out);
   };

@@ -765,9 +765,12 @@ static WarpKernel<W> warp_kernel(const stdg_solver* s) {
   switch (s->N) {
     case 10: return k_apply_warp<W, NG, 10>;
     case 20: return k_apply_warp<W, NG, 20>;
-    case 35: return k_apply_warp<W, NG, 35>;
+    case 35:
+      if constexpr (W::kPlanes == 2 || sizeof(typename W::TB) == 2) return k_apply_warp<W, NG, 35>;
+      else break;                                 // cta_serves at every size
     default: return k_apply_warp<W, NG, 0>;
   }
+  return nullptr;
 }
 
 // Launch shape (warps per CTA, persistent grid) from the occupancy of this layout; sets the

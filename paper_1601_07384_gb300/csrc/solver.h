@@ -75,7 +75,6 @@ struct stdg_solver {
   double *opdot = nullptr;                    // per-block p.q partials of the binary32 operator launch
   float *lpBinv = nullptr;                    // block-Jacobi inverses in binary32
   float *fr = nullptr, *fp = nullptr, *fq = nullptr, *fz = nullptr, *fx = nullptr, *fb = nullptr;
-  double* dmix = nullptr;                     // device copy of K (time mixing)
   int* derr = nullptr;                        // device error word (bounded waits)
   // state
   double *P = nullptr, *V = nullptr;
@@ -158,15 +157,10 @@ inline FaceOps face_ops(const stdg_solver* s) {
 }
 // binary32 Krylov kernels (lowprec.cu), exposed as launch functions
 struct LpKernels {
-  void (*coldot)(cudaStream_t, int64_t, int, int, const float*, const float*, double*);
-  void (*update)(cudaStream_t, int64_t, int, int, const double*, float*, float*, const float*, const float*,
-                 const double*, double*, int);
   void (*dir)(cudaStream_t, int64_t, int, int, const double*, const float*, float*);
   void (*bjacobi)(cudaStream_t, int, int, int, const float*, const float*, float*, double*);
-  void (*from64)(cudaStream_t, int64_t, int, int, const double*, double, const double*, float*);
   void (*accum)(cudaStream_t, int64_t, double, const float*, double*);
   void (*f32)(cudaStream_t, int64_t, const double*, float*);
-  void (*scale)(cudaStream_t, int64_t, float, float*);
   void (*f32s)(cudaStream_t, int64_t, double, const double*, float*);
 };
 LpKernels lp_kernels();
