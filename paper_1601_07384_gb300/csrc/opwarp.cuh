@@ -226,7 +226,13 @@ __global__ void __launch_bounds__(128, 1) k_apply_warp(WarpArgs a, const typenam
       gf_c = gf_n; gn_c = gn_n;
       if (inx + nw < a.ne) { gf_n = a.gface[inx + nw]; gn_n = a.gnbr[inx + nw]; }
     }
-    if (warp_wait_gave_up(&bar[st], (uint32_t)((it / S) & 1), kWarpSpin)) { abort = true; break; }
+    {                                             // warp_wait_gave_up written out: as a call it takes 26 registers
+      long spins = 0;                             // more at Ng = 5 (bfloat16, N = 20: 170 -> 196), and fewer warps fit
+      const uint32_t par = (uint32_t)((it / S) & 1);
+      while (!mbar_wait_hint(&bar[st], par))
+        if (++spins > kWarpSpin) { abort = true; break; }
+    }
+    if (__any_sync(0xffffffffu, abort)) { abort = true; break; }
     __syncwarp();
     if (kPrefetch && lane == 0 && i + S * nw < a.ne) {   // the blocks after the next staged tet: towards L2
       const int ip = i + S * nw;
