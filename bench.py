@@ -575,8 +575,9 @@ def main():
     out = {
         "metric": METRIC, "value": s_per_step * 1.0, "unit": "s/step", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": s_per_step * 1e3, "higher_is_better": False, "scaling": "weak",
-        "vs_baseline": None, "dtype": {"fp64": "f64", "df32": "f64 (products from fp32 pairs)",
-                                       "mixed_f32": "f64 outer (pair products) / f32 inner", "mixed_bf16": "f64 outer (pair products) / bf16 inner"}[args.precision],
+        "vs_baseline": None, "dtype": {"fp64": "f64", "df32": "f64 (fixed-point products)",
+                                       "mixed_f32": "f64 outer (fixed-point products) / f32 inner",
+                                       "mixed_bf16": "f64 outer (fixed-point products) / bf16 inner"}[args.precision],
         "data": "synthetic",
         "config": {"workload": workload_name(w) + (f", theta={args.theta}" if args.theta != 1.0 else "")
                    + (f" (dt overridden to {w['dt']})" if args.dt > 0 else ""),

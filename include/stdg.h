@@ -246,7 +246,8 @@ typedef struct {
  * orthonormal dual basis, Q_{i,j} (Eq. MD_6, spatial part), M_{i,j} (Eq. vis3), and the
  * assembled five-point spatial blocks B_i and A_{l r} of Sum_j D M^-1 Q (Eq. CS_19).
  * cuda_stream may be NULL (default stream).  opts may be NULL (defaults).
- * Device memory: ~ (ne + nf) * N^2 * 8 * 4 bytes + nf * N^2 * 8 * 9 bytes. */
+ * Device memory: about 8 bytes x ((10 nf + 2 ne) N^2 + (6 nf + ne) Nst): blocks, state, and room for the limbs of
+ * the products' input vectors (3 nf Nst entries). */
 stdg_status stdg_solver_create(const stdg_mesh* mesh, const stdg_ref* ref, double dt,
                                const stdg_solver_options* opts, void* cuda_stream,
                                stdg_solver** out);
@@ -459,7 +460,7 @@ typedef struct {
   int64_t kernel_launches;   /* CUDA kernels this library launched since stdg_profile      */
   int64_t operator_launches; /* five-point operator launches (pressure and viscous)        */
   double operator_ms;        /* summed CUDA-event time of the operator launches (enabled)  */
-  int64_t kind_launches[4];  /* timed operator launches by kernel: [0] binary64 blocks,     */
+  int64_t kind_launches[4];  /* timed operator launches by kernel: [0] fixed-point blocks,  */
   double kind_ms[4];         /* [1] binary32-pair blocks, [2] binary32, [3] bfloat16 blocks */
   double phase_ms[8];        /* stdg_step by phase (CUDA events, enabled): [0] slab setup
                                 (averages, boundary data, trace), [1] averaging and Lambda,

@@ -1265,9 +1265,9 @@ static stdg_status solve_mixed(stdg_solver* s, const double* b, double* x, doubl
     rfull = std::sqrt(s->hostbuf[880 + Ng]);
     if (!std::isfinite(rfull)) { set_error("mixed solve: non-finite residual"); return STDG_ENAN; }
     if (rfull <= tol * bn || rdec == 0.0) {
-      // the recurrence says converged: evaluate b - A x with the binary64 kernel (the pair kernel's
-      // rounding, ~1e-14 of |A| |x|, can exceed tol |b|); if it misses the tolerance, continue from
-      // that residual with a fresh set of directions (at most 3 times)
+      // the recurrence says converged: evaluate b - A x with the fixed-point kernel (the recurrence drifts by
+      // rounding, and the pair kernels' own, ~1e-14 of |A| |x|, can exceed tol |b|); if it misses the tolerance,
+      // continue from that residual with a fresh set of directions (at most 3 times)
       if ((e = op_apply(s, pressure_op(s, 1, 0, 1.0, -1.0), x, s->kq, true)) != STDG_OK) return e;
       k_scale_copy<<<rb, kRedThreads, 0, s->stream>>>(n, b, nullptr, 1, s->kq);   // kq = b - A x
       ++s->nlaunch;
