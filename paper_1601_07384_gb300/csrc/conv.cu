@@ -15,10 +15,10 @@
 //    Jacobian are applied to the moments: 130 + 31 instead of 540;
 //  * a trace lies in P_p of the triangle (15 functions): restricted there once, evaluated at the 49 points
 //    with 15 terms instead of 35, once per face for both tets, and the flux tested against 15 functions.
-// In sum 560.  Bound: issue and latency at 25 to 30 % occupancy (the sums of a point fill the registers).
-// Measured, one kernel per tet -> these two: 13,182 tets, p = 3, p_t = 1, 4.19 -> 0.70 ms (faces 0.38, tets 0.33); 10,368
-// tets, p = p_t = 4, 10.0 -> 3.7 ms (1.3 and 2.4).  The face kernel spent 70 % of the binary64 pipe on splitting the
-// velocities and on the square roots (0.51 ms): both are done without it now (pair_split_int, pair_sqrt).  Threads
+// In sum 560.  Bound: issue and latency with 24 to 27 % of the warps (the sums of a point fill the registers).
+// Measured, one kernel per tet -> these two: 13,182 tets, p = 3, p_t = 1, 4.19 -> 0.73 ms (faces 0.39, tets 0.34); 10,368
+// tets, p = p_t = 4, 10.0 -> 3.6 ms (1.2 and 2.4).  The face kernel kept 70 % of the binary64 pipe busy with splitting
+// the velocities and with the square roots (0.51 ms); without them (pair_split_int, pair_sqrt) 51 %: conversions.  Threads
 // own quadrature points for the evaluation (all columns of a point in registers, the basis table
 // coalesced over the points), and outputs for the tests; all pair
 // products run two at a time in packed binary32 operations.
