@@ -97,9 +97,10 @@ struct ConvDim {
   // Sums of few terms add more rounding than the shorter sums save: fine sums for the traces, moments and outputs at
   // p = 1 and for the moments at p = 2.  Relative rms error against binary64 at p_t = 0, a kernel per tet that sums
   // over the points -> plain sums here -> as built: p = 1 5.1e-15 -> 6.6e-15 -> 4.5e-15, p = 2 1.0e-14 -> 9.3e-15 ->
-  // 7.6e-15, p = 3 2.0e-14 -> 1.5e-14 -> 1.4e-14, p = 4 2.4e-14 -> 2.1e-14 -> 2.0e-14; with random coefficients of
-  // order 1, plain sums were also worse at p = 2 (8.0e-15 -> 8.2e-15 -> 6.5e-15).  Cost at p_t = 0: 82,944 tets,
-  // p = 1, 206 -> 228 us; 34,992 tets, p = 2, 256 -> 275 us; at p = 3 and 4 below 1 %.
+  // 7.9e-15, p = 3 2.0e-14 -> 1.5e-14 -> 1.4e-14, p = 4 2.4e-14 -> 2.1e-14 -> 2.0e-14; with random coefficients of
+  // order 1, plain sums were also worse at p = 2 (8.0e-15 -> 8.2e-15 -> 7.3e-15).  Cost at p_t = 0: 82,944 tets,
+  // p = 1, 206 -> 218 us; 34,992 tets, p = 2, 256 -> 267 us; at p = 3 and 4 below 1 %.  (Fine sums that keep the
+  // rounding of c's two parts apart: 4.0e-15 and 227 us at p = 1.)
   static constexpr bool FINE = P == 1, FINE_M = P <= 2;
   // faces per CTA of 256 threads: all points of a face side by side
   static constexpr int kFT = 256, FB = kFT / NF;

@@ -85,18 +85,17 @@ __device__ __forceinline__ void pair_fma2(float2 ah2, float2 nah2, float2 al2, f
 }
 
 // The same with the error part negated, nc, and the rounding errors of its additions collected in d: the sum
-// s - nc - d is accurate to the rounding of the single terms, at twice the operations
+// s - nc - d is accurate to the rounding of the single terms, at one and a half times the operations
 __device__ __forceinline__ void pair_fma2(float2 ah2, float2 nah2, float2 al2, float2 bh2, float2 bl2, float2& s,
                                           float2& nc, float2& d) {
   const float2 pn = __fmul2_rn(nah2, bh2);
   float2 e = __ffma2_rn(ah2, bh2, pn);
   e = __ffma2_rn(al2, bh2, e);
   e = __ffma2_rn(ah2, bl2, e);
-  float2 s2, err, n1, n2, d1, d2;
+  float2 s2, err, n2, dn;
   df_two_diff2(s, pn, s2, err);
-  df_two_diff2(nc, err, n1, d1);
-  df_two_diff2(n1, e, n2, d2);
-  d = __fadd2_rn(d, __fadd2_rn(d1, d2));
+  df_two_diff2(nc, __fadd2_rn(err, e), n2, dn);
+  d = __fadd2_rn(d, dn);
   s = s2;
   nc = n2;
 }
